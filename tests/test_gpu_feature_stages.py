@@ -1,0 +1,98 @@
+"""The separate feature stages at the edges of their tiles: cepstra, mean and variance,
+filterbank on given power spectra -- against the fp64 checker."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1912_11040_b200 import binding, synth
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -24
+
+
+def context(B, n_mel, n_fft=512):
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=n_fft, n_mel=n_mel, f_lo=0.0, f_hi=8000.0,
+                            rir_taps=64, max_order=1, max_sources=1, frac_half_width=40, sound_speed=343.0,
+                            log_floor=1e-7, pad_value=-3.5, compression=binding.COMPRESS_LOG, max_batch=B,
+                            max_samples=16000, host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0,
+                            host_rows=0)
+    return binding.AugContext(cfg)
+
+
+def draw(B, T_max, D, seed):
+    rng = np.random.default_rng(seed)
+    x = (rng.standard_normal((B, T_max, D)) * 2.0 - 5.0).astype(np.float32)
+    counts = rng.integers(0, T_max + 1, B).astype(np.int32)
+    counts[0] = T_max
+    if B > 1:
+        counts[1] = 0
+    return x, counts
+
+
+# tile edges (128 frames), odd band counts, more than one round of 16 coefficients, one band
+@pytest.mark.parametrize("T_max,M,n_cep", [(1, 40, 13), (127, 80, 13), (128, 23, 23), (129, 128, 128),
+                                           (300, 64, 17), (65, 1, 1), (257, 40, 16)])
+def test_mfcc_tiles(T_max, M, n_cep):
+    import torch
+    B = 3
+    x, counts = draw(B, T_max, M, T_max + M)
+    out = torch.full((B, T_max, n_cep), float("nan"), device="cuda")
+    ctx = context(B, M)
+    ctx.feat_mfcc(torch.from_numpy(x).cuda(), torch.from_numpy(counts).cuda(), B, T_max, n_cep, out)
+    got = out.cpu().numpy()
+    for b in range(B):
+        T = counts[b]
+        assert np.all(got[b, T:] == -3.5)
+        if T:
+            # M products and sums of fp32 numbers, basis values off by up to 4 ulp of an angle of M pi
+            bound = (M + 4 + 4 * np.pi * M) * EPS * np.sqrt(2.0 / M) * np.abs(x[b, :T]).sum(1, keepdims=True)
+            assert np.all(np.abs(got[b, :T] - oracle.mfcc(x[b, :T], n_cep)) <= bound)
+
+
+# one column, columns that do not fill the CTA, rows of 16-byte multiples, more columns than a round
+@pytest.mark.parametrize("T_max,D", [(1, 1), (5, 3), (33, 80), (700, 23), (97, 256), (40, 300), (9, 1028),
+                                     (3001, 4)])
+def test_mean_var_shapes(T_max, D):
+    import torch
+    B = 3
+    x, counts = draw(B, T_max, D, T_max + D)
+    mean = torch.full((B, D), float("nan"), device="cuda")
+    var = torch.full_like(mean, float("nan"))
+    context(B, 40).feat_mean_var(torch.from_numpy(x).cuda(), torch.from_numpy(counts).cuda(), B, T_max, D, mean, var)
+    mean, var = mean.cpu().numpy(), var.cpu().numpy()
+    for b in range(B):
+        T = counts[b]
+        if T == 0:
+            assert not mean[b].any() and not var[b].any()
+            continue
+        y = x[b, :T].astype(np.float64)
+        mu = y.mean(0)
+        # fp64 sums, one rounding to fp32; the variance is a difference of fp64 sums of about mu^2 + var
+        assert np.all(np.abs(mean[b] - mu) <= 2 * EPS * np.abs(mu))
+        vr = y.var(0)
+        assert np.all(np.abs(var[b] - vr) <= 2 * EPS * vr + 4 * T * 2.0 ** -53 * (mu * mu + vr))
+
+
+# rows that start at any offset from a 16-byte boundary, tiles of 32 frames, widest and narrowest bands
+@pytest.mark.parametrize("T_max,M,n_fft", [(1, 40, 512), (31, 80, 512), (33, 128, 1024), (66, 1, 512), (35, 23, 1024)])
+def test_logmel_tiles(T_max, M, n_fft):
+    import torch
+    B = 3
+    rng = np.random.default_rng(T_max + M)
+    K = n_fft // 2 + 1
+    P = np.exp(rng.standard_normal((B, T_max, K)) * 3.0).astype(np.float32)
+    counts = np.array([T_max, 0, T_max // 2], dtype=np.int32)
+    tab = np.zeros(B, dtype=synth.UTT_DTYPE)
+    tab["alpha"] = [1.0, 0.9, 1.13]
+    out = torch.full((B, T_max, M), float("nan"), device="cuda")
+    ctx = context(B, M, n_fft)
+    ctx.feat_vtlp_logmel(torch.from_numpy(P).cuda(), torch.from_numpy(counts).cuda(), binding.table_to_device(tab),
+                         B, T_max, out)
+    got = out.cpu().numpy()
+    for b in range(B):
+        T = counts[b]
+        assert np.all(got[b, T:] == -3.5)
+        if T:
+            ref = oracle.logmel(P[b, :T].astype(np.float64), float(tab["alpha"][b]), n_fft, M, floor=1e-7)
+            # positive terms: relative error of a sum of K of them, plus that of the logarithm
+            assert np.all(np.abs(got[b, :T] - ref) <= (K + 4) * EPS + 4 * EPS * np.abs(ref))
