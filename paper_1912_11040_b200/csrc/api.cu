@@ -556,7 +556,7 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     t1(5, sm);
     if ((rc = joined(AUG_OK)) != AUG_OK) return rc;
     t0(6, sm);
-    rc = launch_fused_features(ctx, lengths_dev, table_dev, B, feats_dev, T_max, frame_counts_dev, max_len);
+    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len);
     t1(6, sm);
     if (ev && rc == AUG_OK) ctx->ev_n++;
     return rc;

@@ -419,7 +419,10 @@ spectral_convolve_kernel(const int *__restrict__ lengths, const float *__restric
 
 // ---------------------------------------------------------------- mixing
 // g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise or with a silent side:
-// once per utterance, in fp64, after the convolution has finished the two sums.
+// once per utterance, in fp64, after the convolution has finished the two sums.  (Worked out by
+// every feature CTA instead, the chain of fp64 operations cost 13 us on 256 utterances of
+// 2-20 s where this launch costs 2.6; by the last CTA of the convolution, the fence it needs
+// cost as much.)
 __global__ void __launch_bounds__(256)
 snr_gain_kernel(const double *__restrict__ energy, const AugUttParams *__restrict__ table, int B,
                 float *__restrict__ gain) {
@@ -428,29 +431,46 @@ snr_gain_kernel(const double *__restrict__ energy, const AugUttParams *__restric
     const double es = energy[2 * utt], ev = energy[2 * utt + 1];
     float g = 0.f;
     if (table[utt].n_src > 1 && es > 0.0 && ev > 0.0)
-        g = (float)sqrt(es / (ev * pow(10.0, (double)table[utt].snr_db / 10.0)));
+        g = (float)sqrt(es / (ev * exp10((double)table[utt].snr_db / 10.0)));
     gain[utt] = g;
 }
 
+// A pass over y_s and v, bound by memory: 4096 samples per CTA, eight 128-bit loads in flight per
+// thread.
+constexpr int MIX_GROUPS = 4;              // 128-bit groups per thread
 __global__ void __launch_bounds__(256)
 mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t ws_stride,
            const float *__restrict__ gain, const int *__restrict__ lengths,
            float *__restrict__ out, int64_t out_stride, int n_cap) {
-    const int utt = blockIdx.y;
+    const int utt = blockIdx.y, tid = threadIdx.x;
     const int N = min(max(lengths[utt], 0), n_cap);
-    const int i = (blockIdx.x * 256 + threadIdx.x) * 4;
-    if (i >= N) return;
+    const int i0 = blockIdx.x * (MIX_GROUPS * 1024) + 4 * tid;
+    if (blockIdx.x * (MIX_GROUPS * 1024) >= N) return;
+    const float *a = ys + (int64_t)utt * ws_stride;
+    const float *b = vv + (int64_t)utt * ws_stride;
+    float *o = out + (int64_t)utt * out_stride;
+    float4 x[MIX_GROUPS], y[MIX_GROUPS];
+#pragma unroll
+    for (int u = 0; u < MIX_GROUPS; ++u) {
+        const int i = i0 + 1024 * u;           // (workspace rows are allocated up to a multiple of 4)
+        if (i < N) {
+            x[u] = __ldg(reinterpret_cast<const float4 *>(a + i));
+            y[u] = __ldg(reinterpret_cast<const float4 *>(b + i));
+        }
+    }
     const float g = gain[utt];
-    const float *a = ys + (int64_t)utt * ws_stride + i;
-    const float *b = vv + (int64_t)utt * ws_stride + i;
-    float *o = out + (int64_t)utt * out_stride + i;
-    if (i + 3 < N) {
-        const float4 x = *reinterpret_cast<const float4 *>(a);
-        const float4 y = *reinterpret_cast<const float4 *>(b);
-        *reinterpret_cast<float4 *>(o) =
-            make_float4(fmaf(g, y.x, x.x), fmaf(g, y.y, x.y), fmaf(g, y.z, x.z), fmaf(g, y.w, x.w));
-    } else {
-        for (int j = 0; j < 4 && i + j < N; ++j) o[j] = fmaf(g, b[j], a[j]);
+#pragma unroll
+    for (int u = 0; u < MIX_GROUPS; ++u) {
+        const int i = i0 + 1024 * u;
+        const float4 z = make_float4(fmaf(g, y[u].x, x[u].x), fmaf(g, y[u].y, x[u].y), fmaf(g, y[u].z, x[u].z),
+                                     fmaf(g, y[u].w, x[u].w));
+        if (i + 3 < N) {
+            *reinterpret_cast<float4 *>(o + i) = z;
+        } else if (i < N) {
+            o[i] = z.x;
+            if (i + 1 < N) o[i + 1] = z.y;
+            if (i + 2 < N) o[i + 2] = z.z;
+        }
     }
 }
 
@@ -1101,7 +1121,7 @@ int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, con
 int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
                float *wave_out, int64_t out_stride) {
     if (max_len <= 0) return AUG_OK;
-    dim3 grid((max_len + 1023) / 1024, B);
+    dim3 grid((max_len + MIX_GROUPS * 1024 - 1) / (MIX_GROUPS * 1024), B);
     mix_kernel<<<grid, 256, 0, ctx->stream>>>(ctx->ys, ctx->vv, ctx->ws_stride, ctx->gain, lengths,
                                               wave_out, out_stride, max_len);
     AUG_CUDA_OK(cudaGetLastError());
