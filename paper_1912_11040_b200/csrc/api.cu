@@ -106,7 +106,7 @@ int check_config(const AugConfig *c) {
 struct Layout {
     int n_part, route, n_bins, t_cap, nblk_cap;
     int64_t ws_stride;
-    int64_t off_xspec, off_park, off_park_flags;
+    int64_t off_xspec, off_park, off_park_flags, off_plans, off_units;
     int64_t off_tw, off_rir, off_hspec, off_ys, off_vv, off_energy, off_leff, off_gain, off_melw, off_melstart,
         off_status, off_warped, off_vtlp_tab, off_st_speech, off_st_bank, off_st_table, off_st_lengths,
         off_st_feats, off_st_counts, total;
@@ -127,14 +127,18 @@ Layout make_layout(const AugConfig &c) {
     l.off_hspec = take(sizeof(float2) * B * S * (l.route == aug::ROUTE_FUSED_8192 ? 2 : l.n_part) * aug::CONV_N2);
     l.nblk_cap = (c.max_samples + aug::CONV_BLK - 1) / aug::CONV_BLK;
     l.off_xspec = l.route == aug::ROUTE_STORED ? take(sizeof(float2) * B * S * l.nblk_cap * aug::CONV_N2) : -1;
-    // parking slots of the fused route, three per multiprocessor, when a row can have several noises
+    // parking slots of the fused route, when a row can have several noises
     const bool parks = c.max_sources >= 3;    // (long-response contexts use the fused route for short responses)
-    l.off_park = parks ? take(sizeof(float2) * (int64_t)aug::PARK_SMS * aug::PARK_PER_SM * 2 * aug::CONV_N2) : -1;
-    l.off_park_flags = parks ? take(sizeof(int) * (int64_t)aug::PARK_SMS * aug::PARK_PER_SM) : -1;
+    l.off_park = parks ? take(sizeof(float2) * (int64_t)aug::PARK_SLOTS * 2 * aug::CONV_N2) : -1;
+    l.off_park_flags = parks ? take(sizeof(int) * aug::PARK_SLOTS) : -1;
+    // its list of work: two outputs of every block, blocks as short as min(rir_taps, 8192) taps make them
+    l.off_plans = take((int64_t)aug::PLAN_BYTES * B);
+    const int ob = (4 * aug::CONV_BLK - std::min(c.rir_taps, 2 * aug::CONV_BLK) + 1) & ~3;
+    l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + ob - 1) / ob));
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take(sizeof(double) * 2 * B);
-    l.off_leff = take(sizeof(int) * (B + 1));
+    l.off_leff = take(sizeof(int) * (B + 3));
     l.off_gain = take(sizeof(float) * B);
     l.off_melw = take(sizeof(aug::MelBin) * B * l.n_bins);
     l.off_melstart = take(sizeof(int) * B * (c.n_mel + 2));
@@ -262,9 +266,10 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     ctx->hspec = reinterpret_cast<float2 *>(base + l.off_hspec);
     ctx->nblk_cap = l.nblk_cap;
     ctx->xspec = l.off_xspec >= 0 ? reinterpret_cast<float2 *>(base + l.off_xspec) : nullptr;
-    ctx->park = l.off_park >= 0 ? reinterpret_cast<float2 *>(base + l.off_park) : nullptr;
+    ctx->park = l.off_park >= 0 ? reinterpret_cast<float4 *>(base + l.off_park) : nullptr;
     ctx->park_flags = l.off_park_flags >= 0 ? reinterpret_cast<int *>(base + l.off_park_flags) : nullptr;
-    ctx->n_sm = aug::PARK_SMS;
+    ctx->plans = base + l.off_plans;
+    ctx->units = base + l.off_units;
     ctx->ys = reinterpret_cast<float *>(base + l.off_ys);
     ctx->vv = reinterpret_cast<float *>(base + l.off_vv);
     ctx->energy = reinterpret_cast<double *>(base + l.off_energy);
@@ -332,7 +337,7 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     }
     const int st0[2] = {-1, 0};
     if (ctx->park_flags &&
-        cudaMemsetAsync(ctx->park_flags, 0, sizeof(int) * aug::PARK_SMS * aug::PARK_PER_SM, ctx->stream) !=
+        cudaMemsetAsync(ctx->park_flags, 0, sizeof(int) * aug::PARK_SLOTS, ctx->stream) !=
             cudaSuccess) {
         if (ctx->leff_seen) cudaFreeHost(ctx->leff_seen);
         cudaFree(ctx->ws_base);
@@ -757,7 +762,7 @@ int aug_hold_parking_slots(AugCtx *ctx, int hold) {
     if (!ctx) return AUG_EINVAL;
     if (!ctx->park_flags) return AUG_OK;   // this context has no parking area
     // all slots marked taken: every CTA then sums its noise sources in the time domain
-    std::vector<int> v((size_t)aug::PARK_SMS * aug::PARK_PER_SM, hold ? 1 : 0);
+    std::vector<int> v((size_t)aug::PARK_SLOTS, hold ? 1 : 0);
     AUG_CUDA_OK(cudaStreamSynchronize(ctx->stream));
     AUG_CUDA_OK(cudaMemcpyAsync(ctx->park_flags, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice,
                                 ctx->stream));

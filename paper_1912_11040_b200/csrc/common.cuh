@@ -12,8 +12,8 @@ namespace aug {
 constexpr int CONV_BLK = 4096;          // output samples per convolution block
 constexpr int CONV_F = 2 * CONV_BLK;    // real FFT size of one block
 constexpr int CONV_N2 = CONV_F / 2;     // complex FFT size
-constexpr int PARK_SMS = 160;       // multiprocessors that get parking slots in the fused convolution
-constexpr int PARK_PER_SM = 3;      // slots per multiprocessor = resident CTAs of that kernel
+constexpr int PARK_SLOTS = 320;     // parking slots of the fused convolution = most CTAs it runs with
+constexpr int PLAN_BYTES = 96;      // per utterance, see conv.cu
 constexpr int MAX_TAPS = 24576;
 constexpr int MAX_ORDER = 32;
 constexpr int MAX_HALF_W = 47;
@@ -61,15 +61,16 @@ struct AugCtx {
     float2 *hspec;         // [max_batch][max_sources][n_part][CONV_N2]
     float2 *xspec;         // [max_batch][max_sources][nblk_cap][CONV_N2]; NULL unless route == ROUTE_STORED
     int nblk_cap;          // blocks of an utterance of max_samples
-    float2 *park;          // [PARK_SMS * PARK_PER_SM][8192] products of noise sources waiting for the last one; NULL if unused
-    int *park_flags;       // [PARK_SMS * PARK_PER_SM] 1 = slot taken
-    int n_sm;              // multiprocessors with slots (PARK_SMS); CTAs on others sum in the time domain
+    float4 *park;          // [PARK_SLOTS][4096] products of noise sources waiting for the last one; NULL if unused
+    int *park_flags;       // [PARK_SLOTS] 1 = slot held: that CTA sums in the time domain
+    void *plans;           // [max_batch][PLAN_BYTES] what the fused convolution has to know of an utterance
+    void *units;           // its list of work
     float *warped;         // [max_batch][ws_stride] speech after the waveform warp; NULL unless cfg.vtlp_win
     void *vtlp_tab;        // [max_batch][513] lower source bin (int), then [max_batch][513] fraction (float)
     float *ys;             // [max_batch][ws_stride]
     float *vv;             // [max_batch][ws_stride]
     double *energy;        // [max_batch][2]
-    int *leff;             // [max_batch + 1] (last entry: largest over the batch)
+    int *leff;             // [max_batch + 3] (then: largest over the batch, units of work listed, drawn)
     int *leff_seen;        // pinned host copy of that last entry from an earlier call (long-response contexts)
     int stored_only;       // this call launches the stored-spectra kernels alone taps up to the last non-zero one, largest over the utterance's sources
     float *gain;           // [max_batch] noise gain g for the requested SNR

@@ -42,8 +42,11 @@
 // the bin pairs (k, F/2-k), k = t + 256 q.  Spectra are stored as F/2 complex numbers
 // with the two real bins (0 and F/2) packed into slot 0; the partition spectra of
 // the responses carry the noise weight and the 1/F of the inverse.
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft.cuh"
+#include "fft_pair.cuh"
 
 namespace {
 
@@ -57,7 +60,7 @@ constexpr int SM_POINTS = padded_points(N2);
 #ifndef CONV_MINB
 #define CONV_MINB 3                  // CTAs per SM the register budget is set for
 #endif
-static_assert(CONV_MINB == aug::PARK_PER_SM, "one parking slot per resident CTA of the fused convolution");
+constexpr int FUSED_MINB = 2;          // CTAs per SM of the fused convolution
 
 __device__ __forceinline__ void fft4096_from_regs(float2 (*v)[E], float2 *s, int t,
                                                   const float2 *__restrict__ tw) {
@@ -120,7 +123,7 @@ __device__ __forceinline__ void mac_pair(float2 &acc_a, float2 &acc_b, float2 a,
 // 2*BLK input samples starting at `base` as 16 (even, odd) pairs per thread in the
 // order the first FFT pass wants them.  Speech reads x[i]; a noise source reads
 // its stretch of the bank end to end (x[i mod nlen]).  Outside [0, N): zero.
-__device__ __forceinline__ void load_segment(float2 (*v)[E], const float *__restrict__ x, bool looped,
+__device__ __forceinline__ void load_block(float2 (*v)[E], const float *__restrict__ x, bool looped,
                                              int nlen, int base, int N, int t) {
     // A segment inside the utterance, and for a looped stretch inside one period of it on
     // 8-byte boundaries, needs no test per pair (the same for the whole CTA).
@@ -352,7 +355,7 @@ block_spectra_kernel(const float *__restrict__ speech, int64_t stride,
         return;
     }
     float2 v[1][E];
-    load_segment(v, x, s != 0, nlen, (b - 1) * BLK, N, t);
+    load_block(v, x, s != 0, nlen, (b - 1) * BLK, N, t);
     fft4096_from_regs(v, sm, t, tw);
     float2 *out = xspec + (((int64_t)utt * S_max + s) * nblk_cap + b) * N2;
 #pragma unroll
@@ -475,548 +478,516 @@ mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t w
 }
 
 // ================================================================ 8192-sample blocks
-// Impulse responses of 4097..8192 taps fit one partition of a 16384-point real
-// transform, so a CTA can do the whole block -- forward, multiply, inverse --
-// without any stored spectra.  The 8192-point complex transform of the (even, odd)
-// pairs is run as two 4096-point transforms (pairs 0, 2, 4, ... in buffer A, pairs
-// 1, 3, 5, ... in buffer B: one 128-bit load feeds one point of each) joined by a
-// radix-2 step.  Thread t owns, for k = t + 256 q < 2048, slots k and 4096-k of
-// both buffers; from those four numbers it forms bins k, 8192-k, 4096-k and
-// 4096+k of the real signal's spectrum, multiplies them with the response's
-// bins, and folds the products back into the two half-size inputs of the inverse
-// transform -- in place, with no exchange between threads.  Spectra are stored as
-// 8192 complex numbers, bins 0 and 8192 (both real) packed into slot 0.
-constexpr int BLK2 = 2 * BLK;          // output samples per block
+// Impulse responses of up to 8192 taps fit one partition of a 16384-point real
+// transform, so a CTA can do a whole block of one output -- forward, multiply, inverse --
+// without any stored spectra.  The even and the odd samples of a segment are two real
+// sequences of 8192 points, each a complex transform of 4096 points on pairs of its
+// samples: four consecutive samples x0..x3 are one point of both, (x0, x1) their real and
+// (x2, x3) their imaginary parts, which is the layout the packed arithmetic of
+// fft_pair.cuh wants.  After the forward transform thread t holds, for r < 8, the
+// frequencies k = j + 256 r and (from its partner lane) 4096 - k of both; from these it forms
+// the bins k, 8192-k, 4096-k and 4096+k of the segment's spectrum, multiplies them with the
+// response's and folds the products back, all in registers.  The response's spectra are
+// stored in the order the threads read them.
+constexpr int BLK2 = 2 * BLK;          // most taps; output samples per block are F2 - taps + 1
 constexpr int F2 = 2 * BLK2;           // real transform size
-constexpr int NB2 = F2 / 2;            // complex bins stored per spectrum
-constexpr int NQ2 = N2 / 2 / CT;       // slot pairs per thread and buffer
+constexpr int NB2 = F2 / 2;            // complex numbers stored per spectrum
+constexpr int CF = fftpair::THREADS;   // threads per CTA
+constexpr int NP2 = N2 / CF;           // points per thread
+constexpr int NS2 = NP2 / 2;           // slots (k, 4096-k) per thread
+using fftpair::C2;
+using fftpair::u64;
 
-// 2*BLK2 input samples starting at `base`: thread t gets samples
-// base + 4 (t + 256 r) + {0,1} as point r of buffer A and + {2,3} as point r of B.
-__device__ __forceinline__ void load_segment4(float2 (*va)[E], float2 (*vb)[E],
-                                              const float *__restrict__ x, bool looped, int nlen,
-                                              int base, int N, int t, const float *xend) {
+// Asynchronous copy global -> shared; `bytes` are read, the rest is zero.
+__device__ __forceinline__ void copy4_async(float *dst_smem, const float *src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst_smem)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// F2 input samples starting at `base`: thread t gets samples base + 4 (t + 256 r) + {0, 1} and
+// + {2, 3} as the real and imaginary parts of point r.  Speech reads x[i]; a noise source
+// reads its stretch of the bank end to end (x[i mod nlen]).  Outside [0, N): zero.  The
+// exchange buffer must be free.
+__device__ __forceinline__ void load_segment(C2 *v, fftpair::Shared &sh, const float *__restrict__ x, bool looped,
+                                             int nlen, int base, int N, int t) {
     // A segment that lies inside the utterance (most do), and for a looped stretch inside one
-    // period of it on 16-byte boundaries, needs no test per group: the same for the whole CTA.
+    // period of it, is read straight into registers: the same for the whole CTA.
     if (base >= 0 && base + F2 <= N) {
-        int m0 = base;
-        bool plain = !looped;
-        if (looped && (nlen & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-            m0 = base % nlen;
-            plain = m0 + F2 <= nlen;
-        }
-        if (plain) {
-            const float4 *x4 = reinterpret_cast<const float4 *>(x + m0) + t;
+        const int m0 = looped ? base % nlen : base;
+        if (!looped || m0 + F2 <= nlen) {
+            const float *p = x + m0 + 4 * t;
+            if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
-            for (int r = 0; r < E; ++r) {
-                const float4 z = __ldg(x4 + CT * r);
-                va[0][r] = make_float2(z.x, z.y);
-                vb[0][r] = make_float2(z.z, z.w);
+                for (int r = 0; r < NP2; ++r)
+                    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];"
+                        : "=l"(v[r].re), "=l"(v[r].im)
+                        : "l"(p + 4 * CF * r));
+            } else {
+                // any other offset: single words, which the four loads of a group share in L1
+#pragma unroll
+                for (int r = 0; r < NP2; ++r) {
+                    const float *q = p + 4 * CF * r;
+                    v[r] = {fftpair::pack(__ldg(q), __ldg(q + 1)), fftpair::pack(__ldg(q + 2), __ldg(q + 3))};
+                }
             }
             return;
         }
     }
-    if (!looped) {
+    if (!looped || ((nlen & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
+        // groups of four lie on 16-byte boundaries and never wrap; rows and stretches hold whole groups
+        int i = base + 4 * t, m = i, step = 4 * CF, wrap = 0x7fffffff;
+        if (looped) {
+            m = i >= 0 ? i % nlen : (nlen - (-i) % nlen) % nlen;
+            step %= nlen;
+            wrap = nlen;
+        }
 #pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int i0 = base + 4 * (t + CT * r);
+        for (int r = 0; r < NP2; ++r) {
             float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i0 >= 0) {
-                if (i0 + 3 < N) {
-                    z = __ldg(reinterpret_cast<const float4 *>(x + i0));
-                } else {
-                    if (i0 < N) z.x = x[i0];
-                    if (i0 + 1 < N) z.y = x[i0 + 1];
-                    if (i0 + 2 < N) z.z = x[i0 + 2];
-                }
-            }
-            va[0][r] = make_float2(z.x, z.y);
-            vb[0][r] = make_float2(z.z, z.w);
+            if ((unsigned)i < (unsigned)N) z = __ldg(reinterpret_cast<const float4 *>(x + m));
+            v[r] = {fftpair::pack(z.x, i + 1 < N ? z.y : 0.f),
+                    fftpair::pack(i + 2 < N ? z.z : 0.f, i + 3 < N ? z.w : 0.f)};
+            i += 4 * CF;
+            m += step;
+            if (m >= wrap) m -= wrap;
         }
         return;
     }
-    const int first = base + 4 * t;
-    const int step = (4 * CT) % nlen;
-    int m = first >= 0 ? first % nlen : (nlen - (-first) % nlen) % nlen;
-    if ((nlen & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-        // A stretch that starts on a 16-byte boundary and whose length is a multiple
-        // of four samples never wraps inside a group of four: one 128-bit load each.
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int i0 = first + 4 * CT * r;
-            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i0 >= 0 && i0 < N) {
-                z = __ldg(reinterpret_cast<const float4 *>(x + m));
-                if (i0 + 3 >= N) {
-                    z.w = 0.f;
-                    if (i0 + 2 >= N) z.z = 0.f;
-                    if (i0 + 1 >= N) z.y = 0.f;
-                }
-            }
-            va[0][r] = make_float2(z.x, z.y);
-            vb[0][r] = make_float2(z.z, z.w);
+    // sample by sample through the exchange buffer, neighbouring threads neighbouring samples
+    {
+        __syncthreads();
+        int i = base + t, m = i >= 0 ? i % nlen : (nlen - (-i) % nlen) % nlen;
+        const int step = CF % nlen;
+        float *dst = reinterpret_cast<float *>((t & 2 ? sh.im : sh.re) + fftpair::slot(t >> 2)) + (t & 1);
+#pragma unroll 4
+        for (int r = 0; r < F2 / CF; ++r) {
+            copy4_async(dst, x + m, (unsigned)i < (unsigned)N ? 4 : 0);
+            dst += 2 * fftpair::slot(CF / 4);
+            i += CF;
             m += step;
             if (m >= nlen) m -= nlen;
         }
-        return;
+        copies_done();
+        __syncthreads();
     }
-    // Any other stretch: a group of four that does not wrap is read as the aligned
-    // 128-bit word it starts in and, if it starts a samples into that word, the next
-    // word as well (a second round, so that the first loads are all in flight
-    // together; neighbouring threads bring that word into L1).  Groups that wrap, end
-    // with the utterance or would touch bytes past the bank are read sample by sample.
-    const int m0 = m;
-    const int room = (int)min((int64_t)0x7fffffff, (int64_t)(xend - x));   // samples from x to the end of the bank
-    const int a0 = (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3);       // where in a 128-bit word x starts
-    unsigned amask = 0;                  // 2 bits per group: a, where the second round is needed
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int i0 = first + 4 * CT * r;
-        float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i0 >= 0 && i0 < N) {
-            const int a = (a0 + m) & 3;
-            if (m + 3 < nlen && i0 + 3 < N && (a == 0 || m - a + 8 <= room)) {
-                z = __ldg(reinterpret_cast<const float4 *>(x + (m - a)));
-                amask |= (unsigned)a << (2 * r);
-            } else {
-                int j = m;
-                z.x = x[j];
-                j = j + 1 == nlen ? 0 : j + 1;
-                if (i0 + 1 < N) z.y = x[j];
-                j = j + 1 == nlen ? 0 : j + 1;
-                if (i0 + 2 < N) z.z = x[j];
-                j = j + 1 == nlen ? 0 : j + 1;
-                if (i0 + 3 < N) z.w = x[j];
-            }
-        }
-        va[0][r] = make_float2(z.x, z.y);
-        vb[0][r] = make_float2(z.z, z.w);
-        m += step;
-        if (m >= nlen) m -= nlen;
-    }
-    if (__any_sync(0xffffffffu, amask != 0)) {
-        m = m0;
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int a = (int)(amask >> (2 * r)) & 3;
-            if (a) {
-                const float4 q = __ldg(reinterpret_cast<const float4 *>(x + m - a + 4));
-                const float2 lo = va[0][r], hi = vb[0][r];
-                // samples a .. a+3 of the eight in (lo, hi, q)
-                va[0][r] = a == 1 ? make_float2(lo.y, hi.x) : a == 2 ? hi : make_float2(hi.y, q.x);
-                vb[0][r] = a == 1 ? make_float2(hi.y, q.x) : a == 2 ? make_float2(q.x, q.y) : make_float2(q.y, q.z);
-            }
-            m += step;
-            if (m >= nlen) m -= nlen;
-            // four second-round loads at a time: more in flight would not fit the registers
-            if ((r & 3) == 3) asm volatile("" ::: "memory");
-        }
-    }
+    fftpair::load16<fftpair::slot(CF)>(v, sh, fftpair::slot(t));
 }
 
-// Passes two and three of both half transforms, shared by the forward and the
-// inverse direction (a real call: the kernel's instruction footprint matters).
-// On entry A is complete and visible and B at most one barrier away from it.
-// Returns with B written but not yet synchronised: the caller's barrier finishes it
-// (loads that do not depend on the transform go in front of that barrier).
-__device__ __noinline__ void fft2x4096_tail(float2 *A, float2 *B, int t, const float2 *__restrict__ tw) {
-    pass_pair<N2, E, 16, 16, 1>(A, B, t, tw, CtaSync());
-    pass_pair<N2, E, 16, 256, 16>(A, B, t, tw, CtaSync());
-}
-
-// Both half transforms of a segment held in registers; on return A and B hold the
-// 4096-point transforms of the even and odd pairs, complete and synchronised.
-__device__ __forceinline__ void fft2x4096_from_regs(float2 (*va)[E], float2 (*vb)[E], float2 *A,
-                                                    float2 *B, int t, const float2 *__restrict__ tw) {
-    pass_from_regs<N2, E, 16, 1>(va, A, t, tw);
-    pass_from_regs<N2, E, 16, 1>(vb, B, t, tw);
-    __syncthreads();
-    fft2x4096_tail(A, B, t, tw);
-}
-// (both variants leave the closing barrier to the caller)
-
-__device__ __forceinline__ void fft2x4096_in_place(float2 *A, float2 *B, int t,
-                                                   const float2 *__restrict__ tw) {
-    pass_pair<N2, E, 16, 1, 0>(A, B, t, tw, CtaSync());
-    fft2x4096_tail(A, B, t, tw);
-}
-
-// Inverse of real_split, unnormalised (twice the value): the half-size spectrum
-// at the bin pair (k, M-k) from the real signal's bins Y[k], Y[M-k]; W = W_{2M}^k.
-__device__ __forceinline__ void real_unsplit(float2 yk, float2 ym, float2 w, float2 &zk, float2 &zm) {
-    const float2 a = make_float2(yk.x + ym.x, yk.y - ym.y);          // Yk + conj Ym
-    const float2 d = make_float2(yk.x - ym.x, yk.y + ym.y);          // Yk - conj Ym
-    const float2 e = cmul(make_float2(w.y, w.x), d);                 // i conj(W) d
-    zk = make_float2(a.x + e.x, a.y + e.y);
-    const float2 e2 = cmul(make_float2(-w.y, w.x), make_float2(d.x, -d.y));   // i W conj(d)
-    zm = make_float2(a.x + e2.x, -a.y + e2.y);
-}
-
-// The four bins a thread forms for slot k (1 <= k < 2048) from the two half
-// transforms: X[k], X[8192-k], X[4096-k], X[4096+k].
-struct Quad {
-    float2 k, nk, mk, pk;
+// The four bins a thread forms from frequencies k and m = 4096-k of the two half
+// transforms, lanes (k, m):  p = X[k], conj X[m];  q = conj X[8192-k], X[4096+k].
+// Thread j = 0 has in its first slot the frequencies 0 and 2048 instead:
+// p = (X[0], Re X[4096]; X[8192], Im X[4096]), q = (X[2048], conj X[6144]).
+// All are twice the value of the transform (the factor sits in the stored responses).
+struct Bins {
+    u64 pr, pi, qr, qi;
 };
-__device__ __forceinline__ Quad quad_forward(float2 ze_k, float2 ze_m, float2 zo_k, float2 zo_m,
-                                             float2 w, float2 u) {
-    // radix-2 join: Z[k], Z[k+4096], Z[4096-k], Z[8192-k]
-    const float2 t1 = cmul(w, zo_k), t2 = cmul(cconj(w), zo_m);
-    const float2 z_k = cadd(ze_k, t1), z_pk = csub(ze_k, t1);
-    const float2 z_mk = csub(ze_m, t2), z_nk = cadd(ze_m, t2);
-    Quad x;
-    real_split(z_k, z_nk, u, x.k, x.nk);
-    real_split(z_mk, z_pk, make_float2(-u.y, -u.x), x.mk, x.pk);    // W_F^(4096-k) = -i conj(u)
-    return x;
-}
-// Products back to the inputs of the two half-size inverse transforms, real and
-// imaginary parts swapped (the forward code then computes the inverse).
-__device__ __forceinline__ void quad_inverse(const Quad &y, float2 w, float2 u, float2 &a_k,
-                                             float2 &a_m, float2 &b_k, float2 &b_m) {
-    float2 z_k, z_nk, z_mk, z_pk;
-    real_unsplit(y.k, y.nk, u, z_k, z_nk);
-    real_unsplit(y.mk, y.pk, make_float2(-u.y, -u.x), z_mk, z_pk);
-    const float2 s1 = cadd(z_k, z_pk), d1 = cmul(csub(z_k, z_pk), cconj(w));
-    const float2 s2 = cadd(z_mk, z_nk), d2 = cmul(csub(z_nk, z_mk), w);   // -(Z[4096-k]-Z[8192-k]) w
-    a_k = make_float2(s1.y, s1.x);
-    b_k = make_float2(d1.y, d1.x);
-    a_m = make_float2(s2.y, s2.x);
-    b_m = make_float2(d2.y, d2.x);
-}
+__device__ __forceinline__ u64 low2(u64 a, u64 b) { return fftpair::pack(fftpair::unpack(a).x, fftpair::unpack(b).x); }
+__device__ __forceinline__ u64 high2(u64 a, u64 b) { return fftpair::pack(fftpair::unpack(a).y, fftpair::unpack(b).y); }
 
-// Slots 0 and 2048 of both buffers (thread 0): bins 0, 8192 (packed), 4096, 2048, 6144.
-struct Edge {
-    float2 dc;       // (X[0], X[8192]), both real
-    float2 mid;      // X[4096]
-    float2 q1, q3;   // X[2048], X[6144]
+// U = exp(-2 pi i k / 16384) of slot r and, by squaring, W = exp(-2 pi i k / 8192), from
+// u = exp(-2 pi i j / 16384), k = j + 256 r
+struct SplitTwiddle {
+    u64 ur, ui;            // lanes (U^k, conj U^m), conj U^m = i U^k
+    u64 wx, wy;
+    __device__ __forceinline__ SplitTwiddle(float2 u, int r) {
+        using namespace fftpair;
+        // exp(-i pi r / 32)
+        const float cr[8] = {1.f, 0.99518472667219688624f, 0.98078528040323044913f, 0.95694033573220886494f,
+                             0.92387953251128675613f, 0.88192126434835502971f, 0.83146961230254523708f,
+                             0.77301045336273696081f};
+        const float ci[8] = {0.f, -0.09801714032956060199f, -0.19509032201612826785f, -0.29028467725446236764f,
+                             -0.38268343236508977173f, -0.47139673682599764856f, -0.55557023301960222474f,
+                             -0.63439328416364549822f};
+        const float x = r ? fmaf(u.x, cr[r], -u.y * ci[r]) : u.x, y = r ? fmaf(u.x, ci[r], u.y * cr[r]) : u.y;
+        ur = pack(x, -y);
+        ui = pack(y, x);
+        const float p = fmaf(x, x, -y * y), q = 2.f * x * y;
+        wx = both(p);
+        wy = both(q);
+    }
 };
-__device__ __forceinline__ Edge edge_forward(float2 ze0, float2 zo0, float2 zeh, float2 zoh, float2 uh) {
-    Edge x;
-    const float2 z0 = cadd(ze0, zo0), z4 = csub(ze0, zo0);
-    x.dc = make_float2(z0.x + z0.y, z0.x - z0.y);
-    x.mid = cconj(z4);
-    const float2 th = cmul_mi(zoh);                                 // W_8192^2048 = -i
-    real_split(cadd(zeh, th), csub(zeh, th), uh, x.q1, x.q3);
-    return x;
+// Spectra E, O of the even and odd samples at k and (conjugated) at m = 4096-k; then
+// X = E +- U^k O in lanes (X[k], conj X[m]).
+__device__ __forceinline__ Bins bins_forward(C2 zk, C2 zm, const SplitTwiddle &w) {
+    using namespace fftpair;
+    const u64 evr = add2(zk.re, zm.re), evi = sub2(zk.im, zm.im);
+    const u64 odr = add2(zk.im, zm.im), nodi = sub2(zk.re, zm.re);
+    const u64 wor = fma2(w.wy, nodi, mul2(w.wx, odr));
+    const u64 nwoi = sub2(mul2(w.wx, nodi), mul2(w.wy, odr));
+    const C2 ek = {add2(evr, wor), sub2(evi, nwoi)}, em = {sub2(evr, wor), add2(evi, nwoi)};
+    // lanes from (even, odd) to (k, m)
+    const u64 er = low2(ek.re, em.re), ei = low2(ek.im, em.im);
+    const u64 orr = high2(ek.re, em.re), oi = high2(ek.im, em.im);
+    const u64 tr = sub2(mul2(w.ur, orr), mul2(w.ui, oi)), ti = fma2(w.ui, orr, mul2(w.ur, oi));
+    return {add2(er, tr), add2(ei, ti), sub2(er, tr), sub2(ei, ti)};
 }
-__device__ __forceinline__ void edge_inverse(const Edge &y, float2 uh, float2 &a0, float2 &b0,
-                                             float2 &ah, float2 &bh) {
-    const float2 z0 = make_float2(y.dc.x + y.dc.y, y.dc.x - y.dc.y);
-    const float2 z4 = make_float2(2.f * y.mid.x, -2.f * y.mid.y);
-    const float2 s0 = cadd(z0, z4), d0 = csub(z0, z4);
-    float2 z2, z6;
-    real_unsplit(y.q1, y.q3, uh, z2, z6);
-    const float2 sh = cadd(z2, z6), dd = csub(z2, z6);
-    const float2 dh = make_float2(-dd.y, dd.x);                     // times conj(-i) = i
-    a0 = make_float2(s0.y, s0.x);
-    b0 = make_float2(d0.y, d0.x);
-    ah = make_float2(sh.y, sh.x);
-    bh = make_float2(dh.y, dh.x);
+// Products back to the frequencies of the two half-size transforms (again twice the value),
+// real and imaginary parts swapped for the inverse.
+__device__ __forceinline__ void bins_inverse(const Bins &y, const SplitTwiddle &w, C2 &zk, C2 &zm) {
+    using namespace fftpair;
+    const u64 er = add2(y.pr, y.qr), ei = add2(y.pi, y.qi);
+    const u64 dr = sub2(y.pr, y.qr), di = sub2(y.pi, y.qi);
+    const u64 orr = fma2(w.ui, di, mul2(w.ur, dr)), oi = sub2(mul2(w.ur, di), mul2(w.ui, dr));
+    // lanes from (k, m) to (even, odd)
+    const u64 ekr = low2(er, orr), emr = high2(er, orr), eki = low2(ei, oi), emi = high2(ei, oi);
+    const u64 ar = add2(ekr, emr), ai = add2(eki, emi);           // Ek + conj Em
+    const u64 cr = sub2(ekr, emr), ci = sub2(eki, emi);           // Ek - conj Em
+    // i conj(W) c, its real part with the other sign
+    const u64 nqr = sub2(mul2(w.wx, ci), mul2(w.wy, cr)), qi = fma2(w.wy, ci, mul2(w.wx, cr));
+    zk = {add2(ai, qi), sub2(ar, nqr)};
+    zm = {sub2(qi, ai), add2(ar, nqr)};
+}
+__device__ __forceinline__ Bins edge_forward(C2 z0, C2 zh) {
+    using namespace fftpair;
+    const float h = 0.70710678118654752440f;                      // U^2048 = (h, -h)
+    const float2 r = unpack(z0.re), i = unpack(z0.im), hr = unpack(zh.re), hi = unpack(zh.im);
+    const float e0 = 2.f * (r.x + i.x), e4 = 2.f * (r.x - i.x), o0 = 2.f * (r.y + i.y), o4 = 2.f * (r.y - i.y);
+    const float er = 2.f * hr.x, ei = -2.f * hi.x, orr = 2.f * hr.y, oi = -2.f * hi.y;
+    const float tr = h * (orr + oi), ti = h * (oi - orr);
+    return {pack(e0 + o0, e4), pack(e0 - o0, -o4), pack(er + tr, er - tr), pack(ei + ti, ei - ti)};
+}
+__device__ __forceinline__ void edge_inverse(const Bins &y, C2 &z0, C2 &zh) {
+    using namespace fftpair;
+    const float h = 0.70710678118654752440f;
+    const float2 pr = unpack(y.pr), pi = unpack(y.pi), qr = unpack(y.qr), qi = unpack(y.qi);
+    const float e0 = pr.x + pi.x, o0 = pr.x - pi.x, e4 = 2.f * pr.y, o4 = -2.f * pi.y;
+    z0 = {pack(e0 - e4, o0 - o4), pack(e0 + e4, o0 + o4)};
+    const float er = qr.x + qr.y, ei = qi.x + qi.y, dr = qr.x - qr.y, di = qi.x - qi.y;
+    const float orr = h * (dr - di), oi = h * (di + dr);
+    zh = {pack(-2.f * ei, -2.f * oi), pack(2.f * er, 2.f * orr)};
+}
+__device__ __forceinline__ void multiply(u64 &xr, u64 &xi, u64 hr, u64 hi) {
+    using namespace fftpair;
+    const u64 yr = sub2(mul2(xr, hr), mul2(xi, hi));
+    xi = fma2(xi, hr, mul2(xr, hi));
+    xr = yr;
+}
+__device__ __forceinline__ void edge_multiply(Bins &y, const Bins &h) {
+    using namespace fftpair;
+    const float2 pr = unpack(y.pr), pi = unpack(y.pi), hr = unpack(h.pr), hi = unpack(h.pi);
+    y.pr = pack(pr.x * hr.x, pr.y * hr.y - pi.y * hi.y);
+    y.pi = pack(pi.x * hi.x, pr.y * hi.y + pi.y * hr.y);
+    multiply(y.qr, y.qi, h.qr, h.qi);
+}
+// Bins of a slot of thread t at p + t, the halves CF apart; streamed, not kept in L1.
+__device__ __forceinline__ Bins load_bins(const float4 *p) {
+    Bins z;
+    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.pr), "=l"(z.pi) : "l"(p));
+    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.qr), "=l"(z.qi) : "l"(p + CF));
+    return z;
+}
+__device__ __forceinline__ Bins load_parked(const float4 *p) {
+    const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2 *>(p));
+    const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2 *>(p + CF));
+    return {a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
+    __stcg(reinterpret_cast<ulonglong2 *>(p), make_ulonglong2(z.pr, z.pi));
+    __stcg(reinterpret_cast<ulonglong2 *>(p + CF), make_ulonglong2(z.qr, z.qi));
 }
 
 // Spectrum of one 16384-sample segment of each impulse response (taps beyond L and
-// the whole second half are zero), scaled by the noise weight and 1/F.
-__global__ void __launch_bounds__(CT)
+// the whole second half are zero), scaled by the noise weight and 1/F (and by 1/4 for
+// the two doubled spectra of a product).
+__global__ void __launch_bounds__(CF, FUSED_MINB)
 rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max,
-                    int L, const float2 *__restrict__ tw, float2 *__restrict__ hspec, int64_t hs_stride,
+                    int L, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int64_t hs_stride,
                     const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed) {
-    extern __shared__ __align__(16) float2 sm[];
-    __shared__ int red_i[CT / 32];
-    float2 *A = sm, *Bf = sm + SM_POINTS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
+    __shared__ int red_i[CF / 32];
     const int s = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
     // mixed: the lengths are known already (rir_length_kernel) and decide the route; otherwise
     // this kernel reads every tap anyway and records the length on the way
     if (mixed && !takes_fused_route(*leff_all)) return;
     const AugUttParams &row = table[utt];
     if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
-    const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (float)F2;
+    const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (4.f * (float)F2);
     const float *h = rir + ((int64_t)utt * S_max + s) * L;
-    float2 *out = hspec + ((int64_t)utt * S_max + s) * hs_stride;
-    {
-        float2 va[1][E], vb[1][E];
-        int last = 0;
+    float4 *out = hspec + ((int64_t)utt * S_max + s) * (hs_stride / 2) + t;
+    fftpair::fill_tables(sh, t, tw);
+    C2 v[NP2];
+    int last = 0;
 #pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int i0 = 4 * (t + CT * r);
-            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i0 < BLK2) {
-                if (i0 < L) z.x = h[i0];
-                if (i0 + 1 < L) z.y = h[i0 + 1];
-                if (i0 + 2 < L) z.z = h[i0 + 2];
-                if (i0 + 3 < L) z.w = h[i0 + 3];
-                if (z.x != 0.f) last = i0 + 1;
-                if (z.y != 0.f) last = i0 + 2;
-                if (z.z != 0.f) last = i0 + 3;
-                if (z.w != 0.f) last = i0 + 4;
-            }
-            va[0][r] = make_float2(z.x, z.y);
-            vb[0][r] = make_float2(z.z, z.w);
+    for (int r = 0; r < NP2; ++r) {
+        const int i0 = 4 * (t + CF * r);
+        float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i0 < BLK2) {
+            if (i0 < L) z.x = h[i0];
+            if (i0 + 1 < L) z.y = h[i0 + 1];
+            if (i0 + 2 < L) z.z = h[i0 + 2];
+            if (i0 + 3 < L) z.w = h[i0 + 3];
+            if (z.x != 0.f) last = i0 + 1;
+            if (z.y != 0.f) last = i0 + 2;
+            if (z.z != 0.f) last = i0 + 3;
+            if (z.w != 0.f) last = i0 + 4;
         }
-        if (!mixed) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
-            if ((t & 31) == 0) red_i[t >> 5] = last;
-            __syncthreads();
-            if (t == 0) {
-                int m = 0;
-                for (int i = 0; i < CT / 32; ++i) m = max(m, red_i[i]);
-                if (m > 0) atomicMax(const_cast<int *>(&leff[utt]), m);
-            }
-        }
-        fft2x4096_from_regs(va, vb, A, Bf, t, tw);
-        __syncthreads();
+        v[r] = {fftpair::pack(z.x, z.y), fftpair::pack(z.z, z.w)};
     }
+    if (!mixed) {
 #pragma unroll
-    for (int q = 0; q < NQ2; ++q) {
-        const int k = t + CT * q;
-        if (k == 0) {
-            const Edge x = edge_forward(A[pad0(0)], Bf[pad0(0)], A[pad0(N2 / 2)], Bf[pad0(N2 / 2)],
-                                        __ldg(&tw[tw_index(F2, N2 / 2)]));
-            out[0] = make_float2(x.dc.x * scale, x.dc.y * scale);
-            out[N2] = make_float2(x.mid.x * scale, x.mid.y * scale);
-            out[N2 / 2] = make_float2(x.q1.x * scale, x.q1.y * scale);
-            out[N2 + N2 / 2] = make_float2(x.q3.x * scale, x.q3.y * scale);
-        } else {
-            const Quad x = quad_forward(A[pad0(k)], A[pad0(N2 - k)], Bf[pad0(k)], Bf[pad0(N2 - k)],
-                                        __ldg(&tw[tw_index(NB2, k)]), __ldg(&tw[tw_index(F2, k)]));
-            out[k] = make_float2(x.k.x * scale, x.k.y * scale);
-            out[NB2 - k] = make_float2(x.nk.x * scale, x.nk.y * scale);
-            out[N2 - k] = make_float2(x.mk.x * scale, x.mk.y * scale);
-            out[N2 + k] = make_float2(x.pk.x * scale, x.pk.y * scale);
-        }
+        for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+        if ((t & 31) == 0) red_i[t >> 5] = last;
+    }
+    __syncthreads();
+    if (!mixed && t == 0) {
+        int m = 0;
+        for (int i = 0; i < CF / 32; ++i) m = max(m, red_i[i]);
+        if (m > 0) atomicMax(const_cast<int *>(&leff[utt]), m);
+    }
+    fftpair::forward4096(v, sh, t, tw);
+    fftpair::exchange_mirror(v, t);
+    const u64 sc = fftpair::both(scale);
+    const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
+#pragma unroll
+    for (int r = 0; r < NS2; ++r) {
+        Bins x = r == 0 && fftpair::owns_zero(t) ? edge_forward(v[0], v[NP2 - 1])
+                                                 : bins_forward(v[r], v[NP2 - 1 - r], SplitTwiddle(u, r));
+        x = {fftpair::mul2(x.pr, sc), fftpair::mul2(x.pi, sc), fftpair::mul2(x.qr, sc), fftpair::mul2(x.qi, sc)};
+        store_bins(out + 2 * r * CF, x);
     }
 }
 
-// What the spectral phase reads from global memory for slot k: the join and split
-// twiddles and the four response bins X[k], X[8192-k], X[4096-k], X[4096+k] pair with
-// (slot 0: the split twiddle of bin 2048 and bins 0/8192, 4096, 2048, 6144).
-struct SpecOps {
-    float2 w, u, h0, h1, h2, h3;
+// ---------------------------------------------------------------- what the fused convolution does
+// One unit of work is one block of one output (the reverberant speech, or the sum of the noise
+// sources) of an utterance.  plan_kernel lists the units that exist -- how many blocks an
+// utterance has depends on its length and on where its responses end -- and what they need to
+// know; the convolution's CTAs, as many as fit the device, work through the list.  With one CTA
+// per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
+// (two thirds of them without work) and to each one's chain of loads before its first sample.
+struct Plan {
+    const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
+    int nlen[AUG_S_MAX];           // their lengths ([0] unused)
+    int src[AUG_S_MAX];            // their source numbers
+    int n_src;                     // 0: the row was rejected, both outputs are silence
+    int n_noise;
+    int N;                         // samples of the utterance
+    int ob;                        // outputs per block
 };
-__device__ __forceinline__ SpecOps load_spec_ops(const float2 *__restrict__ H, const float2 *__restrict__ tw,
-                                                 int k) {
-    SpecOps o;
-    const bool z = k == 0;
-    o.w = __ldg(&tw[tw_index(NB2, k)]);
-    o.u = __ldg(&tw[z ? tw_index(F2, N2 / 2) : tw_index(F2, k)]);
-    o.h0 = __ldg(&H[k]);
-    o.h1 = __ldg(&H[z ? N2 : NB2 - k]);
-    o.h2 = __ldg(&H[z ? N2 / 2 : N2 - k]);
-    o.h3 = __ldg(&H[z ? N2 + N2 / 2 : N2 + k]);
-    return o;
+struct Unit {
+    int utt;
+    int block2;                    // 2 block + (1 for the noise sum)
+};
+static_assert(sizeof(Plan) % 4 == 0 && sizeof(Plan) <= aug::PLAN_BYTES && sizeof(Unit) == 8, "");
+
+// One warp per utterance.
+__global__ void __launch_bounds__(256)
+plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restrict__ lengths,
+            const float *__restrict__ bank, int64_t bank_len, const AugUttParams *__restrict__ table, int B,
+            int S_max, int n_cap, const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed,
+            int *status, Plan *__restrict__ plans, Unit *__restrict__ units, int *__restrict__ n_units) {
+    const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (utt >= B || (mixed && !takes_fused_route(*leff_all))) return;
+    const AugUttParams &row = table[utt];
+    const int N = min(max(lengths[utt], 0), n_cap);
+    // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
+    // of 4, where taps counts up to the last non-zero tap of this utterance's responses
+    const int ob = (F2 - min(max(leff[utt], 1), BLK2) + 1) & ~3;
+    const int n = 2 * ((N + ob - 1) / ob);
+    int at = 0;
+    if (lane == 0) {
+        Plan p;
+        p.N = N;
+        p.ob = ob;
+        p.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;    // (reported by step 1)
+        p.n_noise = 0;
+        p.x[0] = speech + (int64_t)utt * stride;
+        p.nlen[0] = 1;
+        p.src[0] = 0;
+        for (int s = 1; s < p.n_src; ++s) {
+            const float *x;
+            int nlen;
+            if (source_of(row, s, nullptr, bank, bank_len, x, nlen)) {
+                ++p.n_noise;
+                p.x[p.n_noise] = x;
+                p.nlen[p.n_noise] = nlen;
+                p.src[p.n_noise] = s;
+            } else if (n > 0 && atomicCAS(&status[0], -1, utt) == -1) {
+                status[1] = aug::R_NOISE;
+            }
+        }
+        plans[utt] = p;
+        if (n > 0) at = atomicAdd(n_units, n);
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (int i = lane; i < n; i += 32) units[at + i] = Unit{utt, i};
 }
 
 // PARK: rows may have several noise sources (the context allows three or more
 // sources); without it the kernel carries none of the parking code.
+//
+// Several noise sources are summed in the frequency domain: the products of all but the last
+// are parked in a 64 KB global slot of the CTA's own (it stays in L2) and added to the last
+// one's before the single inverse transform.  Where the slot is held (park_flags) the sum is
+// done in the time domain instead: v is read back and added to for every source after the
+// first, one inverse transform each.
+enum Fate { DIRECT = 0, PARK_FIRST = 1, PARK_MORE = 2, PARK_JOIN = 3 };
+
 template <bool PARK>
-__global__ void __launch_bounds__(CT, CONV_MINB)
-convolve_fused2_kernel(const float *__restrict__ speech, int64_t stride,
-                       const int *__restrict__ lengths, const float *__restrict__ bank,
-                       int64_t bank_len, const AugUttParams *__restrict__ table, int S_max,
-                       const float2 *__restrict__ hspec, const float2 *__restrict__ tw,
-                       float *__restrict__ ys, float *__restrict__ vv, int64_t ws_stride,
-                       double *__restrict__ energy, int *status, int n_cap,
-                       const int *__restrict__ leff, const int *__restrict__ leff_all, int64_t hs_stride,
-                       int mixed,
-                       float2 *__restrict__ park, int *park_flags, int n_sm) {
-    extern __shared__ __align__(16) float2 sm[];
-    float2 *A = sm, *Bf = sm + SM_POINTS;
-    __shared__ float red[CT / 32];
-    __shared__ int park_slot_s;
-    const int b = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
-    const int N = min(max(lengths[utt], 0), n_cap);
-    // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
-    // of 4, where taps counts up to the last non-zero tap of this utterance's responses
-    if (mixed && !takes_fused_route(*leff_all)) return;
-    const int taps_used = leff[utt];
-    const int ob = (F2 - min(max(taps_used, 1), BLK2) + 1) & ~3;
-    if ((int64_t)b * ob >= N) return;
-    const AugUttParams &row = table[utt];
-    int n_src = row.n_src;
-    if (n_src < 1 || n_src > S_max) n_src = 0;   // rejected row: silence (reported by step 1)
-    const int m0 = (F2 - ob) / 4;            // first point of A and B that belongs to a block
+__global__ void __launch_bounds__(CF, FUSED_MINB)
+convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units,
+                       int *n_units, int S_max, const float4 *__restrict__ hspec,
+                       int64_t hs_stride, const float2 *__restrict__ tw, float *__restrict__ ys,
+                       float *__restrict__ vv, int64_t ws_stride, double *__restrict__ energy,
+                       float4 *__restrict__ park, const int *__restrict__ park_flags) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
+    // The first two units of a CTA follow from its number, the others it draws from a counter (units
+    // differ: more noise sources, more work; dealt out in turn they left CTAs idle, 567 against
+    // 447 us on 256 utterances of 2-20 s).  The unit after next and the next one's plan are
+    // fetched while the current one is worked on; a warp may be up to one unit behind, hence three
+    // places for each.
+    __shared__ Plan plan_s[3];
+    __shared__ Unit unit_s[3];
+    const int t = threadIdx.x, count = *n_units, G = gridDim.x;
+    int *drawn = n_units + 1;
+    if (blockIdx.x >= count) return;
+    if (t == 0) {
+        const int second = blockIdx.x + G;
+        unit_s[0] = units[blockIdx.x];
+        unit_s[1] = second < count ? units[second] : Unit{-1, 0};
+    }
+    if (t < (int)(sizeof(Plan) / 4))
+        reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + units[blockIdx.x].utt)[t];
+    fftpair::fill_tables(sh, t, tw);
+    __syncthreads();
+    const bool own_slot = PARK && park != nullptr && park_flags[blockIdx.x] == 0;
 
-    int last_noise = 0, n_noise = 0;
-    for (int s = 1; s < n_src; ++s) {
-        const float *x;
-        int nlen;
-        if (source_of(row, s, nullptr, bank, bank_len, x, nlen)) {
-            last_noise = s;
-            ++n_noise;
-        } else if (t == 0 && b == 0 && atomicCAS(&status[0], -1, utt) == -1) {
-            status[1] = aug::R_NOISE;
-        }
-    }
-    // Several noise sources are summed in the frequency domain: the products of all
-    // but the last are parked in a 64 KB global slot (one per resident CTA of an SM,
-    // taken with a compare-and-swap; it stays in L2) and added to the last one's
-    // before the single inverse transform.  A CTA that finds no free slot -- more
-    // CTAs on the SM than slots -- sums in the time domain instead: v is read back
-    // and added to for every source after the first, one inverse transform each.
-    int park_slot = -1;
-    if (PARK && n_noise > 1 && park != nullptr) {
-        if (t == 0) {
-            unsigned smid;
-            asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-            int got = -1;
-            if ((int)smid < n_sm) {
-                for (int i = 0; i < CONV_MINB && got < 0; ++i)
-                    if (atomicCAS(&park_flags[smid * CONV_MINB + i], 0, 1) == 0) got = smid * CONV_MINB + i;
-            }
-            park_slot_s = got;
-        }
-        __syncthreads();
-        park_slot = park_slot_s;
-    }
-    float2 *slot = park_slot >= 0 ? park + (int64_t)park_slot * (4 * NQ2 * CT) : nullptr;
-    const int n_left = min(N - b * ob, ob);
-    bool v_written = false, v_parked = false;
-    for (int s = 0; s < n_src; ++s) {
-        const float *x;
-        int nlen;
-        if (!source_of(row, s, speech + (int64_t)utt * stride, bank, bank_len, x, nlen)) continue;
-        {
-            float2 va[1][E], vb[1][E];
-            load_segment4(va, vb, x, s != 0, nlen, (b + 1) * ob - F2, N, t, bank + bank_len);
-            fft2x4096_from_regs(va, vb, A, Bf, t, tw);
-        }
-        const float2 *H = hspec + ((int64_t)utt * S_max + s) * hs_stride;
-        // the first slot's operands are requested before the barrier that completes the transform
-        SpecOps nxt = load_spec_ops(H, tw, t);
-        __syncthreads();
-        // what happens to this source's products: inverse-transformed right away (0),
-        // parked for a later noise source (1: first one, 2: added to what is parked),
-        // or joined by the parked sum before the inverse (3)
-        int mode = 0;
-        if (PARK && s != 0 && slot != nullptr) mode = s == last_noise ? 3 : (v_parked ? 2 : 1);
-#pragma unroll 2
-        for (int q = 0; q < NQ2; ++q) {
-            const int k = t + CT * q;
-            const SpecOps c = nxt;
-            if (q + 1 < NQ2) nxt = load_spec_ops(H, tw, k + CT);     // next slot's operands while this one is worked on
-            float2 *pk = slot + (4 * q) * CT + t;      // this thread's four parked products, CT apart
-            if (k == 0) {
-                const float2 uh = c.u;
-                Edge x4 = edge_forward(A[pad0(0)], Bf[pad0(0)], A[pad0(N2 / 2)], Bf[pad0(N2 / 2)], uh);
-                x4.dc = make_float2(x4.dc.x * c.h0.x, x4.dc.y * c.h0.y);
-                x4.mid = cmul(x4.mid, c.h1);
-                x4.q1 = cmul(x4.q1, c.h2);
-                x4.q3 = cmul(x4.q3, c.h3);
-                if (PARK && mode >= 2) {
-                    x4.dc = cadd(x4.dc, pk[0]);
-                    x4.mid = cadd(x4.mid, pk[CT]);
-                    x4.q1 = cadd(x4.q1, pk[2 * CT]);
-                    x4.q3 = cadd(x4.q3, pk[3 * CT]);
+#pragma unroll 1
+    for (int k = 0;;) {
+        const Plan &p = plan_s[k];
+        const Unit cur = unit_s[k];
+        const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+        const int next_utt = unit_s[k1].utt;
+        if (next_utt >= 0 && t < (int)(sizeof(Plan) / 4))
+            copy4_async(reinterpret_cast<float *>(&plan_s[k1]) + t,
+                        reinterpret_cast<const float *>(plans + next_utt) + t, 4);
+        int ticket = 0;
+        if (t == 0) ticket = 2 * G + atomicAdd(drawn, 1);
+        auto draw = [&]() {                    // (published by the barrier that follows)
+            if (t == 0) unit_s[k2] = ticket < count ? units[ticket] : Unit{-1, 0};
+            copies_done();
+        };
+        const bool noise = cur.block2 & 1;
+        const int b = cur.block2 >> 1;
+        // sources of this output: list entries j .. j_last
+        int j = noise ? 1 : 0;
+        const int j_last = noise ? p.n_noise : 0;
+        if (j > j_last || p.n_src == 0) {
+            // no (usable) source: the output is defined as silence
+            float *dst = (noise ? vv : ys) + (int64_t)cur.utt * ws_stride + (int64_t)b * p.ob;
+            const int n_left = min(p.N - b * p.ob, p.ob);
+            for (int i = t; i < n_left; i += CF) dst[i] = 0.f;
+            draw();
+            __syncthreads();
+        } else {
+            bool added = false;
+#pragma unroll 1
+            for (;; ++j) {
+                Fate fate = DIRECT;
+                if (PARK && own_slot && j_last > 1)
+                    fate = j == j_last ? PARK_JOIN : j > 1 ? PARK_MORE : PARK_FIRST;
+                C2 v[NP2];
+                load_segment(v, sh, p.x[j], noise, p.nlen[j], (b + 1) * p.ob - F2, p.N, t);
+                fftpair::forward4096(v, sh, t, tw);
+                const float4 *H = hspec + ((int64_t)cur.utt * S_max + p.src[j]) * (hs_stride / 2) + t;
+                Bins h = load_bins(H);
+                const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
+                fftpair::exchange_mirror(v, t);
+#pragma unroll
+                for (int r = 0; r < NS2; ++r) {
+                    const Bins hc = h;
+                    if (r + 1 < NS2) h = load_bins(H + 2 * (r + 1) * CF);   // the next slot's meanwhile
+                    const bool edge = r == 0 && fftpair::owns_zero(t);
+                    const SplitTwiddle w(u, r);
+                    Bins y;
+                    if (edge) {
+                        y = edge_forward(v[0], v[NP2 - 1]);
+                        edge_multiply(y, hc);
+                    } else {
+                        y = bins_forward(v[r], v[NP2 - 1 - r], w);
+                        multiply(y.pr, y.pi, hc.pr, hc.pi);
+                        multiply(y.qr, y.qi, hc.qr, hc.qi);
+                    }
+                    if (PARK && fate != DIRECT) {
+                        // this thread's parked products, two words per slot: no other thread reads them
+                        float4 *pk = park + (int64_t)blockIdx.x * (2 * NS2 * CF) + 2 * r * CF + t;
+                        if (fate != PARK_FIRST) {
+                            const Bins z = load_parked(pk);
+                            y = {fftpair::add2(y.pr, z.pr), fftpair::add2(y.pi, z.pi), fftpair::add2(y.qr, z.qr),
+                                 fftpair::add2(y.qi, z.qi)};
+                        }
+                        if (fate != PARK_JOIN) store_bins(pk, y);
+                    }
+                    if (edge) edge_inverse(y, v[0], v[NP2 - 1]);
+                    else bins_inverse(y, w, v[r], v[NP2 - 1 - r]);
                 }
-                if (PARK && (mode == 1 || mode == 2)) {
-                    pk[0] = x4.dc;
-                    pk[CT] = x4.mid;
-                    pk[2 * CT] = x4.q1;
-                    pk[3 * CT] = x4.q3;
-                } else {
-                    edge_inverse(x4, uh, A[pad0(0)], Bf[pad0(0)], A[pad0(N2 / 2)], Bf[pad0(N2 / 2)]);
+                if (PARK && (fate == PARK_FIRST || fate == PARK_MORE)) {
+                    __syncthreads();       // other warps may still read rows of the buffer the next source fills
+                    continue;
                 }
-            } else {
-                const float2 w = c.w, u = c.u;
-                Quad x4 = quad_forward(A[pad0(k)], A[pad0(N2 - k)], Bf[pad0(k)], Bf[pad0(N2 - k)], w, u);
-                x4.k = cmul(x4.k, c.h0);
-                x4.nk = cmul(x4.nk, c.h1);
-                x4.mk = cmul(x4.mk, c.h2);
-                x4.pk = cmul(x4.pk, c.h3);
-                if (PARK && mode >= 2) {
-                    x4.k = cadd(x4.k, pk[0]);
-                    x4.nk = cadd(x4.nk, pk[CT]);
-                    x4.mk = cadd(x4.mk, pk[2 * CT]);
-                    x4.pk = cadd(x4.pk, pk[3 * CT]);
-                }
-                if (PARK && (mode == 1 || mode == 2)) {
-                    pk[0] = x4.k;
-                    pk[CT] = x4.nk;
-                    pk[2 * CT] = x4.mk;
-                    pk[3 * CT] = x4.pk;
-                } else {
-                    quad_inverse(x4, w, u, A[pad0(k)], A[pad0(N2 - k)], Bf[pad0(k)], Bf[pad0(N2 - k)]);
-                }
-            }
-        }
-        if (PARK && (mode == 1 || mode == 2)) {
-            // every thread reads back only what it parked itself: no fence is needed
-            v_parked = true;
-            __syncthreads();   // the buffers are refilled by the next source
-            continue;
-        }
-        __syncthreads();
-        fft2x4096_in_place(A, Bf, t, tw);
-        __syncthreads();
+                fftpair::exchange_back(v, t);
+                if (j == j_last) draw();
+                fftpair::inverse4096(v, sh, t, tw);
 
-        // The last `ob` outputs of the segment are this block: samples 4m, 4m+1 of the
-        // segment are point m of A, samples 4m+2, 4m+3 point m of B.
-        const bool is_speech = s == 0;
-        const bool add = !is_speech && v_written;
-        const bool want_energy = is_speech || s == last_noise;
-        float *dst = (is_speech ? ys : vv) + (int64_t)utt * ws_stride + (int64_t)b * ob;
-        float e2sum = 0.f;
-        if (n_left >= ob) {
-            // a whole block of outputs (the same for the CTA): no test per group
-#pragma unroll 4
-            for (int j = t; m0 + j < N2; j += CT) {
-                const float2 za = A[pad0(m0 + j)], zb = Bf[pad0(m0 + j)];
-                float4 y = make_float4(za.y, za.x, zb.y, zb.x);
-                float4 *p = reinterpret_cast<float4 *>(dst + 4 * j);
-                if (add) {
-                    const float4 o = *p;
-                    y = make_float4(y.x + o.x, y.y + o.y, y.z + o.z, y.w + o.w);
+                // The last `ob` outputs of the segment are this block: samples 4m .. 4m+3 of the
+                // segment are point m = t + CF r, real and imaginary parts swapped.
+                const int ob = p.ob, n_left = min(p.N - b * ob, ob);
+                float *dst = (noise ? vv : ys) + (int64_t)cur.utt * ws_stride + (int64_t)b * ob;
+                u64 e2 = 0;
+                const int o0 = 4 * t - (F2 - ob);         // first of this thread's outputs, 4 CF apart
+                if (n_left == ob && !(PARK && added)) {
+                    // a whole block (most are)
+#pragma unroll
+                    for (int r = 0; r < NP2; ++r) {
+                        if (o0 + 4 * CF * r >= 0) {
+                            const float2 lo = fftpair::unpack(v[r].im), hi = fftpair::unpack(v[r].re);
+                            *reinterpret_cast<float4 *>(dst + o0 + 4 * CF * r) = make_float4(lo.x, lo.y, hi.x, hi.y);
+                            e2 = fftpair::fma2(v[r].re, v[r].re, fftpair::fma2(v[r].im, v[r].im, e2));
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < NP2; ++r) {
+                        const int o = o0 + 4 * CF * r;
+                        if (o >= 0 && o < n_left) {
+                            const float2 lo = fftpair::unpack(v[r].im), hi = fftpair::unpack(v[r].re);
+                            // (workspace rows are allocated up to a multiple of 4)
+                            float4 y = make_float4(lo.x, o + 1 < n_left ? lo.y : 0.f, o + 2 < n_left ? hi.x : 0.f,
+                                                   o + 3 < n_left ? hi.y : 0.f);
+                            float4 *q = reinterpret_cast<float4 *>(dst + o);
+                            if (PARK && added) {
+                                const float4 z = *q;
+                                y = make_float4(y.x + z.x, y.y + z.y, y.z + z.z, y.w + z.w);
+                            }
+                            *q = y;
+                            const u64 a = fftpair::pack(y.x, y.y), c = fftpair::pack(y.z, y.w);
+                            e2 = fftpair::fma2(a, a, fftpair::fma2(c, c, e2));
+                        }
+                    }
                 }
-                *p = y;
-                e2sum += y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w;
-            }
-        } else
-#pragma unroll 4
-        for (int j = t; m0 + j < N2; j += CT) {
-            const float2 za = A[pad0(m0 + j)], zb = Bf[pad0(m0 + j)];
-            float4 y = make_float4(za.y, za.x, zb.y, zb.x);
-            const int i = 4 * j;
-            if (i + 3 < n_left) {
-                float4 *p = reinterpret_cast<float4 *>(dst + i);
-                if (add) {
-                    const float4 o = *p;
-                    y = make_float4(y.x + o.x, y.y + o.y, y.z + o.z, y.w + o.w);
+                added = true;
+                if (j == j_last) {
+                    const float2 e = fftpair::unpack(e2);
+                    float sum = e.x + e.y;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    if ((t & 31) == 0) atomicAdd(&energy[2 * cur.utt + (noise ? 1 : 0)], (double)sum);
+                    break;
                 }
-                *p = y;
-                e2sum += y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w;
-            } else {
-                const float yy[3] = {y.x, y.y, y.z};
-                for (int c = 0; c < 3 && i + c < n_left; ++c) {
-                    const float val = add ? yy[c] + dst[i + c] : yy[c];
-                    dst[i + c] = val;
-                    e2sum += val * val;
-                }
+                if (PARK) __syncthreads();
             }
         }
-        if (want_energy) {
-            const float tot = block_sum(e2sum, red, t);
-            if (t == 0) atomicAdd(&energy[2 * utt + (is_speech ? 0 : 1)], (double)tot);
-        }
-        if (!is_speech) v_written = true;
-        __syncthreads();   // the buffers are refilled by the next source
-    }
-    if (n_src == 0) {
-        // rejected row: y_s is silence too
-        float *dst = ys + (int64_t)utt * ws_stride + (int64_t)b * ob;
-        for (int i = t; i < n_left; i += CT) dst[i] = 0.f;
-    }
-    if (!v_written) {
-        // no (usable) noise: v is defined as silence
-        float *dst = vv + (int64_t)utt * ws_stride + (int64_t)b * ob;
-        for (int i = t; i < n_left; i += CT) dst[i] = 0.f;
-    }
-    if (PARK && park_slot >= 0) {
-        __syncthreads();                                  // all reads of the slot are done
-        if (t == 0) atomicExch(&park_flags[park_slot], 0);
+        if (next_utt < 0) break;
+        k = k1;
     }
 }
 
 constexpr size_t FFT_SMEM = sizeof(float2) * SM_POINTS;
-constexpr size_t FFT2_SMEM = 2 * FFT_SMEM;
+constexpr size_t FFT2_SMEM = sizeof(fftpair::Shared);
 
 }  // namespace
 
@@ -1032,7 +1003,7 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table,
     ctx->stored_only = mixed && ctx->leff_seen && *ctx->leff_seen > BLK2;
     int *leff_all = ctx->leff + ctx->cfg.max_batch;
     AUG_CUDA_OK(cudaMemsetAsync(ctx->leff, 0, sizeof(int) * (size_t)B, st));
-    AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, sizeof(int), st));
+    AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, 3 * sizeof(int), st));      // and the counters of the work list
     dim3 grid2(c.max_sources, B);
     if (mixed) {
         rir_length_kernel<<<grid2, CT, 0, st>>>(rir, table, c.max_sources, c.rir_taps, ctx->leff, leff_all);
@@ -1041,9 +1012,9 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table,
     }
     if (!ctx->stored_only) {
         if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
-        rir_spectra2_kernel<<<grid2, CT, FFT2_SMEM, st>>>(rir, table, c.max_sources, c.rir_taps, ctx->tw,
-                                                          ctx->hspec, hspec_stride(ctx), ctx->leff, leff_all,
-                                                          mixed);
+        rir_spectra2_kernel<<<grid2, CF, FFT2_SMEM, st>>>(
+            rir, table, c.max_sources, c.rir_taps, ctx->tw, reinterpret_cast<float4 *>(ctx->hspec),
+            hspec_stride(ctx), ctx->leff, leff_all, mixed);
         AUG_CUDA_OK(cudaGetLastError());
         ctx->launches++;
     }
@@ -1083,21 +1054,26 @@ int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, con
     const int mixed = stored_route(ctx) ? 1 : 0;
     const int *leff_all = ctx->leff + c.max_batch;
     if (!ctx->stored_only) {
-        // fused route: the grid covers the shortest block an utterance on it can have (a response
-        // that fills min(rir_taps, 8192) taps)
+        plan_kernel<<<(B + 7) / 8, 256, 0, ctx->stream>>>(
+            speech, stride, lengths, bank, bank_len, table, B, c.max_sources, max_len, ctx->leff, leff_all, mixed,
+            ctx->status, reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
+            ctx->leff + c.max_batch + 1);
+        AUG_CUDA_OK(cudaGetLastError());
+        // as many CTAs as fit, but not more than there can be units of work (blocks are shortest
+        // where a response fills min(rir_taps, 8192) taps)
         const int ob_min = (F2 - min(c.rir_taps, BLK2) + 1) & ~3;
-        const int nblk2 = (max_len + ob_min - 1) / ob_min;
-        dim3 grid2(nblk2, B);
+        const int64_t most = 2 * (int64_t)B * ((max_len + ob_min - 1) / ob_min);
+        const int grid2 = (int)std::min<int64_t>(most, std::min(FUSED_MINB * ctx->sm_count, aug::PARK_SLOTS));
         auto kern = ctx->park ? convolve_fused2_kernel<true> : convolve_fused2_kernel<false>;
         if ((ctx->park ? smem_opt_in<convolve_fused2_kernel<true>>(ctx->device)
                        : smem_opt_in<convolve_fused2_kernel<false>>(ctx->device)) != AUG_OK)
             return AUG_ECUDA;
-        kern<<<grid2, CT, FFT2_SMEM, ctx->stream>>>(
-            speech, stride, lengths, bank, bank_len, table, c.max_sources, ctx->hspec, ctx->tw,
-            ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->status, max_len, ctx->leff, leff_all,
-            hspec_stride(ctx), mixed, ctx->park, ctx->park_flags, ctx->n_sm);
+        kern<<<grid2, CF, FFT2_SMEM, ctx->stream>>>(
+            reinterpret_cast<const Plan *>(ctx->plans), reinterpret_cast<const Unit *>(ctx->units),
+            ctx->leff + c.max_batch + 1, c.max_sources, reinterpret_cast<const float4 *>(ctx->hspec),
+            hspec_stride(ctx), ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->park, ctx->park_flags);
         AUG_CUDA_OK(cudaGetLastError());
-        ctx->launches++;
+        ctx->launches += 2;
     }
     if (mixed) {
         const int nblk = (max_len + BLK - 1) / BLK;

@@ -178,4 +178,145 @@ __device__ __forceinline__ void fft512(C2 *v, u64 *buf, float4 c, int l) {
     dft16(v);
 }
 
+// A pair of 4096-point transforms by a CTA of 256 threads, 16 points each, in place in shared
+// memory: three radix-16 passes.  Digits of an index: slot = 256 a + 16 b + c.
+//   forward  pass 1: thread t = 16 b + c transforms the slots 256 r + t over r
+//            pass 2: thread (a, c)       the slots 256 a + 16 r + c
+//            pass 3: thread (a, b)       the slots 256 a + 16 b + r; its outputs, which stay in
+//                    registers, are the frequencies j + 256 r, j = a + 16 b
+//   inverse  the same three passes in the opposite order, from frequencies in the registers
+//            of thread (a, b) to samples t + 256 r in the registers of thread t.
+// Every pass writes the slots it has read, so nothing is overwritten that another thread
+// still wants, and as passes 2 and 3 of the forward and 1 and 2 of the inverse direction
+// with the same digit a are done by the same warp (two values of a per warp), only the
+// boundary between passes 1 and 2 (inverse: 2 and 3) needs a barrier of the whole CTA.
+// Real and imaginary parts lie in separate planes of 8-byte words: a 16-byte word would want
+// both pairs of registers side by side, which costs moves.  Rows of 16 words are padded by
+// one, which keeps all three access patterns free of bank conflicts.
+constexpr int THREADS = 256;
+constexpr int PLANE = 4096 + 256;
+__host__ __device__ constexpr int slot(int i) { return i + (i >> 4); }
+
+// Frequency j = a + 16 b of thread t, whose row of 16 slots is 256 a + 16 b and whose
+// frequencies are j + 256 r.  Warp w works on the digits a = w and 16 - w (w = 0: 8 and 0).
+// Lane and partner (lane ^ 16) own frequencies that mirror each other:
+// 4096 - (j + 256 r) = j' + 256 (15 - r).  j = 128 mirrors itself, and so does j = 0 but with
+// 256 (16 - r); these two threads are their own partners.
+__host__ __device__ constexpr int row_frequency(int t) {
+    const int w = t >> 5, l = t & 31, q = l & 7;
+    if (w != 0) return l < 16 ? w + 16 * l : 16 - w + 16 * (31 - l);
+    // warp 0: lanes 0-7 and 16-23 a = 8, b and 15 - b; lanes 8-15 and 24-31 a = 0, 16 - b and b
+    if (l & 8) return 16 * (l >= 16 ? q : q ? 16 - q : 8);
+    return 8 + 16 * (l < 16 ? q : 15 - q);
+}
+__device__ __forceinline__ bool owns_zero(int t) { return t == 24; }               // j = 0
+__device__ __forceinline__ int partner_of(int t) { return (t & ~16) == 8 ? t : (t & 31) ^ 16; }
+// Digit a of a thread in pass 2: one per half of the warp.
+__device__ __forceinline__ int col_digit(int t) {
+    const int w = t >> 5;
+    return (t & 16) ? (w ? 16 - w : 0) : (w ? w : 8);
+}
+
+struct Shared {
+    u64 re[PLANE], im[PLANE];
+    float4 w256[15][16];            // exp(-2 pi i k r / 256), doubled (x, x, y, y)
+};
+// tw: exp(-2 pi i k / M) at M / 2 + k.  The caller synchronises.
+__device__ __forceinline__ void fill_tables(Shared &sh, int t, const float2 *__restrict__ tw) {
+    if (t < 15 * 16) {
+        const int k = ((t >> 4) + 1) * (t & 15);
+        float2 w = __ldg(&tw[128 + (k & 127)]);
+        if (k & 128) w = make_float2(-w.x, -w.y);
+        (&sh.w256[0][0])[t] = make_float4(w.x, w.x, w.y, w.y);
+    }
+}
+// v[r] *= w[(r - 1) 16]
+__device__ __forceinline__ void twiddle_table(C2 *v, const float4 *w) {
+#pragma unroll
+    for (int r = 1; r < 16; ++r) {
+        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(w + (r - 1) * 16);
+        v[r] = times(v[r], W2{z.x, z.y});
+    }
+}
+template <int STEP>
+__device__ __forceinline__ void load16(C2 *v, const Shared &sh, int at) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r].re = sh.re[at + STEP * r];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r].im = sh.im[at + STEP * r];
+}
+template <int STEP>
+__device__ __forceinline__ void store16(const C2 *v, Shared &sh, int at) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        sh.re[at + STEP * r] = v[r].re;
+        sh.im[at + STEP * r] = v[r].im;
+    }
+}
+__device__ __forceinline__ int row_slot(int t) {
+    const int j = row_frequency(t);
+    return slot(256 * (j & 15) + (j & ~15));
+}
+__device__ __forceinline__ int col_slot(int t) { return slot(256 * col_digit(t)) + (t & 15); }
+
+// Samples t + 256 r in v -> frequencies j + 256 r in v.  The slots t + 256 r must be free for
+// this thread.
+__device__ __forceinline__ void forward4096(C2 *v, Shared &sh, int t, const float2 *__restrict__ tw) {
+    const float2 w1 = __ldg(&tw[2048 + t]);
+    dft16(v);
+    twiddle16(v, w1);
+    store16<slot(256)>(v, sh, slot(t));
+    __syncthreads();
+    load16<slot(16)>(v, sh, col_slot(t));
+    dft16(v);
+    twiddle_table(v, &sh.w256[0][t & 15]);
+    store16<slot(16)>(v, sh, col_slot(t));
+    __syncwarp();
+    load16<1>(v, sh, row_slot(t));
+    dft16(v);
+}
+// Frequencies j + 256 r in v, real and imaginary parts swapped -> 4096 times the samples
+// t + 256 r, swapped too.
+__device__ __forceinline__ void inverse4096(C2 *v, Shared &sh, int t, const float2 *__restrict__ tw) {
+    const float2 w1 = __ldg(&tw[2048 + row_frequency(t)]);
+    dft16(v);
+    twiddle16(v, w1);
+    store16<1>(v, sh, row_slot(t));
+    __syncwarp();
+    load16<slot(16)>(v, sh, col_slot(t));
+    dft16(v);
+    twiddle_table(v, &sh.w256[0][col_digit(t)]);
+    store16<slot(16)>(v, sh, col_slot(t));
+    __syncthreads();
+    load16<slot(256)>(v, sh, slot(t));
+    dft16(v);
+}
+// Give the partner frequencies v[8..15] and take its own: v[15 - r] becomes frequency
+// 4096 - (j + 256 r) for r < 8 (thread j = 0: for 0 < r < 8, and v[15] becomes frequency 2048).
+__device__ __forceinline__ void exchange_mirror(C2 *v, int t) {
+    const int partner = partner_of(t);
+    if (owns_zero(t)) {
+        const C2 x = v[8];
+#pragma unroll
+        for (int r = 8; r < 15; ++r) v[r] = v[r + 1];
+        v[15] = x;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 8; r < 16; ++r) v[r] = {shfl(v[r].re, partner), shfl(v[r].im, partner)};
+}
+// The way back.
+__device__ __forceinline__ void exchange_back(C2 *v, int t) {
+    const int partner = partner_of(t);
+#pragma unroll
+    for (int r = 8; r < 16; ++r) v[r] = {shfl(v[r].re, partner), shfl(v[r].im, partner)};
+    if (owns_zero(t)) {
+        const C2 x = v[15];
+#pragma unroll
+        for (int r = 15; r > 8; --r) v[r] = v[r - 1];
+        v[8] = x;
+    }
+    __syncwarp();
+}
+
 }  // namespace fftpair
