@@ -1,0 +1,70 @@
+"""The fused convolution where its blocks, loads and work list have edges, against the fp64
+checker: utterances that end with a block, one sample around it, within the first group of
+four; noise stretches at every offset from a 16-byte boundary, read inside one period, across
+its end, and looped many times; more units of work than resident CTAs."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1912_11040_b200 import binding, synth
+from helpers import check_wave
+
+pytestmark = pytest.mark.gpu
+TAPS = 300
+OB = (16384 - TAPS + 1) & ~3         # outputs per block
+
+
+def run(lengths, stretches, taps=TAPS, seed=0):
+    """stretches[b] = list of (offset, length); responses dense over `taps`."""
+    import torch
+    rng = np.random.default_rng(seed)
+    B, S = len(lengths), 1 + max(len(s) for s in stretches)
+    stride = (max(lengths) + 3) // 4 * 4
+    bank = (rng.standard_normal(60000) * 0.05).astype(np.float32)
+    speech = np.zeros((B, stride), np.float32)
+    tab = np.zeros(B, dtype=synth.UTT_DTYPE)
+    rir = np.zeros((B, S, taps), np.float32)
+    for b, n in enumerate(lengths):
+        speech[b, :n] = rng.standard_normal(n) * 0.05
+        tab[b]["n_src"], tab[b]["snr_db"] = 1 + len(stretches[b]), 3.0 * b - 4.0
+        for k, (o, m) in enumerate(stretches[b]):
+            tab[b]["noise_offset"][k], tab[b]["noise_len"][k], tab[b]["noise_weight"][k] = o, m, 1.0 - 0.3 * k
+        rir[b, : tab[b]["n_src"]] = rng.standard_normal((tab[b]["n_src"], taps)) * np.exp(-np.arange(taps) / (0.3 * taps)) * 0.1
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
+                            max_order=1, max_sources=S, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=stride,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    out = torch.full((B, stride), float("nan"), device="cuda")
+    ctx.aug_reverb_mix(cu(speech), stride, cu(np.array(lengths, np.int32)), cu(bank), bank.size, cu(rir),
+                       binding.table_to_device(tab), B, out)
+    got = out.cpu().numpy()
+    for b, n in enumerate(lengths):
+        noises = [oracle.looped_noise(bank, o, m, n) for o, m in stretches[b]]
+        ref, *_ = oracle.reverb_mix(speech[b, :n].astype(np.float64),
+                                    [rir[b, s].astype(np.float64) for s in range(int(tab[b]["n_src"]))], noises,
+                                    tab[b]["noise_weight"], tab[b]["snr_db"])
+        check_wave(got[b, :n], ref, f"utt {b} of {n} samples")
+        assert np.all(np.isnan(got[b, n:]))
+
+
+def test_lengths_around_a_block():
+    lengths = [OB, OB - 1, OB + 1, 2 * OB + 3, 3, 1, 401]
+    run(lengths, [[(8, 5000)]] * len(lengths))
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_stretches_at_any_offset(offset):
+    """50003 samples: blocks that lie inside the stretch, across its end, and at both ends of
+    the utterance; the short ones wrap inside a block; lengths that are multiples of 4 and not."""
+    lengths = [50003, 50003, 40000, 33000]
+    run(lengths, [[(100 + offset, 40000 + offset)], [(offset, 44000), (7 + offset, 321)], [], [(4 + offset, 7 + offset)]],
+        seed=offset)
+
+
+def test_more_units_than_resident_ctas():
+    """600 utterances of one block, both outputs: most units are drawn from the counter."""
+    rng = np.random.default_rng(4)
+    lengths = [int(n) for n in rng.integers(1, 900, 600)]
+    run(lengths, [[(4 * (b % 50), 200 + b)] if b % 3 else [] for b in range(600)], taps=50)
