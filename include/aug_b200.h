@@ -356,17 +356,17 @@ int aug_upload_noise_bank(AugCtx *ctx, const float *noise_bank_host, int64_t ban
 /* -------------------------------------------------------------- measurement utilities
  * (instrumentation of this library; the paper has no counterpart) */
 
-#define AUG_N_STAGES 7 /* 0 impulse responses, 1 response lengths and spectra, 2 filterbank tables
-                            (on a stream of their own beside stages 0 and 1: their time is the
-                            time they took there and is not part of the sum of the others),
+#define AUG_N_STAGES 7 /* 0 impulse responses, 1 response lengths and spectra, 2 filterbank tables,
                           3 waveform warp (vtlp_win > 0) and block spectra of the audio (contexts
                             sized for responses of more than 8192 taps),
-                          4 convolution, 5 waveform mix (only when requested), 6 features */
+                          4 convolution, 5 waveform mix (only when requested), 6 features.
+                          Without the events between them the stages overlap at their ends, so the
+                          sum is more than a call takes */
 
 /* The fused convolution (responses of up to 8192 taps) sums several noise sources of an
- * utterance in the frequency domain through parking slots in the workspace, three per
- * multiprocessor; a CTA that finds none free sums in the time domain instead.
- * hold != 0 marks every slot taken, so that this second way can be exercised and
+ * utterance in the frequency domain through parking slots in the workspace, one per
+ * resident CTA; a CTA whose slot is held sums in the time domain instead.
+ * hold != 0 marks every slot held, so that this second way can be exercised and
  * timed; hold == 0 frees them.  Synchronises the stream; call it only between
  * pipeline calls. */
 int aug_hold_parking_slots(AugCtx *ctx, int hold);

@@ -262,6 +262,8 @@ rir_length_kernel(const float *__restrict__ rir, const AugUttParams *__restrict_
                   int *__restrict__ leff, int *__restrict__ leff_all) {
     __shared__ int red_i[CT / 32];
     const int s = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
+    chain_next();
+    chain_wait();
     const AugUttParams &row = table[utt];
     if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
     const float *h = rir + ((int64_t)utt * S_max + s) * L;
@@ -304,6 +306,7 @@ rir_spectra_kernel(const float *__restrict__ rir, const AugUttParams *__restrict
                    const int *__restrict__ leff_all, int always) {
     extern __shared__ __align__(16) float2 sm[];
     const int p = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x;
+    chain_wait();
     if (!always && takes_fused_route(*leff_all)) return;
     const AugUttParams &row = table[utt];
     if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
@@ -324,6 +327,7 @@ rir_spectra_kernel(const float *__restrict__ rir, const AugUttParams *__restrict
         v[0][r] = z;
     }
     fft4096_from_regs(v, sm, t, tw);
+    chain_next();
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const int k = t + CT * q;
@@ -344,6 +348,7 @@ block_spectra_kernel(const float *__restrict__ speech, int64_t stride,
                      int *status, int n_cap, const int *__restrict__ leff_all, int always) {
     extern __shared__ __align__(16) float2 sm[];
     const int b = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x;
+    chain_wait();
     const int N = min(max(lengths[utt], 0), n_cap);
     if ((int64_t)b * BLK >= N || (!always && takes_fused_route(*leff_all))) return;
     const AugUttParams &row = table[utt];
@@ -357,6 +362,7 @@ block_spectra_kernel(const float *__restrict__ speech, int64_t stride,
     float2 v[1][E];
     load_block(v, x, s != 0, nlen, (b - 1) * BLK, N, t);
     fft4096_from_regs(v, sm, t, tw);
+    chain_next();
     float2 *out = xspec + (((int64_t)utt * S_max + s) * nblk_cap + b) * N2;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
@@ -379,6 +385,7 @@ spectral_convolve_kernel(const int *__restrict__ lengths, const float *__restric
     extern __shared__ __align__(16) float2 sm[];
     __shared__ float red[CT / 32];
     const int b = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
+    chain_wait();
     // partitions behind the last non-zero tap of every source of this utterance are zero
     const int P_used = min(P, (max(leff[utt], 1) + BLK - 1) / BLK);
     const int N = min(max(lengths[utt], 0), n_cap);
@@ -414,6 +421,7 @@ spectral_convolve_kernel(const int *__restrict__ lengths, const float *__restric
         float *dst = (o ? vv : ys) + (int64_t)utt * ws_stride + (int64_t)b * BLK;
         finish_block(acc, sm, tw, t, dst, N - b * BLK, &energy[2 * utt + o], red);
     }
+    chain_next();
     if (n_src <= 1) {
         float *dst = vv + (int64_t)utt * ws_stride + (int64_t)b * BLK;
         for (int i = t; i < BLK && b * BLK + i < N; i += CT) dst[i] = 0.f;
@@ -430,6 +438,8 @@ __global__ void __launch_bounds__(256)
 snr_gain_kernel(const double *__restrict__ energy, const AugUttParams *__restrict__ table, int B,
                 float *__restrict__ gain) {
     const int utt = blockIdx.x * 256 + threadIdx.x;
+    chain_next();
+    chain_wait();
     if (utt >= B) return;
     const double es = energy[2 * utt], ev = energy[2 * utt + 1];
     float g = 0.f;
@@ -446,6 +456,7 @@ mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t w
            const float *__restrict__ gain, const int *__restrict__ lengths,
            float *__restrict__ out, int64_t out_stride, int n_cap) {
     const int utt = blockIdx.y, tid = threadIdx.x;
+    chain_wait();
     const int N = min(max(lengths[utt], 0), n_cap);
     const int i0 = blockIdx.x * (MIX_GROUPS * 1024) + 4 * tid;
     if (blockIdx.x * (MIX_GROUPS * 1024) >= N) return;
@@ -700,6 +711,8 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
     fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
     __shared__ int red_i[CF / 32];
     const int s = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
+    fftpair::fill_tables(sh, t, tw);
+    chain_wait();
     // mixed: the lengths are known already (rir_length_kernel) and decide the route; otherwise
     // this kernel reads every tap anyway and records the length on the way
     if (mixed && !takes_fused_route(*leff_all)) return;
@@ -708,7 +721,6 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
     const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (4.f * (float)F2);
     const float *h = rir + ((int64_t)utt * S_max + s) * L;
     float4 *out = hspec + ((int64_t)utt * S_max + s) * (hs_stride / 2) + t;
-    fftpair::fill_tables(sh, t, tw);
     C2 v[NP2];
     int last = 0;
 #pragma unroll
@@ -739,6 +751,7 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
         if (m > 0) atomicMax(const_cast<int *>(&leff[utt]), m);
     }
     fftpair::forward4096(v, sh, t, tw);
+    chain_next();
     fftpair::exchange_mirror(v, t);
     const u64 sc = fftpair::both(scale);
     const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
@@ -780,6 +793,8 @@ plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restr
             int S_max, int n_cap, const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed,
             int *status, Plan *__restrict__ plans, Unit *__restrict__ units, int *__restrict__ n_units) {
     const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    chain_next();
+    chain_wait();
     if (utt >= B || (mixed && !takes_fused_route(*leff_all))) return;
     const AugUttParams &row = table[utt];
     const int N = min(max(lengths[utt], 0), n_cap);
@@ -842,7 +857,10 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
     // places for each.
     __shared__ Plan plan_s[3];
     __shared__ Unit unit_s[3];
-    const int t = threadIdx.x, count = *n_units, G = gridDim.x;
+    const int t = threadIdx.x, G = gridDim.x;
+    fftpair::fill_tables(sh, t, tw);
+    chain_wait();
+    const int count = __ldcg(n_units);
     int *drawn = n_units + 1;
     if (blockIdx.x >= count) return;
     if (t == 0) {
@@ -852,7 +870,6 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
     }
     if (t < (int)(sizeof(Plan) / 4))
         reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + units[blockIdx.x].utt)[t];
-    fftpair::fill_tables(sh, t, tw);
     __syncthreads();
     const bool own_slot = PARK && park != nullptr && park_flags[blockIdx.x] == 0;
 
@@ -862,6 +879,7 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
         const Unit cur = unit_s[k];
         const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
         const int next_utt = unit_s[k1].utt;
+        if (next_utt < 0) chain_next();        // the CTA's last unit
         if (next_utt >= 0 && t < (int)(sizeof(Plan) / 4))
             copy4_async(reinterpret_cast<float *>(&plan_s[k1]) + t,
                         reinterpret_cast<const float *>(plans + next_utt) + t, 4);
@@ -995,35 +1013,38 @@ static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_ST
 // response spectra of one (utterance, source): complex numbers between consecutive ones
 static int64_t hspec_stride(const AugCtx *ctx) { return stored_route(ctx) ? (int64_t)ctx->n_part * N2 : NB2; }
 
-int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table, int B,
-                       cudaStream_t st) {
+int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table, int B, bool reset) {
     const AugConfig &c = ctx->cfg;
+    const cudaStream_t st = ctx->stream;
     const int mixed = stored_route(ctx) ? 1 : 0;
     // long-response context: the last batch size seen decides whether the fused kernels are launched at all
     ctx->stored_only = mixed && ctx->leff_seen && *ctx->leff_seen > BLK2;
     int *leff_all = ctx->leff + ctx->cfg.max_batch;
-    AUG_CUDA_OK(cudaMemsetAsync(ctx->leff, 0, sizeof(int) * (size_t)B, st));
-    AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, 3 * sizeof(int), st));      // and the counters of the work list
+    if (reset) {
+        AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0, sizeof(double) * 2 * (size_t)B, st));
+        AUG_CUDA_OK(cudaMemsetAsync(ctx->leff, 0, sizeof(int) * (size_t)B, st));
+        AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, 3 * sizeof(int), st));      // and the counters of the work list
+    }
     dim3 grid2(c.max_sources, B);
     if (mixed) {
-        rir_length_kernel<<<grid2, CT, 0, st>>>(rir, table, c.max_sources, c.rir_taps, ctx->leff, leff_all);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(rir_length_kernel, grid2, CT, 0, st, rir, table, c.max_sources, c.rir_taps, ctx->leff,
+                           leff_all) != AUG_OK)
+            return AUG_ECUDA;
         ctx->launches++;
     }
     if (!ctx->stored_only) {
         if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
-        rir_spectra2_kernel<<<grid2, CF, FFT2_SMEM, st>>>(
-            rir, table, c.max_sources, c.rir_taps, ctx->tw, reinterpret_cast<float4 *>(ctx->hspec),
-            hspec_stride(ctx), ctx->leff, leff_all, mixed);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(rir_spectra2_kernel, grid2, CF, FFT2_SMEM, st, rir, table, c.max_sources, c.rir_taps,
+                           ctx->tw, reinterpret_cast<float4 *>(ctx->hspec), hspec_stride(ctx), ctx->leff, leff_all,
+                           mixed) != AUG_OK)
+            return AUG_ECUDA;
         ctx->launches++;
     }
     if (mixed) {
         dim3 grid(ctx->n_part, c.max_sources, B);
-        rir_spectra_kernel<<<grid, CT, FFT_SMEM, st>>>(rir, table, c.max_sources, c.rir_taps,
-                                                       ctx->n_part, ctx->tw, ctx->hspec, leff_all,
-                                                       ctx->stored_only);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(rir_spectra_kernel, grid, CT, FFT_SMEM, st, rir, table, c.max_sources, c.rir_taps,
+                           ctx->n_part, ctx->tw, ctx->hspec, leff_all, ctx->stored_only) != AUG_OK)
+            return AUG_ECUDA;
         ctx->launches++;
     }
     return AUG_OK;
@@ -1034,14 +1055,13 @@ int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, co
                             int max_len) {
     const AugConfig &c = ctx->cfg;
     if (max_len <= 0) return AUG_OK;
-    AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0, sizeof(double) * 2 * (size_t)B, ctx->stream));
     if (!stored_route(ctx)) return AUG_OK;
     const int nblk = (max_len + BLK - 1) / BLK;
     dim3 grid_x(nblk, c.max_sources, B);
-    block_spectra_kernel<<<grid_x, CT, FFT_SMEM, ctx->stream>>>(
-        speech, stride, lengths, bank, bank_len, table, c.max_sources, ctx->tw, ctx->xspec,
-        ctx->nblk_cap, ctx->status, max_len, ctx->leff + c.max_batch, ctx->stored_only);
-    AUG_CUDA_OK(cudaGetLastError());
+    if (launch_chained(block_spectra_kernel, grid_x, CT, FFT_SMEM, ctx->stream, speech, stride, lengths, bank,
+                       bank_len, table, c.max_sources, ctx->tw, ctx->xspec, ctx->nblk_cap, ctx->status, max_len,
+                       ctx->leff + c.max_batch, ctx->stored_only) != AUG_OK)
+        return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
 }
@@ -1054,11 +1074,11 @@ int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, con
     const int mixed = stored_route(ctx) ? 1 : 0;
     const int *leff_all = ctx->leff + c.max_batch;
     if (!ctx->stored_only) {
-        plan_kernel<<<(B + 7) / 8, 256, 0, ctx->stream>>>(
-            speech, stride, lengths, bank, bank_len, table, B, c.max_sources, max_len, ctx->leff, leff_all, mixed,
-            ctx->status, reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
-            ctx->leff + c.max_batch + 1);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, speech, stride, lengths, bank,
+                           bank_len, table, B, c.max_sources, max_len, ctx->leff, leff_all, mixed, ctx->status,
+                           reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
+                           ctx->leff + c.max_batch + 1) != AUG_OK)
+            return AUG_ECUDA;
         // as many CTAs as fit, but not more than there can be units of work (blocks are shortest
         // where a response fills min(rir_taps, 8192) taps)
         const int ob_min = (F2 - min(c.rir_taps, BLK2) + 1) & ~3;
@@ -1068,28 +1088,29 @@ int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, con
         if ((ctx->park ? smem_opt_in<convolve_fused2_kernel<true>>(ctx->device)
                        : smem_opt_in<convolve_fused2_kernel<false>>(ctx->device)) != AUG_OK)
             return AUG_ECUDA;
-        kern<<<grid2, CF, FFT2_SMEM, ctx->stream>>>(
-            reinterpret_cast<const Plan *>(ctx->plans), reinterpret_cast<const Unit *>(ctx->units),
-            ctx->leff + c.max_batch + 1, c.max_sources, reinterpret_cast<const float4 *>(ctx->hspec),
-            hspec_stride(ctx), ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->park, ctx->park_flags);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(kern, grid2, CF, FFT2_SMEM, ctx->stream, reinterpret_cast<const Plan *>(ctx->plans),
+                           reinterpret_cast<const Unit *>(ctx->units), ctx->leff + c.max_batch + 1, c.max_sources,
+                           reinterpret_cast<const float4 *>(ctx->hspec), hspec_stride(ctx), ctx->tw, ctx->ys, ctx->vv,
+                           ctx->ws_stride, ctx->energy, ctx->park, ctx->park_flags) != AUG_OK)
+            return AUG_ECUDA;
         ctx->launches += 2;
     }
     if (mixed) {
         const int nblk = (max_len + BLK - 1) / BLK;
         dim3 grid(nblk, B);
-        spectral_convolve_kernel<<<grid, CT, FFT_SMEM, ctx->stream>>>(
-            lengths, bank, bank_len, table, c.max_sources, ctx->n_part, ctx->hspec, ctx->xspec,
-            ctx->nblk_cap, ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, max_len, ctx->leff, leff_all,
-            ctx->stored_only);
-        AUG_CUDA_OK(cudaGetLastError());
+        if (launch_chained(spectral_convolve_kernel, grid, CT, FFT_SMEM, ctx->stream, lengths, bank, bank_len, table,
+                           c.max_sources, ctx->n_part, ctx->hspec, ctx->xspec, ctx->nblk_cap, ctx->tw, ctx->ys,
+                           ctx->vv, ctx->ws_stride, ctx->energy, max_len, ctx->leff, leff_all,
+                           ctx->stored_only) != AUG_OK)
+            return AUG_ECUDA;
         ctx->launches++;
         // for the next call's choice (not waited for)
         if (ctx->leff_seen)
             AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, leff_all, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     }
-    snr_gain_kernel<<<(B + 255) / 256, 256, 0, ctx->stream>>>(ctx->energy, table, B, ctx->gain);
-    AUG_CUDA_OK(cudaGetLastError());
+    if (launch_chained(snr_gain_kernel, dim3((B + 255) / 256), 256, 0, ctx->stream, ctx->energy, table, B,
+                       ctx->gain) != AUG_OK)
+        return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
 }
@@ -1098,9 +1119,9 @@ int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B
                float *wave_out, int64_t out_stride) {
     if (max_len <= 0) return AUG_OK;
     dim3 grid((max_len + MIX_GROUPS * 1024 - 1) / (MIX_GROUPS * 1024), B);
-    mix_kernel<<<grid, 256, 0, ctx->stream>>>(ctx->ys, ctx->vv, ctx->ws_stride, ctx->gain, lengths,
-                                              wave_out, out_stride, max_len);
-    AUG_CUDA_OK(cudaGetLastError());
+    if (launch_chained(mix_kernel, grid, 256, 0, ctx->stream, ctx->ys, ctx->vv, ctx->ws_stride, ctx->gain, lengths,
+                       wave_out, out_stride, max_len) != AUG_OK)
+        return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
 }

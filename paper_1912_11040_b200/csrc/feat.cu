@@ -24,8 +24,16 @@ __host__ __device__ __forceinline__ int frame_count(int n, int win, int hop) {
 // rounding), then the first bin of every interval.
 __global__ void __launch_bounds__(256)
 mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double f_lo,
-                  double f_hi, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped) {
+                  double f_hi, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped,
+                  int *leff, int *counters, double *energy) {
     __shared__ int seg_s[513];
+    chain_next();
+    // first kernel of aug_pipeline: the convolution's sums and counters start from zero
+    if (leff != nullptr && threadIdx.x == 0) {
+        leff[blockIdx.x] = 0;
+        energy[2 * blockIdx.x] = energy[2 * blockIdx.x + 1] = 0.0;
+        if (blockIdx.x == 0) counters[0] = counters[1] = counters[2] = 0;
+    }
     const int utt = blockIdx.x, nb = K / 2 + 1;
     // (unwarped: the warp was already applied to the waveform)
     const double a = unwarped ? 0.0 : 1.0 - (double)table[utt].alpha;
@@ -254,6 +262,13 @@ frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, in
 
     const int utt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int run0 = blockIdx.x * (FT * TILES);
+    for (int n = tid; n < K; n += FEAT_THREADS)
+        win_s[n] = n < win ? 0.25f - 0.25f * cospif(2.f * (float)n / (float)win) : 0.f;
+    if (tid < 32) {
+        const float2 w1 = __ldg(&tw[256 + tid]), wh = tid < 16 ? make_float2(1.f, 0.f) : __ldg(&tw[tid]);
+        reinterpret_cast<float4 *>(sm + lay.lanes)[tid] = make_float4(w1.x, w1.y, wh.x, wh.y);
+    }
+    chain_wait();
     const int N = min(max(lengths[utt], 0), n_cap);
     const int T = min(frame_count(N, win, hop), T_max);
     if (blockIdx.x == 0 && tid == 0) counts[utt] = T;
@@ -320,12 +335,6 @@ frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, in
     };
     if (lay.ahead) stage_issue(0);
 
-    for (int n = tid; n < K; n += FEAT_THREADS)
-        win_s[n] = n < win ? 0.25f - 0.25f * cospif(2.f * (float)n / (float)win) : 0.f;
-    if (tid < 32) {
-        const float2 w1 = __ldg(&tw[256 + tid]), wh = tid < 16 ? make_float2(1.f, 0.f) : __ldg(&tw[tid]);
-        reinterpret_cast<float4 *>(sm + lay.lanes)[tid] = make_float4(w1.x, w1.y, wh.x, wh.y);
-    }
     constexpr int RUNS = 2 * FEAT_THREADS / FT;       // runs of bands, one per FT / 2 lanes
     if (MODE == 1) {
         for (int k = tid; k < NBP; k += FEAT_THREADS) {
@@ -504,9 +513,13 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
     const int rows = min(LM_FT, T_max - t0);
     const int T = min(max(counts[utt], 0), T_max);
     const int nf = max(0, min(rows, T - t0));
+    // (the tables come from the kernel before; everything else was there when that one started)
     float *o = feats + ((int64_t)utt * T_max + t0) * M;
     fill_floats(o + nf * M, (rows - nf) * M, pad_v, tid, 256);
-    if (nf == 0) return;
+    if (nf == 0) {
+        chain_wait();
+        return;
+    }
     const float *p = power + ((int64_t)utt * T_max + t0) * NBP;
     const int n = nf * NBP, shift = (int)((reinterpret_cast<uintptr_t>(p) >> 2) & 3);
     const int head = min(n, (4 - shift) & 3), n4 = (n - head) >> 2;
@@ -519,6 +532,7 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
     if (tid < head) pt[tid] = p[tid];
     const int tail = head + 4 * n4 + tid;
     if (tail < n) pt[tail] = p[tail];
+    chain_wait();
     for (int k = tid; k < NBP; k += 256) {
         const aug::MelBin w = melw[(int64_t)utt * NBP + k];
         mw[k] = make_float2(w.up, w.down);
@@ -587,22 +601,29 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
     if ((runs ? smem_opt_in<frames_kernel<K, MODE, RUN_TILES>>(ctx->device)
               : smem_opt_in<frames_kernel<K, MODE, 1>>(ctx->device)) != AUG_OK)
         return AUG_ECUDA;
-    kern<<<grid, FEAT_THREADS, smem, ctx->stream>>>(
-        a, b, stride, ctx->gain, lengths, c.win, c.hop, c.n_mel, T_max, ctx->melw,
-        ctx->melstart, ctx->tw, c.log_floor, c.pad_value, c.compression, out, counts,
-        n_cap, lay);
-    AUG_CUDA_OK(cudaGetLastError());
+    // (MODE 0 reads what the caller's kernels wrote: launched the ordinary way)
+    if (MODE == 1) {
+        if (launch_chained(kern, grid, FEAT_THREADS, smem, ctx->stream, a, b, stride, ctx->gain, lengths, c.win, c.hop,
+                           c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw, c.log_floor, c.pad_value, c.compression,
+                           out, counts, n_cap, lay) != AUG_OK)
+            return AUG_ECUDA;
+    } else {
+        kern<<<grid, FEAT_THREADS, smem, ctx->stream>>>(
+            a, b, stride, ctx->gain, lengths, c.win, c.hop, c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw,
+            c.log_floor, c.pad_value, c.compression, out, counts, n_cap, lay);
+        AUG_CUDA_OK(cudaGetLastError());
+    }
     ctx->launches++;
     return AUG_OK;
 }
 
 }  // namespace
 
-int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, cudaStream_t st) {
+int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset) {
     const AugConfig &c = ctx->cfg;
-    mel_tables_kernel<<<B, 256, 0, st>>>(table, c.n_fft, c.n_mel, (double)c.fs,
-                                                  (double)c.f_lo, (double)c.f_hi, ctx->melw,
-                                                  ctx->melstart, c.vtlp_win > 0 ? 1 : 0);
+    mel_tables_kernel<<<B, 256, 0, ctx->stream>>>(
+        table, c.n_fft, c.n_mel, (double)c.fs, (double)c.f_lo, (double)c.f_hi, ctx->melw, ctx->melstart,
+        c.vtlp_win > 0 ? 1 : 0, reset ? ctx->leff : nullptr, ctx->leff + c.max_batch, ctx->energy);
     AUG_CUDA_OK(cudaGetLastError());
     ctx->launches++;
     return AUG_OK;
@@ -634,10 +655,9 @@ int launch_logmel(AugCtx *ctx, const float *power, const int *counts, int B, int
     const int NBP = ctx->n_bins;
     if (smem_opt_in<logmel_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
     dim3 grid((T_max + LM_FT - 1) / LM_FT, B);
-    logmel_kernel<<<grid, 256, logmel_smem(NBP, c.n_mel), ctx->stream>>>(power, counts, NBP, c.n_mel, T_max, ctx->melw,
-                                                    ctx->melstart, c.log_floor, c.pad_value,
-                                                    c.compression, feats);
-    AUG_CUDA_OK(cudaGetLastError());
+    if (launch_chained(logmel_kernel, grid, 256, logmel_smem(NBP, c.n_mel), ctx->stream, power, counts, NBP, c.n_mel,
+                       T_max, ctx->melw, ctx->melstart, c.log_floor, c.pad_value, c.compression, feats) != AUG_OK)
+        return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
 }
@@ -717,7 +737,8 @@ extern "C" int feat_vtlp_logmel_noalloc(const AugConfig *cfg, const float *power
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int nbp = cfg->n_fft / 2 + 1;
     mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs,
-                                         (double)cfg->f_lo, (double)cfg->f_hi, melw, melstart, 0);
+                                         (double)cfg->f_lo, (double)cfg->f_hi, melw, melstart, 0, nullptr,
+                                         nullptr, nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     int dev = -1;
     AUG_CUDA_OK(cudaGetDevice(&dev));

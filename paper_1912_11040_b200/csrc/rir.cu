@@ -93,6 +93,7 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
         if (bad && tid == 0 && s == 0) {
             if (atomicCAS(&status[0], -1, utt) == -1) status[1] = bad;
         }
+        chain_wait();
         return;
     }
 
@@ -242,6 +243,7 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
         __syncwarp();   // the ring slots are rewritten by the next batch
     }
     __syncthreads();
+    chain_next();
     if ((reinterpret_cast<uintptr_t>(out) & 15) == 0 && (L & 3) == 0) {
         for (int i = tid; i < (L >> 2); i += THREADS) {
             const int4 q = reinterpret_cast<const int4 *>(h)[i];
@@ -251,20 +253,27 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
     } else {
         for (int i = tid; i < L; i += THREADS) out[i] = (float)h[i] * inv_scale;
     }
+    chain_wait();
 }
 
 }  // namespace
 
-int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, cudaStream_t st) {
+int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
     const AugConfig &c = ctx->cfg;
     const size_t smem = rir_smem_bytes(THREADS, c.rir_taps);
     const double fs_over_c = (double)c.fs / (double)c.sound_speed;
     const int cube = c.image_lattice == AUG_LATTICE_CUBE ? 1 : 0;
     dim3 grid(c.max_sources, B);
     if (smem_opt_in<rir_image_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
-    rir_image_kernel<<<grid, THREADS, smem, st>>>(table, c.max_sources, c.rir_taps, c.frac_half_width,
-                                                  fs_over_c, c.max_order, cube, rir, ctx->status);
-    AUG_CUDA_OK(cudaGetLastError());
+    if (beside) {
+        if (launch_chained(rir_image_kernel, grid, THREADS, smem, ctx->stream, table, c.max_sources, c.rir_taps,
+                           c.frac_half_width, fs_over_c, c.max_order, cube, rir, ctx->status) != AUG_OK)
+            return AUG_ECUDA;
+    } else {
+        rir_image_kernel<<<grid, THREADS, smem, ctx->stream>>>(table, c.max_sources, c.rir_taps, c.frac_half_width,
+                                                               fs_over_c, c.max_order, cube, rir, ctx->status);
+        AUG_CUDA_OK(cudaGetLastError());
+    }
     ctx->launches++;
     return AUG_OK;
 }
