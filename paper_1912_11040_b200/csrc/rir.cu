@@ -8,13 +8,21 @@
 //      an integer n0 and a fraction phi; the five numbers the taps need are
 //      written, compacted over the images that contribute, to a slot of a small
 //      shared-memory ring owned by the warp.
-//   B  one image at a time, its 2 W_h + 1 taps over the lanes: lane l owns taps
-//      l, l + 32, l + 64, so everything that depends only on the tap (its offset,
-//      the cosine and sine of its Hann angle, its sign) sits in registers, and
-//      the image's numbers arrive with two broadcast loads.  With tau = n0 + phi,
+//   B  two images at a time, their 2 W_h taps over the lanes: lane l owns taps l and l + 32
+//      of both, and of the 16 taps that are left (W_h = 40) the lower half-warp does those of
+//      the first image and the upper half those of the second.  Everything that depends only
+//      on the tap (its offset, the cosine and sine of its Hann angle, its sign) sits in
+//      registers, and the images' numbers arrive as pairs, the operands of packed (f32x2)
+//      arithmetic, by broadcast loads.  With tau = n0 + phi, 0 <= phi < 1,
 //      sin(pi (n - tau)) = -(-1)^(n - n0) sin(pi phi), and the Hann factor follows
-//      from the angle-sum identity, so a tap costs one reciprocal, three FMAs
-//      and one shared-memory reduction.
+//      from the angle-sum identity, so a tap costs one reciprocal, three to four fused
+//      multiply-adds -- the last one adds 1.5 2^23, which leaves the fixed-point value in the
+//      low bits -- and one shared-memory reduction.  n0 is rounded down so that the window
+//      always covers the same taps -W_h + 1 .. W_h and none has to be masked.
+//
+// Bound by instruction issue (45 warp instructions an image, 72 % of the slots).  One image at
+// a time in scalar arithmetic, with a conversion instruction per tap and masks, it was 58, and
+// the quarter-rate pipe of reciprocals and conversions was 62 % busy too.
 //
 // The response is accumulated in 32-bit fixed point: a shared-memory fp32 atomic
 // add is a compare-and-swap loop on this hardware, an integer one is a single
@@ -30,6 +38,7 @@
 // prefix over kx, then closed forms inside the diamond of (ky, kz)), so every
 // lane of a warp carries a real image.
 #include "common.cuh"
+#include "fft_pair.cuh"
 
 namespace {
 
@@ -56,27 +65,42 @@ __device__ __forceinline__ void red_shared_add(unsigned a, int iv) {
 // Bytes of dynamic shared memory of a CTA of `threads` threads for responses of L taps.
 __host__ __device__ constexpr size_t rir_smem_bytes(int threads, int L) {
     return sizeof(double) * 3 * AX + sizeof(float) * 3 * AX + sizeof(int) * (AX + 3) +
-           sizeof(float4) * threads + sizeof(float) * threads + sizeof(float) * (size_t)((L + 3) & ~3);
+           5 * sizeof(float) * threads + sizeof(float) * (size_t)((L + 3) & ~3);
 }
 
-#ifndef RIR_THREADS
-#define RIR_THREADS 512
-#endif
-#ifndef RIR_MINB
-#define RIR_MINB 3
-#endif
-constexpr int THREADS = RIR_THREADS;      // 16 warps; two or three CTAs per multiprocessor
 constexpr float HEADROOM_LOG2 = 6.f;   // full scale = 2^6 times the direct-path amplitude
 
-__global__ void __launch_bounds__(THREADS, RIR_MINB)
+// Entries of a warp's ring, each an array of 32: delay (first sample of the window plus BIAS; the bit
+// STRONG set if the image's taps may exceed 2^22 steps), phi, P0, P1, P2.
+enum Ring { R_N = 0, R_PHI = 32, R_P0 = 64, R_P1 = 96, R_P2 = 128, RING = 160 };
+constexpr int STRONG = 1 << 29, BIAS = 64;
+static_assert(BIAS >= aug::MAX_HALF_W, "delays are not negative");
+
+// round(v) by additions (the conversion instruction shares the quarter-rate pipe with the
+// reciprocals): adding 1.5 2^23 leaves the nearest integer, |v| < 2^22, in the low bits.
+constexpr float TO_INT = 12582912.f;
+constexpr int INT_BITS = 0x4B400000;
+// Images as loud as the direct path reach 2^25 steps: multiples of 16 first, then the rest.
+__device__ __forceinline__ int2 round_strong(fftpair::u64 v) {
+    using namespace fftpair;
+    const u64 m = both(TO_INT);
+    const u64 t = fma2(v, both(0.0625f), m);
+    const u64 rest = add2(fma2(sub2(m, t), both(16.f), v), m);
+    const float2 hi = unpack(t), lo = unpack(rest);
+    return make_int2(16 * __float_as_int(hi.x) + __float_as_int(lo.x) - (int)(17u * INT_BITS),
+                     16 * __float_as_int(hi.y) + __float_as_int(lo.y) - (int)(17u * INT_BITS));
+}
+
+// NARROW: half_w <= 40, at most 80 taps.
+template <bool NARROW, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int half_w,
                  double fs_over_c, int max_order, int cube, float *__restrict__ rir, int *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *ring4 = reinterpret_cast<float4 *>(smem_raw);          // [THREADS] n0, phi, P0, P1 of an image
-    int *h = reinterpret_cast<int *>(ring4 + THREADS);             // [L rounded up to 4] fixed-point response
+    int *ring = reinterpret_cast<int *>(smem_raw);                 // [THREADS / 32][RING]
+    int *h = ring + THREADS / 32 * RING;                           // [L rounded up to 4] fixed-point response
     double *dsq = reinterpret_cast<double *>(h + ((L + 3) & ~3));  // [3][AX] squared coordinate differences
-    float *ring1 = reinterpret_cast<float *>(dsq + 3 * AX);        // [THREADS] P2
-    float *gain = ring1 + THREADS;                                 // [3][AX] wall gains per axis
+    float *gain = reinterpret_cast<float *>(dsq + 3 * AX);         // [3][AX] wall gains per axis
     int *xpre = reinterpret_cast<int *>(gain + 3 * AX);            // [AX + 1] images before slab kx
 
     const int utt = blockIdx.y, s = blockIdx.x;
@@ -125,33 +149,34 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
     const float e2 = d0sq > 0.f ? floorf(31.f - HEADROOM_LOG2 + 0.5f * log2f(d0sq)) : 0.f;
     const float scale = exp2f(fminf(fmaxf(e2, -60.f), 60.f)), inv_scale = exp2f(-fminf(fmaxf(e2, -60.f), 60.f));
 
-    // Per-lane tap constants: this lane owns taps j = lane + 32 i - half_w, i < 3.  The
-    // sign (-1)^j is the same for all three and is folded into the Hann constants; a
-    // tap beyond 2 half_w gets an offset no window reaches.
+    // Per-lane tap constants.  Tap jj = 0 .. 2 half_w - 1 lies at offset j = jj - half_w + 1 from n0.
+    // The sign (-1)^j (with that of the sine) is the same for all taps of a lane; it goes into the
+    // offset, whose reciprocal is taken.  A tap beyond the window gets an offset so large that its
+    // value rounds to zero.
+    using fftpair::u64;
     const float fhw = (float)half_w;
-    const float sgn = ((lane - half_w) & 1) ? -1.f : 1.f;
+    const float sgn = ((lane - half_w + 1) & 1) ? -1.f : 1.f;
     float fj[3], cj[3], sj[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const int jj = lane + 32 * i, j = jj - half_w;
-        fj[i] = jj <= 2 * half_w ? (float)j : 3e9f;
-        cj[i] = sgn * cospif((float)j / fhw);
-        sj[i] = sgn * sinpif((float)j / fhw);
+        const int jj = i < 2 ? lane + 32 * i : NARROW ? 64 + (lane & 15) : 64 + lane, j = jj - half_w + 1;
+        fj[i] = jj < 2 * half_w ? sgn * (float)j : 3e18f;
+        cj[i] = cospif((float)j / fhw);
+        sj[i] = sinpif((float)j / fhw);
     }
+    const u64 nsgn = fftpair::both(-sgn);
     constexpr int NW = THREADS / 32;
-    const unsigned h_addr = (unsigned)__cvta_generic_to_shared(h);
-    // first-tap samples for which all 96 lane slots (81 of them taps) stay inside the response
+    const unsigned h_addr = (unsigned)__cvta_generic_to_shared(h) + 4u * lane - 4u * BIAS;
+    // first-tap samples for which all 96 lane slots (80 of them taps) stay inside the response
     const unsigned inside = (unsigned)max(L - 96, 0);
-    const bool mid_always = half_w >= 32;                       // taps 32..63 lie inside every window
-    float4 *my4 = ring4 + warp * 32;
-    float *my1 = ring1 + warp * 32;
+    int *my = ring + warp * RING;
 
     for (int base = warp * 32; base < total; base += NW * 32) {
         // ---- phase A: one image per lane
         const int idx = base + lane;
         bool valid = idx < total;
-        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-        float p2 = 0.f;
+        int n_first = BIAS;
+        float phi = 0.5f, p0 = 0.f, p1 = 0.f, p2 = 0.f;
         if (valid) {
             int ix, ky, kz;
             if (cube) {
@@ -189,54 +214,113 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             double d = d2 * rd;
             d = fma(0.5 * rd, fma(-d, d, d2), d);
             const double tau = d * fs_over_c;
-            const int n0 = __double2int_rn(tau);
-            float phi = (float)(tau - (double)n0);
+            int n0 = __double2int_rd(tau);
+            phi = (float)(tau - (double)n0);
+            if (phi >= 1.f) {                  // rounded up to the next sample
+                ++n0;
+                phi = 0.f;
+            }
             // a fraction of exactly zero would make the centre tap 0/0: 1e-7 of a sample
             // away from it the tap is the same to 3e-7 of its size
-            if (fabsf(phi) < 1e-7f) phi = copysignf(1e-7f, phi);
+            phi = fmaxf(phi, 1e-7f);
+            n_first = n0 - half_w + 1 + BIAS;
             const float A = g * (float)rd;
-            valid = d2 > 0.0 && A != 0.f && n0 - half_w < L;
+            valid = d2 > 0.0 && A != 0.f && n_first < L + BIAS;
+            // no tap is larger than A
+            if (fabsf(A) * scale >= 4194303.f) n_first |= STRONG;
             const float As = -A * scale * sinpif(phi) * 0.318309886183790671538f;
             float sps, cps;
             sincospif(phi / fhw, &sps, &cps);
-            q = make_float4(__int_as_float(n0), phi, 0.5f * As, 0.5f * As * cps);
-            p2 = 0.5f * As * sps;
+            p0 = 0.5f * As;
+            p1 = p0 * cps;
+            p2 = p0 * sps;
         }
         const unsigned mask = __ballot_sync(0xffffffffu, valid);
-        if (valid) {
-            const int pos = __popc(mask & ((1u << lane) - 1u));
-            my4[pos] = q;
-            my1[pos] = p2;
+        const int cnt = __popc(mask);
+        {
+            // contributing images to the front; one that adds nothing pairs with an odd last one
+            const int pos = valid ? __popc(mask & ((1u << lane) - 1u)) : cnt + __popc(~mask & ((1u << lane) - 1u));
+            if (!valid) {
+                n_first = BIAS;
+                phi = 0.5f;
+                p0 = p1 = p2 = 0.f;
+            }
+            my[R_N + pos] = n_first;
+            my[R_PHI + pos] = __float_as_int(phi);
+            my[R_P0 + pos] = __float_as_int(p0);
+            my[R_P1 + pos] = __float_as_int(p1);
+            my[R_P2 + pos] = __float_as_int(p2);
         }
         __syncwarp();
-        // ---- phase B: the taps of one image over the lanes
-        const int cnt = __popc(mask);
-        for (int k = 0; k < cnt; ++k) {
-            const float4 im = my4[k];
-            const float P2 = my1[k];
-            const int n_first = __float_as_int(im.x) - half_w;      // sample of tap -half_w
-            const float phi = im.y, P0 = sgn * im.z, P1 = im.w;
-            // A sinc(x) hann(x) = (1/x) (-A sin(pi phi)/pi) (-1)^j (1/2 + 1/2 cos(pi x / W_h)), x = j - phi
-            if ((unsigned)n_first < inside) {
-                // every tap of the window falls inside the response: no index checks, the
-                // three adds go to fixed offsets from one address
-                const unsigned a = h_addr + 4u * (unsigned)(n_first + lane);
-                // (a predicated reduction compiles to a branch around it: a tap outside the
-                // window adds zero instead; taps 32..63 are always inside it)
-                const float x0 = fj[0] - phi, x1 = fj[1] - phi, x2 = fj[2] - phi;
-                const float v0 = rcp_approx(x0) * fmaf(sj[0], P2, fmaf(cj[0], P1, P0));
-                const float v1 = rcp_approx(x1) * fmaf(sj[1], P2, fmaf(cj[1], P1, P0));
-                const float v2 = rcp_approx(x2) * fmaf(sj[2], P2, fmaf(cj[2], P1, P0));
-                red_shared_add<0>(a, __float2int_rn(fabsf(x0) <= fhw ? v0 : 0.f));
-                red_shared_add<128>(a, __float2int_rn(mid_always ? v1 : (fabsf(x1) <= fhw ? v1 : 0.f)));
-                red_shared_add<256>(a, __float2int_rn(fabsf(x2) <= fhw ? v2 : 0.f));
-            } else {
+        // ---- phase B: the taps of two images over the lanes
+        // A sinc(x) hann(x) = (1/x) (-A sin(pi phi)/pi) (-1)^j (1/2 + 1/2 cos(pi x / W_h)), x = j - phi
+        for (int k = 0; k < cnt; k += 2) {
+            using namespace fftpair;
+            const int2 n = *reinterpret_cast<const int2 *>(my + R_N + k);
+            const int na = n.x & ~STRONG, nb = n.y & ~STRONG;
+            if ((unsigned)(na - BIAS) < inside && (unsigned)(nb - BIAS) < inside) {
+                // every tap of both windows falls inside the response: no index checks, the adds of an
+                // image go to fixed offsets from one address
+                const u64 ph = *reinterpret_cast<const u64 *>(my + R_PHI + k);
+                const u64 q0 = *reinterpret_cast<const u64 *>(my + R_P0 + k);
+                const u64 q1 = *reinterpret_cast<const u64 *>(my + R_P1 + k);
+                const u64 q2 = *reinterpret_cast<const u64 *>(my + R_P2 + k);
+                const unsigned a = h_addr + 4u * (unsigned)na, b = h_addr + 4u * (unsigned)nb;
+                const bool strong = ((n.x | n.y) & STRONG) != 0;
+                constexpr int PAIRS = NARROW ? 2 : 3;
+                u64 rx[PAIRS], num[PAIRS];
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const float x = fj[i] - phi;
-                    const int n = n_first + lane + 32 * i;
-                    const float v = rcp_approx(x) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
-                    if (fabsf(x) <= fhw && (unsigned)n < (unsigned)L) atomicAdd(&h[n], __float2int_rn(v));
+                for (int i = 0; i < PAIRS; ++i) {
+                    const float2 x = unpack(fma2(nsgn, ph, both(fj[i])));
+                    rx[i] = pack(rcp_approx(x.x), rcp_approx(x.y));
+                    num[i] = fma2(both(sj[i]), q2, fma2(both(cj[i]), q1, q0));
+                }
+                float rs = 0.f, nums = 0.f;
+                if (NARROW) {
+                    // the last 16 taps, lower half-warp: first image, upper half: second
+                    const int w = k + (lane >> 4);
+                    rs = rcp_approx(fmaf(-sgn, __int_as_float(my[R_PHI + w]), fj[2]));
+                    nums = fmaf(sj[2], __int_as_float(my[R_P2 + w]),
+                                fmaf(cj[2], __int_as_float(my[R_P1 + w]), __int_as_float(my[R_P0 + w])));
+                }
+                int2 t[PAIRS];
+                int ts = 0;
+                if (!strong) {
+#pragma unroll
+                    for (int i = 0; i < PAIRS; ++i) {
+                        const float2 v = unpack(fma2(rx[i], num[i], both(TO_INT)));
+                        t[i] = make_int2(__float_as_int(v.x) - INT_BITS, __float_as_int(v.y) - INT_BITS);
+                    }
+                    if (NARROW) ts = __float_as_int(fmaf(rs, nums, TO_INT)) - INT_BITS;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < PAIRS; ++i) t[i] = round_strong(mul2(rx[i], num[i]));
+                    if (NARROW) ts = __float2int_rn(rs * nums);
+                }
+                red_shared_add<0>(a, t[0].x);
+                red_shared_add<0>(b, t[0].y);
+                red_shared_add<128>(a, t[1].x);
+                red_shared_add<128>(b, t[1].y);
+                if (NARROW) {
+                    red_shared_add<256>(lane < 16 ? a : b - 64u, ts);
+                } else {
+                    red_shared_add<256>(a, t[PAIRS - 1].x);
+                    red_shared_add<256>(b, t[PAIRS - 1].y);
+                }
+            } else {
+#pragma unroll 1
+                for (int w = k; w < min(k + 2, cnt); ++w) {
+                    const int n_f = (my[R_N + w] & ~STRONG) - BIAS;
+                    const float f = __int_as_float(my[R_PHI + w]), P0 = __int_as_float(my[R_P0 + w]);
+                    const float P1 = __int_as_float(my[R_P1 + w]), P2 = __int_as_float(my[R_P2 + w]);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        const float x = fmaf(-sgn, f, fj[i]);
+                        const int m = n_f + lane + 32 * i;
+                        const float v = rcp_approx(x) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
+                        const bool mine = !NARROW || i < 2 || lane < 16;
+                        if (mine && (unsigned)m < (unsigned)L) atomicAdd(&h[m], __float2int_rn(v));
+                    }
                 }
             }
         }
@@ -258,22 +342,38 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
 
 }  // namespace
 
-int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
+template <int THREADS>
+static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
     const AugConfig &c = ctx->cfg;
     const size_t smem = rir_smem_bytes(THREADS, c.rir_taps);
     const double fs_over_c = (double)c.fs / (double)c.sound_speed;
     const int cube = c.image_lattice == AUG_LATTICE_CUBE ? 1 : 0;
     dim3 grid(c.max_sources, B);
-    if (smem_opt_in<rir_image_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
+    const bool narrow = c.frac_half_width <= 40;
+    auto kern = narrow ? rir_image_kernel<true, THREADS> : rir_image_kernel<false, THREADS>;
+    if ((narrow ? smem_opt_in<rir_image_kernel<true, THREADS>>(ctx->device)
+                : smem_opt_in<rir_image_kernel<false, THREADS>>(ctx->device)) != AUG_OK)
+        return AUG_ECUDA;
     if (beside) {
-        if (launch_chained(rir_image_kernel, grid, THREADS, smem, ctx->stream, table, c.max_sources, c.rir_taps,
-                           c.frac_half_width, fs_over_c, c.max_order, cube, rir, ctx->status) != AUG_OK)
+        if (launch_chained(kern, grid, THREADS, smem, ctx->stream, table, c.max_sources, c.rir_taps, c.frac_half_width,
+                           fs_over_c, c.max_order, cube, rir, ctx->status) != AUG_OK)
             return AUG_ECUDA;
     } else {
-        rir_image_kernel<<<grid, THREADS, smem, ctx->stream>>>(table, c.max_sources, c.rir_taps, c.frac_half_width,
-                                                               fs_over_c, c.max_order, cube, rir, ctx->status);
+        kern<<<grid, THREADS, smem, ctx->stream>>>(table, c.max_sources, c.rir_taps, c.frac_half_width, fs_over_c,
+                                                   c.max_order, cube, rir, ctx->status);
         AUG_CUDA_OK(cudaGetLastError());
     }
     ctx->launches++;
     return AUG_OK;
+}
+
+// Both sizes keep 32 warps with 64 registers on a multiprocessor.  Four CTAs of 256 threads
+// balance better where the responses fit four times and there are enough of them: 4096 x 2
+// responses of 4096 taps 355 us against 399 with two of 512, 512 x 4 of 8192 taps 204 against
+// 213.  Long responses fit twice (128 x 4 of 24000 taps: 313 against 383), and a few responses
+// are done sooner by more warps each (8 x 2: 12.7 against 14.8).
+int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
+    const bool fit = 4 * (rir_smem_bytes(256, ctx->cfg.rir_taps) + 1024) <= (size_t)ctx->smem_per_sm;
+    const bool many = (int64_t)B * ctx->cfg.max_sources >= 4 * (int64_t)ctx->sm_count;
+    return fit && many ? launch_rir_as<256>(ctx, table, B, rir, beside) : launch_rir_as<512>(ctx, table, B, rir, beside);
 }

@@ -1,0 +1,41 @@
+"""The response kernel at the edges of its windows, buffers and CTA sizes: half widths on both
+sides of 40 (where the window stops fitting two and a half taps a lane) and the smallest,
+buffers shorter than a window, images that begin before or end behind the buffer, odd
+numbers of images, and batches large enough for the 256-thread CTAs."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1912_11040_b200 import binding, synth
+from helpers import RIR_REL_TOL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("half_w", [1, 16, 39, 40, 41, 47])
+@pytest.mark.parametrize("taps,B", [(60, 3), (97, 3), (700, 3), (333, 600)])
+def test_windows_and_buffers(half_w, taps, B):
+    import torch
+    rng = np.random.default_rng(half_w * taps + B)
+    tab = np.zeros(B, dtype=synth.UTT_DTYPE)
+    tab["n_src"], tab["order"] = 1, rng.integers(0, 4, B)
+    for b in range(B):
+        tab[b]["room"] = rng.uniform(0.8, 6.0, 3)
+        tab[b]["beta"] = rng.uniform(0.2, 1.0, 6)
+        tab[b]["mic"] = tab[b]["room"] * rng.uniform(0.1, 0.45, 3)
+        tab[b]["src_pos"][0] = tab[b]["room"] * rng.uniform(0.5, 0.9, 3)
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
+                            max_order=3, max_sources=1, frac_half_width=half_w, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=4,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    out = torch.full((B, 1, taps), float("nan"), device="cuda")
+    ctx.aug_rir_image_method(binding.table_to_device(tab), B, out)
+    h = out.cpu().numpy()[:, 0]
+    for b in range(0, B, 1 if B < 10 else 29):
+        r = tab[b]
+        ref = oracle.rir_image_method(r["room"], r["beta"], r["mic"], r["src_pos"][0], int(r["order"]), taps,
+                                      half_width=half_w)
+        # fixed-point steps follow the direct path, which may lie behind a short buffer
+        d0 = np.linalg.norm(r["mic"].astype(np.float64) - r["src_pos"][0])
+        assert np.max(np.abs(h[b] - ref)) <= RIR_REL_TOL * max(np.max(np.abs(ref)), 1.0 / d0), b
