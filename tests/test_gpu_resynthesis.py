@@ -1,0 +1,38 @@
+"""The waveform warp in runs of several rounds per CTA: batches large enough for them, windows
+whose hop is a multiple of four (samples are added four at a time), even, and odd, the longest
+window, utterances that end inside every part of a run."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1912_11040_b200 import binding, synth
+from helpers import check_wave
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("win,n_max,B", [(64, 9000, 64), (60, 9000, 64), (56, 3001, 200), (800, 30000, 160),
+                                         (1024, 13000, 600)])
+def test_runs_of_rounds(win, n_max, B):
+    import torch
+    rng = np.random.default_rng(win)
+    lengths = rng.integers(1, n_max + 1, B).astype(np.int32)
+    lengths[0], lengths[1] = n_max, 0
+    stride = (n_max + 3) // 4 * 4
+    speech = (rng.standard_normal((B, stride)) * 0.05).astype(np.float32)
+    tab = np.zeros(B, dtype=synth.UTT_DTYPE)
+    tab["alpha"] = rng.uniform(0.8, 1.2, B)
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=64,
+                            max_order=1, max_sources=1, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=stride,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=win, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    out = torch.full((B, stride), float("nan"), device="cuda")
+    ctx.aug_vtlp_resynth(torch.from_numpy(speech).cuda(), stride, torch.from_numpy(lengths).cuda(),
+                         binding.table_to_device(tab), B, out, stride)
+    got = out.cpu().numpy()
+    for b in [0, 1] + list(range(2, B, max(1, B // 12))):
+        n = int(lengths[b])
+        check_wave(got[b, :n], oracle.vtlp_resynth(speech[b, :n].astype(np.float64), float(tab[b]["alpha"]), win),
+                   f"utt {b} of {n} samples")
+        assert np.all(np.isnan(got[b, n:]))
