@@ -910,15 +910,20 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
                     fate = j == j_last ? PARK_JOIN : j > 1 ? PARK_MORE : PARK_FIRST;
                 C2 v[NP2];
                 load_segment(v, sh, p.x[j], noise, p.nlen[j], (b + 1) * p.ob - F2, p.N, t);
-                fftpair::forward4096(v, sh, t, tw);
+                // the response's bins are brought into L2 meanwhile (they may have been pushed out by the
+                // audio), and the first two slots' requested before the exchange
                 const float4 *H = hspec + ((int64_t)cur.utt * S_max + p.src[j]) * (hs_stride / 2) + t;
-                Bins h = load_bins(H);
+                if (t == 0)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(H), "n"(8 * NB2) : "memory");
+                fftpair::forward4096(v, sh, t, tw);
+                Bins h = load_bins(H), h1 = load_bins(H + 2 * CF);
                 const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
                 fftpair::exchange_mirror(v, t);
 #pragma unroll
                 for (int r = 0; r < NS2; ++r) {
                     const Bins hc = h;
-                    if (r + 1 < NS2) h = load_bins(H + 2 * (r + 1) * CF);   // the next slot's meanwhile
+                    h = h1;
+                    if (r + 2 < NS2) h1 = load_bins(H + 2 * (r + 2) * CF);
                     const bool edge = r == 0 && fftpair::owns_zero(t);
                     const SplitTwiddle w(u, r);
                     Bins y;
