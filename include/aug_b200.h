@@ -329,7 +329,8 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
  * back, and the call returns after synchronising, so the host buffers are free
  * again.  The longest rows of a chunk go by the copy engine while the kernel fetches
  * the others, and valid feature rows are written by a kernel straight into a pinned
- * (mapped) feature buffer, else by one copy per utterance.  Internally the batch is cut into up to 8 chunks of utterances that are
+ * (mapped) feature buffer, else by one copy per utterance.  Internally the batch is cut into up to 8 chunks of
+ * sixteen or more utterances that are
  * copied in, computed and copied out concurrently on three streams; speech rows
  * are copied only up to their length when that saves more than the extra copy
  * calls cost.  Host buffers should be pinned: copies then run asynchronously, and

@@ -22,7 +22,7 @@ inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 // size (about 40 of 54 GB/s each), so a chunk's longest rows, AUG_DMA_SHARE_PCT percent
 // of its samples, go by the copy engine at the same time on a stream of their own.
 #ifndef AUG_DMA_SHARE_PCT
-#define AUG_DMA_SHARE_PCT 40
+#define AUG_DMA_SHARE_PCT 60
 #endif
 #ifndef AUG_COPY_CTAS
 #define AUG_COPY_CTAS 48
@@ -31,6 +31,7 @@ inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 #define AUG_COPY_UNROLL 16
 #endif
 constexpr int COPY_CTAS = AUG_COPY_CTAS, COPY_THREADS = 256, COPY_UNROLL = AUG_COPY_UNROLL;
+constexpr int CHUNK_UTTS = 16;
 #ifndef AUG_DMA_MIN_BYTES
 #define AUG_DMA_MIN_BYTES (512 << 10)
 #endif
@@ -299,10 +300,13 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
         *ctx->leff_seen = 0;
     }
     if (cfg->host_staging) {
+        // the copying kernels' CTAs go first where they compete with the computation of a chunk
+        int prio_lo = 0, prio_hi = 0;
+        cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
         bool ok_s = cudaStreamCreateWithFlags(&ctx->s_h2d, cudaStreamNonBlocking) == cudaSuccess &&
-                    cudaStreamCreateWithFlags(&ctx->s_h2d2, cudaStreamNonBlocking) == cudaSuccess &&
+                    cudaStreamCreateWithPriority(&ctx->s_h2d2, cudaStreamNonBlocking, prio_hi) == cudaSuccess &&
                     cudaEventCreateWithFlags(&ctx->ev_len, cudaEventDisableTiming) == cudaSuccess &&
-                    cudaStreamCreateWithFlags(&ctx->s_d2h, cudaStreamNonBlocking) == cudaSuccess &&
+                    cudaStreamCreateWithPriority(&ctx->s_d2h, cudaStreamNonBlocking, prio_hi) == cudaSuccess &&
                     cudaEventCreateWithFlags(&ctx->ev_start, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < aug::HOST_CHUNKS && ok_s; ++i)
             ok_s = cudaEventCreateWithFlags(&ctx->ev_in[i], cudaEventDisableTiming) == cudaSuccess &&
@@ -562,7 +566,13 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
     // of a few hundred kilobytes each reach about 70 % of the link's rate).
     const float *speech_alias = ragged && (reinterpret_cast<uintptr_t>(speech_host) & 15) == 0
                                     ? mapped_alias(speech_host) : nullptr;
-    const int n_chunk = B >= 2 * aug::HOST_CHUNKS ? aug::HOST_CHUNKS : 1;
+    // What a chunk of eight utterances takes on the device is mostly latency, so chunks hold sixteen
+    // or more (64 utterances of 2-20 s: 1364 us in 8 chunks, 1200 in 4; 16: 892 in 8, 380 in 2).  Only the last chunk's
+    // computation and copy back are not hidden behind the copies in: the last two are smaller.
+    const int n_chunk = B >= 8 ? std::max(2, std::min(aug::HOST_CHUNKS, B / CHUNK_UTTS)) : 1;
+    double share[aug::HOST_CHUNKS], shares = 0.0;
+    for (int c = 0; c < n_chunk; ++c)
+        shares += share[c] = c < n_chunk - 2 ? 1.0 : c == n_chunk - 2 ? 0.8 : 0.5;
 
     AUG_CUDA_OK(cudaEventRecord(ctx->ev_start, sc));          // earlier work on the context's stream
     AUG_CUDA_OK(cudaStreamWaitEvent(si, ctx->ev_start, 0));
@@ -601,11 +611,12 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
         feats_alias = const_cast<float *>(mapped_alias(feats_host));
     int b0 = 0;
     int64_t done = 0;
+    double goal = 0.0;
     for (int c = 0; c < n_chunk; ++c) {
-        // chunk boundaries at equal shares of the samples
+        // chunk boundaries at these shares of the samples
         int b1 = b0;
-        const int64_t goal = total * (c + 1) / n_chunk;
-        while (b1 < B && (done < goal || b1 == b0)) done += lengths_host[b1++];
+        goal += share[c] / shares * (double)total;
+        while (b1 < B && ((double)done < goal || b1 == b0)) done += lengths_host[b1++];
         if (c == n_chunk - 1) b1 = B;
         if (b1 == b0) continue;
         const int nb = b1 - b0;

@@ -60,6 +60,7 @@ constexpr int SM_POINTS = padded_points(N2);
 #ifndef CONV_MINB
 #define CONV_MINB 3                  // CTAs per SM the register budget is set for
 #endif
+constexpr int HOST_ROOM = 16;          // CTAs left out in contexts with host staging, for the copying kernels
 constexpr int FUSED_MINB = 2;          // CTAs per SM of the fused convolution
 
 __device__ __forceinline__ void fft4096_from_regs(float2 (*v)[E], float2 *s, int t,
@@ -1088,7 +1089,7 @@ int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, con
         // where a response fills min(rir_taps, 8192) taps)
         const int ob_min = (F2 - min(c.rir_taps, BLK2) + 1) & ~3;
         const int64_t most = 2 * (int64_t)B * ((max_len + ob_min - 1) / ob_min);
-        const int grid2 = (int)std::min<int64_t>(most, std::min(FUSED_MINB * ctx->sm_count, aug::PARK_SLOTS));
+        const int grid2 = (int)std::min<int64_t>(most, std::min(FUSED_MINB * ctx->sm_count - (ctx->st_speech ? HOST_ROOM : 0), aug::PARK_SLOTS));
         auto kern = ctx->park ? convolve_fused2_kernel<true> : convolve_fused2_kernel<false>;
         if ((ctx->park ? smem_opt_in<convolve_fused2_kernel<true>>(ctx->device)
                        : smem_opt_in<convolve_fused2_kernel<false>>(ctx->device)) != AUG_OK)
