@@ -43,8 +43,8 @@ NCU_TRAFFIC = {
         5: {"convolve": 46.3e6 / 240.0, "features": 34.1e6 / 240.0}},
     "captured_on": {2: "96 utterances", 3: "16 utterances", 5: "4 utterances"},
     # kernel -> (its source files, sha256[:16] of them when the counters were taken)
-    "sources": {"convolve": (("conv.cu", "fft.cuh"), "7a79969eb6513345"),
-                "features": (("feat.cu", "fft.cuh"), "6b90b8e67ab940e5"),
+    "sources": {"convolve": (("conv.cu", "fft_pair.cuh"), "7a79969eb6513345"),
+                "features": (("feat.cu", "fft_pair.cuh"), "6b90b8e67ab940e5"),
                 "rir_image": (("rir.cu",), "9c178fa666e60507")}}
 
 

@@ -7,7 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "fft.cuh"
+#include "fft_pair.cuh"
 
 namespace {
 
@@ -115,31 +115,31 @@ struct Layout {
 
 Layout make_layout(const AugConfig &c) {
     Layout l;
-    l.n_part = (c.rir_taps + aug::CONV_BLK - 1) / aug::CONV_BLK;
-    l.route = l.n_part <= 2 ? aug::ROUTE_FUSED_8192 : aug::ROUTE_STORED;
+    l.n_part = (c.rir_taps + aug::CONV_TAPS - 1) / aug::CONV_TAPS;
+    l.route = l.n_part == 1 ? aug::ROUTE_FUSED_8192 : aug::ROUTE_STORED;
     l.n_bins = c.n_fft / 2 + 1;
     l.t_cap = aug_frame_count(c.max_samples, c.win, c.hop);
     l.ws_stride = align_up(c.max_samples, 4);
     const int64_t B = c.max_batch, S = c.max_sources;
     int64_t o = 0;
     auto take = [&](int64_t bytes) { int64_t r = o; o = align_up(o + bytes, 256); return r; };
-    l.off_tw = take(sizeof(float2) * augfft::TW_N);
+    l.off_tw = take(sizeof(float2) * fftpair::TW_N);
     l.off_rir = take(sizeof(float) * B * S * c.rir_taps);
-    l.off_hspec = take(sizeof(float2) * B * S * (l.route == aug::ROUTE_FUSED_8192 ? 2 : l.n_part) * aug::CONV_N2);
-    l.nblk_cap = (c.max_samples + aug::CONV_BLK - 1) / aug::CONV_BLK;
-    l.off_xspec = l.route == aug::ROUTE_STORED ? take(sizeof(float2) * B * S * l.nblk_cap * aug::CONV_N2) : -1;
+    l.off_hspec = take(sizeof(float2) * B * S * l.n_part * aug::CONV_BINS);
+    l.nblk_cap = (c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS;
+    l.off_xspec = l.route == aug::ROUTE_STORED ? take(sizeof(float2) * B * S * l.nblk_cap * aug::CONV_BINS) : -1;
     // parking slots of the fused route, when a row can have several noises
     const bool parks = c.max_sources >= 3;    // (long-response contexts use the fused route for short responses)
-    l.off_park = parks ? take(sizeof(float2) * (int64_t)aug::PARK_SLOTS * 2 * aug::CONV_N2) : -1;
+    l.off_park = parks ? take(sizeof(float2) * (int64_t)aug::PARK_SLOTS * aug::CONV_BINS) : -1;
     l.off_park_flags = parks ? take(sizeof(int) * aug::PARK_SLOTS) : -1;
     // its list of work: two outputs of every block, blocks as short as min(rir_taps, 8192) taps make them
     l.off_plans = take((int64_t)aug::PLAN_BYTES * B);
-    const int ob = (4 * aug::CONV_BLK - std::min(c.rir_taps, 2 * aug::CONV_BLK) + 1) & ~3;
+    const int ob = (2 * aug::CONV_TAPS - std::min(c.rir_taps, aug::CONV_TAPS) + 1) & ~3;
     l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + ob - 1) / ob));
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take(sizeof(double) * 2 * B);
-    l.off_leff = take(sizeof(int) * (B + 3));
+    l.off_leff = take(sizeof(int) * (B + aug::N_COUNTERS));
     l.off_gain = take(sizeof(float) * B);
     l.off_melw = take(sizeof(aug::MelBin) * B * l.n_bins);
     l.off_melstart = take(sizeof(int) * B * (c.n_mel + 2));
@@ -320,12 +320,12 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
         }
     }
     // twiddles, evaluated in double: block [M/2, M) = exp(-2 pi i k / M), k < M/2
-    std::vector<float2> tw(augfft::TW_N);
+    std::vector<float2> tw(fftpair::TW_N);
     tw[0] = make_float2(1.f, 0.f);
-    for (int M = 2; M <= augfft::TW_N; M *= 2) {
+    for (int M = 2; M <= fftpair::TW_N; M *= 2) {
         for (int k = 0; k < M / 2; ++k) {
             const double a = -2.0 * 3.14159265358979323846 * k / M;
-            tw[augfft::tw_index(M, k)] = make_float2((float)cos(a), (float)sin(a));
+            tw[fftpair::tw_index(M, k)] = make_float2((float)cos(a), (float)sin(a));
         }
     }
     const int st0[2] = {-1, 0};
@@ -337,7 +337,7 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
         delete ctx;
         return AUG_ECUDA;
     }
-    bool ok = cudaMemcpyAsync(ctx->tw, tw.data(), sizeof(float2) * augfft::TW_N,
+    bool ok = cudaMemcpyAsync(ctx->tw, tw.data(), sizeof(float2) * fftpair::TW_N,
                               cudaMemcpyHostToDevice, ctx->stream) == cudaSuccess &&
               cudaMemcpyAsync(ctx->status, st0, sizeof(st0), cudaMemcpyHostToDevice,
                               ctx->stream) == cudaSuccess &&
@@ -434,8 +434,7 @@ int aug_reverb_mix(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if ((rc = launch_rir_spectra(ctx, rir_dev, table_dev, B, true)) != AUG_OK) return rc;
     if ((rc = launch_convolve_prepare(ctx, speech_dev, speech_stride, lengths_dev, noise_bank_dev,
                                       bank_len, table_dev, B, max_len)) != AUG_OK) return rc;
-    if ((rc = launch_convolve_finish(ctx, speech_dev, speech_stride, lengths_dev, noise_bank_dev,
-                                     bank_len, table_dev, B, max_len)) != AUG_OK) return rc;
+    if ((rc = launch_convolve_finish(ctx, table_dev, B, max_len)) != AUG_OK) return rc;
     return launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out_dev, speech_stride);
 }
 
@@ -519,8 +518,7 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     t1(3, sm);
     if (rc != AUG_OK) return rc;
     t0(4, sm);
-    rc = launch_convolve_finish(ctx, speech_dev, speech_stride, lengths_dev, noise_bank_dev, bank_len,
-                                table_dev, B, max_len);
+    rc = launch_convolve_finish(ctx, table_dev, B, max_len);
     t1(4, sm);
     if (rc != AUG_OK) return rc;
     t0(5, sm);

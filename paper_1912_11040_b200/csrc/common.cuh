@@ -9,9 +9,12 @@
 
 namespace aug {
 
-constexpr int CONV_BLK = 4096;          // output samples per convolution block
-constexpr int CONV_F = 2 * CONV_BLK;    // real FFT size of one block
-constexpr int CONV_N2 = CONV_F / 2;     // complex FFT size
+constexpr int CONV_TAPS = 8192;         // taps of a partition: half a transform of the convolution
+constexpr int CONV_BINS = 8192;         // complex numbers of a stored spectrum
+// Counters of the convolution behind the batch's largest response length: units of work listed for
+// the two routes, units drawn from the lists.
+enum Counter { LIST_FUSED, LIST_STORED, DRAWN_FUSED, DRAWN_SPECTRA, DRAWN_STORED };
+constexpr int N_COUNTERS = 6;
 constexpr int PARK_SLOTS = 320;     // parking slots of the fused convolution = most CTAs it runs with
 constexpr int PLAN_BYTES = 96;      // per utterance, see conv.cu
 constexpr int MAX_TAPS = 24576;
@@ -28,7 +31,7 @@ constexpr int HOST_CHUNKS = AUG_HOST_CHUNKS;   // pipeline depth of aug_pipeline
 // How step 2 is run, fixed by the response length at aug_create:
 //   ROUTE_FUSED_8192  rir_taps <= 8192: one partition of a 16384-point transform
 //                     (16384 - taps + 1 outputs per block), one kernel
-//   ROUTE_STORED      longer: partitions of 4096 taps, block spectra stored once and reused
+//   ROUTE_STORED      longer: partitions of 8192 taps, block spectra stored once and reused
 enum Route { ROUTE_FUSED_8192 = 1, ROUTE_STORED = 2 };
 
 enum Reason { R_NONE = 0, R_NSRC = 1, R_ORDER = 2, R_NOISE = 3 };
@@ -48,7 +51,7 @@ struct AugCtx {
     int device;
     int sm_count;          // multiprocessors of the device
     int smem_per_sm;       // shared memory of one multiprocessor, bytes
-    int n_part;            // RIR partitions of CONV_BLK taps
+    int n_part;            // partitions of CONV_TAPS taps
     int route;             // aug::Route
     int n_bins;            // n_fft/2 + 1
     int t_cap;             // frames of an utterance of max_samples
@@ -58,8 +61,8 @@ struct AugCtx {
     int64_t ws_bytes;
     float2 *tw;            // [TW_N] twiddles
     float *rir;            // [max_batch][max_sources][rir_taps]
-    float2 *hspec;         // [max_batch][max_sources][n_part][CONV_N2]
-    float2 *xspec;         // [max_batch][max_sources][nblk_cap][CONV_N2]; NULL unless route == ROUTE_STORED
+    float2 *hspec;         // [max_batch][max_sources][n_part][CONV_BINS]
+    float2 *xspec;         // [max_batch][max_sources][nblk_cap][CONV_BINS]; NULL unless route == ROUTE_STORED
     int nblk_cap;          // blocks of an utterance of max_samples
     float4 *park;          // [PARK_SLOTS][4096] products of noise sources waiting for the last one; NULL if unused
     int *park_flags;       // [PARK_SLOTS] 1 = slot held: that CTA sums in the time domain
@@ -70,7 +73,7 @@ struct AugCtx {
     float *ys;             // [max_batch][ws_stride]
     float *vv;             // [max_batch][ws_stride]
     double *energy;        // [max_batch][2]
-    int *leff;             // [max_batch + 3] (then: largest over the batch, units of work listed, drawn)
+    int *leff;             // [max_batch + N_COUNTERS] (behind the lengths: largest over the batch, counters)
     int *leff_seen;        // pinned host copy of that last entry from an earlier call (long-response contexts)
     int stored_only;       // this call launches the stored-spectra kernels alone taps up to the last non-zero one, largest over the utterance's sources
     float *gain;           // [max_batch] noise gain g for the requested SNR
@@ -161,9 +164,7 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table,
 int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
                             const float *bank, int64_t bank_len, const AugUttParams *table, int B,
                             int max_len);
-int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
-                           const float *bank, int64_t bank_len, const AugUttParams *table, int B,
-                           int max_len);
+int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len);
 int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
                float *wave_out, int64_t out_stride);
 int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset);

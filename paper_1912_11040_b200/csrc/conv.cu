@@ -3,23 +3,20 @@
 // Every route is overlap-save in form: an output block is computed from the input
 // segment that ends with it (the block plus the samples before it that the response
 // reaches back to), which is the overlap-add tail sum moved to the input side, so
-// output blocks never exchange data.  The route is fixed by the response length:
+// output blocks never exchange data.  All transforms are real ones of 16384 points
+// (fft_pair.cuh).  The route is fixed by the response length:
 //
-//   up to 8192 taps   convolve_fused2_kernel: ONE partition of a 16384-point real
-//                     transform, 16384 - taps + 1 outputs per block.  A CTA does the
-//                     whole block per source -- forward, multiply, inverse -- and
-//                     nothing but y_s and v is stored.  The 8192-point complex
-//                     transform of the (even, odd) sample pairs runs as two
-//                     4096-point transforms joined by a radix-2 step (second half
-//                     of this file).  Several noise sources are summed in the frequency domain
+//   up to 8192 taps   ONE partition, 16384 - taps + 1 outputs per block: a block of one output is
+//                     done in one go -- forward, multiply, inverse -- and nothing but y_s and v
+//                     is stored.  Several noise sources are summed in the frequency domain
 //                     through a small parking area in global memory (one inverse).
-//   longer            partitions of CONV_BLK = 4096 taps of an 8192-point transform,
-//                     Y_b = sum_p X_{b-p} H_p with X_j the spectrum of the 8192
-//                     samples that end with block j: block_spectra_kernel stores
-//                     every X_j once; spectral_convolve_kernel reads the P spectra a
-//                     block needs (mostly from L2), multiply-accumulates in registers
-//                     and inverse-transforms.  Noise sources are summed in the
-//                     frequency domain: two inverse transforms per block.
+//   longer            partitions of 8192 taps, blocks of 8192 outputs, Y_b = sum_p X_{b-p} H_p with
+//                     X_j the spectrum of the 16384 samples that end with block j: every X_j is
+//                     stored once; the spectra a block needs are read back (mostly from L2),
+//                     multiplied and accumulated in registers -- all noise sources in one sum --
+//                     and inverse-transformed.  On 128 x 8 s with 24000 taps and three noises
+//                     this takes 488 us; 4096-tap partitions of 8192-point scalar transforms,
+//                     twice the products per sample and twice the bytes from L2, took 534.
 //
 // Responses are often shorter than their buffer: behind the last image source's window
 // every tap is exactly zero.  The kernels that transform the responses record, per
@@ -36,143 +33,16 @@
 // utterance by utterance was
 // measured too: a minority of long CTAs of the fused kernel beside the stored-spectra
 // kernels balanced badly.)  The result is the same convolution.
-//
-// A real transform of F points is a complex transform of F/2 points on (even, odd)
-// sample pairs followed by the usual split; in the 8192-point routes thread t owns
-// the bin pairs (k, F/2-k), k = t + 256 q.  Spectra are stored as F/2 complex numbers
-// with the two real bins (0 and F/2) packed into slot 0; the partition spectra of
-// the responses carry the noise weight and the 1/F of the inverse.
 #include <algorithm>
 
 #include "common.cuh"
-#include "fft.cuh"
 #include "fft_pair.cuh"
 
 namespace {
 
-using namespace augfft;
-constexpr int N2 = aug::CONV_N2;      // 4096 complex points
-constexpr int BLK = aug::CONV_BLK;
-constexpr int CT = 256;               // threads per CTA
-constexpr int E = N2 / CT;            // 16 points per thread: three radix-16 passes
-constexpr int NQ = N2 / 2 / CT;       // 8 bin pairs per thread
-constexpr int SM_POINTS = padded_points(N2);
-#ifndef CONV_MINB
-#define CONV_MINB 3                  // CTAs per SM the register budget is set for
-#endif
+constexpr int CT = 256;                // threads per CTA of the smaller kernels
 constexpr int HOST_ROOM = 16;          // CTAs left out in contexts with host staging, for the copying kernels
-constexpr int FUSED_MINB = 2;          // CTAs per SM of the fused convolution
-
-__device__ __forceinline__ void fft4096_from_regs(float2 (*v)[E], float2 *s, int t,
-                                                  const float2 *__restrict__ tw) {
-    pass_from_regs<N2, E, 16, 1>(v, s, t, tw);
-    __syncthreads();
-    pass<N2, E, 16, 16, 1>(s, t, tw, CtaSync());
-    pass<N2, E, 16, 256, 16>(s, t, tw, CtaSync());
-}
-
-__device__ __forceinline__ void fft4096_in_place(float2 *s, int t, const float2 *__restrict__ tw) {
-    pass<N2, E, 16, 1, 0>(s, t, tw, CtaSync());
-    pass<N2, E, 16, 16, 1>(s, t, tw, CtaSync());
-    pass<N2, E, 16, 256, 16>(s, t, tw, CtaSync());
-}
-
-// Split of the half-size transform Z into the spectrum X of the real signal at the
-// bin pair (k, N2-k):  X[k] = Ev + W^k Od,  X[N2-k] = conj(Ev - W^k Od),
-// Ev = (Z[k] + conj Z[N2-k])/2, Od = -i (Z[k] - conj Z[N2-k])/2, W = exp(-2 pi i/F).
-__device__ __forceinline__ void real_split(float2 zk, float2 zm, float2 w, float2 &xk, float2 &xm) {
-    const float2 ev = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-    const float2 od = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-    const float2 wo = cmul(w, od);
-    xk = make_float2(ev.x + wo.x, ev.y + wo.y);
-    xm = make_float2(ev.x - wo.x, -(ev.y - wo.y));
-}
-
-// The pair a thread owns for k = t + CT q, read from a finished transform in `sm`:
-//   k != 0:  a = X[k],            b = X[N2-k]
-//   k == 0:  a = (X[0], X[N2])    b = X[N2/2]      (X[0], X[N2] are real)
-__device__ __forceinline__ void spectrum_pair(const float2 *sm, const float2 *__restrict__ tw, int k,
-                                              float2 &a, float2 &b) {
-    const float2 zk = sm[pad0(k)], zm = sm[pad0((N2 - k) & (N2 - 1))];
-    const float2 w = __ldg(&tw[tw_index(aug::CONV_F, k)]);
-    float2 xk, xm;
-    real_split(zk, zm, w, xk, xm);
-    if (k == 0) {
-        const float2 zh = sm[pad0(N2 / 2)];
-        a = make_float2(xk.x, xm.x);
-        b = make_float2(zh.x, -zh.y);
-    } else {
-        a = xk;
-        b = xm;
-    }
-}
-// Slots of that pair in a stored spectrum.
-__device__ __forceinline__ int slot_a(int k) { return k; }
-__device__ __forceinline__ int slot_b(int k) { return k == 0 ? N2 / 2 : N2 - k; }
-
-__device__ __forceinline__ void mac_pair(float2 &acc_a, float2 &acc_b, float2 a, float2 b, float2 ha,
-                                         float2 hb, int k) {
-    if (k == 0) {
-        acc_a.x = fmaf(a.x, ha.x, acc_a.x);
-        acc_a.y = fmaf(a.y, ha.y, acc_a.y);
-    } else {
-        acc_a = cadd(acc_a, cmul(a, ha));
-    }
-    acc_b = cadd(acc_b, cmul(b, hb));
-}
-
-// 2*BLK input samples starting at `base` as 16 (even, odd) pairs per thread in the
-// order the first FFT pass wants them.  Speech reads x[i]; a noise source reads
-// its stretch of the bank end to end (x[i mod nlen]).  Outside [0, N): zero.
-__device__ __forceinline__ void load_block(float2 (*v)[E], const float *__restrict__ x, bool looped,
-                                             int nlen, int base, int N, int t) {
-    // A segment inside the utterance, and for a looped stretch inside one period of it on
-    // 8-byte boundaries, needs no test per pair (the same for the whole CTA).
-    if (base >= 0 && base + 2 * BLK <= N) {
-        int m0 = base;
-        bool plain = !looped;
-        if (looped && (nlen & 1) == 0 && (reinterpret_cast<uintptr_t>(x) & 7) == 0) {
-            m0 = base % nlen;
-            plain = (m0 & 1) == 0 && m0 + 2 * BLK <= nlen;
-        }
-        if (plain) {
-            const float2 *x2 = reinterpret_cast<const float2 *>(x + m0) + t;
-#pragma unroll
-            for (int r = 0; r < E; ++r) v[0][r] = __ldg(x2 + CT * r);
-            return;
-        }
-    }
-    if (!looped) {
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int i0 = base + 2 * (t + CT * r);
-            float2 z = make_float2(0.f, 0.f);
-            if (i0 >= 0) {
-                if (i0 + 1 < N) z = *reinterpret_cast<const float2 *>(x + i0);
-                else if (i0 < N) z.x = x[i0];
-            }
-            v[0][r] = z;
-        }
-        return;
-    }
-    // Looped source: one division for the first sample, then the position advances
-    // by 2*CT (mod nlen) from one pair to the next.
-    const int first = base + 2 * t;
-    const int step = (2 * CT) % nlen;
-    int m = first >= 0 ? first % nlen : (nlen - (-first) % nlen) % nlen;
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int i0 = first + 2 * CT * r;
-        float2 z = make_float2(0.f, 0.f);
-        if (i0 >= 0) {
-            if (i0 < N) z.x = x[m];
-            if (i0 + 1 < N) z.y = x[m + 1 == nlen ? 0 : m + 1];
-        }
-        v[0][r] = z;
-        m += step;
-        if (m >= nlen) m -= nlen;
-    }
-}
+constexpr int FUSED_MINB = 2;          // CTAs per SM of the transforming kernels
 
 // Source s of an utterance: pointer to its samples, loop length; false if the row's
 // noise stretch is unusable (reported once through the status word).
@@ -189,71 +59,6 @@ __device__ __forceinline__ bool source_of(const AugUttParams &row, int s, const 
     if (nlen <= 0 || off < 0 || off + nlen > bank_len || bank == nullptr) return false;
     x = bank + off;
     return true;
-}
-
-__device__ __forceinline__ float block_sum(float x, float *red, int t) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    __syncthreads();
-    if ((t & 31) == 0) red[t >> 5] = x;
-    __syncthreads();
-    float tot = 0.f;
-    if (t < 32) {
-        tot = (t < CT / 32) ? red[t] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    return tot;   // valid in warp 0
-}
-
-// Accumulated block spectrum -> CONV_BLK output samples at dst, plus their energy.
-// The half-size spectrum is rebuilt with real and imaginary parts swapped, which
-// turns the forward transform into the (unnormalised) inverse; the scale 1/F sits
-// in the stored partition spectra.  The second half of the 2*BLK outputs is kept.
-__device__ __forceinline__ void finish_block(const float2 (*acc)[2], float2 *sm,
-                                             const float2 *__restrict__ tw, int t, float *dst,
-                                             int n_left, double *energy_slot, float *red) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int k = t + CT * q;
-        const float2 yk = acc[q][0], ym = acc[q][1];
-        if (k == 0) {
-            // yk = (Y[0], Y[N2]) real pair; ym = Y[N2/2]
-            sm[pad0(0)] = make_float2(yk.x - yk.y, yk.x + yk.y);
-            sm[pad0(N2 / 2)] = make_float2(-2.f * ym.y, 2.f * ym.x);
-        } else {
-            const float2 w = __ldg(&tw[tw_index(aug::CONV_F, k)]);
-            // Z[k] = (Yk + conj Ym) + i conj(W)(Yk - conj Ym)
-            const float2 a = make_float2(yk.x + ym.x, yk.y - ym.y);
-            const float2 d = make_float2(yk.x - ym.x, yk.y + ym.y);
-            const float2 e = cmul(make_float2(w.y, w.x), d);       // i conj(W) = (w.y, w.x)
-            const float2 zk = make_float2(a.x + e.x, a.y + e.y);
-            // Z[N2-k] = (Ym + conj Yk) - i W (Ym - conj Yk)
-            const float2 e2 = cmul(make_float2(-w.y, w.x), make_float2(-d.x, d.y));   // i W = (-w.y, w.x)
-            const float2 zm = make_float2(a.x - e2.x, -a.y - e2.y);
-            sm[pad0(k)] = make_float2(zk.y, zk.x);
-            sm[pad0(N2 - k)] = make_float2(zm.y, zm.x);
-        }
-    }
-    __syncthreads();
-    fft4096_in_place(sm, t, tw);
-    float e2sum = 0.f;
-#pragma unroll
-    for (int r = 0; r < BLK / 2 / CT; ++r) {
-        const int n = t + CT * r;                       // pair index within the block
-        const float2 z = sm[pad0(N2 / 2 + n)];          // second half; swapped back here
-        const float y0 = z.y, y1 = z.x;
-        if (2 * n + 1 < n_left) {
-            *reinterpret_cast<float2 *>(dst + 2 * n) = make_float2(y0, y1);
-            e2sum += y0 * y0 + y1 * y1;
-        } else if (2 * n < n_left) {
-            dst[2 * n] = y0;
-            e2sum += y0 * y0;
-        }
-    }
-    const float tot = block_sum(e2sum, red, t);
-    if (t == 0) atomicAdd(energy_slot, (double)tot);
-    __syncthreads();
 }
 
 // Effective length of the responses: (index + 1) of the last non-zero tap, largest over the
@@ -298,136 +103,7 @@ rir_length_kernel(const float *__restrict__ rir, const AugUttParams *__restrict_
 }
 
 // Which route a batch takes in a context sized for responses of more than 8192 taps.
-__device__ __forceinline__ bool takes_fused_route(int leff_batch) { return leff_batch <= 2 * BLK; }
-
-// ---------------------------------------------------------------- partition spectra
-__global__ void __launch_bounds__(CT)
-rir_spectra_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max,
-                   int L, int P, const float2 *__restrict__ tw, float2 *__restrict__ hspec,
-                   const int *__restrict__ leff_all, int always) {
-    extern __shared__ __align__(16) float2 sm[];
-    const int p = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x;
-    chain_wait();
-    if (!always && takes_fused_route(*leff_all)) return;
-    const AugUttParams &row = table[utt];
-    if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
-    const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (float)aug::CONV_F;
-    const float *h = rir + ((int64_t)utt * S_max + s) * L;
-    float2 *out = hspec + (((int64_t)utt * S_max + s) * P + p) * N2;
-
-    float2 v[1][E];
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int n = t + CT * r;                 // complex index; taps 2n, 2n+1 of the partition
-        const int i0 = p * BLK + 2 * n;
-        float2 z = make_float2(0.f, 0.f);
-        if (n < BLK / 2) {
-            if (i0 < L) z.x = h[i0];
-            if (i0 + 1 < L) z.y = h[i0 + 1];
-        }
-        v[0][r] = z;
-    }
-    fft4096_from_regs(v, sm, t, tw);
-    chain_next();
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int k = t + CT * q;
-        float2 a, b;
-        spectrum_pair(sm, tw, k, a, b);
-        out[slot_a(k)] = make_float2(a.x * scale, a.y * scale);
-        out[slot_b(k)] = make_float2(b.x * scale, b.y * scale);
-    }
-}
-
-// ---------------------------------------------------------------- several partitions
-// Spectrum of every 2*BLK input segment of every source, stored once.
-__global__ void __launch_bounds__(CT, CONV_MINB)
-block_spectra_kernel(const float *__restrict__ speech, int64_t stride,
-                     const int *__restrict__ lengths, const float *__restrict__ bank,
-                     int64_t bank_len, const AugUttParams *__restrict__ table, int S_max,
-                     const float2 *__restrict__ tw, float2 *__restrict__ xspec, int nblk_cap,
-                     int *status, int n_cap, const int *__restrict__ leff_all, int always) {
-    extern __shared__ __align__(16) float2 sm[];
-    const int b = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x;
-    chain_wait();
-    const int N = min(max(lengths[utt], 0), n_cap);
-    if ((int64_t)b * BLK >= N || (!always && takes_fused_route(*leff_all))) return;
-    const AugUttParams &row = table[utt];
-    if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
-    const float *x;
-    int nlen;
-    if (!source_of(row, s, speech + (int64_t)utt * stride, bank, bank_len, x, nlen)) {
-        if (t == 0 && b == 0 && atomicCAS(&status[0], -1, utt) == -1) status[1] = aug::R_NOISE;
-        return;
-    }
-    float2 v[1][E];
-    load_block(v, x, s != 0, nlen, (b - 1) * BLK, N, t);
-    fft4096_from_regs(v, sm, t, tw);
-    chain_next();
-    float2 *out = xspec + (((int64_t)utt * S_max + s) * nblk_cap + b) * N2;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int k = t + CT * q;
-        float2 a, bb;
-        spectrum_pair(sm, tw, k, a, bb);
-        out[slot_a(k)] = a;
-        out[slot_b(k)] = bb;
-    }
-}
-
-__global__ void __launch_bounds__(CT, CONV_MINB)
-spectral_convolve_kernel(const int *__restrict__ lengths, const float *__restrict__ bank,
-                         int64_t bank_len, const AugUttParams *__restrict__ table, int S_max, int P,
-                         const float2 *__restrict__ hspec, const float2 *__restrict__ xspec,
-                         int nblk_cap, const float2 *__restrict__ tw, float *__restrict__ ys,
-                         float *__restrict__ vv, int64_t ws_stride, double *__restrict__ energy,
-                         int n_cap, const int *__restrict__ leff, const int *__restrict__ leff_all,
-                         int always) {
-    extern __shared__ __align__(16) float2 sm[];
-    __shared__ float red[CT / 32];
-    const int b = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
-    chain_wait();
-    // partitions behind the last non-zero tap of every source of this utterance are zero
-    const int P_used = min(P, (max(leff[utt], 1) + BLK - 1) / BLK);
-    const int N = min(max(lengths[utt], 0), n_cap);
-    if ((int64_t)b * BLK >= N || (!always && takes_fused_route(*leff_all))) return;
-    const AugUttParams &row = table[utt];
-    int n_src = row.n_src;
-    if (n_src < 1 || n_src > S_max) n_src = 0;
-    const int n_out = n_src > 1 ? 2 : (n_src == 1 ? 1 : 0);
-
-    for (int o = 0; o < n_out; ++o) {
-        float2 acc[NQ][2];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q][0] = acc[q][1] = make_float2(0.f, 0.f);
-        const int s_lo = o ? 1 : 0, s_hi = o ? n_src : 1;
-        for (int s = s_lo; s < s_hi; ++s) {
-            const float *x;
-            int nlen;
-            if (!source_of(row, s, nullptr, bank, bank_len, x, nlen)) continue;   // no spectra stored
-            const float2 *Hs = hspec + ((int64_t)utt * S_max + s) * P * N2;
-            const float2 *Xs = xspec + ((int64_t)utt * S_max + s) * nblk_cap * N2;
-            for (int p = 0; p < P_used && p <= b; ++p) {
-                const float2 *H = Hs + (int64_t)p * N2;
-                const float2 *X = Xs + (int64_t)(b - p) * N2;
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const int k = t + CT * q;
-                    const int ia = slot_a(k), ib = slot_b(k);
-                    mac_pair(acc[q][0], acc[q][1], __ldg(&X[ia]), __ldg(&X[ib]), __ldg(&H[ia]),
-                             __ldg(&H[ib]), k);
-                }
-            }
-        }
-        float *dst = (o ? vv : ys) + (int64_t)utt * ws_stride + (int64_t)b * BLK;
-        finish_block(acc, sm, tw, t, dst, N - b * BLK, &energy[2 * utt + o], red);
-    }
-    chain_next();
-    if (n_src <= 1) {
-        float *dst = vv + (int64_t)utt * ws_stride + (int64_t)b * BLK;
-        for (int i = t; i < BLK && b * BLK + i < N; i += CT) dst[i] = 0.f;
-    }
-}
+__device__ __forceinline__ bool takes_fused_route(int leff_batch) { return leff_batch <= aug::CONV_TAPS; }
 
 // ---------------------------------------------------------------- mixing
 // g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise or with a silent side:
@@ -501,11 +177,11 @@ mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t w
 // the bins k, 8192-k, 4096-k and 4096+k of the segment's spectrum, multiplies them with the
 // response's and folds the products back, all in registers.  The response's spectra are
 // stored in the order the threads read them.
-constexpr int BLK2 = 2 * BLK;          // most taps; output samples per block are F2 - taps + 1
+constexpr int BLK2 = aug::CONV_TAPS;   // most taps of a partition
 constexpr int F2 = 2 * BLK2;           // real transform size
 constexpr int NB2 = F2 / 2;            // complex numbers stored per spectrum
 constexpr int CF = fftpair::THREADS;   // threads per CTA
-constexpr int NP2 = N2 / CF;           // points per thread
+constexpr int NP2 = 4096 / CF;         // points per thread
 constexpr int NS2 = NP2 / 2;           // slots (k, 4096-k) per thread
 using fftpair::C2;
 using fftpair::u64;
@@ -691,6 +367,10 @@ __device__ __forceinline__ Bins load_bins(const float4 *p) {
     asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.qr), "=l"(z.qi) : "l"(p + CF));
     return z;
 }
+// A whole spectrum into L2, by one thread.
+__device__ __forceinline__ void prefetch_spectrum(const float4 *p) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "n"(8 * NB2) : "memory");
+}
 __device__ __forceinline__ Bins load_parked(const float4 *p) {
     const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2 *>(p));
     const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2 *>(p + CF));
@@ -701,34 +381,33 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
     __stcg(reinterpret_cast<ulonglong2 *>(p + CF), make_ulonglong2(z.qr, z.qi));
 }
 
-// Spectrum of one 16384-sample segment of each impulse response (taps beyond L and
-// the whole second half are zero), scaled by the noise weight and 1/F (and by 1/4 for
+// Spectra of the partitions of each impulse response: 8192 taps (those beyond L are zero) and as many
+// zeros, scaled by the noise weight and 1/F (and by 1/4 for
 // the two doubled spectra of a product).
 __global__ void __launch_bounds__(CF, FUSED_MINB)
 rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max,
-                    int L, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int64_t hs_stride,
-                    const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed) {
+                    int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int *leff, int mixed) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
     __shared__ int red_i[CF / 32];
-    const int s = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
+    const int part = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x, from = part * BLK2;
     fftpair::fill_tables(sh, t, tw);
     chain_wait();
-    // mixed: the lengths are known already (rir_length_kernel) and decide the route; otherwise
+    // mixed: the lengths are known already (rir_length_kernel); otherwise there is one partition, and
     // this kernel reads every tap anyway and records the length on the way
-    if (mixed && !takes_fused_route(*leff_all)) return;
+    if (mixed && part > 0 && from >= leff[utt]) return;
     const AugUttParams &row = table[utt];
     if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
     const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (4.f * (float)F2);
     const float *h = rir + ((int64_t)utt * S_max + s) * L;
-    float4 *out = hspec + ((int64_t)utt * S_max + s) * (hs_stride / 2) + t;
+    float4 *out = hspec + (((int64_t)utt * S_max + s) * P + part) * (NB2 / 2) + t;
     C2 v[NP2];
     int last = 0;
 #pragma unroll
     for (int r = 0; r < NP2; ++r) {
-        const int i0 = 4 * (t + CF * r);
+        const int i0 = from + 4 * (t + CF * r);
         float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i0 < BLK2) {
+        if (4 * (t + CF * r) < BLK2) {
             if (i0 < L) z.x = h[i0];
             if (i0 + 1 < L) z.y = h[i0 + 1];
             if (i0 + 2 < L) z.z = h[i0 + 2];
@@ -749,7 +428,7 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
     if (!mixed && t == 0) {
         int m = 0;
         for (int i = 0; i < CF / 32; ++i) m = max(m, red_i[i]);
-        if (m > 0) atomicMax(const_cast<int *>(&leff[utt]), m);
+        if (m > 0) atomicMax(&leff[utt], m);
     }
     fftpair::forward4096(v, sh, t, tw);
     chain_next();
@@ -765,11 +444,11 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
     }
 }
 
-// ---------------------------------------------------------------- what the fused convolution does
+// ---------------------------------------------------------------- the list of work
 // One unit of work is one block of one output (the reverberant speech, or the sum of the noise
 // sources) of an utterance.  plan_kernel lists the units that exist -- how many blocks an
 // utterance has depends on its length and on where its responses end -- and what they need to
-// know; the convolution's CTAs, as many as fit the device, work through the list.  With one CTA
+// know; the convolving kernels' CTAs, as many as fit the device, work through the list.  With one CTA
 // per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
 // (two thirds of them without work) and to each one's chain of loads before its first sample.
 struct Plan {
@@ -780,6 +459,7 @@ struct Plan {
     int n_noise;
     int N;                         // samples of the utterance
     int ob;                        // outputs per block
+    int parts;                     // partitions that are not zero throughout (stored-spectra route)
 };
 struct Unit {
     int utt;
@@ -792,22 +472,24 @@ __global__ void __launch_bounds__(256)
 plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restrict__ lengths,
             const float *__restrict__ bank, int64_t bank_len, const AugUttParams *__restrict__ table, int B,
             int S_max, int n_cap, const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed,
-            int *status, Plan *__restrict__ plans, Unit *__restrict__ units, int *__restrict__ n_units) {
+            int stored_only, int *status, Plan *__restrict__ plans, Unit *__restrict__ units, int *__restrict__ n_units) {
     const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     chain_next();
     chain_wait();
-    if (utt >= B || (mixed && !takes_fused_route(*leff_all))) return;
+    if (utt >= B) return;
+    const bool stored = mixed && (stored_only || !takes_fused_route(*leff_all));
     const AugUttParams &row = table[utt];
     const int N = min(max(lengths[utt], 0), n_cap);
     // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
     // of 4, where taps counts up to the last non-zero tap of this utterance's responses
-    const int ob = (F2 - min(max(leff[utt], 1), BLK2) + 1) & ~3;
+    const int ob = stored ? BLK2 : (F2 - min(max(leff[utt], 1), BLK2) + 1) & ~3;
     const int n = 2 * ((N + ob - 1) / ob);
     int at = 0;
     if (lane == 0) {
         Plan p;
         p.N = N;
         p.ob = ob;
+        p.parts = (max(leff[utt], 1) + BLK2 - 1) / BLK2;
         p.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;    // (reported by step 1)
         p.n_noise = 0;
         p.x[0] = speech + (int64_t)utt * stride;
@@ -826,13 +508,16 @@ plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restr
             }
         }
         plans[utt] = p;
-        if (n > 0) at = atomicAdd(n_units, n);
+        if (n > 0) at = atomicAdd(n_units + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
     }
     at = __shfl_sync(0xffffffffu, at, 0);
     for (int i = lane; i < n; i += 32) units[at + i] = Unit{utt, i};
 }
 
-// PARK: rows may have several noise sources (the context allows three or more
+// KIND  FUSED    a block of one output from its samples (responses of one partition)
+//       SPECTRA  the spectra of a block's segments, one per source, stored
+//       STORED   a block of one output from stored spectra
+// PARK (FUSED): rows may have several noise sources (the context allows three or more
 // sources); without it the kernel carries none of the parking code.
 //
 // Several noise sources are summed in the frequency domain: the products of all but the last
@@ -842,13 +527,15 @@ plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restr
 // first, one inverse transform each.
 enum Fate { DIRECT = 0, PARK_FIRST = 1, PARK_MORE = 2, PARK_JOIN = 3 };
 
-template <bool PARK>
+enum Kind { FUSED, SPECTRA, STORED };
+
+template <Kind KIND, bool PARK>
 __global__ void __launch_bounds__(CF, FUSED_MINB)
-convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units,
-                       int *n_units, int S_max, const float4 *__restrict__ hspec,
-                       int64_t hs_stride, const float2 *__restrict__ tw, float *__restrict__ ys,
-                       float *__restrict__ vv, int64_t ws_stride, double *__restrict__ energy,
-                       float4 *__restrict__ park, const int *__restrict__ park_flags) {
+convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, const int *__restrict__ n_units,
+                int *drawn, int S_max, int P, const float4 *__restrict__ hspec, float4 *__restrict__ xspec,
+                int nblk_cap, const float2 *__restrict__ tw, float *__restrict__ ys, float *__restrict__ vv,
+                int64_t ws_stride, double *__restrict__ energy, float4 *__restrict__ park,
+                const int *__restrict__ park_flags) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
     // The first two units of a CTA follow from its number, the others it draws from a counter (units
@@ -862,7 +549,6 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
     fftpair::fill_tables(sh, t, tw);
     chain_wait();
     const int count = __ldcg(n_units);
-    int *drawn = n_units + 1;
     if (blockIdx.x >= count) return;
     if (t == 0) {
         const int second = blockIdx.x + G;
@@ -872,7 +558,7 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
     if (t < (int)(sizeof(Plan) / 4))
         reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + units[blockIdx.x].utt)[t];
     __syncthreads();
-    const bool own_slot = PARK && park != nullptr && park_flags[blockIdx.x] == 0;
+    const bool own_slot = KIND == FUSED && PARK && park != nullptr && park_flags[blockIdx.x] == 0;
 
 #pragma unroll 1
     for (int k = 0;;) {
@@ -899,59 +585,133 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
             // no (usable) source: the output is defined as silence
             float *dst = (noise ? vv : ys) + (int64_t)cur.utt * ws_stride + (int64_t)b * p.ob;
             const int n_left = min(p.N - b * p.ob, p.ob);
-            for (int i = t; i < n_left; i += CF) dst[i] = 0.f;
+            if (KIND != SPECTRA)
+                for (int i = t; i < n_left; i += CF) dst[i] = 0.f;
             draw();
             __syncthreads();
         } else {
             bool added = false;
 #pragma unroll 1
             for (;; ++j) {
-                Fate fate = DIRECT;
-                if (PARK && own_slot && j_last > 1)
-                    fate = j == j_last ? PARK_JOIN : j > 1 ? PARK_MORE : PARK_FIRST;
                 C2 v[NP2];
-                load_segment(v, sh, p.x[j], noise, p.nlen[j], (b + 1) * p.ob - F2, p.N, t);
-                // the response's bins are brought into L2 meanwhile (they may have been pushed out by the
-                // audio), and the first two slots' requested before the exchange
-                const float4 *H = hspec + ((int64_t)cur.utt * S_max + p.src[j]) * (hs_stride / 2) + t;
-                if (t == 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(H), "n"(8 * NB2) : "memory");
-                fftpair::forward4096(v, sh, t, tw);
-                Bins h = load_bins(H), h1 = load_bins(H + 2 * CF);
-                const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
-                fftpair::exchange_mirror(v, t);
+                Fate fate = DIRECT;
+                if constexpr (KIND == SPECTRA) {
+                    if (j == j_last) draw();
+                    load_segment(v, sh, p.x[j], noise, p.nlen[j], (b + 1) * p.ob - F2, p.N, t);
+                    fftpair::forward4096(v, sh, t, tw);
+                    float4 *X = xspec + (((int64_t)cur.utt * S_max + p.src[j]) * nblk_cap + b) * (NB2 / 2) + t;
+                    const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
+                    fftpair::exchange_mirror(v, t);
 #pragma unroll
-                for (int r = 0; r < NS2; ++r) {
-                    const Bins hc = h;
-                    h = h1;
-                    if (r + 2 < NS2) h1 = load_bins(H + 2 * (r + 2) * CF);
-                    const bool edge = r == 0 && fftpair::owns_zero(t);
-                    const SplitTwiddle w(u, r);
-                    Bins y;
-                    if (edge) {
-                        y = edge_forward(v[0], v[NP2 - 1]);
-                        edge_multiply(y, hc);
-                    } else {
-                        y = bins_forward(v[r], v[NP2 - 1 - r], w);
-                        multiply(y.pr, y.pi, hc.pr, hc.pi);
-                        multiply(y.qr, y.qi, hc.qr, hc.qi);
-                    }
-                    if (PARK && fate != DIRECT) {
-                        // this thread's parked products, two words per slot: no other thread reads them
-                        float4 *pk = park + (int64_t)blockIdx.x * (2 * NS2 * CF) + 2 * r * CF + t;
-                        if (fate != PARK_FIRST) {
-                            const Bins z = load_parked(pk);
-                            y = {fftpair::add2(y.pr, z.pr), fftpair::add2(y.pi, z.pi), fftpair::add2(y.qr, z.qr),
-                                 fftpair::add2(y.qi, z.qi)};
-                        }
-                        if (fate != PARK_JOIN) store_bins(pk, y);
-                    }
-                    if (edge) edge_inverse(y, v[0], v[NP2 - 1]);
-                    else bins_inverse(y, w, v[r], v[NP2 - 1 - r]);
-                }
-                if (PARK && (fate == PARK_FIRST || fate == PARK_MORE)) {
-                    __syncthreads();       // other warps may still read rows of the buffer the next source fills
+                    for (int r = 0; r < NS2; ++r)
+                        store_bins(X + 2 * r * CF,
+                                   r == 0 && fftpair::owns_zero(t) ? edge_forward(v[0], v[NP2 - 1])
+                                                                   : bins_forward(v[r], v[NP2 - 1 - r], SplitTwiddle(u, r)));
+                    __syncthreads();           // other warps may still read rows of the buffer the next source fills
+                    if (j == j_last) break;
                     continue;
+                }
+                if constexpr (KIND == STORED) {
+                    // All sources of the output and all partitions into one sum.  Bound by the latency of the
+                    // spectra (128 KB per product; half of those of the audio come from memory): the next
+                    // product's are brought into L2 while one is worked on, and each slot's are
+                    // requested one slot ahead (319 -> 248 us on 128 x 8 s).
+                    Bins acc[NS2], xa, ha;
+#pragma unroll
+                    for (int r = 0; r < NS2; ++r) acc[r] = {0, 0, 0, 0};
+                    const int parts = min(p.parts, b + 1);
+#pragma unroll 1
+                    for (; j <= j_last; ++j) {
+                        const int64_t row = (int64_t)cur.utt * S_max + p.src[j];
+                        const float4 *H = hspec + row * P * (NB2 / 2) + t;
+                        const float4 *X = xspec + (row * nblk_cap + b) * (NB2 / 2) + t;
+                        xa = load_parked(X);
+                        ha = load_bins(H);
+#pragma unroll 1
+                        for (int q = 0; q < parts; ++q) {
+                            const bool more = q + 1 < parts;
+                            if (t == 0 && (more || j < j_last)) {
+                                const int64_t row_n = (int64_t)cur.utt * S_max + p.src[min(j + 1, j_last)];
+                                prefetch_spectrum(more ? H + NB2 / 2 : hspec + row_n * P * (NB2 / 2));
+                                prefetch_spectrum(more ? X - NB2 / 2 : xspec + (row_n * nblk_cap + b) * (NB2 / 2));
+                            }
+#pragma unroll
+                            for (int r = 0; r < NS2; ++r) {
+                                using namespace fftpair;
+                                Bins x = xa;
+                                const Bins h = ha;
+                                if (r + 1 < NS2 || more) {
+                                    xa = load_parked(r + 1 < NS2 ? X + 2 * (r + 1) * CF : X - NB2 / 2);
+                                    ha = load_bins(r + 1 < NS2 ? H + 2 * (r + 1) * CF : H + NB2 / 2);
+                                }
+                                if (r == 0 && owns_zero(t)) {
+                                    edge_multiply(x, h);
+                                    acc[0] = {add2(acc[0].pr, x.pr), add2(acc[0].pi, x.pi), add2(acc[0].qr, x.qr),
+                                              add2(acc[0].qi, x.qi)};
+                                } else {
+                                    acc[r].pr = sub2(fma2(x.pr, h.pr, acc[r].pr), mul2(x.pi, h.pi));
+                                    acc[r].pi = fma2(x.pi, h.pr, fma2(x.pr, h.pi, acc[r].pi));
+                                    acc[r].qr = sub2(fma2(x.qr, h.qr, acc[r].qr), mul2(x.qi, h.qi));
+                                    acc[r].qi = fma2(x.qi, h.qr, fma2(x.qr, h.qi, acc[r].qi));
+                                }
+                            }
+                            H += NB2 / 2;
+                            X -= NB2 / 2;
+                        }
+                    }
+                    j = j_last;
+                    const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
+#pragma unroll
+                    for (int r = 0; r < NS2; ++r) {
+                        if (r == 0 && fftpair::owns_zero(t)) edge_inverse(acc[0], v[0], v[NP2 - 1]);
+                        else bins_inverse(acc[r], SplitTwiddle(u, r), v[r], v[NP2 - 1 - r]);
+                    }
+                }
+                if constexpr (KIND == FUSED) {
+                    if (PARK && own_slot && j_last > 1)
+                        fate = j == j_last ? PARK_JOIN : j > 1 ? PARK_MORE : PARK_FIRST;
+                    load_segment(v, sh, p.x[j], noise, p.nlen[j], (b + 1) * p.ob - F2, p.N, t);
+                    // the response's bins are brought into L2 meanwhile (they may have been pushed out by the
+                    // audio), and the first two slots' requested before the exchange
+                    const float4 *H = hspec + ((int64_t)cur.utt * S_max + p.src[j]) * P * (NB2 / 2) + t;
+                    if (t == 0) prefetch_spectrum(H);
+                    fftpair::forward4096(v, sh, t, tw);
+                    Bins h = load_bins(H), h1 = load_bins(H + 2 * CF);
+                    const float2 u = __ldg(&tw[8192 + fftpair::row_frequency(t)]);
+                    fftpair::exchange_mirror(v, t);
+#pragma unroll
+                    for (int r = 0; r < NS2; ++r) {
+                        const Bins hc = h;
+                        h = h1;
+                        if (r + 2 < NS2) h1 = load_bins(H + 2 * (r + 2) * CF);
+                        const bool edge = r == 0 && fftpair::owns_zero(t);
+                        const SplitTwiddle w(u, r);
+                        Bins y;
+                        if (edge) {
+                            y = edge_forward(v[0], v[NP2 - 1]);
+                            edge_multiply(y, hc);
+                        } else {
+                            y = bins_forward(v[r], v[NP2 - 1 - r], w);
+                            multiply(y.pr, y.pi, hc.pr, hc.pi);
+                            multiply(y.qr, y.qi, hc.qr, hc.qi);
+                        }
+                        if (PARK && fate != DIRECT) {
+                            // this thread's parked products, two words per slot: no other thread reads them
+                            float4 *pk = park + (int64_t)blockIdx.x * (2 * NS2 * CF) + 2 * r * CF + t;
+                            if (fate != PARK_FIRST) {
+                                const Bins z = load_parked(pk);
+                                y = {fftpair::add2(y.pr, z.pr), fftpair::add2(y.pi, z.pi), fftpair::add2(y.qr, z.qr),
+                                     fftpair::add2(y.qi, z.qi)};
+                            }
+                            if (fate != PARK_JOIN) store_bins(pk, y);
+                        }
+                        if (edge) edge_inverse(y, v[0], v[NP2 - 1]);
+                        else bins_inverse(y, w, v[r], v[NP2 - 1 - r]);
+                    }
+                    if (PARK && (fate == PARK_FIRST || fate == PARK_MORE)) {
+                        __syncthreads();       // other warps may still read rows of the buffer the next source fills
+                        continue;
+                    }
                 }
                 fftpair::exchange_back(v, t);
                 if (j == j_last) draw();
@@ -1010,14 +770,11 @@ convolve_fused2_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ 
     }
 }
 
-constexpr size_t FFT_SMEM = sizeof(float2) * SM_POINTS;
 constexpr size_t FFT2_SMEM = sizeof(fftpair::Shared);
 
 }  // namespace
 
 static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_STORED; }
-// response spectra of one (utterance, source): complex numbers between consecutive ones
-static int64_t hspec_stride(const AugCtx *ctx) { return stored_route(ctx) ? (int64_t)ctx->n_part * N2 : NB2; }
 
 int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table, int B, bool reset) {
     const AugConfig &c = ctx->cfg;
@@ -1029,31 +786,44 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table,
     if (reset) {
         AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0, sizeof(double) * 2 * (size_t)B, st));
         AUG_CUDA_OK(cudaMemsetAsync(ctx->leff, 0, sizeof(int) * (size_t)B, st));
-        AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, 3 * sizeof(int), st));      // and the counters of the work list
-    }
-    dim3 grid2(c.max_sources, B);
-    if (mixed) {
-        if (launch_chained(rir_length_kernel, grid2, CT, 0, st, rir, table, c.max_sources, c.rir_taps, ctx->leff,
-                           leff_all) != AUG_OK)
-            return AUG_ECUDA;
-        ctx->launches++;
-    }
-    if (!ctx->stored_only) {
-        if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
-        if (launch_chained(rir_spectra2_kernel, grid2, CF, FFT2_SMEM, st, rir, table, c.max_sources, c.rir_taps,
-                           ctx->tw, reinterpret_cast<float4 *>(ctx->hspec), hspec_stride(ctx), ctx->leff, leff_all,
-                           mixed) != AUG_OK)
-            return AUG_ECUDA;
-        ctx->launches++;
+        AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, sizeof(int) * aug::N_COUNTERS, st));
     }
     if (mixed) {
-        dim3 grid(ctx->n_part, c.max_sources, B);
-        if (launch_chained(rir_spectra_kernel, grid, CT, FFT_SMEM, st, rir, table, c.max_sources, c.rir_taps,
-                           ctx->n_part, ctx->tw, ctx->hspec, leff_all, ctx->stored_only) != AUG_OK)
+        if (launch_chained(rir_length_kernel, dim3(c.max_sources, B), CT, 0, st, rir, table, c.max_sources, c.rir_taps,
+                           ctx->leff, leff_all) != AUG_OK)
             return AUG_ECUDA;
         ctx->launches++;
     }
+    if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
+    if (launch_chained(rir_spectra2_kernel, dim3(ctx->n_part, c.max_sources, B), CF, FFT2_SMEM, st, rir, table,
+                       c.max_sources, c.rir_taps, ctx->n_part, ctx->tw, reinterpret_cast<float4 *>(ctx->hspec),
+                       ctx->leff, mixed) != AUG_OK)
+        return AUG_ECUDA;
+    ctx->launches++;
     return AUG_OK;
+}
+
+template <Kind KIND, bool PARK>
+static int launch_convolve(AugCtx *ctx, int grid) {
+    const AugConfig &c = ctx->cfg;
+    int *counters = ctx->leff + c.max_batch;
+    if (smem_opt_in<convolve_kernel<KIND, PARK>>(ctx->device) != AUG_OK) return AUG_ECUDA;
+    const int list = KIND == FUSED ? aug::LIST_FUSED : aug::LIST_STORED;
+    const int drawn = KIND == FUSED ? aug::DRAWN_FUSED : KIND == SPECTRA ? aug::DRAWN_SPECTRA : aug::DRAWN_STORED;
+    if (launch_chained(convolve_kernel<KIND, PARK>, dim3(grid), CF, FFT2_SMEM, ctx->stream,
+                       reinterpret_cast<const Plan *>(ctx->plans), reinterpret_cast<const Unit *>(ctx->units),
+                       counters + 1 + list, counters + 1 + drawn, c.max_sources, ctx->n_part,
+                       reinterpret_cast<const float4 *>(ctx->hspec), reinterpret_cast<float4 *>(ctx->xspec),
+                       ctx->nblk_cap, ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->park,
+                       ctx->park_flags) != AUG_OK)
+        return AUG_ECUDA;
+    ctx->launches++;
+    return AUG_OK;
+}
+// As many CTAs as fit, but not more than there can be units of work.
+static int convolve_grid(const AugCtx *ctx, int B, int max_len, int ob) {
+    const int fit = std::min(FUSED_MINB * ctx->sm_count - (ctx->st_speech ? HOST_ROOM : 0), aug::PARK_SLOTS);
+    return (int)std::min<int64_t>(2 * (int64_t)B * ((max_len + ob - 1) / ob), fit);
 }
 
 int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
@@ -1061,61 +831,35 @@ int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, co
                             int max_len) {
     const AugConfig &c = ctx->cfg;
     if (max_len <= 0) return AUG_OK;
-    if (!stored_route(ctx)) return AUG_OK;
-    const int nblk = (max_len + BLK - 1) / BLK;
-    dim3 grid_x(nblk, c.max_sources, B);
-    if (launch_chained(block_spectra_kernel, grid_x, CT, FFT_SMEM, ctx->stream, speech, stride, lengths, bank,
-                       bank_len, table, c.max_sources, ctx->tw, ctx->xspec, ctx->nblk_cap, ctx->status, max_len,
-                       ctx->leff + c.max_batch, ctx->stored_only) != AUG_OK)
+    int *counters = ctx->leff + c.max_batch;
+    if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, speech, stride, lengths, bank, bank_len,
+                       table, B, c.max_sources, max_len, ctx->leff, counters, stored_route(ctx) ? 1 : 0,
+                       ctx->stored_only, ctx->status, reinterpret_cast<Plan *>(ctx->plans),
+                       reinterpret_cast<Unit *>(ctx->units), counters + 1) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
-    return AUG_OK;
+    return stored_route(ctx) ? launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, B, max_len, BLK2)) : AUG_OK;
 }
 
-int launch_convolve_finish(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
-                           const float *bank, int64_t bank_len, const AugUttParams *table, int B,
-                           int max_len) {
+int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len) {
     const AugConfig &c = ctx->cfg;
     if (max_len <= 0) return AUG_OK;
-    const int mixed = stored_route(ctx) ? 1 : 0;
-    const int *leff_all = ctx->leff + c.max_batch;
+    int rc = AUG_OK;
     if (!ctx->stored_only) {
-        if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, speech, stride, lengths, bank,
-                           bank_len, table, B, c.max_sources, max_len, ctx->leff, leff_all, mixed, ctx->status,
-                           reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
-                           ctx->leff + c.max_batch + 1) != AUG_OK)
-            return AUG_ECUDA;
-        // as many CTAs as fit, but not more than there can be units of work (blocks are shortest
-        // where a response fills min(rir_taps, 8192) taps)
-        const int ob_min = (F2 - min(c.rir_taps, BLK2) + 1) & ~3;
-        const int64_t most = 2 * (int64_t)B * ((max_len + ob_min - 1) / ob_min);
-        const int grid2 = (int)std::min<int64_t>(most, std::min(FUSED_MINB * ctx->sm_count - (ctx->st_speech ? HOST_ROOM : 0), aug::PARK_SLOTS));
-        auto kern = ctx->park ? convolve_fused2_kernel<true> : convolve_fused2_kernel<false>;
-        if ((ctx->park ? smem_opt_in<convolve_fused2_kernel<true>>(ctx->device)
-                       : smem_opt_in<convolve_fused2_kernel<false>>(ctx->device)) != AUG_OK)
-            return AUG_ECUDA;
-        if (launch_chained(kern, grid2, CF, FFT2_SMEM, ctx->stream, reinterpret_cast<const Plan *>(ctx->plans),
-                           reinterpret_cast<const Unit *>(ctx->units), ctx->leff + c.max_batch + 1, c.max_sources,
-                           reinterpret_cast<const float4 *>(ctx->hspec), hspec_stride(ctx), ctx->tw, ctx->ys, ctx->vv,
-                           ctx->ws_stride, ctx->energy, ctx->park, ctx->park_flags) != AUG_OK)
-            return AUG_ECUDA;
-        ctx->launches += 2;
+        // blocks are shortest where a response fills min(rir_taps, 8192) taps
+        const int grid = convolve_grid(ctx, B, max_len, (F2 - std::min(c.rir_taps, BLK2) + 1) & ~3);
+        rc = ctx->park ? launch_convolve<FUSED, true>(ctx, grid) : launch_convolve<FUSED, false>(ctx, grid);
+        if (rc != AUG_OK) return rc;
     }
-    if (mixed) {
-        const int nblk = (max_len + BLK - 1) / BLK;
-        dim3 grid(nblk, B);
-        if (launch_chained(spectral_convolve_kernel, grid, CT, FFT_SMEM, ctx->stream, lengths, bank, bank_len, table,
-                           c.max_sources, ctx->n_part, ctx->hspec, ctx->xspec, ctx->nblk_cap, ctx->tw, ctx->ys,
-                           ctx->vv, ctx->ws_stride, ctx->energy, max_len, ctx->leff, leff_all,
-                           ctx->stored_only) != AUG_OK)
-            return AUG_ECUDA;
-        ctx->launches++;
+    if (stored_route(ctx)) {
+        if ((rc = launch_convolve<STORED, false>(ctx, convolve_grid(ctx, B, max_len, BLK2))) != AUG_OK) return rc;
         // for the next call's choice (not waited for)
         if (ctx->leff_seen)
-            AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, leff_all, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+            AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, ctx->leff + c.max_batch, sizeof(int), cudaMemcpyDeviceToHost,
+                                        ctx->stream));
     }
-    if (launch_chained(snr_gain_kernel, dim3((B + 255) / 256), 256, 0, ctx->stream, ctx->energy, table, B,
-                       ctx->gain) != AUG_OK)
+    if (launch_chained(snr_gain_kernel, dim3((B + 255) / 256), 256, 0, ctx->stream, ctx->energy, table, B, ctx->gain) !=
+        AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;

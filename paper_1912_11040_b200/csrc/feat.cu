@@ -29,10 +29,10 @@ mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double f
     __shared__ int seg_s[513];
     chain_next();
     // first kernel of aug_pipeline: the convolution's sums and counters start from zero
+    if (leff != nullptr && blockIdx.x == 0 && threadIdx.x < aug::N_COUNTERS) counters[threadIdx.x] = 0;
     if (leff != nullptr && threadIdx.x == 0) {
         leff[blockIdx.x] = 0;
         energy[2 * blockIdx.x] = energy[2 * blockIdx.x + 1] = 0.0;
-        if (blockIdx.x == 0) counters[0] = counters[1] = counters[2] = 0;
     }
     const int utt = blockIdx.x, nb = K / 2 + 1;
     // (unwarped: the warp was already applied to the waveform)

@@ -11,6 +11,12 @@
 
 namespace fftpair {
 
+// Twiddle table, TW_N entries: for every power of two M <= TW_N the block
+// [M/2, M) holds exp(-2 pi i k / M), k < M/2, so that the factors one pass or one
+// real-FFT split needs are contiguous in k (coalesced loads).
+constexpr int TW_N = 16384;
+__host__ __device__ constexpr int tw_index(int M, int k) { return M / 2 + k; }
+
 typedef unsigned long long u64;
 
 __device__ __forceinline__ u64 pack(float lo, float hi) {
