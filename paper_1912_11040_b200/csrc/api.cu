@@ -132,10 +132,9 @@ Layout make_layout(const AugConfig &c) {
     const bool parks = c.max_sources >= 3;    // (long-response contexts use the fused route for short responses)
     l.off_park = parks ? take(sizeof(float2) * (int64_t)aug::PARK_SLOTS * aug::CONV_BINS) : -1;
     l.off_park_flags = parks ? take(sizeof(int) * aug::PARK_SLOTS) : -1;
-    // its list of work: two outputs of every block, blocks as short as min(rir_taps, 8192) taps make them
+    // its list of work: two outputs of every block, blocks as short as 8192 taps make them
     l.off_plans = take((int64_t)aug::PLAN_BYTES * B);
-    const int ob = (2 * aug::CONV_TAPS - std::min(c.rir_taps, aug::CONV_TAPS) + 1) & ~3;
-    l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + ob - 1) / ob));
+    l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS));
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take(sizeof(double) * 2 * B);
