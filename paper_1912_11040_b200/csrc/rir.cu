@@ -8,11 +8,11 @@
 //      an integer n0 and a fraction phi; the five numbers the taps need are
 //      written, compacted over the images that contribute, to a slot of a small
 //      shared-memory ring owned by the warp.
-//   B  two images at a time, their 2 W_h taps over the lanes: lane l owns taps l and l + 32
-//      of both, and of the 16 taps that are left (W_h = 40) the lower half-warp does those of
-//      the first image and the upper half those of the second.  Everything that depends only
-//      on the tap (its offset, the cosine and sine of its Hann angle, its sign) sits in
-//      registers, and the images' numbers arrive as pairs, the operands of packed (f32x2)
+//   B  four images at a time, their 2 W_h taps over the lanes: lane l owns taps l and l + 32
+//      of all four, and of the 16 taps that are left (W_h = 40) the lower half-warp does those
+//      of the first two images and the upper half those of the others.  Everything that
+//      depends only on the tap (its offset, the cosine and sine of its Hann angle, its sign) sits
+//      in registers, and the images' numbers arrive as pairs, the operands of packed (f32x2)
 //      arithmetic, by broadcast loads.  With tau = n0 + phi, 0 <= phi < 1,
 //      sin(pi (n - tau)) = -(-1)^(n - n0) sin(pi phi), and the Hann factor follows
 //      from the angle-sum identity, so a tap costs one reciprocal, three to four fused
@@ -20,9 +20,14 @@
 //      low bits -- and one shared-memory reduction.  n0 is rounded down so that the window
 //      always covers the same taps -W_h + 1 .. W_h and none has to be masked.
 //
-// Bound by instruction issue (45 warp instructions an image, 72 % of the slots).  One image at
-// a time in scalar arithmetic, with a conversion instruction per tap and masks, it was 58, and
-// the quarter-rate pipe of reciprocals and conversions was 62 % busy too.
+//      Phase A orders the images of a batch: loud ones (their taps need more than 22 bits) first,
+//      then the others whose window lies inside the response, then those at its edges, which are
+//      done one by one with tests.  No test is left in the loops over the first two.
+//
+// Bound by instruction issue (30 warp instructions an image, 70 % of the slots; reciprocal pipe 60 %).  One image at a time in scalar
+// arithmetic, with a conversion instruction per tap and masks, it was 58, and the quarter-rate
+// pipe of reciprocals and conversions was 62 % busy too; two at a time with tests of strength and
+// range per pair 45.
 //
 // The response is accumulated in 32-bit fixed point: a shared-memory fp32 atomic
 // add is a compare-and-swap loop on this hardware, an integer one is a single
@@ -37,6 +42,8 @@
 // The lattice points with |kx|+|ky|+|kz| <= order are enumerated compactly (a
 // prefix over kx, then closed forms inside the diamond of (ky, kz)), so every
 // lane of a warp carries a real image.
+#include <type_traits>
+
 #include "common.cuh"
 #include "fft_pair.cuh"
 
@@ -70,11 +77,8 @@ __host__ __device__ constexpr size_t rir_smem_bytes(int threads, int L) {
 
 constexpr float HEADROOM_LOG2 = 6.f;   // full scale = 2^6 times the direct-path amplitude
 
-// Entries of a warp's ring, each an array of 32: delay (first sample of the window plus BIAS; the bit
-// STRONG set if the image's taps may exceed 2^22 steps), phi, P0, P1, P2.
+// Entries of a warp's ring, each an array of 32: first sample of the window, phi, P0, P1, P2.
 enum Ring { R_N = 0, R_PHI = 32, R_P0 = 64, R_P1 = 96, R_P2 = 128, RING = 160 };
-constexpr int STRONG = 1 << 29, BIAS = 64;
-static_assert(BIAS >= aug::MAX_HALF_W, "delays are not negative");
 
 // round(v) by additions (the conversion instruction shares the quarter-rate pipe with the
 // reciprocals): adding 1.5 2^23 leaves the nearest integer, |v| < 2^22, in the low bits.
@@ -166,7 +170,8 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
     }
     const u64 nsgn = fftpair::both(-sgn);
     constexpr int NW = THREADS / 32;
-    const unsigned h_addr = (unsigned)__cvta_generic_to_shared(h) + 4u * lane - 4u * BIAS;
+    const unsigned h_addr = (unsigned)__cvta_generic_to_shared(h) + 4u * lane;
+    const unsigned h_rest = h_addr + (lane < 16 ? 256u : 192u);      // of this lane's tap among the last 16
     // first-tap samples for which all 96 lane slots (80 of them taps) stay inside the response
     const unsigned inside = (unsigned)max(L - 96, 0);
     int *my = ring + warp * RING;
@@ -175,7 +180,8 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
         // ---- phase A: one image per lane
         const int idx = base + lane;
         bool valid = idx < total;
-        int n_first = BIAS;
+        int n_first = 0;
+        bool strong = false;
         float phi = 0.5f, p0 = 0.f, p1 = 0.f, p2 = 0.f;
         if (valid) {
             int ix, ky, kz;
@@ -223,11 +229,11 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             // a fraction of exactly zero would make the centre tap 0/0: 1e-7 of a sample
             // away from it the tap is the same to 3e-7 of its size
             phi = fmaxf(phi, 1e-7f);
-            n_first = n0 - half_w + 1 + BIAS;
+            n_first = n0 - half_w + 1;
             const float A = g * (float)rd;
-            valid = d2 > 0.0 && A != 0.f && n_first < L + BIAS;
+            valid = d2 > 0.0 && A != 0.f && n_first < L;
             // no tap is larger than A
-            if (fabsf(A) * scale >= 4194303.f) n_first |= STRONG;
+            strong = fabsf(A) * scale >= 4194303.f;
             const float As = -A * scale * sinpif(phi) * 0.318309886183790671538f;
             float sps, cps;
             sincospif(phi / fhw, &sps, &cps);
@@ -235,13 +241,18 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             p1 = p0 * cps;
             p2 = p0 * sps;
         }
-        const unsigned mask = __ballot_sync(0xffffffffu, valid);
-        const int cnt = __popc(mask);
+        const bool in = valid && (unsigned)n_first < inside;
+        const unsigned below = (1u << lane) - 1u;
+        const unsigned m_strong = __ballot_sync(0xffffffffu, in && strong), m_in = __ballot_sync(0xffffffffu, in);
+        const unsigned m_valid = __ballot_sync(0xffffffffu, valid);
+        const int n_strong = __popc(m_strong), n_in = __popc(m_in), cnt = __popc(m_valid);
         {
-            // contributing images to the front; one that adds nothing pairs with an odd last one
-            const int pos = valid ? __popc(mask & ((1u << lane) - 1u)) : cnt + __popc(~mask & ((1u << lane) - 1u));
+            // strong ones, other ones inside, those at the edges, and lanes without an image, which add
+            // nothing if they fill up a group of four
+            const int pos = in ? (strong ? __popc(m_strong & below) : n_strong + __popc(m_in & ~m_strong & below))
+                               : valid ? n_in + __popc(m_valid & ~m_in & below) : cnt + __popc(~m_valid & below);
             if (!valid) {
-                n_first = BIAS;
+                n_first = 0;
                 phi = 0.5f;
                 p0 = p1 = p2 = 0.f;
             }
@@ -252,76 +263,73 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             my[R_P2 + pos] = __float_as_int(p2);
         }
         __syncwarp();
-        // ---- phase B: the taps of two images over the lanes
+        // ---- phase B: the taps of four images over the lanes
         // A sinc(x) hann(x) = (1/x) (-A sin(pi phi)/pi) (-1)^j (1/2 + 1/2 cos(pi x / W_h)), x = j - phi
-        for (int k = 0; k < cnt; k += 2) {
-            using namespace fftpair;
-            const int2 n = *reinterpret_cast<const int2 *>(my + R_N + k);
-            const int na = n.x & ~STRONG, nb = n.y & ~STRONG;
-            if ((unsigned)(na - BIAS) < inside && (unsigned)(nb - BIAS) < inside) {
-                // every tap of both windows falls inside the response: no index checks, the adds of an
-                // image go to fixed offsets from one address
-                const u64 ph = *reinterpret_cast<const u64 *>(my + R_PHI + k);
-                const u64 q0 = *reinterpret_cast<const u64 *>(my + R_P0 + k);
-                const u64 q1 = *reinterpret_cast<const u64 *>(my + R_P1 + k);
-                const u64 q2 = *reinterpret_cast<const u64 *>(my + R_P2 + k);
-                const unsigned a = h_addr + 4u * (unsigned)na, b = h_addr + 4u * (unsigned)nb;
-                const bool strong = ((n.x | n.y) & STRONG) != 0;
-                constexpr int PAIRS = NARROW ? 2 : 3;
-                u64 rx[PAIRS], num[PAIRS];
-#pragma unroll
-                for (int i = 0; i < PAIRS; ++i) {
-                    const float2 x = unpack(fma2(nsgn, ph, both(fj[i])));
-                    rx[i] = pack(rcp_approx(x.x), rcp_approx(x.y));
-                    num[i] = fma2(both(sj[i]), q2, fma2(both(cj[i]), q1, q0));
-                }
-                float rs = 0.f, nums = 0.f;
-                if (NARROW) {
-                    // the last 16 taps, lower half-warp: first image, upper half: second
-                    const int w = k + (lane >> 4);
-                    rs = rcp_approx(fmaf(-sgn, __int_as_float(my[R_PHI + w]), fj[2]));
-                    nums = fmaf(sj[2], __int_as_float(my[R_P2 + w]),
-                                fmaf(cj[2], __int_as_float(my[R_P1 + w]), __int_as_float(my[R_P0 + w])));
-                }
-                int2 t[PAIRS];
-                int ts = 0;
-                if (!strong) {
-#pragma unroll
-                    for (int i = 0; i < PAIRS; ++i) {
-                        const float2 v = unpack(fma2(rx[i], num[i], both(TO_INT)));
-                        t[i] = make_int2(__float_as_int(v.x) - INT_BITS, __float_as_int(v.y) - INT_BITS);
-                    }
-                    if (NARROW) ts = __float_as_int(fmaf(rs, nums, TO_INT)) - INT_BITS;
+        using namespace fftpair;
+        const int n_fast = inside == 0 ? 0 : cnt == n_in ? (n_in + 3) & ~3 : n_in & ~3;
+        const int n_loud = min((n_strong + 3) & ~3, n_fast);
+        auto four = [&](int k, auto loud) {
+            auto taps = [&](u64 ph, u64 q0, u64 q1, u64 q2, int i) {
+                const float2 x = unpack(fma2(nsgn, ph, both(fj[i])));
+                const u64 rx = pack(rcp_approx(x.x), rcp_approx(x.y));
+                const u64 num = fma2(both(sj[i]), q2, fma2(both(cj[i]), q1, q0));
+                if constexpr (decltype(loud)::value) {
+                    return round_strong(mul2(rx, num));
                 } else {
-#pragma unroll
-                    for (int i = 0; i < PAIRS; ++i) t[i] = round_strong(mul2(rx[i], num[i]));
-                    if (NARROW) ts = __float2int_rn(rs * nums);
+                    const float2 v = unpack(fma2(rx, num, both(TO_INT)));
+                    return make_int2(__float_as_int(v.x) - INT_BITS, __float_as_int(v.y) - INT_BITS);
                 }
-                red_shared_add<0>(a, t[0].x);
-                red_shared_add<0>(b, t[0].y);
-                red_shared_add<128>(a, t[1].x);
-                red_shared_add<128>(b, t[1].y);
-                if (NARROW) {
-                    red_shared_add<256>(lane < 16 ? a : b - 64u, ts);
-                } else {
-                    red_shared_add<256>(a, t[PAIRS - 1].x);
-                    red_shared_add<256>(b, t[PAIRS - 1].y);
-                }
+            };
+            // every tap of the windows falls inside the response: no index checks, the adds of an image
+            // go to fixed offsets from one address
+            const int4 n = *reinterpret_cast<const int4 *>(my + R_N + k);
+            const ulonglong2 ph = *reinterpret_cast<const ulonglong2 *>(my + R_PHI + k);
+            const ulonglong2 q0 = *reinterpret_cast<const ulonglong2 *>(my + R_P0 + k);
+            const ulonglong2 q1 = *reinterpret_cast<const ulonglong2 *>(my + R_P1 + k);
+            const ulonglong2 q2 = *reinterpret_cast<const ulonglong2 *>(my + R_P2 + k);
+            const unsigned a = h_addr + 4u * n.x, b = h_addr + 4u * n.y, c = h_addr + 4u * n.z, d = h_addr + 4u * n.w;
+            const int2 s0 = taps(ph.x, q0.x, q1.x, q2.x, 0), t0 = taps(ph.y, q0.y, q1.y, q2.y, 0);
+            red_shared_add<0>(a, s0.x);
+            red_shared_add<0>(b, s0.y);
+            red_shared_add<0>(c, t0.x);
+            red_shared_add<0>(d, t0.y);
+            const int2 s1 = taps(ph.x, q0.x, q1.x, q2.x, 1), t1 = taps(ph.y, q0.y, q1.y, q2.y, 1);
+            red_shared_add<128>(a, s1.x);
+            red_shared_add<128>(b, s1.y);
+            red_shared_add<128>(c, t1.x);
+            red_shared_add<128>(d, t1.y);
+            if constexpr (NARROW) {
+                // the last 16 taps, lower half-warp: first two images, upper half: the others
+                const int *w = my + k + 2 * (lane >> 4);
+                const int2 m = *reinterpret_cast<const int2 *>(w + R_N);
+                const int2 s2 = taps(*reinterpret_cast<const u64 *>(w + R_PHI), *reinterpret_cast<const u64 *>(w + R_P0),
+                                     *reinterpret_cast<const u64 *>(w + R_P1), *reinterpret_cast<const u64 *>(w + R_P2), 2);
+                red_shared_add<0>(h_rest + 4u * m.x, s2.x);
+                red_shared_add<0>(h_rest + 4u * m.y, s2.y);
             } else {
+                const int2 s2 = taps(ph.x, q0.x, q1.x, q2.x, 2), t2 = taps(ph.y, q0.y, q1.y, q2.y, 2);
+                red_shared_add<256>(a, s2.x);
+                red_shared_add<256>(b, s2.y);
+                red_shared_add<256>(c, t2.x);
+                red_shared_add<256>(d, t2.y);
+            }
+        };
 #pragma unroll 1
-                for (int w = k; w < min(k + 2, cnt); ++w) {
-                    const int n_f = (my[R_N + w] & ~STRONG) - BIAS;
-                    const float f = __int_as_float(my[R_PHI + w]), P0 = __int_as_float(my[R_P0 + w]);
-                    const float P1 = __int_as_float(my[R_P1 + w]), P2 = __int_as_float(my[R_P2 + w]);
+        for (int k = 0; k < n_loud; k += 4) four(k, std::true_type());
+#pragma unroll 1
+        for (int k = n_loud; k < n_fast; k += 4) four(k, std::false_type());
+#pragma unroll 1
+        for (int w = n_fast; w < cnt; ++w) {
+            const int n_f = my[R_N + w];
+            const float f = __int_as_float(my[R_PHI + w]), P0 = __int_as_float(my[R_P0 + w]);
+            const float P1 = __int_as_float(my[R_P1 + w]), P2 = __int_as_float(my[R_P2 + w]);
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        const float x = fmaf(-sgn, f, fj[i]);
-                        const int m = n_f + lane + 32 * i;
-                        const float v = rcp_approx(x) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
-                        const bool mine = !NARROW || i < 2 || lane < 16;
-                        if (mine && (unsigned)m < (unsigned)L) atomicAdd(&h[m], __float2int_rn(v));
-                    }
-                }
+            for (int i = 0; i < 3; ++i) {
+                const float x = fmaf(-sgn, f, fj[i]);
+                const int m = n_f + lane + 32 * i;
+                const float v = rcp_approx(x) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
+                const bool mine = !NARROW || i < 2 || lane < 16;
+                if (mine && (unsigned)m < (unsigned)L) atomicAdd(&h[m], __float2int_rn(v));
             }
         }
         __syncwarp();   // the ring slots are rewritten by the next batch
@@ -368,10 +376,11 @@ static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *r
 }
 
 // Both sizes keep 32 warps with 64 registers on a multiprocessor.  Four CTAs of 256 threads
-// balance better where the responses fit four times and there are enough of them: 4096 x 2
-// responses of 4096 taps 355 us against 399 with two of 512, 512 x 4 of 8192 taps 204 against
-// 213.  Long responses fit twice (128 x 4 of 24000 taps: 313 against 383), and a few responses
-// are done sooner by more warps each (8 x 2: 12.7 against 14.8).
+// balance better where the responses fit four times and there are enough of them (measured on
+// the form with two images at a time: 4096 x 2 responses of 4096 taps 355 us against 399 with
+// two of 512, 512 x 4 of 8192 taps 204 against 213).  Long responses fit twice (128 x 4 of
+// 24000 taps: 313 against 383), and a few responses are done sooner by more warps each
+// (8 x 2: 12.7 against 14.8).
 int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
     const bool fit = 4 * (rir_smem_bytes(256, ctx->cfg.rir_taps) + 1024) <= (size_t)ctx->smem_per_sm;
     const bool many = (int64_t)B * ctx->cfg.max_sources >= 4 * (int64_t)ctx->sm_count;
