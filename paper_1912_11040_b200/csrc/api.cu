@@ -138,7 +138,7 @@ Layout make_layout(const AugConfig &c) {
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take(sizeof(double) * 2 * B);
-    l.off_leff = take(sizeof(int) * (B + aug::N_COUNTERS));
+    l.off_leff = take(sizeof(int) * (2 * B + aug::N_COUNTERS));     // (right behind the sums: one memset sets both to zero)
     l.off_gain = take(sizeof(float) * B);
     l.off_melw = take(sizeof(aug::MelBin) * B * l.n_bins);
     l.off_melstart = take(sizeof(int) * B * (c.n_mel + 2));
@@ -430,9 +430,9 @@ int aug_reverb_mix(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if (speech_stride <= 0 || (speech_stride & 3) || bank_len < 0) return AUG_EINVAL;
     const int max_len = (int)(speech_stride < ctx->cfg.max_samples ? speech_stride : ctx->cfg.max_samples);
     if (speech_stride > ctx->ws_stride) return AUG_ECAP;
-    if ((rc = launch_rir_spectra(ctx, rir_dev, table_dev, B, true)) != AUG_OK) return rc;
-    if ((rc = launch_convolve_prepare(ctx, speech_dev, speech_stride, lengths_dev, noise_bank_dev,
-                                      bank_len, table_dev, B, max_len)) != AUG_OK) return rc;
+    const ConvInput in = {speech_dev, speech_stride, lengths_dev, noise_bank_dev, bank_len, max_len};
+    if ((rc = launch_rir_spectra(ctx, rir_dev, in, table_dev, B, true)) != AUG_OK) return rc;
+    if ((rc = launch_convolve_prepare(ctx, in, table_dev, B)) != AUG_OK) return rc;
     if ((rc = launch_convolve_finish(ctx, table_dev, B, max_len)) != AUG_OK) return rc;
     return launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out_dev, speech_stride);
 }
@@ -493,6 +493,9 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     // the stages follow one another, chained (see chain_wait).  The filterbank tables depend on
     // the parameter table alone and come first: the impulse responses start beside them.
     cudaStream_t sm = ctx->stream;
+    // with a waveform-domain warp the simulator sees the warped speech
+    const ConvInput in = {ctx->warped ? ctx->warped : speech_dev, ctx->warped ? ctx->ws_stride : speech_stride,
+                          lengths_dev, noise_bank_dev, bank_len, max_len};
     t0(2, sm);
     rc = launch_mel_tables(ctx, table_dev, B, true);
     t1(2, sm);
@@ -500,20 +503,15 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if (rc == AUG_OK) rc = launch_rir(ctx, table_dev, B, ctx->rir, true);
     t1(0, sm);
     t0(1, sm);
-    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, table_dev, B, false);
+    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, false);
     t1(1, sm);
 
-    // waveform-domain warp first: the simulator then sees the warped speech (timed with stage 3)
+    // waveform-domain warp (timed with stage 3)
     t0(3, sm);
-    if (rc == AUG_OK && ctx->warped) {
+    if (rc == AUG_OK && ctx->warped)
         rc = launch_vtlp_resynth(ctx, speech_dev, speech_stride, lengths_dev, table_dev, B, max_len,
                                  ctx->warped, ctx->ws_stride);
-        speech_dev = ctx->warped;
-        speech_stride = ctx->ws_stride;
-    }
-    if (rc == AUG_OK)
-        rc = launch_convolve_prepare(ctx, speech_dev, speech_stride, lengths_dev, noise_bank_dev,
-                                     bank_len, table_dev, B, max_len);
+    if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B);
     t1(3, sm);
     if (rc != AUG_OK) return rc;
     t0(4, sm);

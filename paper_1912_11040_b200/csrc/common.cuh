@@ -73,7 +73,7 @@ struct AugCtx {
     float *ys;             // [max_batch][ws_stride]
     float *vv;             // [max_batch][ws_stride]
     double *energy;        // [max_batch][2]
-    int *leff;             // [max_batch + N_COUNTERS] (behind the lengths: largest over the batch, counters)
+    int *leff;             // [2 max_batch + N_COUNTERS] (behind the lengths: largest over the batch, counters; sources transformed)
     int *leff_seen;        // pinned host copy of that last entry from an earlier call (long-response contexts)
     int stored_only;       // this call launches the stored-spectra kernels alone taps up to the last non-zero one, largest over the utterance's sources
     float *gain;           // [max_batch] noise gain g for the requested SNR
@@ -151,19 +151,28 @@ inline int launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t sme
 }
 #endif
 
+// What the convolution reads besides the responses; samples beyond max_len of a row are not used.
+struct ConvInput {
+    const float *speech;
+    int64_t stride;
+    const int *lengths;
+    const float *bank;
+    int64_t bank_len;
+    int max_len;
+};
+
 // Launchers (defined next to their kernels).  They enqueue on ctx->stream unless a
 // stream is passed.
 // `beside`: may run beside the kernel before it on the stream, one of this library that calls chain_next()
 int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside);
 // `reset`: set the counters and sums of the convolution to zero first (aug_pipeline has had it done by
 // launch_mel_tables)
-int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table, int B, bool reset);
+int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
+                       bool reset);
 // Convolution in two parts: `prepare` needs only the input audio (block spectra when
 // the response has several partitions, else nothing), `finish` also needs the
 // partition spectra of the impulse responses.
-int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
-                            const float *bank, int64_t bank_len, const AugUttParams *table, int B,
-                            int max_len);
+int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
 int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len);
 int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
                float *wave_out, int64_t out_stride);

@@ -381,12 +381,100 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
     __stcg(reinterpret_cast<ulonglong2 *>(p + CF), make_ulonglong2(z.qr, z.qi));
 }
 
+// ---------------------------------------------------------------- the list of work
+// One unit of work is one block of one output (the reverberant speech, or the sum of the noise
+// sources) of an utterance.  plan_kernel lists the units that exist -- how many blocks an
+// utterance has depends on its length and on where its responses end -- and what they need to
+// know; the convolving kernels' CTAs, as many as fit the device, work through the list.  With one CTA
+// per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
+// (two thirds of them without work) and to each one's chain of loads before its first sample.
+struct Plan {
+    const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
+    int nlen[AUG_S_MAX];           // their lengths ([0] unused)
+    int src[AUG_S_MAX];            // their source numbers
+    int n_src;                     // 0: the row was rejected, both outputs are silence
+    int n_noise;
+    int N;                         // samples of the utterance
+    int ob;                        // outputs per block
+    int parts;                     // partitions that are not zero throughout (stored-spectra route)
+};
+struct Unit {
+    int utt;
+    int block2;                    // 2 block + (1 for the noise sum)
+};
+static_assert(sizeof(Plan) % 4 == 0 && sizeof(Plan) <= aug::PLAN_BYTES && sizeof(Unit) == 8, "");
+
+// All that planning an utterance takes; n_cap: rows are not read beyond.
+struct PlanArgs {
+    const float *speech;
+    int64_t stride;
+    const int *lengths;
+    const float *bank;
+    int64_t bank_len;
+    int n_cap;
+    int *status;
+    Plan *plans;
+    Unit *units;
+    int *lists;                    // counters of the two lists
+};
+// By one warp; leff: taps up to the last non-zero one.
+__device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttParams &row, int utt, int S_max, int leff,
+                                               bool stored, int lane) {
+    const int N = min(max(a.lengths[utt], 0), a.n_cap);
+    // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
+    // of 4, where taps counts up to the last non-zero tap of this utterance's responses
+    const int ob = stored ? BLK2 : (F2 - min(max(leff, 1), BLK2) + 1) & ~3;
+    const int n = 2 * ((N + ob - 1) / ob);
+    int at = 0;
+    if (lane == 0) {
+        Plan p;
+        p.N = N;
+        p.ob = ob;
+        p.parts = (max(leff, 1) + BLK2 - 1) / BLK2;
+        p.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;    // (reported by step 1)
+        p.n_noise = 0;
+        p.x[0] = a.speech + (int64_t)utt * a.stride;
+        p.nlen[0] = 1;
+        p.src[0] = 0;
+        for (int s = 1; s < p.n_src; ++s) {
+            const float *x;
+            int nlen;
+            if (source_of(row, s, nullptr, a.bank, a.bank_len, x, nlen)) {
+                ++p.n_noise;
+                p.x[p.n_noise] = x;
+                p.nlen[p.n_noise] = nlen;
+                p.src[p.n_noise] = s;
+            } else if (n > 0 && atomicCAS(&a.status[0], -1, utt) == -1) {
+                a.status[1] = aug::R_NOISE;
+            }
+        }
+        a.plans[utt] = p;
+        if (n > 0) at = atomicAdd(a.lists + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (int i = lane; i < n; i += 32) a.units[at + i] = Unit{utt, i};
+}
+
+// One warp per utterance (contexts for long responses: the route follows from the whole batch;
+// elsewhere rir_spectra2_kernel plans on the way).
+__global__ void __launch_bounds__(256)
+plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restrict__ table, int B, int S_max,
+            const int *__restrict__ leff, const int *__restrict__ leff_all, int stored_only) {
+    const int utt = blockIdx.x * 8 + (threadIdx.x >> 5);
+    chain_next();
+    chain_wait();
+    if (utt < B)
+        plan_utterance(args, table[utt], utt, S_max, leff[utt], stored_only || !takes_fused_route(*leff_all),
+                       threadIdx.x & 31);
+}
+
 // Spectra of the partitions of each impulse response: 8192 taps (those beyond L are zero) and as many
 // zeros, scaled by the noise weight and 1/F (and by 1/4 for
 // the two doubled spectra of a product).
 __global__ void __launch_bounds__(CF, FUSED_MINB)
 rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max,
-                    int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int *leff, int mixed) {
+                    int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int *leff, int mixed,
+                    int *transformed, const __grid_constant__ PlanArgs plan) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
     __shared__ int red_i[CF / 32];
@@ -397,7 +485,11 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
     // this kernel reads every tap anyway and records the length on the way
     if (mixed && part > 0 && from >= leff[utt]) return;
     const AugUttParams &row = table[utt];
-    if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) return;
+    if (row.n_src < 1 || row.n_src > S_max) {
+        if (!mixed && s == 0 && t < 32) plan_utterance(plan, row, utt, S_max, 1, false, t);
+        return;
+    }
+    if (s >= row.n_src) return;
     const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (4.f * (float)F2);
     const float *h = rir + ((int64_t)utt * S_max + s) * L;
     float4 *out = hspec + (((int64_t)utt * S_max + s) * P + part) * (NB2 / 2) + t;
@@ -425,10 +517,20 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
         if ((t & 31) == 0) red_i[t >> 5] = last;
     }
     __syncthreads();
-    if (!mixed && t == 0) {
-        int m = 0;
-        for (int i = 0; i < CF / 32; ++i) m = max(m, red_i[i]);
-        if (m > 0) atomicMax(&leff[utt], m);
+    if (!mixed && t < 32) {
+        int m = t < CF / 32 ? red_i[t] : 0;
+#pragma unroll
+        for (int o = CF / 64; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        // the CTA that adds the last source's length plans the utterance's work
+        int done = 0;
+        if (t == 0) {
+            atomicMax(&leff[utt], m);
+            __threadfence();
+            done = atomicAdd(&transformed[utt], 1) + 1;
+            __threadfence();
+        }
+        if (__shfl_sync(0xffffffffu, done, 0) == row.n_src)
+            plan_utterance(plan, row, utt, S_max, __ldcg(&leff[utt]), false, t);
     }
     fftpair::forward4096(v, sh, t, tw);
     chain_next();
@@ -442,76 +544,6 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
         x = {fftpair::mul2(x.pr, sc), fftpair::mul2(x.pi, sc), fftpair::mul2(x.qr, sc), fftpair::mul2(x.qi, sc)};
         store_bins(out + 2 * r * CF, x);
     }
-}
-
-// ---------------------------------------------------------------- the list of work
-// One unit of work is one block of one output (the reverberant speech, or the sum of the noise
-// sources) of an utterance.  plan_kernel lists the units that exist -- how many blocks an
-// utterance has depends on its length and on where its responses end -- and what they need to
-// know; the convolving kernels' CTAs, as many as fit the device, work through the list.  With one CTA
-// per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
-// (two thirds of them without work) and to each one's chain of loads before its first sample.
-struct Plan {
-    const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
-    int nlen[AUG_S_MAX];           // their lengths ([0] unused)
-    int src[AUG_S_MAX];            // their source numbers
-    int n_src;                     // 0: the row was rejected, both outputs are silence
-    int n_noise;
-    int N;                         // samples of the utterance
-    int ob;                        // outputs per block
-    int parts;                     // partitions that are not zero throughout (stored-spectra route)
-};
-struct Unit {
-    int utt;
-    int block2;                    // 2 block + (1 for the noise sum)
-};
-static_assert(sizeof(Plan) % 4 == 0 && sizeof(Plan) <= aug::PLAN_BYTES && sizeof(Unit) == 8, "");
-
-// One warp per utterance.
-__global__ void __launch_bounds__(256)
-plan_kernel(const float *__restrict__ speech, int64_t stride, const int *__restrict__ lengths,
-            const float *__restrict__ bank, int64_t bank_len, const AugUttParams *__restrict__ table, int B,
-            int S_max, int n_cap, const int *__restrict__ leff, const int *__restrict__ leff_all, int mixed,
-            int stored_only, int *status, Plan *__restrict__ plans, Unit *__restrict__ units, int *__restrict__ n_units) {
-    const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    chain_next();
-    chain_wait();
-    if (utt >= B) return;
-    const bool stored = mixed && (stored_only || !takes_fused_route(*leff_all));
-    const AugUttParams &row = table[utt];
-    const int N = min(max(lengths[utt], 0), n_cap);
-    // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
-    // of 4, where taps counts up to the last non-zero tap of this utterance's responses
-    const int ob = stored ? BLK2 : (F2 - min(max(leff[utt], 1), BLK2) + 1) & ~3;
-    const int n = 2 * ((N + ob - 1) / ob);
-    int at = 0;
-    if (lane == 0) {
-        Plan p;
-        p.N = N;
-        p.ob = ob;
-        p.parts = (max(leff[utt], 1) + BLK2 - 1) / BLK2;
-        p.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;    // (reported by step 1)
-        p.n_noise = 0;
-        p.x[0] = speech + (int64_t)utt * stride;
-        p.nlen[0] = 1;
-        p.src[0] = 0;
-        for (int s = 1; s < p.n_src; ++s) {
-            const float *x;
-            int nlen;
-            if (source_of(row, s, nullptr, bank, bank_len, x, nlen)) {
-                ++p.n_noise;
-                p.x[p.n_noise] = x;
-                p.nlen[p.n_noise] = nlen;
-                p.src[p.n_noise] = s;
-            } else if (n > 0 && atomicCAS(&status[0], -1, utt) == -1) {
-                status[1] = aug::R_NOISE;
-            }
-        }
-        plans[utt] = p;
-        if (n > 0) at = atomicAdd(n_units + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
-    }
-    at = __shfl_sync(0xffffffffu, at, 0);
-    for (int i = lane; i < n; i += 32) units[at + i] = Unit{utt, i};
 }
 
 // KIND  FUSED    a block of one output from its samples (responses of one partition)
@@ -548,15 +580,17 @@ convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, 
     const int t = threadIdx.x, G = gridDim.x;
     fftpair::fill_tables(sh, t, tw);
     chain_wait();
+    // (the list has room for every CTA's first unit: it is read beside the count)
+    const Unit first = units[blockIdx.x];
     const int count = __ldcg(n_units);
     if (blockIdx.x >= count) return;
-    if (t == 0) {
+    if (t == 32) {
         const int second = blockIdx.x + G;
-        unit_s[0] = units[blockIdx.x];
+        unit_s[0] = first;
         unit_s[1] = second < count ? units[second] : Unit{-1, 0};
     }
     if (t < (int)(sizeof(Plan) / 4))
-        reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + units[blockIdx.x].utt)[t];
+        reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + first.utt)[t];
     __syncthreads();
     const bool own_slot = KIND == FUSED && PARK && park != nullptr && park_flags[blockIdx.x] == 0;
 
@@ -776,18 +810,24 @@ constexpr size_t FFT2_SMEM = sizeof(fftpair::Shared);
 
 static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_STORED; }
 
-int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table, int B, bool reset) {
+static PlanArgs plan_args(const AugCtx *ctx, const ConvInput &in) {
+    return {in.speech, in.stride, in.lengths, in.bank, in.bank_len, in.max_len, ctx->status,
+            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
+            ctx->leff + ctx->cfg.max_batch + 1};
+}
+
+int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
+                       bool reset) {
     const AugConfig &c = ctx->cfg;
     const cudaStream_t st = ctx->stream;
     const int mixed = stored_route(ctx) ? 1 : 0;
     // long-response context: the last batch size seen decides whether the fused kernels are launched at all
     ctx->stored_only = mixed && ctx->leff_seen && *ctx->leff_seen > BLK2;
     int *leff_all = ctx->leff + ctx->cfg.max_batch;
-    if (reset) {
-        AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0, sizeof(double) * 2 * (size_t)B, st));
-        AUG_CUDA_OK(cudaMemsetAsync(ctx->leff, 0, sizeof(int) * (size_t)B, st));
-        AUG_CUDA_OK(cudaMemsetAsync(leff_all, 0, sizeof(int) * aug::N_COUNTERS, st));
-    }
+    if (reset)                       // sums, lengths and counters, which lie one behind the other
+        AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0,
+                                    reinterpret_cast<char *>(ctx->leff + 2 * (size_t)c.max_batch + aug::N_COUNTERS) -
+                                        reinterpret_cast<char *>(ctx->energy), st));
     if (mixed) {
         if (launch_chained(rir_length_kernel, dim3(c.max_sources, B), CT, 0, st, rir, table, c.max_sources, c.rir_taps,
                            ctx->leff, leff_all) != AUG_OK)
@@ -797,7 +837,7 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const AugUttParams *table,
     if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
     if (launch_chained(rir_spectra2_kernel, dim3(ctx->n_part, c.max_sources, B), CF, FFT2_SMEM, st, rir, table,
                        c.max_sources, c.rir_taps, ctx->n_part, ctx->tw, reinterpret_cast<float4 *>(ctx->hspec),
-                       ctx->leff, mixed) != AUG_OK)
+                       ctx->leff, mixed, leff_all + aug::N_COUNTERS, plan_args(ctx, in)) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
@@ -826,19 +866,14 @@ static int convolve_grid(const AugCtx *ctx, int B, int max_len, int ob) {
     return (int)std::min<int64_t>(2 * (int64_t)B * ((max_len + ob - 1) / ob), fit);
 }
 
-int launch_convolve_prepare(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
-                            const float *bank, int64_t bank_len, const AugUttParams *table, int B,
-                            int max_len) {
+int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B) {
     const AugConfig &c = ctx->cfg;
-    if (max_len <= 0) return AUG_OK;
-    int *counters = ctx->leff + c.max_batch;
-    if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, speech, stride, lengths, bank, bank_len,
-                       table, B, c.max_sources, max_len, ctx->leff, counters, stored_route(ctx) ? 1 : 0,
-                       ctx->stored_only, ctx->status, reinterpret_cast<Plan *>(ctx->plans),
-                       reinterpret_cast<Unit *>(ctx->units), counters + 1) != AUG_OK)
+    if (in.max_len <= 0 || !stored_route(ctx)) return AUG_OK;
+    if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, plan_args(ctx, in), table, B, c.max_sources,
+                       ctx->leff, ctx->leff + c.max_batch, ctx->stored_only) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
-    return stored_route(ctx) ? launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, B, max_len, BLK2)) : AUG_OK;
+    return launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, B, in.max_len, BLK2));
 }
 
 int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len) {

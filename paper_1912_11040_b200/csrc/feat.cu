@@ -32,6 +32,7 @@ mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double f
     if (leff != nullptr && blockIdx.x == 0 && threadIdx.x < aug::N_COUNTERS) counters[threadIdx.x] = 0;
     if (leff != nullptr && threadIdx.x == 0) {
         leff[blockIdx.x] = 0;
+        counters[aug::N_COUNTERS + blockIdx.x] = 0;
         energy[2 * blockIdx.x] = energy[2 * blockIdx.x + 1] = 0.0;
     }
     const int utt = blockIdx.x, nb = K / 2 + 1;

@@ -36,3 +36,28 @@ def test_runs_of_rounds(win, n_max, B):
         check_wave(got[b, :n], oracle.vtlp_resynth(speech[b, :n].astype(np.float64), float(tab[b]["alpha"]), win),
                    f"utt {b} of {n} samples")
         assert np.all(np.isnan(got[b, n:]))
+
+
+def test_wave_of_a_warped_batch_keeps_the_callers_row_stride():
+    """The mixed waveform of a call with the waveform warp goes to rows of the caller's stride, also in
+    a context made for longer utterances."""
+    import torch
+    w = synth.make_workload(2, seed=0, batch=4, dur_scale=0.1)
+    w.cfg["vtlp_win"] = 400
+    waves = []
+    for room in (0, 5000):
+        cfg = binding.make_config(w.cfg, w.B, w.stride + room)
+        ctx = binding.AugContext(cfg)
+        cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        T = binding.aug_frame_count(int(w.lengths.max()), cfg.win, cfg.hop)
+        feats = torch.empty((w.B, T, cfg.n_mel), device="cuda")
+        wave = torch.full((w.B, w.stride), float("nan"), device="cuda")
+        ctx.aug_pipeline(cu(w.speech), w.stride, cu(w.lengths), w.lengths, cu(w.bank), w.bank.size,
+                         binding.table_to_device(w.table), w.B, feats, T,
+                         torch.empty(w.B, dtype=torch.int32, device="cuda"), wave)
+        waves.append(wave.cpu().numpy())
+    for b in range(w.B):
+        n = int(w.lengths[b])
+        assert np.all(np.isfinite(waves[0][b, :n])) and np.all(np.isnan(waves[1][b, n:]))
+        # same arithmetic; the gain's sums may be added in another order
+        np.testing.assert_allclose(waves[1][b, :n], waves[0][b, :n], rtol=0, atol=1e-6 * np.abs(waves[0][b, :n]).max())
