@@ -360,7 +360,8 @@ int aug_upload_noise_bank(AugCtx *ctx, const float *noise_bank_host, int64_t ban
 #define AUG_N_STAGES 7 /* 0 impulse responses, 1 response lengths and spectra, 2 filterbank tables,
                           3 waveform warp (vtlp_win > 0) and block spectra of the audio (contexts
                             sized for responses of more than 8192 taps),
-                          4 convolution, 5 waveform mix (only when requested), 6 features.
+                          4 convolution, 5 waveform mix (where the hop exceeds the
+                            window; otherwise stage 6 writes the waveform), 6 features.
                           Without the events between them the stages overlap at their ends, so the
                           sum is more than a call takes */
 

@@ -519,12 +519,14 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     t1(4, sm);
     if (rc != AUG_OK) return rc;
     t0(5, sm);
-    if (wave_out &&
+    const bool on_the_way = features_write_wave(ctx);       // the feature kernel writes the waveform too
+    if (wave_out && !on_the_way &&
         (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
         return rc;
     t1(5, sm);
     t0(6, sm);
-    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len);
+    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
+                               on_the_way ? wave_out : nullptr, speech_stride);
     t1(6, sm);
     if (ev && rc == AUG_OK) ctx->ev_n++;
     return rc;

@@ -96,3 +96,38 @@ def test_logmel_tiles(T_max, M, n_fft):
             ref = oracle.logmel(P[b, :T].astype(np.float64), float(tab["alpha"][b]), n_fft, M, floor=1e-7)
             # positive terms: relative error of a sum of K of them, plus that of the logarithm
             assert np.all(np.abs(got[b, :T] - ref) <= (K + 4) * EPS + 4 * EPS * np.abs(ref))
+
+
+# the waveform written by the feature kernel: full and single tiles, hops that are no multiple of 4,
+# both transforms, and the pass of its own where frames leave gaps; utterances without a frame
+@pytest.mark.parametrize("n_fft,win,hop,batch", [(512, 400, 160, 7), (512, 400, 160, 300), (512, 401, 125, 7),
+                                                 (512, 160, 160, 7), (512, 200, 300, 7), (1024, 800, 200, 300)])
+def test_waveform_written_with_the_features(n_fft, win, hop, batch):
+    import torch
+    w = synth.make_workload(2, seed=1, batch=7, dur_scale=0.12)
+    w.lengths[1], w.lengths[2], w.lengths[3] = 0, win - 1, win
+    rep = lambda a: np.ascontiguousarray(np.tile(a, (-(-batch // 7),) + (1,) * (a.ndim - 1))[:batch])
+    speech, lengths, table = rep(w.speech), rep(w.lengths), rep(w.table)
+    w.cfg.update(n_fft=n_fft, win=win, hop=hop)
+    cfg = binding.make_config(w.cfg, batch, w.stride)
+    ctx = binding.AugContext(cfg)
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    d_speech, d_len, d_bank, d_tab = cu(speech), cu(lengths), cu(w.bank), binding.table_to_device(table)
+    T = binding.aug_frame_count(int(lengths.max()), win, hop)
+    feats = torch.empty((batch, T, cfg.n_mel), device="cuda")
+    wave = torch.full((batch, w.stride), float("nan"), device="cuda")
+    ctx.aug_pipeline(d_speech, w.stride, d_len, lengths, d_bank, w.bank.size, d_tab, batch, feats, T,
+                     torch.empty(batch, dtype=torch.int32, device="cuda"), wave)
+    # the separate steps: responses, convolution and mix
+    rir = torch.empty((batch, cfg.max_sources, cfg.rir_taps), device="cuda")
+    ctx.aug_rir_image_method(d_tab, batch, rir)
+    ref = torch.full_like(wave, float("nan"))
+    ctx.aug_reverb_mix(d_speech, w.stride, d_len, d_bank, w.bank.size, rir, d_tab, batch, ref)
+    wave, ref = wave.cpu().numpy(), ref.cpu().numpy()
+    for b in range(batch):
+        n = int(lengths[b])
+        # same arithmetic but for the order in which the blocks' energies are added (fp64, then one
+        # fp32 rounding of the gain): two roundings of the sum of both sides
+        if n:
+            assert np.max(np.abs(wave[b, :n] - ref[b, :n])) <= 4 * EPS * np.max(np.abs(ref[b, :n]))
+        assert np.all(np.isnan(wave[b, n:]))
