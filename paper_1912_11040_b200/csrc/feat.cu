@@ -92,6 +92,79 @@ __device__ __forceinline__ float compress(float e, float floor_v, int mode) {
     return mode == AUG_COMPRESS_LOG ? l : expf(l * (1.f / 15.f));
 }
 
+// ---------------------------------------------------------------- filterbank
+// Bands are dealt out in RUNS runs of consecutive ones, cut so that all cost about the same: a band
+// costs its bins and about four bins' worth of set-up.  By the first RUNS + 1 threads.
+template <int RUNS>
+__device__ __forceinline__ void cut_bands(int *cut, const int *mst, int M, int tid) {
+    if (tid > RUNS) return;
+    const int base = mst[0], total = mst[M + 1] - base + 4 * M, want = total * tid / RUNS;
+    int lo = 0, hi = M;
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (mst[m] - base + 4 * m < want) lo = m + 1;
+        else hi = m;
+    }
+    cut[tid] = tid == RUNS ? M : lo;
+}
+// Where the powers of two frames come from: words that hold both, or two rows of floats.
+struct PairRow {
+    const fftpair::u64 *p;
+    __device__ __forceinline__ fftpair::u64 at(int i) const { return p[i]; }
+    __device__ __forceinline__ void step(int n) { p += n; }
+};
+struct TwoRows {
+    const float *p;
+    int next;
+    __device__ __forceinline__ fftpair::u64 at(int i) const { return fftpair::pack(p[i], p[next + i]); }
+    __device__ __forceinline__ void step(int n) { p += n; }
+};
+// Energies of bands m0 .. m1 - 1 of two frames: w4[k] the doubled weights of bin k (rising, falling),
+// `power` at bin 0, fs[m] and fs[m + next] the results.  The bins of edge interval j
+// give the falling sum of band j - 1 and the rising sum of band j.
+template <typename Power>
+__device__ __forceinline__ void walk_bands(const ulonglong2 *w4, const int *mst, int m0, int m1, Power power,
+                                           float *fs, int next) {
+    using namespace fftpair;
+    if (m0 >= m1) return;
+    int k = mst[m0];
+    w4 += k;
+    power.step(k);
+    fs += m0;
+    u64 u = 0, d = 0;              // rising and falling sums
+    auto walk = [&](int j) {
+        int n = mst[j + 1] - k;
+        k += n;
+#pragma unroll 1
+        for (; n >= 2; n -= 2, w4 += 2, power.step(2)) {
+            const ulonglong2 wa = w4[0], wb = w4[1];
+            const u64 pa = power.at(0), pb = power.at(1);
+            u = fma2(wa.x, pa, u);
+            d = fma2(wa.y, pa, d);
+            u = fma2(wb.x, pb, u);
+            d = fma2(wb.y, pb, d);
+        }
+        if (n > 0) {
+            const ulonglong2 wa = *w4++;
+            const u64 pa = power.at(0);
+            power.step(1);
+            u = fma2(wa.x, pa, u);
+            d = fma2(wa.y, pa, d);
+        }
+    };
+    walk(m0);
+#pragma unroll 1
+    for (int j = m0 + 1; j <= m1; ++j) {
+        d = u;                     // rising sum of band j - 1, to which its falling one is added
+        u = 0;
+        walk(j);
+        const float2 e = unpack(d);
+        fs[0] = e.x;
+        fs[next] = e.y;
+        ++fs;
+    }
+}
+
 // ---------------------------------------------------------------- frames -> spectra -> features
 // A warp takes four frames (512-point transform) or two (1024) from their samples to their
 // power spectra with one pair of 512-point transforms (fft_pair.cuh):
@@ -353,17 +426,7 @@ frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, in
         }
         for (int m = tid; m < M + 2; m += FEAT_THREADS) mst[m] = melstart[(int64_t)utt * (M + 2) + m];
         __syncthreads();
-        if (tid <= RUNS) {
-            // first band of run `tid`: a band costs its bins and about four bins' worth of set-up
-            const int base = mst[0], total = mst[M + 1] - base + 4 * M, want = total * tid / RUNS;
-            int lo = 0, hi = M;
-            while (lo < hi) {
-                const int m = (lo + hi) >> 1;
-                if (mst[m] - base + 4 * m < want) lo = m + 1;
-                else hi = m;
-            }
-            cut[tid] = tid == RUNS ? M : lo;
-        }
+        cut_bands<RUNS>(cut, mst, M, tid);
     }
     fftpair::u64 *xb = reinterpret_cast<fftpair::u64 *>(sm + warp * SPAN);
 
@@ -429,48 +492,8 @@ frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, in
             const int pr = tid & (PT - 1), run = tid / PT, w = pr / (QF / 2), q = pr % (QF / 2);
             const int f = QF * w + q;                // and f + QF / 2
             if (f < nf) {
-                const u64 *p = reinterpret_cast<const u64 *>(sm + w * SPAN) + q * NBP;
-                const ulonglong2 *w4 = reinterpret_cast<const ulonglong2 *>(mw);
-                float *fs = chunk + f * lay.fs_ld;
-                const int m0 = cut[run], m1 = cut[run + 1];
-                if (m0 < m1) {
-                    int k = mst[m0];
-                    const ulonglong2 *wp = w4 + k;
-                    p += k;
-                    fs += m0;
-                    // interval j: (u, d) its rising and falling sums
-                    u64 u = 0, d = 0;
-                    auto walk = [&](int j) {
-                        int n = mst[j + 1] - k;
-                        k += n;
-#pragma unroll 1
-                        for (; n >= 2; n -= 2, wp += 2, p += 2) {
-                            const ulonglong2 wa = wp[0], wb = wp[1];
-                            const u64 pa = p[0], pb = p[1];
-                            u = fma2(wa.x, pa, u);
-                            d = fma2(wa.y, pa, d);
-                            u = fma2(wb.x, pb, u);
-                            d = fma2(wb.y, pb, d);
-                        }
-                        if (n > 0) {
-                            const ulonglong2 wa = *wp++;
-                            const u64 pa = *p++;
-                            u = fma2(wa.x, pa, u);
-                            d = fma2(wa.y, pa, d);
-                        }
-                    };
-                    walk(m0);
-#pragma unroll 1
-                    for (int j = m0 + 1; j <= m1; ++j) {
-                        d = u;                       // rising sum of band j - 1, to which its falling one is added
-                        u = 0;
-                        walk(j);
-                        const float2 e = unpack(d);
-                        fs[0] = e.x;
-                        fs[(QF / 2) * lay.fs_ld] = e.y;
-                        ++fs;
-                    }
-                }
+                walk_bands(reinterpret_cast<const ulonglong2 *>(mw), mst, cut[run], cut[run + 1],
+                           PairRow{reinterpret_cast<const u64 *>(sm + w * SPAN) + q * NBP}, chunk + f * lay.fs_ld, (QF / 2) * lay.fs_ld);
             }
         }
         __syncthreads();                      // band energies in place
@@ -508,27 +531,27 @@ frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, in
 }
 
 // ---------------------------------------------------------------- step 4 alone
-// Bound by reading the power spectra (1 KB a frame).  A CTA copies a tile of 32 frames, which
-// are contiguous, into shared memory (16-byte asynchronous copies; the tile starts at the same
-// offset from a 16-byte boundary as in global memory) and walks the filterbank with the
-// frames over the lanes, as the fused kernels do.  Gathering every band's bins from global
-// memory one thread per band and frame took 203 us for 205 k frames (80 bands) where the
-// bytes take 51.
-constexpr int LM_FT = 32;
+// A CTA copies a tile of 32 frames, which are contiguous, into shared memory (16-byte asynchronous
+// copies; the tile starts at the same offset from a 16-byte boundary as in global memory) and walks
+// the filterbank as the fused kernels do, half a warp per run of bands, two frames a lane.
+// Bound by issue: 80 bands, 205 k frames 86 us where the bytes take 51; with one frame a lane and
+// the interval sums in shared memory 101, gathered from global memory one thread per band and
+// frame 203.
+constexpr int LM_FT = 32, LM_RUNS = 16;
+__host__ __device__ constexpr int logmel_fs(int NBP) { return ((LM_FT * NBP + 4) + 3) & ~3; }
+__host__ __device__ constexpr int logmel_mw(int NBP, int M) { return (logmel_fs(NBP) + LM_FT * (M | 1) + 3) & ~3; }
 __host__ __device__ constexpr size_t logmel_smem(int NBP, int M) {
-    return sizeof(float) * (LM_FT * NBP + 4 + 2 * LM_FT * (M + 1)) + sizeof(float2) * NBP + sizeof(int) * (M + 2);
+    return sizeof(float) * (size_t)(logmel_mw(NBP, M) + 4 * NBP + M + 2 + LM_RUNS + 1);
 }
 __global__ void __launch_bounds__(256)
 logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, int NBP, int M,
               int T_max, const aug::MelBin *__restrict__ melw, const int *__restrict__ melstart,
               float floor_v, float pad_v, int comp, float *__restrict__ feats) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *tile = reinterpret_cast<float *>(smem_raw);              // [LM_FT * NBP + 4]
-    float *up_s = tile + ((LM_FT * NBP + 4 + 1) & ~1);              // [LM_FT][M + 1]
-    float *dn_s = up_s + LM_FT * (M + 1);                           // [LM_FT][M + 1]
-    float2 *mw = reinterpret_cast<float2 *>(dn_s + LM_FT * (M + 1));   // [NBP]
-    int *mst = reinterpret_cast<int *>(mw + NBP);                   // [M + 2]
-    const int utt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ __align__(16) float sm[];
+    float *fs = sm + logmel_fs(NBP);                                // [LM_FT][M | 1] band energies
+    float4 *mw = reinterpret_cast<float4 *>(sm + logmel_mw(NBP, M));   // [NBP] (up, up, down, down)
+    int *mst = reinterpret_cast<int *>(mw + NBP), *cut = mst + M + 2;
+    const int utt = blockIdx.y, tid = threadIdx.x, ld = M | 1;
     const int t0 = blockIdx.x * LM_FT;
     const int rows = min(LM_FT, T_max - t0);
     const int T = min(max(counts[utt], 0), T_max);
@@ -543,7 +566,7 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
     const float *p = power + ((int64_t)utt * T_max + t0) * NBP;
     const int n = nf * NBP, shift = (int)((reinterpret_cast<uintptr_t>(p) >> 2) & 3);
     const int head = min(n, (4 - shift) & 3), n4 = (n - head) >> 2;
-    float *pt = tile + shift;
+    float *pt = sm + shift;
     for (int i = tid; i < n4; i += 256)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                          (unsigned)__cvta_generic_to_shared(pt + head + 4 * i)),
@@ -555,45 +578,38 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
     chain_wait();
     for (int k = tid; k < NBP; k += 256) {
         const aug::MelBin w = melw[(int64_t)utt * NBP + k];
-        mw[k] = make_float2(w.up, w.down);
+        mw[k] = make_float4(w.up, w.up, w.down, w.down);
     }
     for (int m = tid; m < M + 2; m += 256) mst[m] = melstart[(int64_t)utt * (M + 2) + m];
+    __syncthreads();
+    cut_bands<LM_RUNS>(cut, mst, M, tid);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    // edge interval j: rising sum of band j, falling sum of band j - 1; the widest first
-    if (lane < nf) {
-        const float *f = pt + lane * NBP;
-        for (int j = M - warp; j >= 0; j -= 8) {
-            float u0 = 0.f, d0 = 0.f, u1 = 0.f, d1 = 0.f;
-            int k = mst[j];
-            const int k1 = mst[j + 1];
-            for (; k + 1 < k1; k += 2) {
-                const float2 wa = mw[k], wb = mw[k + 1];
-                const float pa = f[k], pb = f[k + 1];
-                u0 = fmaf(wa.x, pa, u0);
-                d0 = fmaf(wa.y, pa, d0);
-                u1 = fmaf(wb.x, pb, u1);
-                d1 = fmaf(wb.y, pb, d1);
-            }
-            if (k < k1) {
-                const float2 wa = mw[k];
-                u0 = fmaf(wa.x, f[k], u0);
-                d0 = fmaf(wa.y, f[k], d0);
-            }
-            up_s[lane * (M + 1) + j] = u0 + u1;
-            dn_s[lane * (M + 1) + j] = d0 + d1;
-        }
+    const int f = tid & 15, run = tid >> 4;          // frames f and f + 16 (its row may hold no frame)
+    if (f < nf) {
+        walk_bands(reinterpret_cast<const ulonglong2 *>(mw), mst, cut[run], cut[run + 1],
+                   TwoRows{pt + f * NBP, f + 16 < nf ? 16 * NBP : 0}, fs + f * ld, 16 * ld);
     }
     __syncthreads();
-    int ff = tid / M, m = tid - ff * M;
-    const int step_f = 256 / M, step_m = 256 - step_f * M;
-    for (int i = tid; i < nf * M; i += 256) {
-        o[i] = compress(up_s[i + ff] + dn_s[i + ff + 1], floor_v, comp);
-        ff += step_f;
-        m += step_m;
-        if (m >= M) {
-            m -= M;
-            ++ff;
+    if ((M & 3) == 0 && (reinterpret_cast<uintptr_t>(feats) & 15) == 0) {
+        const int m4 = M >> 2, step_f = 256 / m4, step_m = 256 - step_f * m4;
+        int ff = tid / m4, m = tid - ff * m4;
+        for (int i = tid; i < nf * m4; i += 256) {
+            const float *e = fs + ff * ld + 4 * m;
+            reinterpret_cast<float4 *>(o)[i] =
+                make_float4(compress(e[0], floor_v, comp), compress(e[1], floor_v, comp),
+                            compress(e[2], floor_v, comp), compress(e[3], floor_v, comp));
+            ff += step_f;
+            m += step_m;
+            if (m >= m4) {
+                m -= m4;
+                ++ff;
+            }
+        }
+    } else {
+        for (int i = tid; i < nf * M; i += 256) {
+            const int ff = i / M;
+            o[i] = compress(fs[i + ff * (ld - M)], floor_v, comp);
         }
     }
 }

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fft_pair.cuh"
 
 namespace {
 
@@ -72,26 +73,31 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
             basis[i] = c < n_cep ? s * cospif((float)c * ((float)m + 0.5f) / (float)M) : 0.f;
         }
         __syncthreads();
-        float a[8], b[8];
+        // pairs of coefficients, as the basis is read
+        fftpair::u64 a[4], b[4];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) a[c] = b[c] = 0.f;
+        for (int c = 0; c < 4; ++c) a[c] = b[c] = 0;
         const float *x0 = xs + f0 * ld, *x1 = x0 + 64 * ld, *bz = basis + 8 * half;
 #pragma unroll 4
         for (int m = 0; m < M; ++m) {
-            const float u = x0[m], v = x1[m];
-            const float4 p = *reinterpret_cast<const float4 *>(bz + MFCC_CB * m);
-            const float4 q = *reinterpret_cast<const float4 *>(bz + MFCC_CB * m + 4);
-            const float w[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+            const fftpair::u64 u = fftpair::both(x0[m]), v = fftpair::both(x1[m]);
+            const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * m);
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * m + 4);
+            const fftpair::u64 w[4] = {p.x, p.y, q.x, q.y};
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                a[c] = fmaf(u, w[c], a[c]);
-                b[c] = fmaf(v, w[c], b[c]);
+            for (int c = 0; c < 4; ++c) {
+                a[c] = fftpair::fma2(u, w[c], a[c]);
+                b[c] = fftpair::fma2(v, w[c], b[c]);
             }
         }
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            os[f0 * (MFCC_CB + 1) + 8 * half + c] = a[c];
-            os[(f0 + 64) * (MFCC_CB + 1) + 8 * half + c] = b[c];
+        for (int c = 0; c < 4; ++c) {
+            const float2 ua = fftpair::unpack(a[c]), ub = fftpair::unpack(b[c]);
+            float *oa = os + f0 * (MFCC_CB + 1) + 8 * half + 2 * c, *ob = oa + 64 * (MFCC_CB + 1);
+            oa[0] = ua.x;
+            oa[1] = ua.y;
+            ob[0] = ub.x;
+            ob[1] = ub.y;
         }
         __syncthreads();
         for (int i = tid; i < nf * nc; i += MFCC_THREADS) {
@@ -128,7 +134,7 @@ mean_var_kernel(const float *__restrict__ feats, const int *__restrict__ counts,
         for (int v = 0; v < VEC; ++v) a[v] = b[v] = 0.0;
         if (slice < slices) {
             const float *x = feats + (int64_t)utt * T_max * D + d0 + g * VEC;
-#pragma unroll 4
+#pragma unroll 8
             for (int t = rank * slices + slice; t < T; t += MV_CLUSTER * slices) {
                 float z[VEC];
                 if constexpr (VEC == 4) {
