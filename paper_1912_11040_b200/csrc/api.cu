@@ -564,8 +564,9 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
     const float *speech_alias = ragged && (reinterpret_cast<uintptr_t>(speech_host) & 15) == 0
                                     ? mapped_alias(speech_host) : nullptr;
     // What a chunk of eight utterances takes on the device is mostly latency, so chunks hold sixteen
-    // or more (64 utterances of 2-20 s: 1364 us in 8 chunks, 1200 in 4; 16: 892 in 8, 380 in 2).  Only the last chunk's
-    // computation and copy back are not hidden behind the copies in: the last two are smaller.
+    // or more (64 utterances of 2-20 s: 1364 us in 8 chunks, 1200 in 4; 16: 892 in 8, 380 in 2).
+    // Only the last chunk's computation and copy back are not hidden behind the copies in: the
+    // last two are smaller.
     const int n_chunk = B >= 8 ? std::max(2, std::min(aug::HOST_CHUNKS, B / CHUNK_UTTS)) : 1;
     double share[aug::HOST_CHUNKS], shares = 0.0;
     for (int c = 0; c < n_chunk; ++c)

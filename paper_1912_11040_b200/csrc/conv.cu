@@ -557,6 +557,11 @@ rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restric
 // one's before the single inverse transform.  Where the slot is held (park_flags) the sum is
 // done in the time domain instead: v is read back and added to for every source after the
 // first, one inverse transform each.
+//
+// FUSED is bound by the issue of instructions, SPECTRA by those and its stores, STORED by the
+// latency of the spectra.  FUSED on 256 utterances of 2-20 s: 538 us with scalar transforms, one
+// CTA per possible block and three CTAs per multiprocessor (80 registers); 418 with two transforms
+// side by side in packed arithmetic, 128 registers, two CTAs and the list of work.
 enum Fate { DIRECT = 0, PARK_FIRST = 1, PARK_MORE = 2, PARK_JOIN = 3 };
 
 enum Kind { FUSED, SPECTRA, STORED };
