@@ -32,25 +32,19 @@ METRIC = "audio-seconds augmented+featurised per second"
 UNIT = "audio-s/s"
 FP32_LANES = 128          # fp32 lanes of one multiprocessor
 
-# DRAM bytes per audio-second (dram__bytes_read.sum + dram__bytes_write.sum of one ncu --set full
+# DRAM bytes per audio-second (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture per kernel on a reduced batch: profiles/ncu_config{2,3,5}_kernels.md; traffic grows in
 # proportion to the audio processed).  Valid only for the kernel sources the captures were taken
 # from: the hashes guard that.
 NCU_TRAFFIC = {
     "bytes_per_audio_s": {
-        2: {"convolve": 263.7e6 / 1039.18, "features": 150.9e6 / 1039.18, "rir_image": 45.6e6 / 1039.18},
-        3: {"convolve": (79.2e6 + 30.9e6) / 128.0, "rir_image": 32.8e6 / 128.0},
-        5: {"convolve": 46.3e6 / 240.0, "features": 34.1e6 / 240.0}},
+        2: {"convolve": 283.1e6 / 1039.18, "features": 149.5e6 / 1039.18},
+        3: {"convolve": (29.8e6 + 81.1e6) / 128.0},
+        5: {"features": 30.8e6 / 240.0}},
     "captured_on": {2: "96 utterances", 3: "16 utterances", 5: "4 utterances"},
     # kernel -> (its source files, sha256[:16] of them when the counters were taken)
-    "sources": {"convolve": (("conv.cu", "fft_pair.cuh"), "7a79969eb6513345"),
-                "features": (("feat.cu", "fft_pair.cuh"), "6b90b8e67ab940e5"),
-                "rir_image": (("rir.cu",), "9c178fa666e60507")}}
-
-
-# nominal FMAs / fp32 instructions executed: convolution 480 / 736 per thread and 4096-point
-# transform; fused 512-point features 6274 / 11680 per frame
-FP32_INSTRUCTION_CEILING = {"convolve": 0.652, "features": 0.537}
+    "sources": {"convolve": (("conv.cu", "fft_pair.cuh"), "80f9a83b65f26053"),
+                "features": (("feat.cu", "fft_pair.cuh"), "c82b1361896e6434")}}
 
 
 def kernel_sources_sha(files):
@@ -530,12 +524,6 @@ def run_ours(args):
             "ms": ms, "bound": bound,
             "tflops": flops / (ms * 1e-3) / 1e12, "frac_fp32": flops / (ms * 1e-3) / 1e12 / fp32_measured,
             "gbs": byts / (ms * 1e-3) / 1e9, "frac_hbm": byts / (ms * 1e-3) / 1e9 / hbm_peak}
-    # fp32 instructions executed per nominal FMA (ncu instruction counts in profiles/): no SIMT
-    # kernel that issues one instruction per slot can exceed this share of the nominal-flop roofline
-    for name, ceil in FP32_INSTRUCTION_CEILING.items():
-        if name in per_kernel and not (name == "features" and int(w.cfg["n_fft"]) != 512):
-            per_kernel[name]["fp32_instruction_ceiling"] = ceil
-            per_kernel[name]["frac_of_instruction_ceiling"] = per_kernel[name]["frac_fp32"] / ceil
     d = per_kernel[dom]
     if d["bound"] == "alu":
         roofline = {"kernel": dom, "bound": "alu", "achieved": d["tflops"], "peak": fp32_measured,
