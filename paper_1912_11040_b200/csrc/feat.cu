@@ -183,7 +183,7 @@ __device__ __forceinline__ void walk_bands(const ulonglong2 *w4, const int *mst,
 // scalar arithmetic, three radix-8 passes with two exchanges through shared memory, band sums
 // in shared memory) issued 829 warp instructions a frame: 295 us on 256 utterances of 2-20 s
 // (K = 512, 40 bands) where this one takes 249, and 874 against 653 on 64 of 60 s (K = 1024, 128
-// bands); the bytes take 61 and 105.  Tiles of a run, on the former batch and on 4096 of 0.5-5 s: two
+// bands); the bytes take 61 and 105.  Tiles of a run, on the former batch and on 4096 of 1-6 s: two
 // 264 and 1302 us, four 249 and 1179, six 249 and 1190.
 constexpr int WARPS = FEAT_THREADS / 32;
 
