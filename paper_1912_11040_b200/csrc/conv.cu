@@ -594,7 +594,11 @@ convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, 
     // differ: more noise sources, more work; dealt out in turn they left CTAs idle, 567 against
     // 447 us on 256 utterances of 2-20 s).  The unit after next and the next one's plan are
     // fetched while the current one is worked on; a warp may be up to one unit behind, hence three
-    // places for each.
+    // places for each.  The exchange buffer of the unit before may still be read by such a warp (the
+    // inverse transform ends with reads of all rows).  FUSED and SPECTRA go on with a forward transform,
+    // which first writes the slots its own thread has read last and then waits for all, SPECTRA behind a
+    // barrier after its own last reads; STORED goes on with an inverse one, which writes whole rows, and
+    // has a barrier behind the one before.
     __shared__ Plan plan_s[3];
     __shared__ Unit unit_s[3];
     const int t = threadIdx.x, G = gridDim.x;
@@ -785,6 +789,9 @@ convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, 
                 fftpair::exchange_back(v, t);
                 if (j == j_last) draw();
                 fftpair::inverse4096(v, sh, t, tw);
+                // (here, where the warps are close together, 128 x 8 s with 24000 taps take what they took
+                // without it, 863 us; between the products and the inverse transform it cost 5)
+                if constexpr (KIND == STORED) __syncthreads();
 
                 // The last `ob` outputs of the segment are this block: samples 4m .. 4m+3 of the
                 // segment are point m = t + CF r, real and imaginary parts swapped.

@@ -282,7 +282,9 @@ __device__ __forceinline__ void forward4096(C2 *v, Shared &sh, int t, const floa
     dft16(v);
 }
 // Frequencies j + 256 r in v, real and imaginary parts swapped -> 4096 times the samples
-// t + 256 r, swapped too.
+// t + 256 r, swapped too.  The row of slots that holds the thread's frequencies must be free: where
+// the thread has not just read it itself (forward4096), all threads must have passed a barrier since
+// the buffer was last read.
 __device__ __forceinline__ void inverse4096(C2 *v, Shared &sh, int t, const float2 *__restrict__ tw) {
     const float2 w1 = __ldg(&tw[2048 + row_frequency(t)]);
     dft16(v);

@@ -1,7 +1,7 @@
-"""The fused convolution where its blocks, loads and work list have edges, against the fp64
+"""The convolution where its blocks, loads and work list have edges, against the fp64
 checker: utterances that end with a block, one sample around it, within the first group of
 four; noise stretches at every offset from a 16-byte boundary, read inside one period, across
-its end, and looped many times; more units of work than resident CTAs."""
+its end, and looped many times; more units of work than resident CTAs, on every route."""
 import numpy as np
 import pytest
 
@@ -14,8 +14,9 @@ TAPS = 300
 OB = (16384 - TAPS + 1) & ~3         # outputs per block
 
 
-def run(lengths, stretches, taps=TAPS, seed=0):
-    """stretches[b] = list of (offset, length); responses dense over `taps`."""
+def run(lengths, stretches, taps=TAPS, seed=0, copies=1, calls=1, hold=False):
+    """stretches[b] = list of (offset, length); responses dense over `taps`.  The batch holds every
+    utterance `copies` times and goes through the same context `calls` times; every result is compared."""
     import torch
     rng = np.random.default_rng(seed)
     B, S = len(lengths), 1 + max(len(s) for s in stretches)
@@ -32,21 +33,30 @@ def run(lengths, stretches, taps=TAPS, seed=0):
         rir[b, : tab[b]["n_src"]] = rng.standard_normal((tab[b]["n_src"], taps)) * np.exp(-np.arange(taps) / (0.3 * taps)) * 0.1
     cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
                             max_order=1, max_sources=S, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
-                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=stride,
-                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B * copies,
+                            max_samples=stride, host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0,
+                            host_rows=0)
     ctx = binding.AugContext(cfg)
+    if hold:
+        ctx.aug_hold_parking_slots(True)
+    rep = lambda a: np.tile(a, (copies,) + (1,) * (a.ndim - 1))
     cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
-    out = torch.full((B, stride), float("nan"), device="cuda")
-    ctx.aug_reverb_mix(cu(speech), stride, cu(np.array(lengths, np.int32)), cu(bank), bank.size, cu(rir),
-                       binding.table_to_device(tab), B, out)
-    got = out.cpu().numpy()
+    args = [cu(rep(speech)), stride, cu(rep(np.array(lengths, np.int32))), cu(bank), bank.size, cu(rep(rir)),
+            binding.table_to_device(rep(tab)), B * copies]
+    got = []
+    for _ in range(calls):
+        out = torch.full((B * copies, stride), float("nan"), device="cuda")
+        ctx.aug_reverb_mix(*args, out)
+        torch.cuda.synchronize()
+        got += list(out.cpu().numpy().reshape(copies, B, stride))
     for b, n in enumerate(lengths):
         noises = [oracle.looped_noise(bank, o, m, n) for o, m in stretches[b]]
         ref, *_ = oracle.reverb_mix(speech[b, :n].astype(np.float64),
                                     [rir[b, s].astype(np.float64) for s in range(int(tab[b]["n_src"]))], noises,
                                     tab[b]["noise_weight"], tab[b]["snr_db"])
-        check_wave(got[b, :n], ref, f"utt {b} of {n} samples")
-        assert np.all(np.isnan(got[b, n:]))
+        for i, g in enumerate(got):
+            check_wave(g[b, :n], ref, f"utt {b} of {n} samples, copy {i}")
+            assert np.all(np.isnan(g[b, n:]))
 
 
 def test_lengths_around_a_block():
@@ -68,3 +78,19 @@ def test_more_units_than_resident_ctas():
     rng = np.random.default_rng(4)
     lengths = [int(n) for n in rng.integers(1, 900, 600)]
     run(lengths, [[(4 * (b % 50), 200 + b)] if b % 3 else [] for b in range(600)], taps=50)
+
+
+@pytest.mark.parametrize("taps", [8193, 16385, 24576])
+def test_long_responses_with_many_units(taps):
+    """The stored-spectra route: lengths around its blocks of 8192, several units a CTA in each of its
+    kernels; the first call of a context launches the fused kernels too, the later ones know better."""
+    lengths = [8192 * k + d for k in (1, 2, 4) for d in (-1, 0, 1)] + [49153]
+    loops = [[(8, 40000)], [(5, 8193), (4, 16384)], []]
+    run(lengths, [loops[b % 3] for b in range(len(lengths))], taps=taps, copies=16, calls=3)
+
+
+@pytest.mark.parametrize("hold", [False, True])
+def test_parking_slots_used_by_many_units(hold):
+    """Three noise sources, several units a CTA: a slot is written again by the unit after."""
+    run([3 * OB + 5, 2 * OB, 700], [[(8, 40000), (3, 9000), (100, 777)], [(0, 50000), (16, 20000)],
+                                    [(4, 400), (1, 333), (7, 50)]], copies=80, calls=2, hold=hold)
