@@ -64,7 +64,7 @@ __device__ __forceinline__ bool source_of(const AugUttParams &row, int s, const 
 // Effective length of the responses: (index + 1) of the last non-zero tap, largest over the
 // sources of an utterance (leff[utt]) and over the batch (*leff_all); both zeroed before the launch.
 __global__ void __launch_bounds__(CT)
-rir_length_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max, int L,
+rir_length_kernel(const float *rir, const AugUttParams *__restrict__ table, int S_max, int L,
                   int *__restrict__ leff, int *__restrict__ leff_all) {
     __shared__ int red_i[CT / 32];
     const int s = blockIdx.x, utt = blockIdx.y, t = threadIdx.x;
@@ -76,7 +76,7 @@ rir_length_kernel(const float *__restrict__ rir, const AugUttParams *__restrict_
     int last = 0;
     if ((reinterpret_cast<uintptr_t>(h) & 15) == 0) {
         for (int i = 4 * t; i + 3 < L; i += 4 * CT) {
-            const float4 z = __ldg(reinterpret_cast<const float4 *>(h + i));
+            const float4 z = *reinterpret_cast<const float4 *>(h + i);
             if (z.x != 0.f) last = i + 1;
             if (z.y != 0.f) last = i + 2;
             if (z.z != 0.f) last = i + 3;
@@ -112,7 +112,7 @@ __device__ __forceinline__ bool takes_fused_route(int leff_batch) { return leff_
 // 2-20 s where this launch costs 2.6; by the last CTA of the convolution, the fence it needs
 // cost as much.)
 __global__ void __launch_bounds__(256)
-snr_gain_kernel(const double *__restrict__ energy, const AugUttParams *__restrict__ table, int B,
+snr_gain_kernel(const double *energy, const AugUttParams *__restrict__ table, int B,
                 float *__restrict__ gain) {
     const int utt = blockIdx.x * 256 + threadIdx.x;
     chain_next();
@@ -129,8 +129,8 @@ snr_gain_kernel(const double *__restrict__ energy, const AugUttParams *__restric
 // thread.
 constexpr int MIX_GROUPS = 4;              // 128-bit groups per thread
 __global__ void __launch_bounds__(256)
-mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t ws_stride,
-           const float *__restrict__ gain, const int *__restrict__ lengths,
+mix_kernel(const float *ys, const float *vv, int64_t ws_stride,
+           const float *gain, const int *__restrict__ lengths,
            float *__restrict__ out, int64_t out_stride, int n_cap) {
     const int utt = blockIdx.y, tid = threadIdx.x;
     chain_wait();
@@ -145,8 +145,8 @@ mix_kernel(const float *__restrict__ ys, const float *__restrict__ vv, int64_t w
     for (int u = 0; u < MIX_GROUPS; ++u) {
         const int i = i0 + 1024 * u;           // (workspace rows are allocated up to a multiple of 4)
         if (i < N) {
-            x[u] = __ldg(reinterpret_cast<const float4 *>(a + i));
-            y[u] = __ldg(reinterpret_cast<const float4 *>(b + i));
+            x[u] = *reinterpret_cast<const float4 *>(a + i);
+            y[u] = *reinterpret_cast<const float4 *>(b + i);
         }
     }
     const float g = gain[utt];
@@ -198,7 +198,8 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 // F2 input samples starting at `base`: thread t gets samples base + 4 (t + 256 r) + {0, 1} and
 // + {2, 3} as the real and imaginary parts of point r.  Speech reads x[i]; a noise source
 // reads its stretch of the bank end to end (x[i mod nlen]).  Outside [0, N): zero.  The
-// exchange buffer must be free.
+// exchange buffer must be free.  (Nobody writes the audio while this kernel lives: it is the caller's, or
+// the warped speech, whose kernel lets none start beside it.)
 __device__ __forceinline__ void load_segment(C2 *v, fftpair::Shared &sh, const float *__restrict__ x, bool looped,
                                              int nlen, int base, int N, int t) {
     // A segment that lies inside the utterance (most do), and for a looped stretch inside one
@@ -360,11 +361,12 @@ __device__ __forceinline__ void edge_multiply(Bins &y, const Bins &h) {
     y.pi = pack(pi.x * hi.x, pr.y * hi.y + pi.y * hr.y);
     multiply(y.qr, y.qi, h.qr, h.qi);
 }
-// Bins of a slot of thread t at p + t, the halves CF apart; streamed, not kept in L1.
+// Bins of a slot of thread t at p + t, the halves CF apart; streamed, not kept in L1.  (The address follows
+// from the plan, which is read behind chain_wait().)
 __device__ __forceinline__ Bins load_bins(const float4 *p) {
     Bins z;
-    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.pr), "=l"(z.pi) : "l"(p));
-    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.qr), "=l"(z.qi) : "l"(p + CF));
+    asm("ld.global.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.pr), "=l"(z.pi) : "l"(p));
+    asm("ld.global.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(z.qr), "=l"(z.qi) : "l"(p + CF));
     return z;
 }
 // A whole spectrum into L2, by one thread.
@@ -459,7 +461,7 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttPa
 // elsewhere rir_spectra2_kernel plans on the way).
 __global__ void __launch_bounds__(256)
 plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restrict__ table, int B, int S_max,
-            const int *__restrict__ leff, const int *__restrict__ leff_all, int stored_only) {
+            const int *leff, const int *leff_all, int stored_only) {
     const int utt = blockIdx.x * 8 + (threadIdx.x >> 5);
     chain_next();
     chain_wait();
@@ -475,7 +477,7 @@ plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restric
 // by one, 29.9; a test per group inside the loop parts the loads: 33.6).  Persistent CTAs that work
 // through the partitions, as the kernels below, took 33.2 and, 128 x 4 x 3 partitions, 53 against 43.
 __global__ void __launch_bounds__(CF, FUSED_MINB)
-rir_spectra2_kernel(const float *__restrict__ rir, const AugUttParams *__restrict__ table, int S_max,
+rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, int S_max,
                     int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int *leff, int mixed,
                     int *transformed, const __grid_constant__ PlanArgs plan) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -583,8 +585,8 @@ enum Kind { FUSED, SPECTRA, STORED };
 
 template <Kind KIND, bool PARK>
 __global__ void __launch_bounds__(CF, FUSED_MINB)
-convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, const int *__restrict__ n_units,
-                int *drawn, int S_max, int P, const float4 *__restrict__ hspec, float4 *__restrict__ xspec,
+convolve_kernel(const Plan *plans, const Unit *units, const int *n_units,
+                int *drawn, int S_max, int P, const float4 *hspec, float4 *__restrict__ xspec,
                 int nblk_cap, const float2 *__restrict__ tw, float *__restrict__ ys, float *__restrict__ vv,
                 int64_t ws_stride, double *__restrict__ energy, float4 *__restrict__ park,
                 const int *__restrict__ park_flags) {
@@ -608,7 +610,7 @@ convolve_kernel(const Plan *__restrict__ plans, const Unit *__restrict__ units, 
     // STORED goes through the list backwards: the spectra that SPECTRA wrote last are still in L2
     // (128 x 8 s, four sources: 250 -> 246 us).
     const Unit first_of_list = units[blockIdx.x];
-    const int count = __ldcg(n_units);
+    const int count = *n_units;
     if (blockIdx.x >= count) return;
     auto unit_at = [&](int i) { return units[KIND == STORED ? count - 1 - i : i]; };
     const Unit first = KIND == STORED ? unit_at(blockIdx.x) : first_of_list;

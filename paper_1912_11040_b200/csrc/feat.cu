@@ -326,10 +326,9 @@ __device__ __forceinline__ void power_rows(fftpair::C2 *v, fftpair::u64 *p, cons
 
 template <int K, int MODE, int TILES>
 __global__ void __launch_bounds__(FEAT_THREADS, 2)
-frames_kernel(const float *__restrict__ in_a, const float *__restrict__ in_b, int64_t in_stride,
-              const float *__restrict__ gain, const int *__restrict__ lengths, int win, int hop, int M,
-              int T_max, const aug::MelBin *__restrict__ melw, const int *__restrict__ melstart,
-              const float2 *__restrict__ tw, float floor_v, float pad_v, int comp,
+frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const float *gain,
+              const int *__restrict__ lengths, int win, int hop, int M, int T_max, const aug::MelBin *__restrict__ melw,
+              const int *__restrict__ melstart, const float2 *__restrict__ tw, float floor_v, float pad_v, int comp,
               float *__restrict__ out, int *__restrict__ counts, int n_cap, float *__restrict__ wave, int64_t wave_stride,
               const __grid_constant__ Layout lay) {
     constexpr int QF = Plan<K>::QF, FT = tile_frames<K>(), NBP = K / 2 + 1;
@@ -548,8 +547,8 @@ __host__ __device__ constexpr size_t logmel_smem(int NBP, int M) {
 }
 __global__ void __launch_bounds__(256)
 logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, int NBP, int M,
-              int T_max, const aug::MelBin *__restrict__ melw, const int *__restrict__ melstart,
-              float floor_v, float pad_v, int comp, float *__restrict__ feats) {
+              int T_max, const aug::MelBin *melw, const int *melstart, float floor_v, float pad_v, int comp,
+              float *__restrict__ feats) {
     extern __shared__ __align__(16) float sm[];
     float *fs = sm + logmel_fs(NBP);                                // [LM_FT][M | 1] band energies
     float4 *mw = reinterpret_cast<float4 *>(sm + logmel_mw(NBP, M));   // [NBP] (up, up, down, down)
