@@ -92,8 +92,10 @@ __device__ __forceinline__ int2 round_strong(fftpair::u64 v) {
     const u64 t = fma2(v, both(0.0625f), m);
     const u64 rest = add2(fma2(sub2(m, t), both(16.f), v), m);
     const float2 hi = unpack(t), lo = unpack(rest);
-    return make_int2(16 * __float_as_int(hi.x) + __float_as_int(lo.x) - (int)(17u * INT_BITS),
-                     16 * __float_as_int(hi.y) + __float_as_int(lo.y) - (int)(17u * INT_BITS));
+    // (unsigned: sixteen times the bits exceeds 32 of them, and the excess cancels)
+    constexpr unsigned BITS = 17u * (unsigned)INT_BITS;
+    return make_int2((int)(16u * __float_as_uint(hi.x) + __float_as_uint(lo.x) - BITS),
+                     (int)(16u * __float_as_uint(hi.y) + __float_as_uint(lo.y) - BITS));
 }
 
 // NARROW: half_w <= 40, at most 80 taps.

@@ -1,9 +1,12 @@
-"""Kernels that may start while the one before them is still writing (chained launches) must not
+"""Rules of the kernel sources that no run shows to be broken reliably.
+
+Kernels that may start while the one before them is still writing (chained launches) must not
 read its results through the non-coherent path: that path is for data which nobody writes while
-the kernel lives.  Checked on the sources, as no run shows the difference reliably."""
+the kernel lives.  Words made of a float's bits are multiplied without a sign, as they exceed 32 bits."""
 import os
 import re
 
+import numpy as np
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1912_11040_b200", "csrc")
@@ -42,3 +45,19 @@ def test_explicit_non_coherent_loads_are_of_constant_data():
     assert s.count("ld.global.nc") == body.count("ld.global.nc")
     for m in re.finditer(r"__ldg\(([^)]*)\)", s.replace(body, "")):
         assert "tw[" in m.group(1), m.group(0)
+
+
+def test_bits_of_floats_are_multiplied_without_a_sign():
+    """Rounding of loud taps: 16 times the bits of about 1.5 2^23 wraps, which only unsigned words may."""
+    assert not re.search(r"\*\s*__float_as_int|__float_as_int\([^)]*\)\s*\*", source("rir.cu"))
+    rng = np.random.default_rng(0)
+    v = np.concatenate([rng.uniform(-1, 1, 100000) * 2.0 ** 25, [2.0 ** 25, -2.0 ** 25, 2.0 ** 22, -2.0 ** 22, 0.5, 0.0]])
+    v = v.astype(np.float32)
+    magic = np.float32(1.5 * 2.0 ** 23)
+    f32 = lambda x: x.astype(np.float32)                       # the kernel's fused operations: one rounding each
+    hi = f32(v.astype(np.float64) / 16 + magic)
+    lo = f32(f32(f32(magic - hi).astype(np.float64) * 16 + v) + magic)
+    bits = lambda x: x.view(np.uint32)
+    with np.errstate(over="ignore"):
+        got = (np.uint32(16) * bits(hi) + bits(lo) - np.uint32(17 * 0x4B400000 % 2 ** 32)).view(np.int32)
+    assert np.array_equal(got, np.rint(v.astype(np.float64)).astype(np.int32))
