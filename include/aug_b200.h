@@ -361,7 +361,8 @@ int aug_upload_noise_bank(AugCtx *ctx, const float *noise_bank_host, int64_t ban
                           3 waveform warp (vtlp_win > 0) and block spectra of the audio (contexts
                             sized for responses of more than 8192 taps),
                           4 convolution, 5 waveform mix (where the hop exceeds the
-                            window; otherwise stage 6 writes the waveform), 6 features.
+                            window or the frames exceed T_max; otherwise stage 6 writes the waveform),
+                          6 features.
                           Without the events between them the stages overlap at their ends, so the
                           sum is more than a call takes */
 

@@ -519,7 +519,7 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     t1(4, sm);
     if (rc != AUG_OK) return rc;
     t0(5, sm);
-    const bool on_the_way = features_write_wave(ctx);       // the feature kernel writes the waveform too
+    const bool on_the_way = features_write_wave(ctx, max_len, T_max);   // the feature kernel writes the waveform too
     if (wave_out && !on_the_way &&
         (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
         return rc;

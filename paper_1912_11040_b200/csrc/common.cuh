@@ -185,6 +185,6 @@ int launch_stft_power(AugCtx *ctx, const float *wave, int64_t stride, const int 
                       float *power, int T_max, int *counts);
 int launch_logmel(AugCtx *ctx, const float *power, const int *counts, int B, int T_max,
                   float *feats);
-bool features_write_wave(const AugCtx *ctx);
+bool features_write_wave(const AugCtx *ctx, int max_len, int T_max);
 int launch_fused_features(AugCtx *ctx, const int *lengths, int B, float *feats, int T_max, int *counts,
                           int max_len, float *wave, int64_t wave_stride);

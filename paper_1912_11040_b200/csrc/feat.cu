@@ -680,8 +680,14 @@ int launch_stft_power(AugCtx *ctx, const float *wave, int64_t stride, const int 
 // max_len: the length clamp the convolution used, so that every stage cuts an over-long
 // entry of `lengths` at the same sample.  wave (may be NULL): the mixed waveform is written on the
 // way -- it is in shared memory anyway; a pass of its own over y_s and v took 33 us on 96
-// utterances of 2-20 s -- unless frames leave gaps between them.
-bool features_write_wave(const AugCtx *ctx) { return ctx->cfg.hop <= ctx->cfg.win; }
+// utterances of 2-20 s -- unless frames leave gaps between them, or fewer feature rows than frames are
+// asked for: what lies behind the last row is written by one CTA of the utterance (32 utterances of
+// 20 s with one row 722 us, with a pass of its own 126).  A few frames more are let through,
+// as without lengths on the host max_len is the row stride, which callers round up.
+constexpr int WAVE_SLACK = 8;
+bool features_write_wave(const AugCtx *ctx, int max_len, int T_max) {
+    return ctx->cfg.hop <= ctx->cfg.win && frame_count(max_len, ctx->cfg.win, ctx->cfg.hop) <= (int64_t)T_max + WAVE_SLACK;
+}
 int launch_fused_features(AugCtx *ctx, const int *lengths, int B, float *feats, int T_max, int *counts,
                           int max_len, float *wave, int64_t wave_stride) {
     if (T_max <= 0) return AUG_OK;

@@ -131,3 +131,26 @@ def test_waveform_written_with_the_features(n_fft, win, hop, batch):
         if n:
             assert np.max(np.abs(wave[b, :n] - ref[b, :n])) <= 4 * EPS * np.max(np.abs(ref[b, :n]))
         assert np.all(np.isnan(wave[b, n:]))
+
+
+@pytest.mark.parametrize("rows", [1, 40, 0])
+def test_waveform_with_fewer_feature_rows_than_frames(rows):
+    """The waveform does not depend on how many feature rows are asked for; where most of it lies
+    behind the last row, it has a launch of its own instead of one CTA's loop.  rows = 0: all."""
+    import torch
+    from helpers import Device
+    dev = Device(synth.make_workload(2, seed=3, batch=5, dur_scale=0.2))
+    _, _, ref = dev.pipeline()
+    before = dev.ctx.aug_launch_count()
+    _, _, full = dev.pipeline()
+    base = dev.ctx.aug_launch_count() - before
+    F, counts, wave = dev.pipeline(T_max=rows or dev.T_max, lengths_host=False)
+    launches = dev.ctx.aug_launch_count() - before - base
+    assert launches == base + (1 if rows else 0)
+    assert int(counts.max()) == (rows or dev.T_max)
+    wave, ref = wave.cpu().numpy(), ref.cpu().numpy()
+    for b in range(dev.w.B):
+        n = int(dev.w.lengths[b])
+        # the gain's energies are added in another order: two roundings of the sum of both sides
+        assert np.max(np.abs(wave[b, :n] - ref[b, :n])) <= 4 * EPS * np.max(np.abs(ref[b, :n]))
+        assert np.all(np.isnan(wave[b, n:]))
