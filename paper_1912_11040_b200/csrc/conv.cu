@@ -106,8 +106,8 @@ rir_length_kernel(const float *rir, const AugUttParams *__restrict__ table, int 
 __device__ __forceinline__ bool takes_fused_route(int leff_batch) { return leff_batch <= aug::CONV_TAPS; }
 
 // ---------------------------------------------------------------- mixing
-// g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise or with a silent side:
-// once per utterance, in fp64, after the convolution has finished the two sums.  (Worked out by
+// g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise, with a silent side or with noise that is
+// not finite: once per utterance, in fp64, after the convolution has finished the two sums.  (Worked out by
 // every feature CTA instead, the chain of fp64 operations cost 13 us on 256 utterances of
 // 2-20 s where this launch costs 2.6; by the last CTA of the convolution, the fence it needs
 // cost as much.)
@@ -122,7 +122,8 @@ snr_gain_kernel(const double *energy, const AugUttParams *__restrict__ table, in
     float g = 0.f;
     if (table[utt].n_src > 1 && es > 0.0 && ev > 0.0)
         g = (float)sqrt(es / (ev * exp10((double)table[utt].snr_db / 10.0)));
-    gain[utt] = g;
+    // -0 tells the feature kernel that v, though weighted by zero, is not silence (it may not be finite)
+    gain[utt] = g == 0.f && ev != 0.0 ? -0.f : g;
 }
 
 // A pass over y_s and v, bound by memory: 4096 samples per CTA, eight 128-bit loads in flight per
@@ -149,7 +150,7 @@ mix_kernel(const float *ys, const float *vv, int64_t ws_stride,
             y[u] = *reinterpret_cast<const float4 *>(b + i);
         }
     }
-    const float g = gain[utt];
+    const float g = fabsf(gain[utt]);
 #pragma unroll
     for (int u = 0; u < MIX_GROUPS; ++u) {
         const int i = i0 + 1024 * u;

@@ -353,7 +353,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
     // the last frame (the first one if there is none) what lies behind them.
     float *wrow = MODE == 1 && wave != nullptr ? wave + (int64_t)utt * wave_stride : nullptr;
     if (MODE == 1 && wrow != nullptr && run0 <= max(T - 1, 0) && run0 + FT * TILES > max(T - 1, 0)) {
-        const float gw = gain[utt];
+        const float gw = fabsf(gain[utt]);
         const float *wa = in_a + (int64_t)utt * in_stride, *wb = in_b + (int64_t)utt * in_stride;
         for (int i = T * hop + tid; i < N; i += FEAT_THREADS) wrow[i] = fmaf(gw, wb[i], wa[i]);
     }
@@ -448,7 +448,23 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
         if (MODE == 1 && wrow != nullptr) {
             float *o = wrow + t0 * hop;
             const int n = nf * hop;
-            if (((hop | (int)wave_stride) & 3) == 0 && (reinterpret_cast<uintptr_t>(wave) & 15) == 0) {
+            const bool vec = ((hop | (int)wave_stride) & 3) == 0 && (reinterpret_cast<uintptr_t>(wave) & 15) == 0;
+            const float *pa = ra + t0 * hop, *pb = rb + t0 * hop;
+            if (__float_as_int(g) < 0) {
+                // -0, see snr_gain_kernel: noise that is not finite shows in the waveform, though the features
+                // (of y_s alone) never read it.  (Done for every utterance without noise it cost 4 % of 96
+                // utterances of 2-20 s.)
+                if (vec) {
+#pragma unroll 2
+                    for (int i = 4 * tid; i < n; i += 4 * FEAT_THREADS) {
+                        const float4 x = *reinterpret_cast<const float4 *>(pa + i), y = *reinterpret_cast<const float4 *>(pb + i);
+                        *reinterpret_cast<float4 *>(o + i) =
+                            make_float4(fmaf(0.f, y.x, x.x), fmaf(0.f, y.y, x.y), fmaf(0.f, y.z, x.z), fmaf(0.f, y.w, x.w));
+                    }
+                } else {
+                    for (int i = tid; i < n; i += FEAT_THREADS) o[i] = fmaf(0.f, pb[i], pa[i]);
+                }
+            } else if (vec) {
                 for (int i = 4 * tid; i < n; i += 4 * FEAT_THREADS)
                     *reinterpret_cast<float4 *>(o + i) = *reinterpret_cast<const float4 *>(chunk + i);
             } else {

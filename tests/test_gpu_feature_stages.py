@@ -154,3 +154,29 @@ def test_waveform_with_fewer_feature_rows_than_frames(rows):
         # the gain's energies are added in another order: two roundings of the sum of both sides
         assert np.max(np.abs(wave[b, :n] - ref[b, :n])) <= 4 * EPS * np.max(np.abs(ref[b, :n]))
         assert np.all(np.isnan(wave[b, n:]))
+
+
+@pytest.mark.parametrize("n_fft,hop", [(512, 160), (512, 125), (1024, 200)])
+def test_noise_that_is_not_finite_shows_in_the_waveform_alone(n_fft, hop):
+    """Infinite or undefined noise makes the gain 0; the waveform is still y_s + 0 v, undefined where v is
+    and in all of the utterance alike, as the separate mix gives it, and the features are those of y_s."""
+    import torch
+    from helpers import LOGMEL_ABS_TOL, Device
+    w = synth.make_workload(2, seed=5, batch=3, dur_scale=0.2)
+    w.cfg.update(n_fft=n_fft, win=400, hop=hop)
+    w.table["n_src"][:] = [2, 1, 2]
+    clean = synth.Workload(name=w.name, cfg=w.cfg, lengths=w.lengths, speech=w.speech, bank=w.bank, table=w.table.copy())
+    clean.table["n_src"][:] = 1
+    F_ref, _, _ = Device(clean).pipeline()
+    for bad in (np.nan, np.inf):
+        o, m = int(w.table["noise_offset"][0, 0]), int(w.table["noise_len"][0, 0])
+        w.bank = w.bank.copy()
+        w.bank[o:o + m] = bad
+        dev = Device(w)
+        F, _, wave = dev.pipeline()
+        mixed = dev.reverb_mix(dev.rir())
+        assert torch.equal(torch.isnan(wave), torch.isnan(mixed))
+        assert torch.isnan(wave[0, : int(w.lengths[0])]).all() and torch.isfinite(wave[1, : int(w.lengths[1])]).all()
+        # the same y_s from blocks of other sizes (they follow the longest response of an utterance): each side
+        # is within LOGMEL_ABS_TOL of the exact features
+        assert (F[0] - F_ref[0]).abs().max() <= 2 * LOGMEL_ABS_TOL
