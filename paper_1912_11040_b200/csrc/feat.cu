@@ -210,7 +210,7 @@ static_assert(SPAN >= 2 * fftpair::XBUF && SPAN >= 4 * 257 && SPAN >= 2 * 513 &&
 // Shared memory, in floats.  MODE 0: wave -> power.  MODE 1: y_s + g v -> features.  `ahead`: the
 // next tile is copied in while the current one is worked on (else there is one tile buffer).
 struct Layout {
-    int chunk_cap;      // samples of a tile, rounded up to 4
+    int chunk_cap;      // samples of a tile, in whole groups of 4
     int fs_ld;          // row stride of a tile's band energies
     int ahead;
     int chunk, raw, win, lanes, mw, mst, cut, total;
@@ -221,7 +221,8 @@ Layout make_layout(int win_len, int hop, int M, bool ahead) {
     Layout l;
     l.ahead = ahead;
     l.fs_ld = M | 1;
-    l.chunk_cap = ((FT - 1) * hop + win_len + 3) & ~3;
+    // (where tiles begin anywhere, up to three samples before the first one come along)
+    l.chunk_cap = ((FT - 1) * hop + win_len + ((hop & 3) ? 3 : 0) + 3) & ~3;
     int o = WARPS * SPAN;
     auto take = [&](int n) { const int r = o; o = (o + n + 3) & ~3; return r; };
     // samples of the tile; later (MODE 1) its band energies
@@ -371,25 +372,29 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
     const float *rb = MODE == 1 ? in_b + (int64_t)utt * in_stride : nullptr;
     const int n_tiles = min(TILES, (nfr + FT - 1) / FT);
 
-    // Samples of a tile travel global -> shared asynchronously, one tile ahead.  MODE 1: a thread
-    // copies the 16-byte groups 4 (tid + 256 u) of y_s and v into the raw buffers, and one tile
+    // Samples of a tile travel global -> shared asynchronously, one tile ahead, in the 16-byte groups of
+    // the row: the tile's first sample may be any of its first group (with hops that are no
+    // multiple of 4, one sample after another and one tile at a time, 128 utterances of 10 s took 506 us
+    // at K = 1024 and a hop of 441, and 471 at K = 512 and 125; so 322 and 315).  MODE 1: a thread
+    // copies the groups 4 (tid + 256 u) of y_s and v into the raw buffers, and one tile
     // later mixes the same groups into `chunk`, so the raw slots are private to the thread and need
-    // no barrier.  MODE 0 copies into the two tile buffers in turn.  Beyond the tile: zeros.
+    // no barrier.  MODE 0 copies into the two tile buffers in turn.  Beyond the frames there are: zeros.
     auto stage_issue = [&](int tile) {
-        const int t0 = run0 + tile * FT, s0 = t0 * hop;
-        const int ns = (min(FT, T - t0) - 1) * hop + win;
+        const int t0 = run0 + tile * FT, off = (t0 * hop) & 3, s0 = t0 * hop - off;
+        const int ns = (min(FT, T - t0) - 1) * hop + win + off;
         float *a = MODE == 1 ? sm + lay.raw : sm + ((tile & 1) ? lay.raw : lay.chunk), *b = a + lay.chunk_cap;
-        if (ns + 3 >= lay.chunk_cap && (ns & 3) == 0) {       // a full tile: no test per group
+        if (t0 + FT <= T) {
+            // a full tile: whole groups (rows are allocated up to a multiple of 4 floats), what the last
+            // one holds beyond the tile is not used
             const float *pa = ra + s0, *pb = rb + s0;
 #pragma unroll 2
-            for (int i = 4 * tid; i < lay.chunk_cap; i += 4 * FEAT_THREADS) {
+            for (int i = 4 * tid; i < ns; i += 4 * FEAT_THREADS) {
                 copy16_async(a + i, pa + i, 16);
                 if (noisy) copy16_async(b + i, pb + i, 16);
             }
             return;
         }
         for (int i = 4 * tid; i < lay.chunk_cap; i += 4 * FEAT_THREADS) {
-            // rows are allocated up to a multiple of 4 floats
             const int bytes = 4 * min(max(ns - i, 0), 4), src = bytes ? s0 + i : 0;
             copy16_async(a + i, ra + src, bytes);
             if (noisy) copy16_async(b + i, rb + src, bytes);
@@ -435,6 +440,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
     for (int tile = 0; tile < n_tiles; ++tile) {
         const int t0 = run0 + tile * FT;
         const int nf = min(FT, T - t0);
+        const int off = lay.ahead ? (t0 * hop) & 3 : 0;       // of the tile's first sample in its buffer
         if (lay.ahead) {
             copies_done();
             if (MODE == 1) {
@@ -468,7 +474,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
                 for (int i = 4 * tid; i < n; i += 4 * FEAT_THREADS)
                     *reinterpret_cast<float4 *>(o + i) = *reinterpret_cast<const float4 *>(chunk + i);
             } else {
-                for (int i = tid; i < n; i += FEAT_THREADS) o[i] = chunk[i];
+                for (int i = tid; i < n; i += FEAT_THREADS) o[i] = chunk[off + i];
             }
         }
         if (MODE == 0 && lay.ahead && tile + 1 < n_tiles) stage_issue(tile + 1);
@@ -476,7 +482,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
         const int f0 = QF * warp;
         if (f0 < nf) {
             fftpair::C2 v[16];
-            const float *c0 = (MODE == 0 && lay.ahead && (tile & 1) ? sm + lay.raw : chunk) + f0 * hop;
+            const float *c0 = (MODE == 0 && lay.ahead && (tile & 1) ? sm + lay.raw : chunk) + off + f0 * hop;
             windowed_points<K>(v, c0, win_s, win, hop, lane);
             fftpair::fft512(v, xb, reinterpret_cast<const float4 *>(sm + lay.lanes)[lane], lane);
             power_rows<K>(v, xb, tw, lane);
@@ -638,10 +644,10 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
                   int64_t wave_stride = 0) {
     const AugConfig &c = ctx->cfg;
     constexpr int FT = tile_frames<K>(), RUN_TILES = Plan<K>::TILES;
-    // Copying one tile ahead needs 16-byte aligned tile starts, and room: where the buffers
+    // Copying one tile ahead needs rows that start on 16-byte boundaries, and room: where the buffers
     // for it do not fit (hops of several hundred samples) tiles are loaded when they are needed.
     Layout lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, true);
-    if ((c.hop & 3) != 0 || (stride & 3) != 0 || sizeof(float) * lay.total > 227 * 1024)
+    if ((stride & 3) != 0 || sizeof(float) * lay.total > 227 * 1024)
         lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, false);
     const size_t smem = sizeof(float) * (size_t)lay.total;
     if (smem > 227 * 1024) return AUG_ECAP;

@@ -180,3 +180,42 @@ def test_noise_that_is_not_finite_shows_in_the_waveform_alone(n_fft, hop):
         # the same y_s from blocks of other sizes (they follow the longest response of an utterance): each side
         # is within LOGMEL_ABS_TOL of the exact features
         assert (F[0] - F_ref[0]).abs().max() <= 2 * LOGMEL_ABS_TOL
+
+
+# tiles that begin at any sample of a 16-byte group: rows of whole groups are copied in one tile ahead, other
+# rows sample by sample; single tiles and runs of them, last tiles of any number of frames
+@pytest.mark.parametrize("n_fft,win,hop", [(512, 400, 125), (512, 401, 110), (512, 3, 1), (512, 77, 131),
+                                           (1024, 500, 441), (1024, 1023, 163)])
+@pytest.mark.parametrize("batch", [3, 200])
+def test_power_spectra_of_rows_that_start_anywhere(n_fft, win, hop, batch):
+    import torch
+    T_max = 170
+    n = (T_max - 1) * hop + win + 5
+    rng = np.random.default_rng(win + hop)
+    lengths = rng.integers(0, n + 1, batch).astype(np.int32)
+    lengths[:3] = n, n - hop - 6, min(win + 31 * hop, n)
+    wave = rng.standard_normal((batch, n)).astype(np.float32)
+    for b in range(batch):
+        wave[b, lengths[b]:] = np.nan                  # nothing beyond an utterance's end is used
+    cfg = binding.AugConfig(fs=16000, win=win, hop=hop, n_fft=n_fft, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=64,
+                            max_order=1, max_sources=1, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=-3.5, compression=binding.COMPRESS_LOG, max_batch=batch, max_samples=n + 8,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    got = []
+    for stride in ((n + 3) // 4 * 4, (n + 3) // 4 * 4 + 1):
+        x = torch.full((batch, stride), float("nan"), device="cuda")
+        x[:, :n] = torch.from_numpy(wave)
+        P = torch.full((batch, T_max, n_fft // 2 + 1), float("nan"), device="cuda")
+        counts = torch.full((batch,), -7, dtype=torch.int32, device="cuda")
+        ctx.feat_stft_power(x, stride, torch.from_numpy(lengths).cuda(), batch, P, T_max, counts)
+        got.append((P.cpu().numpy(), counts.cpu().numpy()))
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+    P, counts = got[0]
+    for b in range(3):
+        T = min(binding.aug_frame_count(int(lengths[b]), win, hop), T_max)
+        assert counts[b] == T and not P[b, T:].any()
+        ref = oracle.stft_power(wave[b, : lengths[b]].astype(np.float64), win, hop, n_fft)[:T]
+        if T:
+            # two frames share a transform of 9 (10) levels: a few roundings of the loudest bin around
+            assert np.max(np.abs(P[b, :T] - ref)) <= 2e-6 * ref.max()
