@@ -207,22 +207,32 @@ static_assert(SPAN >= 2 * fftpair::XBUF && SPAN >= 4 * 257 && SPAN >= 2 * 513 &&
 // Powers lie in pairs, as the arithmetic leaves them: one 64-bit word holds a bin of frames
 // 4 w and 4 w + 2 (row 0 of warp w) or 4 w + 1 and 4 w + 3 (row 1); K = 1024: 2 w and 2 w + 1.
 
-// Shared memory, in floats.  MODE 0: wave -> power.  MODE 1: y_s + g v -> features.  `ahead`: the
-// next tile is copied in while the current one is worked on (else there is one tile buffer).
+// Shared memory, in floats.  MODE 0: wave -> power.  MODE 1: y_s + g v -> features.
+//   AHEAD    the next tile is copied in while the current one is worked on
+//   DIRECT   there is one tile buffer, filled when it is needed
+//   PACKED   so too, and without the gaps that hops longer than the window leave between the frames
+enum Staging { AHEAD, DIRECT, PACKED };
 struct Layout {
     int chunk_cap;      // samples of a tile, in whole groups of 4
+    int step;           // between the frames of a tile in its buffer
     int fs_ld;          // row stride of a tile's band energies
-    int ahead;
+    int ahead, packed;
     int chunk, raw, win, lanes, mw, mst, cut, total;
 };
+// Frames lie at the same offset from a 16-byte boundary as in their row, and so far apart that the
+// groups at the ends of two neighbours do not meet.
+inline int packed_step(int win_len, int hop) { return win_len + 6 + ((hop - win_len - 6) & 3); }
 template <int K, int MODE>
-Layout make_layout(int win_len, int hop, int M, bool ahead) {
+Layout make_layout(int win_len, int hop, int M, Staging staging) {
     constexpr int FT = tile_frames<K>();
+    const bool ahead = staging == AHEAD;
     Layout l;
     l.ahead = ahead;
+    l.packed = staging == PACKED;
+    l.step = l.packed ? packed_step(win_len, hop) : hop;
     l.fs_ld = M | 1;
     // (where tiles begin anywhere, up to three samples before the first one come along)
-    l.chunk_cap = ((FT - 1) * hop + win_len + ((hop & 3) ? 3 : 0) + 3) & ~3;
+    l.chunk_cap = ((FT - 1) * l.step + win_len + ((hop & 3) ? 3 : 0) + 3) & ~3;
     int o = WARPS * SPAN;
     auto take = [&](int n) { const int r = o; o = (o + n + 3) & ~3; return r; };
     // samples of the tile; later (MODE 1) its band energies
@@ -249,9 +259,9 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 // The samples of a warp's frames, windowed, as the points l + 32 r of a transform pair.
 template <int K>
 __device__ __forceinline__ void windowed_points(fftpair::C2 *v, const float *c0, const float *win_s, int win,
-                                                int hop, int l) {
+                                                int step, int l) {
     using namespace fftpair;
-    const float *c1 = c0 + hop, *c2 = c1 + hop, *c3 = c2 + hop;      // (K = 512: four frames)
+    const float *c1 = c0 + step, *c2 = c1 + step, *c3 = c2 + step;   // (K = 512: four frames)
     auto point = [&](int i, int j, float2 w) {                       // samples i (and i + 1 = j) of every frame
         if (K == 512) {
             const u64 ww = both(w.x);
@@ -411,16 +421,48 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
             *reinterpret_cast<float4 *>(chunk + i) = x;
         }
     };
-    auto stage_direct = [&](int tile) {
-        const int t0 = run0 + tile * FT, s0 = t0 * hop;
-        const int ns = (min(FT, T - t0) - 1) * hop + win;
-        for (int i = tid; i < lay.chunk_cap; i += FEAT_THREADS) {
-            float x = 0.f;
-            if (i < ns) {
-                x = ra[s0 + i];
-                if (noisy) x = fmaf(g, rb[s0 + i], x);
+    // Where there is one tile buffer: n samples from sample s0 on to chunk[d0], by every `step`-th thread
+    // from `first` on.  Whole groups, four loads (of each array) in flight, where rows hold such.
+    const bool groups = (in_stride & 3) == 0;
+    auto stage_stretch = [&](int s0, int d0, int n, int first, int step) {
+        if (groups) {
+            const int lead = s0 & 3, n4 = (lead + n + 3) >> 2;         // (d0 has the same lead)
+            const float4 *pa = reinterpret_cast<const float4 *>(ra + s0 - lead);
+            const float4 *pb = reinterpret_cast<const float4 *>(rb + s0 - lead);
+            float4 *d = reinterpret_cast<float4 *>(chunk + d0 - lead);
+            for (int i = first; i < n4; i += 4 * step) {
+                float4 x[4], y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    x[u] = y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i + u * step < n4) {
+                        x[u] = pa[i + u * step];
+                        if (noisy) y[u] = pb[i + u * step];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (i + u * step < n4)
+                        d[i + u * step] = !noisy ? x[u] : make_float4(fmaf(g, y[u].x, x[u].x), fmaf(g, y[u].y, x[u].y),
+                                                                      fmaf(g, y[u].z, x[u].z), fmaf(g, y[u].w, x[u].w));
             }
-            chunk[i] = x;
+        } else {
+#pragma unroll 4
+            for (int i = first; i < n; i += step) chunk[d0 + i] = noisy ? fmaf(g, rb[s0 + i], ra[s0 + i]) : ra[s0 + i];
+        }
+    };
+    auto stage_direct = [&](int tile) {
+        const int t0 = run0 + tile * FT, s0 = t0 * hop, off = groups ? s0 & 3 : 0, nf = min(FT, T - t0);
+        if (lay.packed) {
+            for (int f = warp; f < nf; f += WARPS) stage_stretch(s0 + f * hop, off + f * lay.step, win, lane, 32);
+        } else {
+            stage_stretch(s0, off, (nf - 1) * hop + win, tid, FEAT_THREADS);
+        }
+        // frames that there are not are transformed beside others: zeros
+        if (nf < FT) {
+            const int end = off + (nf - 1) * lay.step + win;
+            __syncthreads();                  // (the last group may reach beyond the last frame)
+            for (int i = end + tid; i < lay.chunk_cap; i += FEAT_THREADS) chunk[i] = 0.f;
         }
     };
     if (lay.ahead) stage_issue(0);
@@ -440,7 +482,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
     for (int tile = 0; tile < n_tiles; ++tile) {
         const int t0 = run0 + tile * FT;
         const int nf = min(FT, T - t0);
-        const int off = lay.ahead ? (t0 * hop) & 3 : 0;       // of the tile's first sample in its buffer
+        const int off = groups ? (t0 * hop) & 3 : 0;          // of the tile's first sample in its buffer
         if (lay.ahead) {
             copies_done();
             if (MODE == 1) {
@@ -482,8 +524,8 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
         const int f0 = QF * warp;
         if (f0 < nf) {
             fftpair::C2 v[16];
-            const float *c0 = (MODE == 0 && lay.ahead && (tile & 1) ? sm + lay.raw : chunk) + off + f0 * hop;
-            windowed_points<K>(v, c0, win_s, win, hop, lane);
+            const float *c0 = (MODE == 0 && lay.ahead && (tile & 1) ? sm + lay.raw : chunk) + off + f0 * lay.step;
+            windowed_points<K>(v, c0, win_s, win, lay.step, lane);
             fftpair::fft512(v, xb, reinterpret_cast<const float4 *>(sm + lay.lanes)[lane], lane);
             power_rows<K>(v, xb, tw, lane);
             if (MODE == 0) {
@@ -644,11 +686,17 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
                   int64_t wave_stride = 0) {
     const AugConfig &c = ctx->cfg;
     constexpr int FT = tile_frames<K>(), RUN_TILES = Plan<K>::TILES;
+    // Hops beyond several windows have a limit (AUG_ECAP), in samples of 32 (K = 1024: 8) frames that one
+    // behind the other with their gaps fit a multiprocessor beside the tables.
+    const int64_t reach = ((int64_t)(K == 512 ? 31 : 7) * c.hop + c.win + 3) & ~(int64_t)3;
+    if (reach > (K == 1024 ? 43762 - c.n_mel : MODE == 0 ? 48736 : 47644 - ((c.n_mel + 5) & ~3))) return AUG_ECAP;
     // Copying one tile ahead needs rows that start on 16-byte boundaries, and room: where the buffers
-    // for it do not fit (hops of several hundred samples) tiles are loaded when they are needed.
-    Layout lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, true);
+    // for it do not fit (hops of 500 samples at K = 512, of 1000 at 1024) tiles are loaded when they are
+    // needed, without the gaps where there are any (128 utterances of 10 s, K = 1024: hop 1000, window
+    // 1024 394 us one sample after another, 276; hop 1600, window 800 538 and 240).
+    Layout lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, AHEAD);
     if ((stride & 3) != 0 || sizeof(float) * lay.total > 227 * 1024)
-        lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, false);
+        lay = make_layout<K, MODE>(c.win, c.hop, c.n_mel, packed_step(c.win, c.hop) < c.hop ? PACKED : DIRECT);
     const size_t smem = sizeof(float) * (size_t)lay.total;
     if (smem > 227 * 1024) return AUG_ECAP;
     // A CTA works through a run of tiles (window values, filterbank tables and other

@@ -185,7 +185,8 @@ def test_noise_that_is_not_finite_shows_in_the_waveform_alone(n_fft, hop):
 # tiles that begin at any sample of a 16-byte group: rows of whole groups are copied in one tile ahead, other
 # rows sample by sample; single tiles and runs of them, last tiles of any number of frames
 @pytest.mark.parametrize("n_fft,win,hop", [(512, 400, 125), (512, 401, 110), (512, 3, 1), (512, 77, 131),
-                                           (1024, 500, 441), (1024, 1023, 163)])
+                                           (1024, 500, 441), (1024, 1023, 163), (512, 400, 900), (512, 511, 513),
+                                           (1024, 1024, 1022), (1024, 801, 1599)])
 @pytest.mark.parametrize("batch", [3, 200])
 def test_power_spectra_of_rows_that_start_anywhere(n_fft, win, hop, batch):
     import torch
@@ -219,3 +220,24 @@ def test_power_spectra_of_rows_that_start_anywhere(n_fft, win, hop, batch):
         if T:
             # two frames share a transform of 9 (10) levels: a few roundings of the loudest bin around
             assert np.max(np.abs(P[b, :T] - ref)) <= 2e-6 * ref.max()
+
+
+@pytest.mark.parametrize("n_fft,win,hop", [(512, 200, 600), (512, 512, 1022), (1024, 1024, 1000), (1024, 1024, 1024),
+                                           (1024, 801, 1603), (1024, 400, 3001), (1024, 400, 6188)])
+def test_hops_beyond_the_window(n_fft, win, hop):
+    """Tiles whose samples, with the gaps between frames, fit no buffer for copying ahead, up to the
+    largest hop that is served; one more is refused."""
+    from helpers import Device, check_pipeline_against_oracle, oracle_batch
+    w = synth.make_workload(1, seed=hop, batch=3, dur_scale=9.0 if hop > 2000 else 4.0)
+    w.cfg.update(n_fft=n_fft, win=win, hop=hop)
+    w.lengths[1], w.lengths[2] = win + 4 * hop + 1, win
+    dev = Device(w)
+    F, counts, wave = dev.pipeline()
+    check_pipeline_against_oracle(dev, F, counts, wave, oracle_batch(w))
+    if hop == 6188:
+        w.cfg.update(hop=hop + 1)
+        with pytest.raises(binding.AugError) as e:
+            Device(w).pipeline()
+        assert e.value.code == binding.AUG_ECAP
+        with pytest.raises(binding.AugError):
+            Device(w).stft_power(dev.speech)
