@@ -329,11 +329,10 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
  * back, and the call returns after synchronising, so the host buffers are free
  * again.  The longest rows of a chunk go by the copy engine while the kernel fetches
  * the others, and valid feature rows are written by a kernel straight into a pinned
- * (mapped) feature buffer, else by one copy per utterance.  Internally the batch is cut into up to 8 chunks of
- * sixteen or more utterances that are
- * copied in, computed and copied out concurrently on three streams; speech rows
- * are copied only up to their length when that saves more than the extra copy
- * calls cost.  Host buffers should be pinned: copies then run asynchronously, and
+ * (mapped) feature buffer, else by one copy per utterance.  Internally a batch of more than a few
+ * megabytes is cut into up to 8 chunks of utterances that are copied in, computed and copied out
+ * concurrently on three streams; speech rows are copied only up to their length when that saves
+ * more than the extra copy calls cost.  Host buffers should be pinned: copies then run asynchronously, and
  * the ragged rows of a pinned (mapped) speech buffer are fetched by one small kernel
  * per chunk that reads host memory directly instead of one copy per row.
  * noise_bank_host may be NULL with bank_len > 0

@@ -31,7 +31,7 @@ inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 #define AUG_COPY_UNROLL 16
 #endif
 constexpr int COPY_CTAS = AUG_COPY_CTAS, COPY_THREADS = 256, COPY_UNROLL = AUG_COPY_UNROLL;
-constexpr int CHUNK_UTTS = 16;
+constexpr int64_t CHUNKS_FROM = 12 << 20, CHUNK_BYTES = 13 << 20;   // see aug_pipeline_host
 #ifndef AUG_DMA_MIN_BYTES
 #define AUG_DMA_MIN_BYTES (512 << 10)
 #endif
@@ -563,11 +563,27 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
     // of a few hundred kilobytes each reach about 70 % of the link's rate).
     const float *speech_alias = ragged && (reinterpret_cast<uintptr_t>(speech_host) & 15) == 0
                                     ? mapped_alias(speech_host) : nullptr;
-    // What a chunk of eight utterances takes on the device is mostly latency, so chunks hold sixteen
-    // or more (64 utterances of 2-20 s: 1364 us in 8 chunks, 1200 in 4; 16: 892 in 8, 380 in 2).
-    // Only the last chunk's computation and copy back are not hidden behind the copies in: the
-    // last two are smaller.
-    const int n_chunk = B >= 8 ? std::max(2, std::min(aug::HOST_CHUNKS, B / CHUNK_UTTS)) : 1;
+    const int M = ctx->cfg.n_mel;
+    const bool valid_rows = ctx->cfg.host_rows == AUG_HOST_ROWS_VALID;
+    // frames per utterance as the device will count them (lengths are cut at the row stride)
+    auto frames_of = [&](int b) {
+        return std::min(aug_frame_count((int)std::min<int64_t>(lengths_host[b], speech_stride), ctx->cfg.win,
+                                        ctx->cfg.hop), T_max);
+    };
+    int64_t rows_out = (int64_t)B * T_max;
+    if (valid_rows) {
+        rows_out = 0;
+        for (int b = 0; b < B; ++b) rows_out += frames_of(b);
+    }
+    // Every chunk costs 35-50 us of launches and latency, and hides the others' copies.  How many pay
+    // follows from the bytes that are copied in and out (speech and features of: 8 utterances of 2-20 s, 7 MB,
+    // 275 us in one chunk, 301 in two; 32, 28 MB, 802 in one, 741 in two, 777 in four; 64, 56 MB, 1170, 1105
+    // in four, 1257 in eight; 16 of 60 s with 128 bands, 110 MB, 1909 in two, 1677 in eight; a rule by the
+    // number of utterances took eight chunks for the former and two for the latter).  Only the last chunk's
+    // computation and copy back are not hidden behind the copies in: the last two are smaller.
+    const int64_t moved = (int64_t)sizeof(float) * ((ragged ? total : (int64_t)B * speech_stride) + rows_out * M);
+    const int n_chunk = moved < CHUNKS_FROM ? 1
+        : (int)std::max<int64_t>(2, std::min<int64_t>(std::min(aug::HOST_CHUNKS, B), (moved + CHUNK_BYTES / 2) / CHUNK_BYTES));
     double share[aug::HOST_CHUNKS], shares = 0.0;
     for (int c = 0; c < n_chunk; ++c)
         shares += share[c] = c < n_chunk - 2 ? 1.0 : c == n_chunk - 2 ? 0.8 : 0.5;
@@ -588,21 +604,9 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
                                     cudaMemcpyHostToDevice, si));
         ctx->bank_resident = 0;   // the staging copy now holds this call's bank
     }
-    const int M = ctx->cfg.n_mel;
     ctx->last_h2d = (int64_t)sizeof(AugUttParams) * B + (int64_t)sizeof(int) * B +
                     (int64_t)sizeof(float) * (noise_bank_host ? bank_len : 0) +
                     (int64_t)sizeof(float) * (ragged ? total : (int64_t)B * speech_stride);
-    const bool valid_rows = ctx->cfg.host_rows == AUG_HOST_ROWS_VALID;
-    // frames per utterance as the device will count them (lengths are cut at the row stride)
-    auto frames_of = [&](int b) {
-        return std::min(aug_frame_count((int)std::min<int64_t>(lengths_host[b], speech_stride), ctx->cfg.win,
-                                        ctx->cfg.hop), T_max);
-    };
-    int64_t rows_out = (int64_t)B * T_max;
-    if (valid_rows) {
-        rows_out = 0;
-        for (int b = 0; b < B; ++b) rows_out += frames_of(b);
-    }
     ctx->last_d2h = (int64_t)sizeof(float) * rows_out * M + (int64_t)sizeof(int) * B;
     float *feats_alias = nullptr;
     if (valid_rows && (M & 3) == 0 && aligned16(feats_host))
