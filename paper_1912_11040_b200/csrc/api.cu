@@ -31,6 +31,7 @@ inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 #define AUG_COPY_UNROLL 16
 #endif
 constexpr int COPY_CTAS = AUG_COPY_CTAS, COPY_THREADS = 256, COPY_UNROLL = AUG_COPY_UNROLL;
+constexpr int HOST_ROOM = 16;          // CTAs the convolution leaves to the copying kernels of the other chunks
 constexpr int64_t CHUNKS_FROM = 12 << 20, CHUNK_BYTES = 13 << 20;   // see aug_pipeline_host
 #ifndef AUG_DMA_MIN_BYTES
 #define AUG_DMA_MIN_BYTES (512 << 10)
@@ -166,6 +167,81 @@ int check_batch(const AugCtx *ctx, int B) {
     if (B < 0) return AUG_EINVAL;
     if (B > ctx->cfg.max_batch) return AUG_ECAP;
     return AUG_OK;
+}
+
+// aug_pipeline; `room`: see ConvInput.
+int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
+                 const int *lengths_dev, const int *lengths_host, const float *noise_bank_dev,
+                 int64_t bank_len, const AugUttParams *table_dev, int B, float *feats_dev,
+                 int T_max, int *frame_counts_dev, float *wave_out, int room) {
+    int rc = check_batch(ctx, B);
+    if (rc != AUG_OK) return rc;
+    if (B == 0) return AUG_OK;
+    if (!speech_dev || !lengths_dev || !table_dev || !feats_dev || !frame_counts_dev) return AUG_EINVAL;
+    if (!aligned16(speech_dev) || !aligned16(feats_dev)) return AUG_EINVAL;
+    if (noise_bank_dev && !aligned16(noise_bank_dev)) return AUG_EINVAL;
+    if (wave_out && !aligned16(wave_out)) return AUG_EINVAL;
+    if (speech_stride <= 0 || (speech_stride & 3) || bank_len < 0 || T_max <= 0) return AUG_EINVAL;
+    if (speech_stride > ctx->ws_stride) return AUG_ECAP;
+    int max_len = (int)(speech_stride < ctx->cfg.max_samples ? speech_stride : ctx->cfg.max_samples);
+    if (lengths_host) {
+        int mx = 0;
+        for (int b = 0; b < B; ++b) {
+            if (lengths_host[b] < 0) return AUG_EINVAL;
+            if (lengths_host[b] > max_len) return AUG_ECAP;
+            if (lengths_host[b] > mx) mx = lengths_host[b];
+        }
+        if (aug_frame_count(mx, ctx->cfg.win, ctx->cfg.hop) > T_max) return AUG_ECAP;
+        max_len = mx;
+    }
+    // Stage timing: a start and a stop event per stage, on the stream the stage runs on.
+    cudaEvent_t *ev = nullptr;
+    if (ctx->timing && ctx->ev && ctx->ev_n < aug::EV_RING)
+        ev = ctx->ev + (size_t)ctx->ev_n * (2 * AUG_N_STAGES);
+    auto t0 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage], st); };
+    auto t1 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage + 1], st); };
+    // Running the impulse-response chain beside the block spectra on a second stream was
+    // measured and gained nothing (both saturate the SMs' issue and shared-memory pipes), so
+    // the stages follow one another, chained (see chain_wait).  The filterbank tables depend on
+    // the parameter table alone and come first: the impulse responses start beside them.
+    cudaStream_t sm = ctx->stream;
+    // with a waveform-domain warp the simulator sees the warped speech
+    const ConvInput in = {ctx->warped ? ctx->warped : speech_dev, ctx->warped ? ctx->ws_stride : speech_stride,
+                          lengths_dev, noise_bank_dev, bank_len, max_len, room};
+    t0(2, sm);
+    rc = launch_mel_tables(ctx, table_dev, B, true);
+    t1(2, sm);
+    t0(0, sm);
+    if (rc == AUG_OK) rc = launch_rir(ctx, table_dev, B, ctx->rir, true);
+    t1(0, sm);
+    t0(1, sm);
+    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, false);
+    t1(1, sm);
+
+    // waveform-domain warp (timed with stage 3)
+    t0(3, sm);
+    if (rc == AUG_OK && ctx->warped)
+        rc = launch_vtlp_resynth(ctx, speech_dev, speech_stride, lengths_dev, table_dev, B, max_len,
+                                 ctx->warped, ctx->ws_stride);
+    if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B);
+    t1(3, sm);
+    if (rc != AUG_OK) return rc;
+    t0(4, sm);
+    rc = launch_convolve_finish(ctx, in, table_dev, B);
+    t1(4, sm);
+    if (rc != AUG_OK) return rc;
+    t0(5, sm);
+    const bool on_the_way = features_write_wave(ctx, max_len, T_max);   // the feature kernel writes the waveform too
+    if (wave_out && !on_the_way &&
+        (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
+        return rc;
+    t1(5, sm);
+    t0(6, sm);
+    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
+                               on_the_way ? wave_out : nullptr, speech_stride);
+    t1(6, sm);
+    if (ev && rc == AUG_OK) ctx->ev_n++;
+    return rc;
 }
 
 }  // namespace
@@ -430,10 +506,10 @@ int aug_reverb_mix(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if (speech_stride <= 0 || (speech_stride & 3) || bank_len < 0) return AUG_EINVAL;
     const int max_len = (int)(speech_stride < ctx->cfg.max_samples ? speech_stride : ctx->cfg.max_samples);
     if (speech_stride > ctx->ws_stride) return AUG_ECAP;
-    const ConvInput in = {speech_dev, speech_stride, lengths_dev, noise_bank_dev, bank_len, max_len};
+    const ConvInput in = {speech_dev, speech_stride, lengths_dev, noise_bank_dev, bank_len, max_len, 0};
     if ((rc = launch_rir_spectra(ctx, rir_dev, in, table_dev, B, true)) != AUG_OK) return rc;
     if ((rc = launch_convolve_prepare(ctx, in, table_dev, B)) != AUG_OK) return rc;
-    if ((rc = launch_convolve_finish(ctx, table_dev, B, max_len)) != AUG_OK) return rc;
+    if ((rc = launch_convolve_finish(ctx, in, table_dev, B)) != AUG_OK) return rc;
     return launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out_dev, speech_stride);
 }
 
@@ -462,74 +538,8 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
                  const int *lengths_dev, const int *lengths_host, const float *noise_bank_dev,
                  int64_t bank_len, const AugUttParams *table_dev, int B, float *feats_dev,
                  int T_max, int *frame_counts_dev, float *wave_out) {
-    int rc = check_batch(ctx, B);
-    if (rc != AUG_OK) return rc;
-    if (B == 0) return AUG_OK;
-    if (!speech_dev || !lengths_dev || !table_dev || !feats_dev || !frame_counts_dev) return AUG_EINVAL;
-    if (!aligned16(speech_dev) || !aligned16(feats_dev)) return AUG_EINVAL;
-    if (noise_bank_dev && !aligned16(noise_bank_dev)) return AUG_EINVAL;
-    if (wave_out && !aligned16(wave_out)) return AUG_EINVAL;
-    if (speech_stride <= 0 || (speech_stride & 3) || bank_len < 0 || T_max <= 0) return AUG_EINVAL;
-    if (speech_stride > ctx->ws_stride) return AUG_ECAP;
-    int max_len = (int)(speech_stride < ctx->cfg.max_samples ? speech_stride : ctx->cfg.max_samples);
-    if (lengths_host) {
-        int mx = 0;
-        for (int b = 0; b < B; ++b) {
-            if (lengths_host[b] < 0) return AUG_EINVAL;
-            if (lengths_host[b] > max_len) return AUG_ECAP;
-            if (lengths_host[b] > mx) mx = lengths_host[b];
-        }
-        if (aug_frame_count(mx, ctx->cfg.win, ctx->cfg.hop) > T_max) return AUG_ECAP;
-        max_len = mx;
-    }
-    // Stage timing: a start and a stop event per stage, on the stream the stage runs on.
-    cudaEvent_t *ev = nullptr;
-    if (ctx->timing && ctx->ev && ctx->ev_n < aug::EV_RING)
-        ev = ctx->ev + (size_t)ctx->ev_n * (2 * AUG_N_STAGES);
-    auto t0 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage], st); };
-    auto t1 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage + 1], st); };
-    // Running the impulse-response chain beside the block spectra on a second stream was
-    // measured and gained nothing (both saturate the SMs' issue and shared-memory pipes), so
-    // the stages follow one another, chained (see chain_wait).  The filterbank tables depend on
-    // the parameter table alone and come first: the impulse responses start beside them.
-    cudaStream_t sm = ctx->stream;
-    // with a waveform-domain warp the simulator sees the warped speech
-    const ConvInput in = {ctx->warped ? ctx->warped : speech_dev, ctx->warped ? ctx->ws_stride : speech_stride,
-                          lengths_dev, noise_bank_dev, bank_len, max_len};
-    t0(2, sm);
-    rc = launch_mel_tables(ctx, table_dev, B, true);
-    t1(2, sm);
-    t0(0, sm);
-    if (rc == AUG_OK) rc = launch_rir(ctx, table_dev, B, ctx->rir, true);
-    t1(0, sm);
-    t0(1, sm);
-    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, false);
-    t1(1, sm);
-
-    // waveform-domain warp (timed with stage 3)
-    t0(3, sm);
-    if (rc == AUG_OK && ctx->warped)
-        rc = launch_vtlp_resynth(ctx, speech_dev, speech_stride, lengths_dev, table_dev, B, max_len,
-                                 ctx->warped, ctx->ws_stride);
-    if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B);
-    t1(3, sm);
-    if (rc != AUG_OK) return rc;
-    t0(4, sm);
-    rc = launch_convolve_finish(ctx, table_dev, B, max_len);
-    t1(4, sm);
-    if (rc != AUG_OK) return rc;
-    t0(5, sm);
-    const bool on_the_way = features_write_wave(ctx, max_len, T_max);   // the feature kernel writes the waveform too
-    if (wave_out && !on_the_way &&
-        (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
-        return rc;
-    t1(5, sm);
-    t0(6, sm);
-    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
-                               on_the_way ? wave_out : nullptr, speech_stride);
-    t1(6, sm);
-    if (ev && rc == AUG_OK) ctx->ev_n++;
-    return rc;
+    return run_pipeline(ctx, speech_dev, speech_stride, lengths_dev, lengths_host, noise_bank_dev, bank_len, table_dev,
+                        B, feats_dev, T_max, frame_counts_dev, wave_out, 0);
 }
 
 int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stride,
@@ -666,10 +676,10 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
         AUG_CUDA_OK(cudaEventRecord(ctx->ev_in[c], si));
         AUG_CUDA_OK(cudaStreamWaitEvent(sc, ctx->ev_in[c], 0));
         float *f_dev = ctx->st_feats + (int64_t)b0 * T_max * M;
-        rc = aug_pipeline(ctx, ctx->st_speech + (int64_t)b0 * speech_stride, speech_stride,
+        rc = run_pipeline(ctx, ctx->st_speech + (int64_t)b0 * speech_stride, speech_stride,
                           ctx->st_lengths + b0, lengths_host + b0,
                           bank_len > 0 ? ctx->st_bank : nullptr, bank_len, ctx->st_table + b0, nb,
-                          f_dev, T_max, ctx->st_counts + b0, nullptr);
+                          f_dev, T_max, ctx->st_counts + b0, nullptr, n_chunk > 1 ? HOST_ROOM : 0);
         if (rc != AUG_OK) break;
         AUG_CUDA_OK(cudaEventRecord(ctx->ev_out[c], sc));
         AUG_CUDA_OK(cudaStreamWaitEvent(so, ctx->ev_out[c], 0));

@@ -161,6 +161,7 @@ struct ConvInput {
     const float *bank;
     int64_t bank_len;
     int max_len;
+    int room;              // CTAs of a full device left out for kernels that run beside the convolution
 };
 
 // Launchers (defined next to their kernels).  They enqueue on ctx->stream unless a
@@ -175,7 +176,7 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const
 // the response has several partitions, else nothing), `finish` also needs the
 // partition spectra of the impulse responses.
 int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
-int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len);
+int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
 int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
                float *wave_out, int64_t out_stride);
 int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset);

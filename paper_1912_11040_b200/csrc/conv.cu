@@ -41,7 +41,6 @@
 namespace {
 
 constexpr int CT = 256;                // threads per CTA of the smaller kernels
-constexpr int HOST_ROOM = 16;          // CTAs left out in contexts with host staging, for the copying kernels
 constexpr int FUSED_MINB = 2;          // CTAs per SM of the transforming kernels
 
 // Source s of an utterance: pointer to its samples, loop length; false if the row's
@@ -905,9 +904,11 @@ static int launch_convolve(AugCtx *ctx, int grid) {
     ctx->launches++;
     return AUG_OK;
 }
-// As many CTAs as fit, but not more than there can be units of work.
-static int convolve_grid(const AugCtx *ctx, int B, int max_len, int ob) {
-    const int fit = std::min(FUSED_MINB * ctx->sm_count - (ctx->st_speech ? HOST_ROOM : 0), aug::PARK_SLOTS);
+// As many CTAs as fit (less the room to be left for kernels of other streams), but not more than there
+// can be units of work.
+static int convolve_grid(const AugCtx *ctx, const ConvInput &in, int B, int ob) {
+    const int max_len = in.max_len;
+    const int fit = std::min(FUSED_MINB * ctx->sm_count - in.room, aug::PARK_SLOTS);
     return (int)std::min<int64_t>(2 * (int64_t)B * ((max_len + ob - 1) / ob), fit);
 }
 
@@ -918,21 +919,21 @@ int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams
                        ctx->leff, ctx->leff + c.max_batch, ctx->stored_only) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
-    return launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, B, in.max_len, BLK2));
+    return launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, in, B, BLK2));
 }
 
-int launch_convolve_finish(AugCtx *ctx, const AugUttParams *table, int B, int max_len) {
+int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B) {
     const AugConfig &c = ctx->cfg;
-    if (max_len <= 0) return AUG_OK;
+    if (in.max_len <= 0) return AUG_OK;
     int rc = AUG_OK;
     if (!ctx->stored_only) {
         // blocks are shortest where a response fills min(rir_taps, 8192) taps
-        const int grid = convolve_grid(ctx, B, max_len, (F2 - std::min(c.rir_taps, BLK2) + 1) & ~3);
+        const int grid = convolve_grid(ctx, in, B, (F2 - std::min(c.rir_taps, BLK2) + 1) & ~3);
         rc = ctx->park ? launch_convolve<FUSED, true>(ctx, grid) : launch_convolve<FUSED, false>(ctx, grid);
         if (rc != AUG_OK) return rc;
     }
     if (stored_route(ctx)) {
-        if ((rc = launch_convolve<STORED, false>(ctx, convolve_grid(ctx, B, max_len, BLK2))) != AUG_OK) return rc;
+        if ((rc = launch_convolve<STORED, false>(ctx, convolve_grid(ctx, in, B, BLK2))) != AUG_OK) return rc;
         // for the next call's choice (not waited for)
         if (ctx->leff_seen)
             AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, ctx->leff + c.max_batch, sizeof(int), cudaMemcpyDeviceToHost,
