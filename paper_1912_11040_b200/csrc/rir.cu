@@ -378,14 +378,21 @@ static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *r
     return AUG_OK;
 }
 
-// Both sizes keep 32 warps with 64 registers on a multiprocessor.  Four CTAs of 256 threads
-// balance better where the responses fit four times and there are enough of them (measured on
-// the form with two images at a time: 4096 x 2 responses of 4096 taps 355 us against 399 with
-// two of 512, 512 x 4 of 8192 taps 204 against 213).  Long responses fit twice (128 x 4 of
-// 24000 taps: 313 against 383), and a few responses are done sooner by more warps each
-// (8 x 2: 12.7 against 14.8).
+// Both sizes keep 32 warps with 64 registers on a multiprocessor.  Two CTAs of 512 threads are better
+// as long as one round of them does (100 responses of 8192 taps, order 10: 17 us, with four of 256 threads
+// 21; long responses fit only twice, 300 of 24000 taps: 56 against 64), four of 256 balance better
+// beyond where they fit (300 of 8192 taps, order 6: 16.4 against 14.8, 600 23.1 and 21.0; 1200 of 4096
+// taps, order 8: 56 and 52).  How many responses there are depends on the table: at least one an
+// utterance, at most max_sources.  With so few
+// images that eight warps do them in one pass the first round is mostly set-up, and four CTAs are
+// taken as soon as there may be more than one (300 of 1600 taps, order 4: 13.0 against 8.9).
 int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
-    const bool fit = 4 * (rir_smem_bytes(256, ctx->cfg.rir_taps) + 1024) <= (size_t)ctx->smem_per_sm;
-    const bool many = (int64_t)B * ctx->cfg.max_sources >= 4 * (int64_t)ctx->sm_count;
+    const AugConfig &c = ctx->cfg;
+    const bool fit = 4 * (rir_smem_bytes(256, c.rir_taps) + 1024) <= (size_t)ctx->smem_per_sm;
+    const int side = 2 * c.max_order + 1;
+    const int images = c.image_lattice == AUG_LATTICE_CUBE ? side * side * side
+                                                           : side * (2 * c.max_order * (c.max_order + 1) + 3) / 3;
+    const int64_t most = (int64_t)B * c.max_sources, round = 2 * (int64_t)ctx->sm_count;
+    const bool many = B > round || most >= 2 * round || (images <= 256 && most > round);
     return fit && many ? launch_rir_as<256>(ctx, table, B, rir, beside) : launch_rir_as<512>(ctx, table, B, rir, beside);
 }

@@ -39,3 +39,38 @@ def test_windows_and_buffers(half_w, taps, B):
         # fixed-point steps follow the direct path, which may lie behind a short buffer
         d0 = np.linalg.norm(r["mic"].astype(np.float64) - r["src_pos"][0])
         assert np.max(np.abs(h[b] - ref)) <= RIR_REL_TOL * max(np.max(np.abs(ref)), 1.0 / d0), b
+
+
+@pytest.mark.parametrize("B,S,order", [(296, 1, 4), (297, 1, 4), (100, 3, 4), (90, 3, 5), (297, 1, 6), (297, 1, 10)])
+def test_batches_on_both_sides_of_a_round(B, S, order):
+    """Around the sizes from which smaller CTAs are taken (two 512-thread CTAs a multiprocessor): the responses
+    do not depend on how many others are made."""
+    import torch
+    rng = np.random.default_rng(B + S + order)
+    few, taps = 5, 1600
+    tab = np.zeros(few, dtype=synth.UTT_DTYPE)
+    tab["order"] = order
+    tab["n_src"] = rng.integers(1, S + 1, few)
+    for b in range(few):
+        tab[b]["room"] = rng.uniform(3.0, 6.0, 3)
+        tab[b]["beta"] = rng.uniform(0.5, 0.95, 6)
+        tab[b]["mic"] = tab[b]["room"] * rng.uniform(0.1, 0.45, 3)
+        for k in range(S):
+            tab[b]["src_pos"][k] = tab[b]["room"] * rng.uniform(0.5, 0.9, 3)
+    rows = np.tile(tab, -(-B // few))[:B]
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
+                            max_order=order, max_sources=S, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=4,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    out = torch.full((B, S, taps), float("nan"), device="cuda")
+    ctx.aug_rir_image_method(binding.table_to_device(rows), B, out)
+    h = out.cpu().numpy()
+    for b in range(few):
+        for s in range(S):
+            ref = np.zeros(taps)
+            if s < tab[b]["n_src"]:
+                r = tab[b]
+                ref = oracle.rir_image_method(r["room"], r["beta"], r["mic"], r["src_pos"][s], order, taps)
+            for i in range(b, B, few):
+                assert np.max(np.abs(h[i, s] - ref)) <= RIR_REL_TOL * np.max(np.abs(ref)), (i, s)
