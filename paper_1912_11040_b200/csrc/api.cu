@@ -169,16 +169,18 @@ int check_batch(const AugCtx *ctx, int B) {
     return AUG_OK;
 }
 
-// aug_pipeline; `room`: see ConvInput.
+// aug_pipeline; `room`: see ConvInput.  Chunks of the host entry point write feature rows that lie anywhere
+// in the staging (`any_feats`): vectors are stored only where n_mel is a multiple of 4, and all rows then
+// start on 16-byte boundaries.
 int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
                  const int *lengths_dev, const int *lengths_host, const float *noise_bank_dev,
                  int64_t bank_len, const AugUttParams *table_dev, int B, float *feats_dev,
-                 int T_max, int *frame_counts_dev, float *wave_out, int room) {
+                 int T_max, int *frame_counts_dev, float *wave_out, int room, bool any_feats) {
     int rc = check_batch(ctx, B);
     if (rc != AUG_OK) return rc;
     if (B == 0) return AUG_OK;
     if (!speech_dev || !lengths_dev || !table_dev || !feats_dev || !frame_counts_dev) return AUG_EINVAL;
-    if (!aligned16(speech_dev) || !aligned16(feats_dev)) return AUG_EINVAL;
+    if (!aligned16(speech_dev) || (!any_feats && !aligned16(feats_dev))) return AUG_EINVAL;
     if (noise_bank_dev && !aligned16(noise_bank_dev)) return AUG_EINVAL;
     if (wave_out && !aligned16(wave_out)) return AUG_EINVAL;
     if (speech_stride <= 0 || (speech_stride & 3) || bank_len < 0 || T_max <= 0) return AUG_EINVAL;
@@ -539,7 +541,7 @@ int aug_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
                  int64_t bank_len, const AugUttParams *table_dev, int B, float *feats_dev,
                  int T_max, int *frame_counts_dev, float *wave_out) {
     return run_pipeline(ctx, speech_dev, speech_stride, lengths_dev, lengths_host, noise_bank_dev, bank_len, table_dev,
-                        B, feats_dev, T_max, frame_counts_dev, wave_out, 0);
+                        B, feats_dev, T_max, frame_counts_dev, wave_out, 0, false);
 }
 
 int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stride,
@@ -679,7 +681,7 @@ int aug_pipeline_host(AugCtx *ctx, const float *speech_host, int64_t speech_stri
         rc = run_pipeline(ctx, ctx->st_speech + (int64_t)b0 * speech_stride, speech_stride,
                           ctx->st_lengths + b0, lengths_host + b0,
                           bank_len > 0 ? ctx->st_bank : nullptr, bank_len, ctx->st_table + b0, nb,
-                          f_dev, T_max, ctx->st_counts + b0, nullptr, n_chunk > 1 ? HOST_ROOM : 0);
+                          f_dev, T_max, ctx->st_counts + b0, nullptr, n_chunk > 1 ? HOST_ROOM : 0, true);
         if (rc != AUG_OK) break;
         AUG_CUDA_OK(cudaEventRecord(ctx->ev_out[c], sc));
         AUG_CUDA_OK(cudaStreamWaitEvent(so, ctx->ev_out[c], 0));

@@ -12,12 +12,13 @@ pytestmark = pytest.mark.gpu
     (16, 60, 1024, 128, 8),       # 110 MB, the copies far longer than any launch
     (3, 60, 1024, 128, 2),        # 21 MB
     (1, 300, 512, 40, 1),         # 24 MB that cannot be cut
+    (15, 19.99375, 512, 23, 2),   # 22 MB, chunks that begin at any feature row (an odd number of values)
     (24, 2, 512, 40, 1),          # 4 MB in many utterances
     (128, 2, 512, 40, 2)])        # 20 MB
 def test_chunks_follow_the_bytes(utts, seconds, n_fft, n_mel, chunks):
     import torch
     w = synth.make_workload(1, seed=utts, batch=2, dur_scale=0.1)
-    n = seconds * 16000
+    n = int(seconds * 16000)
     gen = torch.Generator().manual_seed(utts)
     speech = (torch.randn((utts, n), generator=gen) * 0.05).pin_memory()
     lengths = np.full(utts, n, np.int32)
