@@ -526,7 +526,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
             fftpair::C2 v[16];
             const float *c0 = (MODE == 0 && lay.ahead && (tile & 1) ? sm + lay.raw : chunk) + off + f0 * lay.step;
             windowed_points<K>(v, c0, win_s, win, lay.step, lane);
-            fftpair::fft512(v, xb, reinterpret_cast<const float4 *>(sm + lay.lanes)[lane], lane);
+            fftpair::fft512<false>(v, xb, reinterpret_cast<const float4 *>(sm + lay.lanes)[lane], lane);
             power_rows<K>(v, xb, tw, lane);
             if (MODE == 0) {
                 __syncwarp();

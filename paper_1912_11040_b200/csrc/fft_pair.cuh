@@ -143,6 +143,16 @@ __device__ __forceinline__ void twiddle16(C2 *v, float2 w) {
     }
 }
 
+// v[r] *= w[(r - 1) STEP], factors doubled (x, x, y, y)
+template <int STEP>
+__device__ __forceinline__ void twiddle_table(C2 *v, const float4 *w) {
+#pragma unroll
+    for (int r = 1; r < 16; ++r) {
+        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(w + (r - 1) * STEP);
+        v[r] = times(v[r], W2{z.x, z.y});
+    }
+}
+
 __device__ __forceinline__ u64 shfl(u64 v, int lane) {
     const float2 z = unpack(v);
     return pack(__shfl_sync(0xffffffffu, z.x, lane), __shfl_sync(0xffffffffu, z.y, lane));
@@ -156,10 +166,14 @@ __device__ __forceinline__ u64 shfl(u64 v, int lane) {
 // passes need two.
 constexpr int XBUF = 32 * 17;
 // c: exp(-2 pi i l / 512) and, for the upper half of the warp, exp(-2 pi i (l - 16) / 32) (lower
-// half: 1).
-__device__ __forceinline__ void fft512(C2 *v, u64 *buf, float4 c, int l) {
+// half: 1).  TABLE: the factors exp(-2 pi i l r / 512) of the first step come from w[32 (r - 1)],
+// each rounded once; built from powers of the first one they double the error of the transform
+// (root mean square 2.5e-7 of the spectrum against 1.1e-7).
+template <bool TABLE>
+__device__ __forceinline__ void fft512(C2 *v, u64 *buf, float4 c, int l, const float4 *w = nullptr) {
     dft16(v);
-    twiddle16(v, make_float2(c.x, c.y));
+    if constexpr (TABLE) twiddle_table<32>(v, w);
+    else twiddle16(v, make_float2(c.x, c.y));
     const u64 sign = both(l < 16 ? 1.f : -1.f);
     const W2 wh = both(make_float2(c.z, c.w));
 #pragma unroll
@@ -236,14 +250,6 @@ __device__ __forceinline__ void fill_tables(Shared &sh, int t, const float2 *__r
         (&sh.w256[0][0])[t] = make_float4(w.x, w.x, w.y, w.y);
     }
 }
-// v[r] *= w[(r - 1) 16]
-__device__ __forceinline__ void twiddle_table(C2 *v, const float4 *w) {
-#pragma unroll
-    for (int r = 1; r < 16; ++r) {
-        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(w + (r - 1) * 16);
-        v[r] = times(v[r], W2{z.x, z.y});
-    }
-}
 template <int STEP>
 __device__ __forceinline__ void load16(C2 *v, const Shared &sh, int at) {
 #pragma unroll
@@ -275,7 +281,7 @@ __device__ __forceinline__ void forward4096(C2 *v, Shared &sh, int t, const floa
     __syncthreads();
     load16<slot(16)>(v, sh, col_slot(t));
     dft16(v);
-    twiddle_table(v, &sh.w256[0][t & 15]);
+    twiddle_table<16>(v, &sh.w256[0][t & 15]);
     store16<slot(16)>(v, sh, col_slot(t));
     __syncwarp();
     load16<1>(v, sh, row_slot(t));
@@ -293,7 +299,7 @@ __device__ __forceinline__ void inverse4096(C2 *v, Shared &sh, int t, const floa
     __syncwarp();
     load16<slot(16)>(v, sh, col_slot(t));
     dft16(v);
-    twiddle_table(v, &sh.w256[0][col_digit(t)]);
+    twiddle_table<16>(v, &sh.w256[0][col_digit(t)]);
     store16<slot(16)>(v, sh, col_slot(t));
     __syncthreads();
     load16<slot(256)>(v, sh, slot(t));

@@ -23,7 +23,8 @@
 // Bound by instruction issue.  The form before (64 threads per pair of frames as real and
 // imaginary part of a 1024-point transform, scalar arithmetic, two exchanges and group
 // barriers per transform, 16 frames for 13 hops) took 360 us for 64 utterances of 2-20 s, this
-// one takes 258.
+// one takes 261.  Its error is 1.8e-7 of the waveform (root mean square; the form before 2.3e-7); with
+// the transforms' factors built from powers instead of a table it took 258 and had 3.1e-7.
 #include "common.cuh"
 #include "fft_pair.cuh"
 
@@ -39,14 +40,15 @@ static_assert(WBUF >= XBUF && 2 * WBUF >= 2 * K, "exchange and frames fit too");
 
 // Shared memory, in floats.  (Passed to the kernel: offsets then cost no registers.)
 struct ResynthLayout {
-    int xin, win, pos, lanes, carry, norm, total;
+    int xin, win, pos, lanes, w512, carry, norm, total;
     explicit ResynthLayout(int w) {
         const int hop = w / 4;
         xin = 2 * WBUF * (RS_THREADS / 32);
         win = xin + (((NF - 1) * hop + w + 3) & ~3);
         pos = win + K;
         lanes = pos + 2 * SPEC + 2;
-        carry = (lanes + 6 * 32 + 3) & ~3;
+        w512 = (lanes + 6 * 32 + 3) & ~3;
+        carry = w512 + 4 * 15 * 32;
         norm = carry + 3 * hop;              // (both on 16-byte boundaries where hops are multiples of 4)
         total = norm + hop;
     }
@@ -123,6 +125,14 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
         lanes4[tid] = make_float4(w1.x, w1.y, wh.x, wh.y);
         lanes2[tid] = __ldg(&tw[512 + tid]);         // exp(-2 pi i l / 1024)
     }
+    // exp(-2 pi i l r / 512) at [r - 1][l], doubled
+    float4 *w512 = reinterpret_cast<float4 *>(sm + lay.w512);
+    for (int i = tid; i < 15 * 32; i += RS_THREADS) {
+        const int k = ((i >> 5) + 1) * (i & 31);
+        float2 w = __ldg(&tw[256 + (k & 255)]);
+        if (k & 256) w = make_float2(-w.x, -w.y);
+        w512[i] = make_float4(w.x, w.x, w.y, w.y);
+    }
 
 #pragma unroll 1
     for (int round = 0; round < ROUNDS; ++round) {
@@ -165,7 +175,7 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
                     v[r] = {pack(w.x * p.x, w.x * q.x), pack(w.y * p.y, w.y * q.y)};
                 }
             }
-            fft512(v, buf, lanes4[lane], lane);
+            fft512<true>(v, buf, lanes4[lane], lane, w512 + lane);
 
             // spectra (twice their value) of both frames into the buffer
             C2 mid = v[8];                           // lane 0: frequency 256
@@ -234,7 +244,7 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
                 v[8] = mid;
             }
             __syncwarp();                            // the buffer is free
-            fft512(v, buf, lanes4[lane], lane);
+            fft512<true>(v, buf, lanes4[lane], lane, w512 + lane);
 
             // both frames, windowed again, one behind the other
             float *fo = reinterpret_cast<float *>(buf);
