@@ -33,7 +33,7 @@ UNIT = "audio-s/s"
 FP32_LANES = 128          # fp32 lanes of one multiprocessor
 
 # DRAM bytes per audio-second (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
-# capture per kernel on a reduced batch: profiles/ncu_config{2,3,5}_kernels.md; traffic grows in
+# capture per kernel on a reduced batch, summarised under profiles/; traffic grows in
 # proportion to the audio processed).  Valid only for the kernel sources the captures were taken
 # from: the hashes guard that.
 NCU_TRAFFIC = {

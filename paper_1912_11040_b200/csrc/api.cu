@@ -196,52 +196,51 @@ int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
         if (aug_frame_count(mx, ctx->cfg.win, ctx->cfg.hop) > T_max) return AUG_ECAP;
         max_len = mx;
     }
-    // Stage timing: a start and a stop event per stage, on the stream the stage runs on.
+    // Stage timing: a start and a stop event per stage.
     cudaEvent_t *ev = nullptr;
     if (ctx->timing && ctx->ev && ctx->ev_n < aug::EV_RING)
         ev = ctx->ev + (size_t)ctx->ev_n * (2 * AUG_N_STAGES);
-    auto t0 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage], st); };
-    auto t1 = [&](int stage, cudaStream_t st) { if (ev) cudaEventRecord(ev[2 * stage + 1], st); };
+    auto t0 = [&](int stage) { if (ev) cudaEventRecord(ev[2 * stage], ctx->stream); };
+    auto t1 = [&](int stage) { if (ev) cudaEventRecord(ev[2 * stage + 1], ctx->stream); };
     // Running the impulse-response chain beside the block spectra on a second stream was
     // measured and gained nothing (both saturate the SMs' issue and shared-memory pipes), so
     // the stages follow one another, chained (see chain_wait).  The filterbank tables depend on
     // the parameter table alone and come first: the impulse responses start beside them.
-    cudaStream_t sm = ctx->stream;
     // with a waveform-domain warp the simulator sees the warped speech
     const ConvInput in = {ctx->warped ? ctx->warped : speech_dev, ctx->warped ? ctx->ws_stride : speech_stride,
                           lengths_dev, noise_bank_dev, bank_len, max_len, room};
-    t0(2, sm);
+    t0(2);
     rc = launch_mel_tables(ctx, table_dev, B, true);
-    t1(2, sm);
-    t0(0, sm);
+    t1(2);
+    t0(0);
     if (rc == AUG_OK) rc = launch_rir(ctx, table_dev, B, ctx->rir, true);
-    t1(0, sm);
-    t0(1, sm);
+    t1(0);
+    t0(1);
     if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, false);
-    t1(1, sm);
+    t1(1);
 
     // waveform-domain warp (timed with stage 3)
-    t0(3, sm);
+    t0(3);
     if (rc == AUG_OK && ctx->warped)
         rc = launch_vtlp_resynth(ctx, speech_dev, speech_stride, lengths_dev, table_dev, B, max_len,
                                  ctx->warped, ctx->ws_stride);
     if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B);
-    t1(3, sm);
+    t1(3);
     if (rc != AUG_OK) return rc;
-    t0(4, sm);
+    t0(4);
     rc = launch_convolve_finish(ctx, in, table_dev, B);
-    t1(4, sm);
+    t1(4);
     if (rc != AUG_OK) return rc;
-    t0(5, sm);
+    t0(5);
     const bool on_the_way = features_write_wave(ctx, max_len, T_max);   // the feature kernel writes the waveform too
     if (wave_out && !on_the_way &&
         (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
         return rc;
-    t1(5, sm);
-    t0(6, sm);
+    t1(5);
+    t0(6);
     rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
                                on_the_way ? wave_out : nullptr, speech_stride);
-    t1(6, sm);
+    t1(6);
     if (ev && rc == AUG_OK) ctx->ev_n++;
     return rc;
 }

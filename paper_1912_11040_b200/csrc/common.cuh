@@ -73,9 +73,10 @@ struct AugCtx {
     float *ys;             // [max_batch][ws_stride]
     float *vv;             // [max_batch][ws_stride]
     double *energy;        // [max_batch][2]
-    int *leff;             // [2 max_batch + N_COUNTERS] (behind the lengths: largest over the batch, counters; sources transformed)
+    int *leff;             // [2 max_batch + N_COUNTERS] taps up to the last non-zero one, largest over the utterance's
+                           // sources; behind them the largest over the batch, counters, sources transformed
     int *leff_seen;        // pinned host copy of that last entry from an earlier call (long-response contexts)
-    int stored_only;       // this call launches the stored-spectra kernels alone taps up to the last non-zero one, largest over the utterance's sources
+    int stored_only;       // this call launches the stored-spectra kernels alone
     float *gain;           // [max_batch] noise gain g for the requested SNR
     aug::MelBin *melw;     // [max_batch][n_bins]
     int *melstart;         // [max_batch][n_mel + 2]
@@ -164,8 +165,7 @@ struct ConvInput {
     int room;              // CTAs of a full device left out for kernels that run beside the convolution
 };
 
-// Launchers (defined next to their kernels).  They enqueue on ctx->stream unless a
-// stream is passed.
+// Launchers (defined next to their kernels).  They enqueue on ctx->stream.
 // `beside`: may run beside the kernel before it on the stream, one of this library that calls chain_next()
 int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside);
 // `reset`: set the counters and sums of the convolution to zero first (aug_pipeline has had it done by

@@ -24,8 +24,8 @@
 //      then the others whose window lies inside the response, then those at its edges, which are
 //      done one by one with tests.  No test is left in the loops over the first two.
 //
-// Bound by instruction issue (30 warp instructions an image, 70 % of the slots; reciprocal pipe
-// 60 %).  One image at a time in scalar arithmetic, with a conversion instruction per tap and
+// Bound by instruction issue (30 warp instructions an image, 58 to 63 % of the slots; reciprocal pipe
+// 47 to 53 %).  One image at a time in scalar arithmetic, with a conversion instruction per tap and
 // masks, it was 58, and the quarter-rate pipe of reciprocals and conversions was 62 % busy too;
 // two at a time with tests of strength and range per pair 45.  128 x 4 responses of 24000 taps,
 // order 20: 393, 312 (two at a time) and 250 us; 4096 x 2 of 4096 taps: 437, 354 and 281.

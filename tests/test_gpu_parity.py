@@ -286,7 +286,7 @@ def test_fused_route_sums_three_noise_sources():
 def test_pipeline_with_other_window_and_hop(n_fft, win, hop):
     """Window and hop are configuration fields: a window as long as the transform with a
     stretch per tile that needs a second round of staging loads, a hop that is not a
-    multiple of four samples (scalar staging), and the 50 ms window of the paper's
+    multiple of four samples (tiles that begin inside a 16-byte group), and the 50 ms window of the paper's
     Section 3 on the 1024-point transform."""
     w = small(1, batch=3, dur_scale=0.8)
     w.cfg.update(n_fft=n_fft, win=win, hop=hop)
