@@ -109,7 +109,7 @@ struct Layout {
     int n_part, route, n_bins, t_cap, nblk_cap;
     int64_t ws_stride;
     int64_t off_xspec, off_park, off_park_flags, off_plans, off_units;
-    int64_t off_tw, off_rir, off_hspec, off_ys, off_vv, off_energy, off_leff, off_gain, off_melw, off_melstart,
+    int64_t off_tw, off_tap_tab, off_rir, off_hspec, off_ys, off_vv, off_energy, off_arrived, off_counters, off_leff, off_gain, off_melw, off_melstart,
         off_status, off_warped, off_vtlp_tab, off_st_speech, off_st_bank, off_st_table, off_st_lengths,
         off_st_feats, off_st_counts, total;
 };
@@ -125,6 +125,7 @@ Layout make_layout(const AugConfig &c) {
     int64_t o = 0;
     auto take = [&](int64_t bytes) { int64_t r = o; o = align_up(o + bytes, 256); return r; };
     l.off_tw = take(sizeof(float2) * fftpair::TW_N);
+    l.off_tap_tab = take(sizeof(float) * 32 * aug::TAP_ROWS);
     l.off_rir = take(sizeof(float) * B * S * c.rir_taps);
     l.off_hspec = take(sizeof(float2) * B * S * l.n_part * aug::CONV_BINS);
     l.nblk_cap = (c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS;
@@ -138,8 +139,10 @@ Layout make_layout(const AugConfig &c) {
     l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS));
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
-    l.off_energy = take(sizeof(double) * 2 * B);
-    l.off_leff = take(sizeof(int) * (2 * B + aug::N_COUNTERS));     // (right behind the sums: one memset sets both to zero)
+    l.off_energy = take((sizeof(double) * 2 + sizeof(unsigned long long)) * B + sizeof(int) * aug::N_COUNTERS);
+    l.off_arrived = l.off_energy + sizeof(double) * 2 * B;
+    l.off_counters = l.off_arrived + sizeof(unsigned long long) * B;
+    l.off_leff = take(sizeof(int) * B * S);
     l.off_gain = take(sizeof(float) * B);
     l.off_melw = take(sizeof(aug::MelBin) * B * l.n_bins);
     l.off_melstart = take(sizeof(int) * B * (c.n_mel + 2));
@@ -216,7 +219,7 @@ int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if (rc == AUG_OK) rc = launch_rir(ctx, table_dev, B, ctx->rir, true);
     t1(0);
     t0(1);
-    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, false);
+    if (rc == AUG_OK) rc = launch_rir_spectra(ctx, ctx->rir, in, table_dev, B, true);
     t1(1);
 
     // waveform-domain warp (timed with stage 3)
@@ -224,7 +227,7 @@ int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if (rc == AUG_OK && ctx->warped)
         rc = launch_vtlp_resynth(ctx, speech_dev, speech_stride, lengths_dev, table_dev, B, max_len,
                                  ctx->warped, ctx->ws_stride);
-    if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B);
+    if (rc == AUG_OK) rc = launch_convolve_prepare(ctx, in, table_dev, B, true);
     t1(3);
     if (rc != AUG_OK) return rc;
     t0(4);
@@ -339,6 +342,7 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     }
     char *base = static_cast<char *>(ctx->ws_base);
     ctx->tw = reinterpret_cast<float2 *>(base + l.off_tw);
+    ctx->tap_tab = reinterpret_cast<float *>(base + l.off_tap_tab);
     ctx->rir = reinterpret_cast<float *>(base + l.off_rir);
     ctx->hspec = reinterpret_cast<float2 *>(base + l.off_hspec);
     ctx->nblk_cap = l.nblk_cap;
@@ -350,6 +354,8 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     ctx->ys = reinterpret_cast<float *>(base + l.off_ys);
     ctx->vv = reinterpret_cast<float *>(base + l.off_vv);
     ctx->energy = reinterpret_cast<double *>(base + l.off_energy);
+    ctx->arrived = reinterpret_cast<unsigned long long *>(base + l.off_arrived);
+    ctx->counters = reinterpret_cast<int *>(base + l.off_counters);
     ctx->leff = reinterpret_cast<int *>(base + l.off_leff);
     ctx->gain = reinterpret_cast<float *>(base + l.off_gain);
     ctx->melw = reinterpret_cast<aug::MelBin *>(base + l.off_melw);
@@ -404,6 +410,8 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
             tw[fftpair::tw_index(M, k)] = make_float2((float)cos(a), (float)sin(a));
         }
     }
+    float taps[32 * aug::TAP_ROWS] = {};
+    rir_tap_table(cfg->frac_half_width, taps);
     const int st0[2] = {-1, 0};
     if (ctx->park_flags &&
         cudaMemsetAsync(ctx->park_flags, 0, sizeof(int) * aug::PARK_SLOTS, ctx->stream) !=
@@ -415,6 +423,7 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     }
     bool ok = cudaMemcpyAsync(ctx->tw, tw.data(), sizeof(float2) * fftpair::TW_N,
                               cudaMemcpyHostToDevice, ctx->stream) == cudaSuccess &&
+              cudaMemcpyAsync(ctx->tap_tab, taps, sizeof(taps), cudaMemcpyHostToDevice, ctx->stream) == cudaSuccess &&
               cudaMemcpyAsync(ctx->status, st0, sizeof(st0), cudaMemcpyHostToDevice,
                               ctx->stream) == cudaSuccess &&
               cudaStreamSynchronize(ctx->stream) == cudaSuccess;
@@ -508,8 +517,8 @@ int aug_reverb_mix(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     const int max_len = (int)(speech_stride < ctx->cfg.max_samples ? speech_stride : ctx->cfg.max_samples);
     if (speech_stride > ctx->ws_stride) return AUG_ECAP;
     const ConvInput in = {speech_dev, speech_stride, lengths_dev, noise_bank_dev, bank_len, max_len, 0};
-    if ((rc = launch_rir_spectra(ctx, rir_dev, in, table_dev, B, true)) != AUG_OK) return rc;
-    if ((rc = launch_convolve_prepare(ctx, in, table_dev, B)) != AUG_OK) return rc;
+    if ((rc = launch_rir_spectra(ctx, rir_dev, in, table_dev, B, false)) != AUG_OK) return rc;
+    if ((rc = launch_convolve_prepare(ctx, in, table_dev, B, false)) != AUG_OK) return rc;
     if ((rc = launch_convolve_finish(ctx, in, table_dev, B)) != AUG_OK) return rc;
     return launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out_dev, speech_stride);
 }

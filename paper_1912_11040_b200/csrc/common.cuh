@@ -11,16 +11,16 @@ namespace aug {
 
 constexpr int CONV_TAPS = 8192;         // taps of a partition: half a transform of the convolution
 constexpr int CONV_BINS = 8192;         // complex numbers of a stored spectrum
-// Counters of the convolution behind the batch's largest response length: units of work listed for
-// the two routes, units drawn from the lists.
-enum Counter { LIST_FUSED, LIST_STORED, DRAWN_FUSED, DRAWN_SPECTRA, DRAWN_STORED };
-constexpr int N_COUNTERS = 6;
+// Counters of the convolution: the batch's largest response length (long-response contexts), units of
+// work listed for the two routes, units drawn from the lists.
+enum Counter { LEFF_ALL, LIST_FUSED, LIST_STORED, DRAWN_FUSED, DRAWN_SPECTRA, DRAWN_STORED, N_COUNTERS };
 constexpr int PARK_SLOTS = 320;     // parking slots of the fused convolution = most CTAs it runs with
 constexpr int PLAN_BYTES = 96;      // per utterance, see conv.cu
 constexpr int MAX_TAPS = 24576;
 constexpr int MAX_ORDER = 32;
 constexpr int MAX_HALF_W = 47;
 constexpr int MAX_MEL = 128;
+constexpr int TAP_ROWS = 13;
 
 constexpr int EV_RING = 256;
 #ifndef AUG_HOST_CHUNKS
@@ -60,6 +60,7 @@ struct AugCtx {
     void *ws_base;
     int64_t ws_bytes;
     float2 *tw;            // [TW_N] twiddles
+    float *tap_tab;        // [TAP_ROWS][32] constants of the taps of an image
     float *rir;            // [max_batch][max_sources][rir_taps]
     float2 *hspec;         // [max_batch][max_sources][n_part][CONV_BINS]
     float2 *xspec;         // [max_batch][max_sources][nblk_cap][CONV_BINS]; NULL unless route == ROUTE_STORED
@@ -72,10 +73,11 @@ struct AugCtx {
     void *vtlp_tab;        // [max_batch][513] lower source bin (int), then [max_batch][513] fraction (float)
     float *ys;             // [max_batch][ws_stride]
     float *vv;             // [max_batch][ws_stride]
-    double *energy;        // [max_batch][2]
-    int *leff;             // [2 max_batch + N_COUNTERS] taps up to the last non-zero one, largest over the utterance's
-                           // sources; behind them the largest over the batch, counters, sources transformed
-    int *leff_seen;        // pinned host copy of that last entry from an earlier call (long-response contexts)
+    double *energy;        // [max_batch][2]; this and the next two lie one behind the other, set to zero together
+    unsigned long long *arrived;   // [max_batch] responses of callers: sources transformed and their lengths
+    int *counters;         // [N_COUNTERS]
+    int *leff;             // [max_batch][max_sources] taps of a response up to the last non-zero one
+    int *leff_seen;        // pinned host copy of LEFF_ALL from an earlier call (long-response contexts)
     int stored_only;       // this call launches the stored-spectra kernels alone
     float *gain;           // [max_batch] noise gain g for the requested SNR
     aug::MelBin *melw;     // [max_batch][n_bins]
@@ -166,16 +168,17 @@ struct ConvInput {
 };
 
 // Launchers (defined next to their kernels).  They enqueue on ctx->stream.
-// `beside`: may run beside the kernel before it on the stream, one of this library that calls chain_next()
-int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside);
-// `reset`: set the counters and sums of the convolution to zero first (aug_pipeline has had it done by
-// launch_mel_tables)
+void rir_tap_table(int half_width, float *tab);
+// `chained`: in aug_pipeline, behind launch_mel_tables; records where the responses end
+int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool chained);
+// `measured`: the responses come from launch_rir, which has recorded where they end (and launch_mel_tables has
+// set the counters and sums of the convolution to zero); otherwise they are the caller's
 int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
-                       bool reset);
+                       bool measured);
 // Convolution in two parts: `prepare` needs only the input audio (block spectra when
 // the response has several partitions, else nothing), `finish` also needs the
 // partition spectra of the impulse responses.
-int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
+int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B, bool measured);
 int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
 int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
                float *wave_out, int64_t out_stride);

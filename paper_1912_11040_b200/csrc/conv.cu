@@ -60,8 +60,8 @@ __device__ __forceinline__ bool source_of(const AugUttParams &row, int s, const 
     return true;
 }
 
-// Effective length of the responses: (index + 1) of the last non-zero tap, largest over the
-// sources of an utterance (leff[utt]) and over the batch (*leff_all); both zeroed before the launch.
+// Effective length of the responses: (index + 1) of the last non-zero tap (leff[utt][source]), and the largest of
+// the batch (*leff_all, zeroed before the launch).  For responses that come from the caller.
 __global__ void __launch_bounds__(CT)
 rir_length_kernel(const float *rir, const AugUttParams *__restrict__ table, int S_max, int L,
                   int *__restrict__ leff, int *__restrict__ leff_all) {
@@ -94,10 +94,8 @@ rir_length_kernel(const float *rir, const AugUttParams *__restrict__ table, int 
     if (t == 0) {
         int m = 0;
         for (int i = 0; i < CT / 32; ++i) m = max(m, red_i[i]);
-        if (m > 0) {
-            atomicMax(&leff[utt], m);
-            atomicMax(leff_all, m);
-        }
+        leff[utt * S_max + s] = m;
+        if (m > 0) atomicMax(leff_all, m);
     }
 }
 
@@ -417,7 +415,7 @@ struct PlanArgs {
     int *status;
     Plan *plans;
     Unit *units;
-    int *lists;                    // counters of the two lists
+    int *counters;                 // [N_COUNTERS]
 };
 // By one warp; leff: taps up to the last non-zero one.
 __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttParams &row, int utt, int S_max, int leff,
@@ -451,23 +449,30 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttPa
             }
         }
         a.plans[utt] = p;
-        if (n > 0) at = atomicAdd(a.lists + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
+        if (n > 0) at = atomicAdd(a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
     }
     at = __shfl_sync(0xffffffffu, at, 0);
     for (int i = lane; i < n; i += 32) a.units[at + i] = Unit{utt, i};
 }
 
-// One warp per utterance (contexts for long responses: the route follows from the whole batch;
-// elsewhere rir_spectra2_kernel plans on the way).
+// The same with the lengths in global memory.
+__device__ __forceinline__ void plan_measured(const PlanArgs &a, const AugUttParams *__restrict__ table, int utt,
+                                              int S_max, const int *leff, const int *leff_all, bool mixed,
+                                              bool stored_only, int lane) {
+    const AugUttParams &row = table[utt];
+    int len = lane < row.n_src && row.n_src <= S_max ? leff[utt * S_max + lane] : 0;
+    len = __reduce_max_sync(0xffffffffu, len);
+    plan_utterance(a, row, utt, S_max, len, mixed && (stored_only || !takes_fused_route(*leff_all)), lane);
+}
+// One warp per utterance (long responses of the caller: the route follows from the whole batch; elsewhere
+// rir_spectra2_kernel plans on the way).
 __global__ void __launch_bounds__(256)
 plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restrict__ table, int B, int S_max,
             const int *leff, const int *leff_all, int stored_only) {
     const int utt = blockIdx.x * 8 + (threadIdx.x >> 5);
     chain_next();
     chain_wait();
-    if (utt < B)
-        plan_utterance(args, table[utt], utt, S_max, leff[utt], stored_only || !takes_fused_route(*leff_all),
-                       threadIdx.x & 31);
+    if (utt < B) plan_measured(args, table, utt, S_max, leff, leff_all, true, stored_only, threadIdx.x & 31);
 }
 
 // Spectra of the partitions of each impulse response: 8192 taps (those beyond L are zero) and as many
@@ -476,28 +481,51 @@ plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restric
 // the taps are requested together, four a load (256 x 3 responses of 8192 taps: 31.1 us one
 // by one, 29.9; a test per group inside the loop parts the loads: 33.6).  Persistent CTAs that work
 // through the partitions, as the kernels below, took 33.2 and, 128 x 4 x 3 partitions, 53 against 43.
+//
+// LENGTHS  KNOWN  where the responses end has been recorded: zeros behind are not read, partitions of zeros left out
+//          FIND   responses of the caller, of one partition: found on the way.  The CTA that adds an utterance's last
+//                 source plans its work; the sum it learns that from holds the lengths too and is asked for before
+//                 the transform, read behind it
+// The first n_plan CTAs plan instead (KNOWN: the kernel that made the responses measured them), a warp an
+// utterance.  With a chain of atomics and the plan of the utterance ahead of the transform, 4096 x 2 responses
+// of 4096 taps took 267 us, so 207.
+enum Lengths { KNOWN, FIND };
+template <Lengths LENGTHS>
 __global__ void __launch_bounds__(CF, FUSED_MINB)
-rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, int S_max,
-                    int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, int *leff, int mixed,
-                    int *transformed, const __grid_constant__ PlanArgs plan) {
+rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, int B, int S_max,
+                    int L, int P, const float2 *__restrict__ tw, float4 *__restrict__ hspec, const int *leff,
+                    unsigned long long *arrived, const __grid_constant__ PlanArgs plan, int n_plan, const int *leff_all,
+                    int mixed, int stored_only) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fftpair::Shared &sh = *reinterpret_cast<fftpair::Shared *>(smem_raw);
     __shared__ int red_i[CF / 32];
-    const int part = blockIdx.x, s = blockIdx.y, utt = blockIdx.z, t = threadIdx.x, from = part * BLK2;
-    fftpair::fill_tables(sh, t, tw);
-    chain_wait();
-    // mixed: the lengths are known already (rir_length_kernel); otherwise there is one partition, and
-    // this kernel reads every tap anyway and records the length on the way
-    if (mixed && part > 0 && from >= leff[utt]) return;
-    const AugUttParams &row = table[utt];
-    if (row.n_src < 1 || row.n_src > S_max) {
-        if (!mixed && s == 0 && t < 32) plan_utterance(plan, row, utt, S_max, 1, false, t);
+    const int t = threadIdx.x;
+    if (LENGTHS == KNOWN && blockIdx.x < n_plan) {
+        chain_wait();
+        const int utt = blockIdx.x * (CF / 32) + (t >> 5);
+        if (utt < B) plan_measured(plan, table, utt, S_max, leff, leff_all, mixed, stored_only, t & 31);
         return;
     }
-    if (s >= row.n_src) return;
+    const int id = blockIdx.x - n_plan, part = id % P, us = id / P, utt = us / S_max, s = us - utt * S_max;
+    const int from = part * BLK2;
+    const AugUttParams &row = table[utt];
+    fftpair::fill_tables(sh, t, tw);
+    if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) {
+        chain_wait();
+        if (LENGTHS == FIND && s == 0 && t < 32) plan_utterance(plan, row, utt, S_max, 1, false, t);
+        return;
+    }
+    chain_wait();
+    const int end = LENGTHS == KNOWN ? min(leff[us], L) : L;
+    if (part > 0 && from >= end) {
+        // (a longer response of the same utterance may be the reason that the products take this partition)
+        int most = 0;
+        for (int i = 0; i < row.n_src; ++i) most = max(most, leff[utt * S_max + i]);
+        if (from >= most) return;
+    }
     const float scale = (s == 0 ? 1.f : row.noise_weight[s - 1]) / (4.f * (float)F2);
-    const float *h = rir + ((int64_t)utt * S_max + s) * L;
-    float4 *out = hspec + (((int64_t)utt * S_max + s) * P + part) * (NB2 / 2) + t;
+    const float *h = rir + (int64_t)us * L;
+    float4 *out = hspec + ((int64_t)us * P + part) * (NB2 / 2) + t;
     static_assert(4 * CF * (NP2 / 2) == BLK2, "");
     C2 v[NP2];
     int last = 0;
@@ -507,47 +535,43 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
 #pragma unroll
         for (int r = 0; r < NP2 / 2; ++r) {
             const int i0 = from + 4 * (t + CF * r);
-            z[r] = i0 < L ? *reinterpret_cast<const float4 *>(h + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
+            z[r] = i0 < end ? *reinterpret_cast<const float4 *>(h + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     } else {
 #pragma unroll
         for (int r = 0; r < NP2 / 2; ++r) {
             const int i0 = from + 4 * (t + CF * r);
-            z[r] = make_float4(i0 < L ? h[i0] : 0.f, i0 + 1 < L ? h[i0 + 1] : 0.f, i0 + 2 < L ? h[i0 + 2] : 0.f,
-                               i0 + 3 < L ? h[i0 + 3] : 0.f);
+            z[r] = make_float4(i0 < end ? h[i0] : 0.f, i0 + 1 < end ? h[i0 + 1] : 0.f, i0 + 2 < end ? h[i0 + 2] : 0.f,
+                               i0 + 3 < end ? h[i0 + 3] : 0.f);
         }
     }
 #pragma unroll
     for (int r = 0; r < NP2 / 2; ++r) {
         const int i0 = from + 4 * (t + CF * r);
-        if (z[r].x != 0.f) last = i0 + 1;
-        if (z[r].y != 0.f) last = i0 + 2;
-        if (z[r].z != 0.f) last = i0 + 3;
-        if (z[r].w != 0.f) last = i0 + 4;
+        if (LENGTHS == FIND) {
+            if (z[r].x != 0.f) last = i0 + 1;
+            if (z[r].y != 0.f) last = i0 + 2;
+            if (z[r].z != 0.f) last = i0 + 3;
+            if (z[r].w != 0.f) last = i0 + 4;
+        }
         v[r] = {fftpair::pack(z[r].x, z[r].y), fftpair::pack(z[r].z, z[r].w)};
     }
 #pragma unroll
     for (int r = NP2 / 2; r < NP2; ++r) v[r] = {0, 0};
-    if (!mixed) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+    if (LENGTHS == FIND) {
+        last = __reduce_max_sync(0xffffffffu, last);
         if ((t & 31) == 0) red_i[t >> 5] = last;
     }
     __syncthreads();
-    if (!mixed && t < 32) {
-        int m = t < CF / 32 ? red_i[t] : 0;
+    // a count of the sources and the length of each in one word
+    static_assert(AUG_S_MAX <= 4 && BLK2 < (1 << 14), "");
+    unsigned long long sum = 0;
+    if (LENGTHS == FIND && t == 0) {
+        int m = 0;
 #pragma unroll
-        for (int o = CF / 64; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        // the CTA that adds the last source's length plans the utterance's work
-        int done = 0;
-        if (t == 0) {
-            atomicMax(&leff[utt], m);
-            __threadfence();
-            done = atomicAdd(&transformed[utt], 1) + 1;
-            __threadfence();
-        }
-        if (__shfl_sync(0xffffffffu, done, 0) == row.n_src)
-            plan_utterance(plan, row, utt, S_max, __ldcg(&leff[utt]), false, t);
+        for (int i = 0; i < CF / 32; ++i) m = max(m, red_i[i]);
+        const unsigned long long mine = (1ull << 56) | ((unsigned long long)m << (14 * s));
+        sum = atomicAdd(&arrived[utt], mine) + mine;
     }
     fftpair::forward4096(v, sh, t, tw);
     chain_next();
@@ -560,6 +584,13 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
                                                  : bins_forward(v[r], v[NP2 - 1 - r], SplitTwiddle(u, r));
         x = {fftpair::mul2(x.pr, sc), fftpair::mul2(x.pi, sc), fftpair::mul2(x.qr, sc), fftpair::mul2(x.qi, sc)};
         store_bins(out + 2 * r * CF, x);
+    }
+    if (LENGTHS == FIND && t < 32) {
+        sum = __shfl_sync(0xffffffffu, sum, 0);
+        if ((int)(sum >> 56) == row.n_src) {
+            const int len = t < 4 ? (int)(sum >> (14 * t)) & ((1 << 14) - 1) : 0;
+            plan_utterance(plan, row, utt, S_max, __reduce_max_sync(0xffffffffu, len), false, t);
+        }
     }
 }
 
@@ -856,47 +887,50 @@ static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_ST
 
 static PlanArgs plan_args(const AugCtx *ctx, const ConvInput &in) {
     return {in.speech, in.stride, in.lengths, in.bank, in.bank_len, in.max_len, ctx->status,
-            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units),
-            ctx->leff + ctx->cfg.max_batch + 1};
+            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units), ctx->counters};
 }
 
-int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
-                       bool reset) {
+template <Lengths LENGTHS>
+static int launch_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
+                          int n_plan) {
     const AugConfig &c = ctx->cfg;
-    const cudaStream_t st = ctx->stream;
-    const int mixed = stored_route(ctx) ? 1 : 0;
-    // long-response context: the last batch size seen decides whether the fused kernels are launched at all
-    ctx->stored_only = mixed && ctx->leff_seen && *ctx->leff_seen > BLK2;
-    int *leff_all = ctx->leff + ctx->cfg.max_batch;
-    if (reset)                       // sums, lengths and counters, which lie one behind the other
-        AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0,
-                                    reinterpret_cast<char *>(ctx->leff + 2 * (size_t)c.max_batch + aug::N_COUNTERS) -
-                                        reinterpret_cast<char *>(ctx->energy), st));
-    if (mixed) {
-        if (launch_chained(rir_length_kernel, dim3(c.max_sources, B), CT, 0, st, rir, table, c.max_sources, c.rir_taps,
-                           ctx->leff, leff_all) != AUG_OK)
-            return AUG_ECUDA;
-        ctx->launches++;
-    }
-    if (smem_opt_in<rir_spectra2_kernel>(ctx->device) != AUG_OK) return AUG_ECUDA;
-    if (launch_chained(rir_spectra2_kernel, dim3(ctx->n_part, c.max_sources, B), CF, FFT2_SMEM, st, rir, table,
-                       c.max_sources, c.rir_taps, ctx->n_part, ctx->tw, reinterpret_cast<float4 *>(ctx->hspec),
-                       ctx->leff, mixed, leff_all + aug::N_COUNTERS, plan_args(ctx, in)) != AUG_OK)
+    if (smem_opt_in<rir_spectra2_kernel<LENGTHS>>(ctx->device) != AUG_OK) return AUG_ECUDA;
+    if (launch_chained(rir_spectra2_kernel<LENGTHS>, dim3(n_plan + ctx->n_part * c.max_sources * B), CF, FFT2_SMEM,
+                       ctx->stream, rir, table, B, c.max_sources, c.rir_taps, ctx->n_part, ctx->tw,
+                       reinterpret_cast<float4 *>(ctx->hspec), ctx->leff, ctx->arrived, plan_args(ctx, in), n_plan,
+                       ctx->counters + aug::LEFF_ALL, stored_route(ctx) ? 1 : 0, ctx->stored_only) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
 }
 
+int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const AugUttParams *table, int B,
+                       bool measured) {
+    const AugConfig &c = ctx->cfg;
+    const bool mixed = stored_route(ctx);
+    // long-response context: the last batch size seen decides whether the fused kernels are launched at all
+    ctx->stored_only = mixed && ctx->leff_seen && *ctx->leff_seen > BLK2;
+    if (measured) return launch_spectra<KNOWN>(ctx, rir, in, table, B, (B + CF / 32 - 1) / (CF / 32));
+    AUG_CUDA_OK(cudaMemsetAsync(ctx->energy, 0, reinterpret_cast<char *>(ctx->counters + aug::N_COUNTERS) -
+                                                    reinterpret_cast<char *>(ctx->energy), ctx->stream));
+    if (!mixed) return launch_spectra<FIND>(ctx, rir, in, table, B, 0);
+    if (launch_chained(rir_length_kernel, dim3(c.max_sources, B), CT, 0, ctx->stream, rir, table, c.max_sources,
+                       c.rir_taps, ctx->leff, ctx->counters + aug::LEFF_ALL) != AUG_OK)
+        return AUG_ECUDA;
+    ctx->launches++;
+    return launch_spectra<KNOWN>(ctx, rir, in, table, B, 0);
+}
+
 template <Kind KIND, bool PARK>
 static int launch_convolve(AugCtx *ctx, int grid) {
     const AugConfig &c = ctx->cfg;
-    int *counters = ctx->leff + c.max_batch;
+    int *counters = ctx->counters;
     if (smem_opt_in<convolve_kernel<KIND, PARK>>(ctx->device) != AUG_OK) return AUG_ECUDA;
     const int list = KIND == FUSED ? aug::LIST_FUSED : aug::LIST_STORED;
     const int drawn = KIND == FUSED ? aug::DRAWN_FUSED : KIND == SPECTRA ? aug::DRAWN_SPECTRA : aug::DRAWN_STORED;
     if (launch_chained(convolve_kernel<KIND, PARK>, dim3(grid), CF, FFT2_SMEM, ctx->stream,
                        reinterpret_cast<const Plan *>(ctx->plans), reinterpret_cast<const Unit *>(ctx->units),
-                       counters + 1 + list, counters + 1 + drawn, c.max_sources, ctx->n_part,
+                       counters + list, counters + drawn, c.max_sources, ctx->n_part,
                        reinterpret_cast<const float4 *>(ctx->hspec), reinterpret_cast<float4 *>(ctx->xspec),
                        ctx->nblk_cap, ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->park,
                        ctx->park_flags) != AUG_OK)
@@ -912,13 +946,15 @@ static int convolve_grid(const AugCtx *ctx, const ConvInput &in, int B, int ob) 
     return (int)std::min<int64_t>(2 * (int64_t)B * ((max_len + ob - 1) / ob), fit);
 }
 
-int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B) {
+int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B, bool measured) {
     const AugConfig &c = ctx->cfg;
     if (in.max_len <= 0 || !stored_route(ctx)) return AUG_OK;
-    if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, plan_args(ctx, in), table, B, c.max_sources,
-                       ctx->leff, ctx->leff + c.max_batch, ctx->stored_only) != AUG_OK)
-        return AUG_ECUDA;
-    ctx->launches++;
+    if (!measured) {
+        if (launch_chained(plan_kernel, dim3((B + 7) / 8), 256, 0, ctx->stream, plan_args(ctx, in), table, B,
+                           c.max_sources, ctx->leff, ctx->counters + aug::LEFF_ALL, ctx->stored_only) != AUG_OK)
+            return AUG_ECUDA;
+        ctx->launches++;
+    }
     return launch_convolve<SPECTRA, false>(ctx, convolve_grid(ctx, in, B, BLK2));
 }
 
@@ -936,7 +972,7 @@ int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams 
         if ((rc = launch_convolve<STORED, false>(ctx, convolve_grid(ctx, in, B, BLK2))) != AUG_OK) return rc;
         // for the next call's choice (not waited for)
         if (ctx->leff_seen)
-            AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, ctx->leff + c.max_batch, sizeof(int), cudaMemcpyDeviceToHost,
+            AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, ctx->counters + aug::LEFF_ALL, sizeof(int), cudaMemcpyDeviceToHost,
                                         ctx->stream));
     }
     if (launch_chained(snr_gain_kernel, dim3((B + 255) / 256), 256, 0, ctx->stream, ctx->energy, table, B, ctx->gain) !=

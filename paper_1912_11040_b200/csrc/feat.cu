@@ -25,15 +25,13 @@ __host__ __device__ __forceinline__ int frame_count(int n, int win, int hop) {
 __global__ void __launch_bounds__(256)
 mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double f_lo,
                   double f_hi, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped,
-                  int *leff, int *counters, double *energy) {
+                  int *counters, double *energy) {
     __shared__ int seg_s[513];
     chain_next();
     // first kernel of aug_pipeline: the convolution's sums and counters start from zero
-    if (leff != nullptr && blockIdx.x == 0 && threadIdx.x < aug::N_COUNTERS) counters[threadIdx.x] = 0;
-    if (leff != nullptr && threadIdx.x == 0) {
-        leff[blockIdx.x] = 0;
-        counters[aug::N_COUNTERS + blockIdx.x] = 0;
-        energy[2 * blockIdx.x] = energy[2 * blockIdx.x + 1] = 0.0;
+    if (energy != nullptr) {
+        if (blockIdx.x == 0 && threadIdx.x < aug::N_COUNTERS) counters[threadIdx.x] = 0;
+        if (threadIdx.x == 0) energy[2 * blockIdx.x] = energy[2 * blockIdx.x + 1] = 0.0;
     }
     const int utt = blockIdx.x, nb = K / 2 + 1;
     // (unwarped: the warp was already applied to the waveform)
@@ -732,7 +730,7 @@ int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset)
     const AugConfig &c = ctx->cfg;
     mel_tables_kernel<<<B, 256, 0, ctx->stream>>>(
         table, c.n_fft, c.n_mel, (double)c.fs, (double)c.f_lo, (double)c.f_hi, ctx->melw, ctx->melstart,
-        c.vtlp_win > 0 ? 1 : 0, reset ? ctx->leff : nullptr, ctx->leff + c.max_batch, ctx->energy);
+        c.vtlp_win > 0 ? 1 : 0, ctx->counters, reset ? ctx->energy : nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     ctx->launches++;
     return AUG_OK;
@@ -858,7 +856,7 @@ extern "C" int feat_vtlp_logmel_noalloc(const AugConfig *cfg, const float *power
     const int nbp = cfg->n_fft / 2 + 1;
     mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs,
                                          (double)cfg->f_lo, (double)cfg->f_hi, melw, melstart, 0, nullptr,
-                                         nullptr, nullptr);
+                                         nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     int dev = -1;
     AUG_CUDA_OK(cudaGetDevice(&dev));

@@ -11,24 +11,28 @@
 //   B  four images at a time, their 2 W_h taps over the lanes: lane l owns taps l and l + 32
 //      of all four, and of the 16 taps that are left (W_h = 40) the lower half-warp does those
 //      of the first two images and the upper half those of the others.  Everything that
-//      depends only on the tap (its offset, the cosine and sine of its Hann angle, its sign) sits
-//      in registers, and the images' numbers arrive as pairs, the operands of packed (f32x2)
-//      arithmetic, by broadcast loads.  With tau = n0 + phi, 0 <= phi < 1,
-//      sin(pi (n - tau)) = -(-1)^(n - n0) sin(pi phi), and the Hann factor follows
-//      from the angle-sum identity, so a tap costs one reciprocal, three to four fused
-//      multiply-adds -- the last one adds 1.5 2^23, which leaves the fixed-point value in the
-//      low bits -- and one shared-memory reduction.  n0 is rounded down so that the window
-//      always covers the same taps -W_h + 1 .. W_h and none has to be masked.
+//      depends only on the tap sits in registers, and the images' numbers arrive as pairs, the
+//      operands of packed (f32x2) arithmetic, by broadcast loads.  With tau = n0 + phi, 0 <= phi < 1,
+//      sin(pi (n - tau)) = -(-1)^(n - n0) sin(pi phi), so tap j is As(phi) times
+//      (1 + cos(pi (j - phi) / W_h)) / (j - phi).  n0 is rounded down so that the window always
+//      covers the same taps -W_h + 1 .. W_h and none has to be masked.  The 32 taps around the
+//      centre take a reciprocal and the angle-sum identity of the Hann factor (three fused
+//      multiply-adds); W_h >= 40 leaves the others at least eight samples away from the image, where that
+//      function of phi is a polynomial of degree four (the first 32 taps) or three (the last 16) to 3e-9 of
+//      the image's amplitude, less than the rounding of the reciprocal form (5e-9).  The last multiply-add
+//      adds 1.5 2^23, which leaves the fixed-point value in the low bits, and one shared-memory reduction
+//      follows.
 //
 //      Phase A orders the images of a batch: loud ones (their taps need more than 22 bits) first,
 //      then the others whose window lies inside the response, then those at its edges, which are
 //      done one by one with tests.  No test is left in the loops over the first two.
 //
-// Bound by instruction issue (30 warp instructions an image, 58 to 63 % of the slots; reciprocal pipe
-// 47 to 53 %).  One image at a time in scalar arithmetic, with a conversion instruction per tap and
-// masks, it was 58, and the quarter-rate pipe of reciprocals and conversions was 62 % busy too;
-// two at a time with tests of strength and range per pair 45.  128 x 4 responses of 24000 taps,
-// order 20: 393, 312 (two at a time) and 250 us; 4096 x 2 of 4096 taps: 437, 354 and 281.
+// Bound by instruction issue (26 warp instructions an image, 68 % of the slots) and shared memory (67 % of its
+// cycles).  128 x 4 responses of 24000 taps, order 20: 393 us one image at a time in scalar arithmetic, 312
+// with two at a time in packed arithmetic, 251 with four at a time and all taps by reciprocals (30
+// instructions an image), 228 with polynomials away from the centre, the lattice without searches, the sines as
+// series and the tap constants from a table; 512 x up to 4 of 8192 taps, order 12: 162 and 147; 4096 x 2 of
+// 4096 taps: 281 and 257.
 //
 // The response is accumulated in 32-bit fixed point: a shared-memory fp32 atomic
 // add is a compare-and-swap loop on this hardware, an integer one is a single
@@ -40,9 +44,10 @@
 // sample is 2-3 A0 in rooms of a few metres and 14 A0 in a 30 cm box; a sample
 // beyond 64 A0 (rooms of a few centimetres) would wrap.
 //
-// The lattice points with |kx|+|ky|+|kz| <= order are enumerated compactly (a
-// prefix over kx, then closed forms inside the diamond of (ky, kz)), so every
-// lane of a warp carries a real image.
+// The lattice points with |kx|+|ky|+|kz| <= order are enumerated compactly in closed
+// form (slab kx, then inside the diamond of (ky, kz)), so every lane of a warp carries a real image.
+#include <math.h>
+
 #include <type_traits>
 
 #include "common.cuh"
@@ -72,8 +77,8 @@ __device__ __forceinline__ void red_shared_add(unsigned a, int iv) {
 
 // Bytes of dynamic shared memory of a CTA of `threads` threads for responses of L taps.
 __host__ __device__ constexpr size_t rir_smem_bytes(int threads, int L) {
-    return sizeof(double) * 3 * AX + sizeof(float) * 3 * AX + sizeof(int) * (AX + 3) +
-           5 * sizeof(float) * threads + sizeof(float) * (size_t)((L + 3) & ~3);
+    return sizeof(double) * 3 * AX + sizeof(float) * 3 * AX + 5 * sizeof(float) * threads +
+           sizeof(float) * (size_t)((L + 3) & ~3);
 }
 
 constexpr float HEADROOM_LOG2 = 6.f;   // full scale = 2^6 times the direct-path amplitude
@@ -98,17 +103,35 @@ __device__ __forceinline__ int2 round_strong(fftpair::u64 v) {
                      (int)(16u * __float_as_uint(hi.y) + __float_as_uint(lo.y) - BITS));
 }
 
-// NARROW: half_w <= 40, at most 80 taps.
-template <bool NARROW, int THREADS>
+// sin(pi x) / pi, 0 <= x <= 1: the Taylor series up to x^13 on the nearer half (rest below 1e-9)
+__device__ __forceinline__ float sin_pi_over_pi(float x) {
+    const float y = fminf(x, 1.f - x), z = y * y;
+    float p = 1.48428793e-4f;
+    p = fmaf(p, z, -2.34608099e-3f);
+    p = fmaf(p, z, 2.61478478e-2f);
+    p = fmaf(p, z, -0.190751824f);
+    p = fmaf(p, z, 0.811742425f);
+    p = fmaf(p, z, -1.64493407f);
+    return fmaf(p * z, y, y);
+}
+
+// The window's half width: below 40, where every tap takes the reciprocal form, 40 (80 taps), and more (at
+// most 96 taps).
+enum Width { SHORT, FORTY, WIDE };
+
+// leff, leff_all (aug_pipeline, else NULL): where each response ends ([utt][source]: taps up to the last
+// non-zero one, at least one of which has to be there) and the largest of all; what lies behind a response's end, and
+// the places of sources that there are not, stay as they are then.
+template <Width WIDTH, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int half_w,
-                 double fs_over_c, int max_order, int cube, float *__restrict__ rir, int *status) {
+                 double fs_over_c, int max_order, int cube, const float *__restrict__ tap_tab, float *__restrict__ rir,
+                 int *status, int *leff, int *leff_all) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *ring = reinterpret_cast<int *>(smem_raw);                 // [THREADS / 32][RING]
     int *h = ring + THREADS / 32 * RING;                           // [L rounded up to 4] fixed-point response
     double *dsq = reinterpret_cast<double *>(h + ((L + 3) & ~3));  // [3][AX] squared coordinate differences
     float *gain = reinterpret_cast<float *>(dsq + 3 * AX);         // [3][AX] wall gains per axis
-    int *xpre = reinterpret_cast<int *>(gain + 3 * AX);            // [AX + 1] images before slab kx
 
     const int utt = blockIdx.y, s = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -120,7 +143,10 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
     if (n_src < 1 || n_src > S_max) bad = aug::R_NSRC;
     else if (order < 0 || order > max_order) bad = aug::R_ORDER;
     if (bad || s >= n_src) {
-        for (int i = tid; i < L; i += THREADS) out[i] = 0.f;
+        if (leff == nullptr)
+            for (int i = tid; i < L; i += THREADS) out[i] = 0.f;
+        else if (bad == aug::R_ORDER && s < n_src && tid == 0)
+            leff[utt * S_max + s] = 0;         // silence
         if (bad && tid == 0 && s == 0) {
             if (atomicCAS(&status[0], -1, utt) == -1) status[1] = bad;
         }
@@ -140,38 +166,41 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
         gain[a * AX + k + order] = (float)(ipow((double)row.beta[2 * a], abs(m - p)) *
                                            ipow((double)row.beta[2 * a + 1], abs(m)));
     }
-    if (tid == 0) {
-        int run = 0;
-        for (int ix = 0; ix < side; ++ix) {
-            const int r = order - abs(ix - order);
-            xpre[ix] = run;
-            run += 2 * r * r + 2 * r + 1;      // points of the diamond |ky|+|kz| <= r
-        }
-        xpre[side] = run;
-    }
     __syncthreads();
-    const int total = cube ? side * side * side : xpre[side];
+    // images in the slabs of radius 0 .. n - 1 of the lattice's lower half: n (2 n^2 + 1) / 3
+    const int lower = (order + 1) * (2 * (order + 1) * (order + 1) + 1) / 3;
+    const int total = cube ? side * side * side : lower + order * (2 * order * order + 1) / 3;
     // fixed-point scale: a power of two with 2^31 / scale >= 2^HEADROOM_LOG2 / d0
     const float d0sq = (float)(dsq[order] + dsq[AX + order] + dsq[2 * AX + order]);
     const float e2 = d0sq > 0.f ? floorf(31.f - HEADROOM_LOG2 + 0.5f * log2f(d0sq)) : 0.f;
     const float scale = exp2f(fminf(fmaxf(e2, -60.f), 60.f)), inv_scale = exp2f(-fminf(fmaxf(e2, -60.f), 60.f));
 
-    // Per-lane tap constants.  Tap jj = 0 .. 2 half_w - 1 lies at offset j = jj - half_w + 1 from n0.
-    // The sign (-1)^j (with that of the sine) is the same for all taps of a lane; it goes into the
-    // offset, whose reciprocal is taken.  A tap beyond the window gets an offset so large that its
-    // value rounds to zero.
+    // Per-lane tap constants, see rir_tap_table.
     using fftpair::u64;
+    constexpr bool POLY = WIDTH != SHORT;
+    constexpr int REST = WIDTH == WIDE ? 4 : 3;          // degree for the last taps
     const float fhw = (float)half_w;
     const float sgn = ((lane - half_w + 1) & 1) ? -1.f : 1.f;
-    float fj[3], cj[3], sj[3];
+    float fj[3], cj[3], sj[3], head[5], rest[REST + 1];
+    if constexpr (POLY) {
+        fj[1] = __ldg(tap_tab + lane);
+        cj[1] = __ldg(tap_tab + 32 + lane);
+        sj[1] = __ldg(tap_tab + 64 + lane);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int jj = i < 2 ? lane + 32 * i : NARROW ? 64 + (lane & 15) : 64 + lane, j = jj - half_w + 1;
-        fj[i] = jj < 2 * half_w ? sgn * (float)j : 3e18f;
-        cj[i] = cospif((float)j / fhw);
-        sj[i] = sinpif((float)j / fhw);
+        for (int i = 0; i < 5; ++i) head[i] = __ldg(tap_tab + 32 * (3 + i) + lane);
+#pragma unroll
+        for (int i = 0; i <= REST; ++i) rest[i] = __ldg(tap_tab + 32 * (8 + i) + lane);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            fj[i] = __ldg(tap_tab + 32 * (3 * i) + lane);
+            cj[i] = __ldg(tap_tab + 32 * (3 * i + 1) + lane);
+            sj[i] = __ldg(tap_tab + 32 * (3 * i + 2) + lane);
+        }
     }
     const u64 nsgn = fftpair::both(-sgn);
+    const float hann = 3.14159265358979323846f / fhw;
+    const double tau_end = (double)(L + half_w - 1);     // windows of later images begin behind the buffer
     constexpr int NW = THREADS / 32;
     const unsigned h_addr = (unsigned)__cvta_generic_to_shared(h) + 4u * lane;
     const unsigned h_rest = h_addr + (lane < 16 ? 256u : 192u);      // of this lane's tap among the last 16
@@ -194,37 +223,33 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
                 ky = rem / side - order;
                 kz = rem % side - order;
             } else {
-                // slab kx: the last ix with xpre[ix] <= idx
-                int lo = 0, hi = side;
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (xpre[mid] <= idx) lo = mid; else hi = mid;
-                }
-                ix = lo;
-                const int r = order - abs(ix - order);
-                int qq = idx - xpre[ix];              // position inside the diamond of radius r
+                // The upper half of the lattice mirrors the lower one.  Radius of the slab: the largest r with
+                // r (2 r^2 + 1) / 3 <= qq; cbrt(1.5 qq) is above it by less than one
+                const bool up = idx >= lower;
+                int qq = up ? total - 1 - idx : idx;
+                int r = (int)exp2f(__log2f(1.5f * (float)qq) * (1.f / 3.f));
+                if (r * (2 * r * r + 1) > 3 * qq) --r;
+                ix = up ? 2 * order - r : r;
+                qq -= r * (2 * r * r + 1) / 3;        // position inside the diamond of radius r
                 // rows ky = -r..0 hold 1, 3, .., 2r+1 points (qq < (r+1)^2, row u has u^2 before it);
                 // rows ky = 1..r mirror rows r-1..0, counted from the end.
                 const bool upper = qq >= (r + 1) * (r + 1);
                 if (upper) qq = 2 * r * r + 2 * r - qq;
-                int u = (int)sqrtf((float)qq);
-                if (u * u > qq) --u;
-                if ((u + 1) * (u + 1) <= qq) ++u;
+                const int u = (int)sqrtf((float)qq + 0.5f);      // (away from whole numbers)
                 ky = upper ? r - u : u - r;
                 kz = qq - u * u - u;
             }
             const int iy = ky + order, iz = kz + order;
             const double d2 = dsq[ix] + dsq[AX + iy] + dsq[2 * AX + iz];
             const float g = gain[ix] * gain[AX + iy] * gain[2 * AX + iz];
-            // 1/d from the fp32 reciprocal square root and one Newton step in fp64
-            // (relative error ~1e-14), d = d2/d with one correction
-            double rd = (double)rsqrtf((float)d2);
-            rd = fma(rd, 0.5 * fma(-d2 * rd, rd, 1.0), rd);
-            double d = d2 * rd;
-            d = fma(0.5 * rd, fma(-d, d, d2), d);
-            const double tau = d * fs_over_c;
-            int n0 = __double2int_rd(tau);
-            phi = (float)(tau - (double)n0);
+            // d from the fp32 reciprocal square root and one Newton step in fp64 (relative error below 1e-13)
+            const float r0 = rsqrtf((float)d2);
+            const double t = d2 * (double)r0, e = fma(-t, (double)r0, 1.0);
+            const double tau = fma(0.5 * t, e, t) * fs_over_c;
+            // its whole part (rounded down): adding 1.5 2^52 leaves the nearest integer in the low word
+            const double m = (tau - 0.5) + 6755399441055744.0;
+            int n0 = __double2loint(m);
+            phi = (float)(tau - (m - 6755399441055744.0));
             if (phi >= 1.f) {                  // rounded up to the next sample
                 ++n0;
                 phi = 0.f;
@@ -233,14 +258,20 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             // away from it the tap is the same to 3e-7 of its size
             phi = fmaxf(phi, 1e-7f);
             n_first = n0 - half_w + 1;
-            const float A = g * (float)rd;
-            valid = d2 > 0.0 && A != 0.f && n_first < L;
+            const float A = g * fmaf(r0, 0.5f * (float)e, r0);
+            valid = d2 > 0.0 && A != 0.f && tau < tau_end;
             // no tap is larger than A
             strong = fabsf(A) * scale >= 4194303.f;
-            const float As = -A * scale * sinpif(phi) * 0.318309886183790671538f;
+            p0 = -0.5f * A * scale * sin_pi_over_pi(phi);
             float sps, cps;
-            sincospif(phi / fhw, &sps, &cps);
-            p0 = 0.5f * As;
+            if constexpr (POLY) {
+                // pi phi / W_h <= 0.08: the series' next terms are below 1e-9
+                const float x = phi * hann, z = x * x;
+                cps = fmaf(z, fmaf(z, 1.f / 24.f, -0.5f), 1.f);
+                sps = fmaf(x * z, fmaf(z, 1.f / 120.f, -1.f / 6.f), x);
+            } else {
+                sincospif(phi / fhw, &sps, &cps);
+            }
             p1 = p0 * cps;
             p2 = p0 * sps;
         }
@@ -272,16 +303,23 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
         const int n_fast = inside == 0 ? 0 : cnt == n_in ? (n_in + 3) & ~3 : n_in & ~3;
         const int n_loud = min((n_strong + 3) & ~3, n_fast);
         auto four = [&](int k, auto loud) {
-            auto taps = [&](u64 ph, u64 q0, u64 q1, u64 q2, int i) {
-                const float2 x = unpack(fma2(nsgn, ph, both(fj[i])));
-                const u64 rx = pack(rcp_approx(x.x), rcp_approx(x.y));
-                const u64 num = fma2(both(sj[i]), q2, fma2(both(cj[i]), q1, q0));
+            auto fixed = [&](u64 x, u64 y) {               // the fixed-point values of x y
                 if constexpr (decltype(loud)::value) {
-                    return round_strong(mul2(rx, num));
+                    return round_strong(mul2(x, y));
                 } else {
-                    const float2 v = unpack(fma2(rx, num, both(TO_INT)));
+                    const float2 v = unpack(fma2(x, y, both(TO_INT)));
                     return make_int2(__float_as_int(v.x) - INT_BITS, __float_as_int(v.y) - INT_BITS);
                 }
+            };
+            auto taps = [&](u64 ph, u64 q0, u64 q1, u64 q2, int i) {
+                const float2 x = unpack(fma2(nsgn, ph, both(fj[i])));
+                return fixed(pack(rcp_approx(x.x), rcp_approx(x.y)), fma2(both(sj[i]), q2, fma2(both(cj[i]), q1, q0)));
+            };
+            auto far = [&](u64 ph, u64 q0, const float *c, int degree) {
+                u64 p = both(c[degree]);
+#pragma unroll
+                for (int i = degree - 1; i >= 0; --i) p = fma2(p, ph, both(c[i]));
+                return fixed(p, q0);
             };
             // every tap of the windows falls inside the response: no index checks, the adds of an image
             // go to fixed offsets from one address
@@ -291,7 +329,14 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             const ulonglong2 q1 = *reinterpret_cast<const ulonglong2 *>(my + R_P1 + k);
             const ulonglong2 q2 = *reinterpret_cast<const ulonglong2 *>(my + R_P2 + k);
             const unsigned a = h_addr + 4u * n.x, b = h_addr + 4u * n.y, c = h_addr + 4u * n.z, d = h_addr + 4u * n.w;
-            const int2 s0 = taps(ph.x, q0.x, q1.x, q2.x, 0), t0 = taps(ph.y, q0.y, q1.y, q2.y, 0);
+            int2 s0, t0;
+            if constexpr (POLY) {
+                s0 = far(ph.x, q0.x, head, 4);
+                t0 = far(ph.y, q0.y, head, 4);
+            } else {
+                s0 = taps(ph.x, q0.x, q1.x, q2.x, 0);
+                t0 = taps(ph.y, q0.y, q1.y, q2.y, 0);
+            }
             red_shared_add<0>(a, s0.x);
             red_shared_add<0>(b, s0.y);
             red_shared_add<0>(c, t0.x);
@@ -301,20 +346,24 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             red_shared_add<128>(b, s1.y);
             red_shared_add<128>(c, t1.x);
             red_shared_add<128>(d, t1.y);
-            if constexpr (NARROW) {
-                // the last 16 taps, lower half-warp: first two images, upper half: the others
-                const int *w = my + k + 2 * (lane >> 4);
-                const int2 m = *reinterpret_cast<const int2 *>(w + R_N);
-                const int2 s2 = taps(*reinterpret_cast<const u64 *>(w + R_PHI), *reinterpret_cast<const u64 *>(w + R_P0),
-                                     *reinterpret_cast<const u64 *>(w + R_P1), *reinterpret_cast<const u64 *>(w + R_P2), 2);
-                red_shared_add<0>(h_rest + 4u * m.x, s2.x);
-                red_shared_add<0>(h_rest + 4u * m.y, s2.y);
-            } else {
-                const int2 s2 = taps(ph.x, q0.x, q1.x, q2.x, 2), t2 = taps(ph.y, q0.y, q1.y, q2.y, 2);
+            if constexpr (WIDTH == WIDE) {
+                const int2 s2 = far(ph.x, q0.x, rest, REST), t2 = far(ph.y, q0.y, rest, REST);
                 red_shared_add<256>(a, s2.x);
                 red_shared_add<256>(b, s2.y);
                 red_shared_add<256>(c, t2.x);
                 red_shared_add<256>(d, t2.y);
+            } else {
+                // the last 16 taps, lower half-warp: first two images, upper half: the others
+                const int *w = my + k + 2 * (lane >> 4);
+                const int2 m = *reinterpret_cast<const int2 *>(w + R_N);
+                const u64 ph2 = *reinterpret_cast<const u64 *>(w + R_PHI), r0 = *reinterpret_cast<const u64 *>(w + R_P0);
+                int2 s2;
+                if constexpr (POLY)
+                    s2 = far(ph2, r0, rest, REST);
+                else
+                    s2 = taps(ph2, r0, *reinterpret_cast<const u64 *>(w + R_P1), *reinterpret_cast<const u64 *>(w + R_P2), 2);
+                red_shared_add<0>(h_rest + 4u * m.x, s2.x);
+                red_shared_add<0>(h_rest + 4u * m.y, s2.y);
             }
         };
 #pragma unroll 1
@@ -328,10 +377,19 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             const float P1 = __int_as_float(my[R_P1 + w]), P2 = __int_as_float(my[R_P2 + w]);
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const float x = fmaf(-sgn, f, fj[i]);
                 const int m = n_f + lane + 32 * i;
-                const float v = rcp_approx(x) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
-                const bool mine = !NARROW || i < 2 || lane < 16;
+                float v;
+                if (POLY && i != 1) {
+                    const float *c = i == 0 ? head : rest;
+                    const int degree = i == 0 ? 4 : REST;
+                    v = c[degree];
+#pragma unroll
+                    for (int k = degree - 1; k >= 0; --k) v = fmaf(v, f, c[k]);
+                    v *= P0;
+                } else {
+                    v = rcp_approx(fmaf(-sgn, f, fj[i])) * fmaf(sj[i], P2, fmaf(cj[i], P1, P0));
+                }
+                const bool mine = WIDTH == WIDE || i < 2 || lane < 16;
                 if (mine && (unsigned)m < (unsigned)L) atomicAdd(&h[m], __float2int_rn(v));
             }
         }
@@ -339,43 +397,112 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
     }
     __syncthreads();
     chain_next();
-    if ((reinterpret_cast<uintptr_t>(out) & 15) == 0 && (L & 3) == 0) {
-        for (int i = tid; i < (L >> 2); i += THREADS) {
+    const bool vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0 && (L & 3) == 0;
+    int end = L;                               // taps to be written
+    if (leff != nullptr) {
+        int last = 0;
+        for (int i = tid; i < ((L + 3) >> 2); i += THREADS) {
+            const int4 q = reinterpret_cast<const int4 *>(h)[i];       // (behind the end of the buffer: zeros)
+            if ((q.x | q.y | q.z | q.w) != 0) last = 4 * i + (q.w ? 4 : q.z ? 3 : q.y ? 2 : 1);
+        }
+        last = __reduce_max_sync(0xffffffffu, last);
+        if (lane == 0) ring[warp] = last;
+        __syncthreads();
+        end = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) end = max(end, ring[w]);
+    }
+    if (vec) {
+        for (int i = tid; i < ((end + 3) >> 2); i += THREADS) {
             const int4 q = reinterpret_cast<const int4 *>(h)[i];
             reinterpret_cast<float4 *>(out)[i] = make_float4((float)q.x * inv_scale, (float)q.y * inv_scale,
                                                              (float)q.z * inv_scale, (float)q.w * inv_scale);
         }
     } else {
-        for (int i = tid; i < L; i += THREADS) out[i] = (float)h[i] * inv_scale;
+        for (int i = tid; i < end; i += THREADS) out[i] = (float)h[i] * inv_scale;
     }
     chain_wait();
+    if (leff != nullptr && tid == 0) {
+        leff[utt * S_max + s] = end;
+        if (leff_all != nullptr) atomicMax(leff_all, end);
+    }
 }
 
 }  // namespace
 
-template <int THREADS>
-static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
+// Constants of the taps, a row of 32 lanes each; lane l's taps are jj = l, l + 32 and l + 64 (half width 40 and
+// below: 64 + l mod 16), tap jj lies at offset j = jj - W + 1 from n0.  The sign (-1)^j (with that of the sine) is the
+// same for all taps of a lane.  Reciprocal form: the signed offset, whose reciprocal is taken, cosine and sine of the
+// Hann angle; a tap beyond the window gets an offset so large that its value rounds to zero.  Polynomials: the
+// coefficients of (1 + cos(pi (j - phi) / W)) / (j - phi) in powers of phi, which interpolate it at the Chebyshev
+// points of 0 <= phi <= 1.  In double, once per context: every warp of the kernel working them out took a tenth of its
+// time (4096 x 2 responses of order 8).
+//   W < 40   three rows for each of the lane's taps
+//   W >= 40  three rows for the middle one, five for the first, five for the last (W = 40: four used)
+void rir_tap_table(int W, float *tab) {
+    const double PI = 3.14159265358979323846;
+    auto reciprocal = [&](int row, int lane, int jj) {
+        const int j = jj - W + 1;
+        const double sgn = ((lane - W + 1) & 1) ? -1.0 : 1.0;
+        tab[32 * row + lane] = jj < 2 * W ? (float)(sgn * j) : 3e18f;
+        tab[32 * (row + 1) + lane] = (float)cos(PI * j / W);
+        tab[32 * (row + 2) + lane] = (float)sin(PI * j / W);
+    };
+    auto polynomial = [&](int row, int lane, int jj, int degree) {
+        const int j = jj - W + 1, n = degree + 1;
+        double x[5], d[5], c[5] = {0, 0, 0, 0, 0};
+        for (int i = 0; i < n; ++i) {                       // divided differences, then powers
+            x[i] = 0.5 + 0.5 * cos(PI * (2 * i + 1) / (2 * n));
+            d[i] = (1.0 + cos(PI * (j - x[i]) / W)) / (j - x[i]);
+        }
+        for (int k = 1; k < n; ++k)
+            for (int i = n - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
+        for (int k = n - 1; k >= 0; --k) {
+            for (int i = n - 1; i > 0; --i) c[i] = c[i - 1] - x[k] * c[i];
+            c[0] = d[k] - x[k] * c[0];
+        }
+        const double sgn = jj >= 2 * W ? 0.0 : ((lane - W + 1) & 1) ? -1.0 : 1.0;
+        for (int i = 0; i < n; ++i) tab[32 * (row + i) + lane] = (float)(sgn * c[i]);
+    };
+    for (int lane = 0; lane < 32; ++lane) {
+        if (W < 40) {
+            for (int i = 0; i < 3; ++i) reciprocal(3 * i, lane, i < 2 ? lane + 32 * i : 64 + (lane & 15));
+        } else {
+            reciprocal(0, lane, lane + 32);
+            polynomial(3, lane, lane, 4);
+            polynomial(8, lane, W == 40 ? 64 + (lane & 15) : 64 + lane, W == 40 ? 3 : 4);
+        }
+    }
+}
+
+template <Width WIDTH, int THREADS>
+static int launch_rir_kernel(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool chained) {
     const AugConfig &c = ctx->cfg;
     const size_t smem = rir_smem_bytes(THREADS, c.rir_taps);
     const double fs_over_c = (double)c.fs / (double)c.sound_speed;
     const int cube = c.image_lattice == AUG_LATTICE_CUBE ? 1 : 0;
     dim3 grid(c.max_sources, B);
-    const bool narrow = c.frac_half_width <= 40;
-    auto kern = narrow ? rir_image_kernel<true, THREADS> : rir_image_kernel<false, THREADS>;
-    if ((narrow ? smem_opt_in<rir_image_kernel<true, THREADS>>(ctx->device)
-                : smem_opt_in<rir_image_kernel<false, THREADS>>(ctx->device)) != AUG_OK)
-        return AUG_ECUDA;
-    if (beside) {
+    auto kern = rir_image_kernel<WIDTH, THREADS>;
+    if (smem_opt_in<rir_image_kernel<WIDTH, THREADS>>(ctx->device) != AUG_OK) return AUG_ECUDA;
+    if (chained) {
+        int *leff_all = ctx->route == aug::ROUTE_STORED ? ctx->counters + aug::LEFF_ALL : nullptr;
         if (launch_chained(kern, grid, THREADS, smem, ctx->stream, table, c.max_sources, c.rir_taps, c.frac_half_width,
-                           fs_over_c, c.max_order, cube, rir, ctx->status) != AUG_OK)
+                           fs_over_c, c.max_order, cube, ctx->tap_tab, rir, ctx->status, ctx->leff, leff_all) != AUG_OK)
             return AUG_ECUDA;
     } else {
         kern<<<grid, THREADS, smem, ctx->stream>>>(table, c.max_sources, c.rir_taps, c.frac_half_width, fs_over_c,
-                                                   c.max_order, cube, rir, ctx->status);
+                                                   c.max_order, cube, ctx->tap_tab, rir, ctx->status, nullptr, nullptr);
         AUG_CUDA_OK(cudaGetLastError());
     }
     ctx->launches++;
     return AUG_OK;
+}
+template <int THREADS>
+static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool chained) {
+    const int w = ctx->cfg.frac_half_width;
+    return w < 40    ? launch_rir_kernel<SHORT, THREADS>(ctx, table, B, rir, chained)
+           : w == 40 ? launch_rir_kernel<FORTY, THREADS>(ctx, table, B, rir, chained)
+                     : launch_rir_kernel<WIDE, THREADS>(ctx, table, B, rir, chained);
 }
 
 // Both sizes keep 32 warps with 64 registers on a multiprocessor.  Two CTAs of 512 threads are better
@@ -386,7 +513,7 @@ static int launch_rir_as(AugCtx *ctx, const AugUttParams *table, int B, float *r
 // utterance, at most max_sources.  With so few
 // images that eight warps do them in one pass the first round is mostly set-up, and four CTAs are
 // taken as soon as there may be more than one (300 of 1600 taps, order 4: 13.0 against 8.9).
-int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool beside) {
+int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool chained) {
     const AugConfig &c = ctx->cfg;
     const bool fit = 4 * (rir_smem_bytes(256, c.rir_taps) + 1024) <= (size_t)ctx->smem_per_sm;
     const int side = 2 * c.max_order + 1;
@@ -394,5 +521,5 @@ int launch_rir(AugCtx *ctx, const AugUttParams *table, int B, float *rir, bool b
                                                            : side * (2 * c.max_order * (c.max_order + 1) + 3) / 3;
     const int64_t most = (int64_t)B * c.max_sources, round = 2 * (int64_t)ctx->sm_count;
     const bool many = B > round || most >= 2 * round || (images <= 256 && most > round);
-    return fit && many ? launch_rir_as<256>(ctx, table, B, rir, beside) : launch_rir_as<512>(ctx, table, B, rir, beside);
+    return fit && many ? launch_rir_as<256>(ctx, table, B, rir, chained) : launch_rir_as<512>(ctx, table, B, rir, chained);
 }
