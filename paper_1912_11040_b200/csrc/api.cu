@@ -237,11 +237,11 @@ int run_pipeline(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     t0(5);
     const bool on_the_way = features_write_wave(ctx, max_len, T_max);   // the feature kernel writes the waveform too
     if (wave_out && !on_the_way &&
-        (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out, speech_stride)) != AUG_OK)
+        (rc = launch_mix(ctx, lengths_dev, table_dev, B, max_len, false, wave_out, speech_stride)) != AUG_OK)
         return rc;
     t1(5);
     t0(6);
-    rc = launch_fused_features(ctx, lengths_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
+    rc = launch_fused_features(ctx, lengths_dev, table_dev, B, feats_dev, T_max, frame_counts_dev, max_len,
                                on_the_way ? wave_out : nullptr, speech_stride);
     t1(6);
     if (ev && rc == AUG_OK) ctx->ev_n++;
@@ -520,7 +520,8 @@ int aug_reverb_mix(AugCtx *ctx, const float *speech_dev, int64_t speech_stride,
     if ((rc = launch_rir_spectra(ctx, rir_dev, in, table_dev, B, false)) != AUG_OK) return rc;
     if ((rc = launch_convolve_prepare(ctx, in, table_dev, B, false)) != AUG_OK) return rc;
     if ((rc = launch_convolve_finish(ctx, in, table_dev, B)) != AUG_OK) return rc;
-    return launch_mix(ctx, lengths_dev, table_dev, B, max_len, wave_out_dev, speech_stride);
+    if ((rc = launch_snr_gain(ctx, table_dev, B)) != AUG_OK) return rc;
+    return launch_mix(ctx, lengths_dev, table_dev, B, max_len, true, wave_out_dev, speech_stride);
 }
 
 int feat_stft_power(AugCtx *ctx, const float *wave_dev, int64_t stride, const int *lengths_dev,

@@ -156,6 +156,24 @@ inline int launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t sme
 }
 #endif
 
+// Where a kernel gets the noise gain from: worked out before (value), or from the two sums of the convolution.
+struct GainSource {
+    const float *value;             // [B], or NULL
+    const double *energy;           // [B][2]
+    const AugUttParams *table;
+};
+#ifdef __CUDACC__
+// g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise, with a silent side or with noise that is not
+// finite, in fp64; `ratio` is 10^(snr/10).  -0 tells the feature kernel that v, though weighted by zero, is
+// not silence (it may not be finite).
+__device__ __forceinline__ bool snr_noisy(double es, double ev, int n_src) { return n_src > 1 && es > 0.0 && ev > 0.0; }
+__device__ __forceinline__ float snr_gain(double es, double ev, double ratio, int n_src) {
+    const float g = snr_noisy(es, ev, n_src) ? (float)sqrt(es / (ev * ratio)) : 0.f;
+    return g == 0.f && ev != 0.0 ? -0.f : g;
+}
+__device__ __forceinline__ double snr_ratio(const AugUttParams &row) { return exp10((double)row.snr_db / 10.0); }
+#endif
+
 // What the convolution reads besides the responses; samples beyond max_len of a row are not used.
 struct ConvInput {
     const float *speech;
@@ -180,7 +198,9 @@ int launch_rir_spectra(AugCtx *ctx, const float *rir, const ConvInput &in, const
 // partition spectra of the impulse responses.
 int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B, bool measured);
 int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B);
-int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
+int launch_snr_gain(AugCtx *ctx, const AugUttParams *table, int B);
+// `ready`: launch_snr_gain has been called
+int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len, bool ready,
                float *wave_out, int64_t out_stride);
 int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset);
 int launch_vtlp_resynth(AugCtx *ctx, const float *speech, int64_t stride, const int *lengths,
@@ -190,5 +210,5 @@ int launch_stft_power(AugCtx *ctx, const float *wave, int64_t stride, const int 
 int launch_logmel(AugCtx *ctx, const float *power, const int *counts, int B, int T_max,
                   float *feats);
 bool features_write_wave(const AugCtx *ctx, int max_len, int T_max);
-int launch_fused_features(AugCtx *ctx, const int *lengths, int B, float *feats, int T_max, int *counts,
-                          int max_len, float *wave, int64_t wave_stride);
+int launch_fused_features(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, float *feats, int T_max,
+                          int *counts, int max_len, float *wave, int64_t wave_stride);

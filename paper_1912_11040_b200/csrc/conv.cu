@@ -103,24 +103,16 @@ rir_length_kernel(const float *rir, const AugUttParams *__restrict__ table, int 
 __device__ __forceinline__ bool takes_fused_route(int leff_batch) { return leff_batch <= aug::CONV_TAPS; }
 
 // ---------------------------------------------------------------- mixing
-// g = sqrt(sum y_s^2 / (sum v^2 10^(snr/10))), 0 without noise, with a silent side or with noise that is
-// not finite: once per utterance, in fp64, after the convolution has finished the two sums.  (Worked out by
-// every feature CTA instead, the chain of fp64 operations cost 13 us on 256 utterances of
-// 2-20 s where this launch costs 2.6; by the last CTA of the convolution, the fence it needs
-// cost as much.)
+// The gain once per utterance, ahead of a mix of its own (aug_reverb_mix), whose many short CTAs would each go
+// through the chain of fp64 operations; the feature kernel works it out while its first samples are on their way.
 __global__ void __launch_bounds__(256)
 snr_gain_kernel(const double *energy, const AugUttParams *__restrict__ table, int B,
                 float *__restrict__ gain) {
     const int utt = blockIdx.x * 256 + threadIdx.x;
+    const double ratio = utt < B ? snr_ratio(table[utt]) : 1.0;
     chain_next();
     chain_wait();
-    if (utt >= B) return;
-    const double es = energy[2 * utt], ev = energy[2 * utt + 1];
-    float g = 0.f;
-    if (table[utt].n_src > 1 && es > 0.0 && ev > 0.0)
-        g = (float)sqrt(es / (ev * exp10((double)table[utt].snr_db / 10.0)));
-    // -0 tells the feature kernel that v, though weighted by zero, is not silence (it may not be finite)
-    gain[utt] = g == 0.f && ev != 0.0 ? -0.f : g;
+    if (utt < B) gain[utt] = snr_gain(energy[2 * utt], energy[2 * utt + 1], ratio, table[utt].n_src);
 }
 
 // A pass over y_s and v, bound by memory: 4096 samples per CTA, eight 128-bit loads in flight per
@@ -128,7 +120,7 @@ snr_gain_kernel(const double *energy, const AugUttParams *__restrict__ table, in
 constexpr int MIX_GROUPS = 4;              // 128-bit groups per thread
 __global__ void __launch_bounds__(256)
 mix_kernel(const float *ys, const float *vv, int64_t ws_stride,
-           const float *gain, const int *__restrict__ lengths,
+           const GainSource gain, const int *__restrict__ lengths,
            float *__restrict__ out, int64_t out_stride, int n_cap) {
     const int utt = blockIdx.y, tid = threadIdx.x;
     chain_wait();
@@ -147,7 +139,10 @@ mix_kernel(const float *ys, const float *vv, int64_t ws_stride,
             y[u] = *reinterpret_cast<const float4 *>(b + i);
         }
     }
-    const float g = fabsf(gain[utt]);
+    const float g = fabsf(gain.value != nullptr
+                              ? gain.value[utt]
+                              : snr_gain(gain.energy[2 * utt], gain.energy[2 * utt + 1], snr_ratio(gain.table[utt]),
+                                         gain.table[utt].n_src));
 #pragma unroll
     for (int u = 0; u < MIX_GROUPS; ++u) {
         const int i = i0 + 1024 * u;
@@ -975,6 +970,10 @@ int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams 
             AUG_CUDA_OK(cudaMemcpyAsync(ctx->leff_seen, ctx->counters + aug::LEFF_ALL, sizeof(int), cudaMemcpyDeviceToHost,
                                         ctx->stream));
     }
+    return AUG_OK;
+}
+
+int launch_snr_gain(AugCtx *ctx, const AugUttParams *table, int B) {
     if (launch_chained(snr_gain_kernel, dim3((B + 255) / 256), 256, 0, ctx->stream, ctx->energy, table, B, ctx->gain) !=
         AUG_OK)
         return AUG_ECUDA;
@@ -982,11 +981,12 @@ int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams 
     return AUG_OK;
 }
 
-int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len,
+int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, int max_len, bool ready,
                float *wave_out, int64_t out_stride) {
     if (max_len <= 0) return AUG_OK;
     dim3 grid((max_len + MIX_GROUPS * 1024 - 1) / (MIX_GROUPS * 1024), B);
-    if (launch_chained(mix_kernel, grid, 256, 0, ctx->stream, ctx->ys, ctx->vv, ctx->ws_stride, ctx->gain, lengths,
+    const GainSource gain = {ready ? ctx->gain : nullptr, ctx->energy, table};
+    if (launch_chained(mix_kernel, grid, 256, 0, ctx->stream, ctx->ys, ctx->vv, ctx->ws_stride, gain, lengths,
                        wave_out, out_stride, max_len) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;

@@ -240,7 +240,7 @@ Layout make_layout(int win_len, int hop, int M, Staging staging) {
     l.lanes = take(4 * 32);
     l.mw = take(MODE == 1 ? 4 * (K / 2 + 1) : 0);
     l.mst = take(MODE == 1 ? M + 2 : 0);
-    l.cut = take(MODE == 1 ? 64 : 0);
+    l.cut = take(MODE == 1 ? 64 : 0);            // (the last one: the gain)
     l.total = o;
     return l;
 }
@@ -335,7 +335,7 @@ __device__ __forceinline__ void power_rows(fftpair::C2 *v, fftpair::u64 *p, cons
 
 template <int K, int MODE, int TILES>
 __global__ void __launch_bounds__(FEAT_THREADS, 2)
-frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const float *gain,
+frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const GainSource gain,
               const int *__restrict__ lengths, int win, int hop, int M, int T_max, const aug::MelBin *__restrict__ melw,
               const int *__restrict__ melstart, const float2 *__restrict__ tw, float floor_v, float pad_v, int comp,
               float *__restrict__ out, int *__restrict__ counts, int n_cap, float *__restrict__ wave, int64_t wave_stride,
@@ -354,28 +354,37 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
         const float2 w1 = __ldg(&tw[256 + tid]), wh = tid < 16 ? make_float2(1.f, 0.f) : __ldg(&tw[tid]);
         reinterpret_cast<float4 *>(sm + lay.lanes)[tid] = make_float4(w1.x, w1.y, wh.x, wh.y);
     }
-    chain_wait();
     const int N = min(max(lengths[utt], 0), n_cap);
     const int T = min(frame_count(N, win, hop), T_max);
     if (blockIdx.x == 0 && tid == 0) counts[utt] = T;
+    const int rows = min(FT * TILES, T_max - run0);
+    const int nfr = max(0, min(FT * TILES, T - run0));
+    const int out_w = MODE == 0 ? NBP : M;
+    float *orun = out + ((int64_t)utt * T_max + run0) * out_w;
+    if (rows > nfr)
+        fill_floats(orun + (int64_t)nfr * out_w, (rows - nfr) * out_w, MODE == 0 ? 0.f : pad_v, tid, FEAT_THREADS);
+    // The gain is one thread's work, done while the first tile's samples travel.
+    const bool gains = MODE == 1 && tid == FEAT_THREADS - 1;
+    const double ratio = gains ? snr_ratio(gain.table[utt]) : 1.0;
+    const int n_src = MODE == 1 ? gain.table[utt].n_src : 0;
+    chain_wait();
+    double es = 0.0, ev = 0.0;
+    if (MODE == 1) {
+        es = gain.energy[2 * utt];
+        ev = gain.energy[2 * utt + 1];
+    }
+    float g = 0.f, *gain_s = sm + lay.cut + 63;
+    const bool noisy = MODE == 1 && snr_noisy(es, ev, n_src);
     // The mixed waveform, where it is wanted: a tile writes the hops that its frames start, the CTA with
     // the last frame (the first one if there is none) what lies behind them.
     float *wrow = MODE == 1 && wave != nullptr ? wave + (int64_t)utt * wave_stride : nullptr;
     if (MODE == 1 && wrow != nullptr && run0 <= max(T - 1, 0) && run0 + FT * TILES > max(T - 1, 0)) {
-        const float gw = fabsf(gain[utt]);
+        const float gw = fabsf(snr_gain(es, ev, snr_ratio(gain.table[utt]), n_src));
         const float *wa = in_a + (int64_t)utt * in_stride, *wb = in_b + (int64_t)utt * in_stride;
         for (int i = T * hop + tid; i < N; i += FEAT_THREADS) wrow[i] = fmaf(gw, wb[i], wa[i]);
     }
-    const int rows = min(FT * TILES, T_max - run0);
-    if (rows <= 0) return;
-    const int nfr = max(0, min(FT * TILES, T - run0));
-    const int out_w = MODE == 0 ? NBP : M;
-    float *orun = out + ((int64_t)utt * T_max + run0) * out_w;
-    fill_floats(orun + (int64_t)nfr * out_w, (rows - nfr) * out_w, MODE == 0 ? 0.f : pad_v, tid, FEAT_THREADS);
     if (nfr == 0) return;
 
-    const float g = MODE == 1 ? gain[utt] : 0.f;
-    const bool noisy = g != 0.f;
     const float *ra = in_a + (int64_t)utt * in_stride;
     const float *rb = MODE == 1 ? in_b + (int64_t)utt * in_stride : nullptr;
     const int n_tiles = min(TILES, (nfr + FT - 1) / FT);
@@ -467,6 +476,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
 
     constexpr int RUNS = 2 * FEAT_THREADS / FT;       // runs of bands, one per FT / 2 lanes
     if (MODE == 1) {
+        if (gains) *gain_s = snr_gain(es, ev, ratio, n_src);
         for (int k = tid; k < NBP; k += FEAT_THREADS) {
             const aug::MelBin w = melw[(int64_t)utt * NBP + k];
             mw[k] = make_float4(w.up, w.up, w.down, w.down);
@@ -474,6 +484,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
         for (int m = tid; m < M + 2; m += FEAT_THREADS) mst[m] = melstart[(int64_t)utt * (M + 2) + m];
         __syncthreads();
         cut_bands<RUNS>(cut, mst, M, tid);
+        g = *gain_s;
     }
     fftpair::u64 *xb = reinterpret_cast<fftpair::u64 *>(sm + warp * SPAN);
 
@@ -497,7 +508,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const flo
             const bool vec = ((hop | (int)wave_stride) & 3) == 0 && (reinterpret_cast<uintptr_t>(wave) & 15) == 0;
             const float *pa = ra + t0 * hop, *pb = rb + t0 * hop;
             if (__float_as_int(g) < 0) {
-                // -0, see snr_gain_kernel: noise that is not finite shows in the waveform, though the features
+                // -0, see snr_gain: noise that is not finite shows in the waveform, though the features
                 // (of y_s alone) never read it.  (Done for every utterance without noise it cost 4 % of 96
                 // utterances of 2-20 s.)
                 if (vec) {
@@ -680,7 +691,7 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
 
 template <int K, int MODE>
 int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, const int *lengths,
-                  int B, float *out, int T_max, int *counts, int n_cap, float *wave = nullptr,
+                  const AugUttParams *table, int B, float *out, int T_max, int *counts, int n_cap, float *wave = nullptr,
                   int64_t wave_stride = 0) {
     const AugConfig &c = ctx->cfg;
     constexpr int FT = tile_frames<K>(), RUN_TILES = Plan<K>::TILES;
@@ -708,15 +719,16 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
     if ((runs ? smem_opt_in<frames_kernel<K, MODE, RUN_TILES>>(ctx->device)
               : smem_opt_in<frames_kernel<K, MODE, 1>>(ctx->device)) != AUG_OK)
         return AUG_ECUDA;
+    const GainSource gain = {nullptr, ctx->energy, table};
     // (MODE 0 reads what the caller's kernels wrote: launched the ordinary way)
     if (MODE == 1) {
-        if (launch_chained(kern, grid, FEAT_THREADS, smem, ctx->stream, a, b, stride, ctx->gain, lengths, c.win, c.hop,
+        if (launch_chained(kern, grid, FEAT_THREADS, smem, ctx->stream, a, b, stride, gain, lengths, c.win, c.hop,
                            c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw, c.log_floor, c.pad_value, c.compression,
                            out, counts, n_cap, wave, wave_stride, lay) != AUG_OK)
             return AUG_ECUDA;
     } else {
         kern<<<grid, FEAT_THREADS, smem, ctx->stream>>>(
-            a, b, stride, ctx->gain, lengths, c.win, c.hop, c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw,
+            a, b, stride, gain, lengths, c.win, c.hop, c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw,
             c.log_floor, c.pad_value, c.compression, out, counts, n_cap, wave, wave_stride, lay);
         AUG_CUDA_OK(cudaGetLastError());
     }
@@ -741,8 +753,8 @@ int launch_stft_power(AugCtx *ctx, const float *wave, int64_t stride, const int 
     if (T_max <= 0) return AUG_OK;
     const int n_cap = (int)(stride < 0x7fffffff ? stride : 0x7fffffff);     // the caller's rows end at their stride
     if (ctx->cfg.n_fft == 512)
-        return launch_frames<512, 0>(ctx, wave, nullptr, stride, lengths, B, power, T_max, counts, n_cap);
-    return launch_frames<1024, 0>(ctx, wave, nullptr, stride, lengths, B, power, T_max, counts, n_cap);
+        return launch_frames<512, 0>(ctx, wave, nullptr, stride, lengths, nullptr, B, power, T_max, counts, n_cap);
+    return launch_frames<1024, 0>(ctx, wave, nullptr, stride, lengths, nullptr, B, power, T_max, counts, n_cap);
 }
 
 // max_len: the length clamp the convolution used, so that every stage cuts an over-long
@@ -756,13 +768,13 @@ constexpr int WAVE_SLACK = 8;
 bool features_write_wave(const AugCtx *ctx, int max_len, int T_max) {
     return ctx->cfg.hop <= ctx->cfg.win && frame_count(max_len, ctx->cfg.win, ctx->cfg.hop) <= (int64_t)T_max + WAVE_SLACK;
 }
-int launch_fused_features(AugCtx *ctx, const int *lengths, int B, float *feats, int T_max, int *counts,
-                          int max_len, float *wave, int64_t wave_stride) {
+int launch_fused_features(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B, float *feats, int T_max,
+                          int *counts, int max_len, float *wave, int64_t wave_stride) {
     if (T_max <= 0) return AUG_OK;
     if (ctx->cfg.n_fft == 512)
-        return launch_frames<512, 1>(ctx, ctx->ys, ctx->vv, ctx->ws_stride, lengths, B, feats, T_max, counts, max_len,
+        return launch_frames<512, 1>(ctx, ctx->ys, ctx->vv, ctx->ws_stride, lengths, table, B, feats, T_max, counts, max_len,
                                      wave, wave_stride);
-    return launch_frames<1024, 1>(ctx, ctx->ys, ctx->vv, ctx->ws_stride, lengths, B, feats, T_max, counts, max_len,
+    return launch_frames<1024, 1>(ctx, ctx->ys, ctx->vv, ctx->ws_stride, lengths, table, B, feats, T_max, counts, max_len,
                                   wave, wave_stride);
 }
 
