@@ -107,7 +107,7 @@ int check_config(const AugConfig *c) {
 
 struct Layout {
     int n_part, route, n_bins, t_cap, nblk_cap;
-    int64_t ws_stride;
+    int64_t ws_stride, unit_cap;
     int64_t off_xspec, off_park, off_park_flags, off_plans, off_units;
     int64_t off_tw, off_tap_tab, off_rir, off_hspec, off_ys, off_vv, off_energy, off_arrived, off_counters, off_leff, off_gain, off_melw, off_melstart,
         off_status, off_warped, off_vtlp_tab, off_st_speech, off_st_bank, off_st_table, off_st_lengths,
@@ -136,7 +136,8 @@ Layout make_layout(const AugConfig &c) {
     l.off_park_flags = parks ? take(sizeof(int) * aug::PARK_SLOTS) : -1;
     // its list of work: two outputs of every block, blocks as short as 8192 taps make them
     l.off_plans = take((int64_t)aug::PLAN_BYTES * B);
-    l.off_units = take(2 * sizeof(int) * 2 * B * ((c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS));
+    l.unit_cap = 2 * B * ((c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS);
+    l.off_units = take(2 * sizeof(int) * l.unit_cap);
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take((sizeof(double) * 2 + sizeof(unsigned long long)) * B + sizeof(int) * aug::N_COUNTERS);
@@ -351,6 +352,7 @@ int aug_create(AugCtx **out, const AugConfig *cfg, void *cuda_stream) {
     ctx->park_flags = l.off_park_flags >= 0 ? reinterpret_cast<int *>(base + l.off_park_flags) : nullptr;
     ctx->plans = base + l.off_plans;
     ctx->units = base + l.off_units;
+    ctx->unit_cap = (int)l.unit_cap;
     ctx->ys = reinterpret_cast<float *>(base + l.off_ys);
     ctx->vv = reinterpret_cast<float *>(base + l.off_vv);
     ctx->energy = reinterpret_cast<double *>(base + l.off_energy);

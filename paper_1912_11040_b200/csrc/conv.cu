@@ -383,6 +383,12 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
 // know; the convolving kernels' CTAs, as many as fit the device, work through the list.  With one CTA
 // per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
 // (two thirds of them without work) and to each one's chain of loads before its first sample.
+//
+// Sums of several noise sources are the heavy units (three transforms and more against two): they are
+// listed from the front, the others from the back, so that the heavy ones are drawn first and none of them is the last
+// that the device waits for (in the order in which they are planned, and so: 64 utterances of 2-16 s, one or two noises,
+// 167 and 153 us; 96 of 2-20 s with up to two 302 and 287; 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and
+// 1376, whole calls each).
 struct Plan {
     const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
     int nlen[AUG_S_MAX];           // their lengths ([0] unused)
@@ -410,6 +416,7 @@ struct PlanArgs {
     int *status;
     Plan *plans;
     Unit *units;
+    int unit_cap;
     int *counters;                 // [N_COUNTERS]
 };
 // By one warp; leff: taps up to the last non-zero one.
@@ -419,8 +426,8 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttPa
     // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
     // of 4, where taps counts up to the last non-zero tap of this utterance's responses
     const int ob = stored ? BLK2 : (F2 - min(max(leff, 1), BLK2) + 1) & ~3;
-    const int n = 2 * ((N + ob - 1) / ob);
-    int at = 0;
+    const int n = (N + ob - 1) / ob;
+    int at = 0, at_heavy = -1;
     if (lane == 0) {
         Plan p;
         p.N = N;
@@ -444,10 +451,20 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttPa
             }
         }
         a.plans[utt] = p;
-        if (n > 0) at = atomicAdd(a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED), n);
+        if (n > 0) {
+            int *list = a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED);
+            const bool heavy = p.n_noise > 1;
+            if (heavy) at_heavy = atomicAdd(list, n);
+            at = atomicAdd(list + 1, heavy ? n : 2 * n);
+        }
     }
     at = __shfl_sync(0xffffffffu, at, 0);
-    for (int i = lane; i < n; i += 32) a.units[at + i] = Unit{utt, i};
+    at_heavy = __shfl_sync(0xffffffffu, at_heavy, 0);
+    const int last = a.unit_cap - 1;
+    for (int i = lane; i < n; i += 32) {
+        a.units[last - at - i] = Unit{utt, 2 * i};
+        a.units[at_heavy >= 0 ? at_heavy + i : last - at - n - i] = Unit{utt, 2 * i + 1};
+    }
 }
 
 // The same with the lengths in global memory.
@@ -611,7 +628,7 @@ enum Kind { FUSED, SPECTRA, STORED };
 
 template <Kind KIND, bool PARK>
 __global__ void __launch_bounds__(CF, FUSED_MINB)
-convolve_kernel(const Plan *plans, const Unit *units, const int *n_units,
+convolve_kernel(const Plan *plans, const Unit *units, const int *n_units, int unit_cap,
                 int *drawn, int S_max, int P, const float4 *hspec, float4 *__restrict__ xspec,
                 int nblk_cap, const float2 *__restrict__ tw, float *__restrict__ ys, float *__restrict__ vv,
                 int64_t ws_stride, double *__restrict__ energy, float4 *__restrict__ park,
@@ -632,14 +649,19 @@ convolve_kernel(const Plan *plans, const Unit *units, const int *n_units,
     const int t = threadIdx.x, G = gridDim.x;
     fftpair::fill_tables(sh, t, tw);
     chain_wait();
-    // (the list has room for every CTA's first unit: it is read beside the count)
-    // STORED goes through the list backwards: the spectra that SPECTRA wrote last are still in L2
+    // (a CTA's first unit, which mostly is one of two, is read beside the counts)
+    // SPECTRA goes through the list backwards: the spectra that it writes last are still in L2 when STORED starts
     // (128 x 8 s, four sources: 250 -> 246 us).
-    const Unit first_of_list = units[blockIdx.x];
-    const int count = *n_units;
+    const Unit front = units[blockIdx.x], back = units[unit_cap - 1 - blockIdx.x];
+    const int heavy = n_units[0], count = heavy + n_units[1];
     if (blockIdx.x >= count) return;
-    auto unit_at = [&](int i) { return units[KIND == STORED ? count - 1 - i : i]; };
-    const Unit first = KIND == STORED ? unit_at(blockIdx.x) : first_of_list;
+    auto unit_at = [&](int i) {
+        if (KIND == SPECTRA) i = count - 1 - i;
+        return units[i < heavy ? i : unit_cap - 1 - (i - heavy)];
+    };
+    const Unit first = KIND != SPECTRA && blockIdx.x < heavy ? front
+                       : KIND != SPECTRA && heavy == 0       ? back
+                                                             : unit_at(blockIdx.x);
     if (t == 32) {
         const int second = blockIdx.x + G;
         unit_s[0] = first;
@@ -882,7 +904,7 @@ static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_ST
 
 static PlanArgs plan_args(const AugCtx *ctx, const ConvInput &in) {
     return {in.speech, in.stride, in.lengths, in.bank, in.bank_len, in.max_len, ctx->status,
-            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units), ctx->counters};
+            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units), ctx->unit_cap, ctx->counters};
 }
 
 template <Lengths LENGTHS>
@@ -925,7 +947,7 @@ static int launch_convolve(AugCtx *ctx, int grid) {
     const int drawn = KIND == FUSED ? aug::DRAWN_FUSED : KIND == SPECTRA ? aug::DRAWN_SPECTRA : aug::DRAWN_STORED;
     if (launch_chained(convolve_kernel<KIND, PARK>, dim3(grid), CF, FFT2_SMEM, ctx->stream,
                        reinterpret_cast<const Plan *>(ctx->plans), reinterpret_cast<const Unit *>(ctx->units),
-                       counters + list, counters + drawn, c.max_sources, ctx->n_part,
+                       counters + list, ctx->unit_cap, counters + drawn, c.max_sources, ctx->n_part,
                        reinterpret_cast<const float4 *>(ctx->hspec), reinterpret_cast<float4 *>(ctx->xspec),
                        ctx->nblk_cap, ctx->tw, ctx->ys, ctx->vv, ctx->ws_stride, ctx->energy, ctx->park,
                        ctx->park_flags) != AUG_OK)
