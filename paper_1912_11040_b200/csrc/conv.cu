@@ -389,6 +389,11 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
 // that the device waits for (in the order in which they are planned, and so: 64 utterances of 2-16 s, one or two noises,
 // 167 and 153 us; 96 of 2-20 s with up to two 302 and 287; 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and
 // 1376, whole calls each).
+//
+// A stretch of noise that is shorter than the utterance repeats, and so does its reverberation as soon as the
+// response has run in: v[n + P] = v[n], n >= taps - 1.  Where there is one noise source, only the blocks
+// up to P + taps - 1 are listed, and those that hold the last period also write it wherever it comes back (4096
+// utterances of 1-6 s, stretches of half to all of their length: convolution 1694 us, so 1585).
 struct Plan {
     const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
     int nlen[AUG_S_MAX];           // their lengths ([0] unused)
@@ -398,6 +403,7 @@ struct Plan {
     int N;                         // samples of the utterance
     int ob;                        // outputs per block
     int parts;                     // partitions that are not zero throughout (stored-spectra route)
+    int period, copy_from;         // v from copy_from on comes back every `period` samples up to the end (0: all of it is computed)
 };
 struct Unit {
     int utt;
@@ -419,72 +425,91 @@ struct PlanArgs {
     int unit_cap;
     int *counters;                 // [N_COUNTERS]
 };
+// What planning reads of the caller's inputs: lane l the length of the utterance and source l (0: the speech) of its row.
+// (Read, where the responses are made by the kernel before, ahead of the wait for it.)
+struct PlanInput {
+    int N, n_src;                  // n_src 0: the row was rejected (reported by step 1)
+    const float *x;                // NULL: the stretch is unusable
+    int nlen;
+};
+__device__ __forceinline__ PlanInput plan_input(const PlanArgs &a, const AugUttParams &row, int utt, int S_max, int lane) {
+    PlanInput in;
+    in.N = min(max(a.lengths[utt], 0), a.n_cap);
+    in.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;
+    in.x = nullptr;
+    in.nlen = 0;
+    if (lane < max(in.n_src, 1) && !source_of(row, lane, a.speech + (int64_t)utt * a.stride, a.bank, a.bank_len, in.x, in.nlen))
+        in.x = nullptr;
+    return in;
+}
 // By one warp; leff: taps up to the last non-zero one.
-__device__ __forceinline__ void plan_utterance(const PlanArgs &a, const AugUttParams &row, int utt, int S_max, int leff,
-                                               bool stored, int lane) {
-    const int N = min(max(a.lengths[utt], 0), a.n_cap);
+__device__ __forceinline__ void plan_utterance(const PlanArgs &a, const PlanInput &in, int utt, int leff, bool stored, int lane) {
+    const int N = in.N;
     // every block yields the F2 - (taps - 1) outputs that see no wrap-around, cut to a multiple
     // of 4, where taps counts up to the last non-zero tap of this utterance's responses
     const int ob = stored ? BLK2 : (F2 - min(max(leff, 1), BLK2) + 1) & ~3;
     const int n = (N + ob - 1) / ob;
+    // usable noises in the order of the sources
+    const unsigned usable = __ballot_sync(0xffffffffu, lane > 0 && lane < in.n_src && in.x != nullptr);
+    const int n_noise = __popc(usable), nlen = __shfl_sync(0xffffffffu, in.nlen, __ffs(usable | 0x80000000u) - 1);
+    if (lane > 0 && lane < in.n_src && in.x == nullptr && n > 0 && atomicCAS(&a.status[0], -1, utt) == -1)
+        a.status[1] = aug::R_NOISE;
+    int n_v = n, period = 0;                       // blocks of v
+    if (!stored && n_noise == 1 && nlen < N) {
+        // (several periods as one where they are shorter than a block: the copies are a whole CTA's work)
+        period = nlen >= ob ? nlen : (ob + nlen - 1) / nlen * nlen;
+        const int blocks = (int)(((unsigned)period + (unsigned)max(leff, 1) - 2u) / (unsigned)ob) + 1;
+        if (blocks < n) n_v = blocks;
+        else period = 0;
+    }
+    Plan *p = a.plans + utt;
+    if (lane == 0 || (usable >> lane & 1)) {
+        const int at = lane == 0 ? 0 : 1 + __popc(usable & ((1u << lane) - 1u));
+        p->x[at] = in.x;
+        p->nlen[at] = in.nlen;
+        p->src[at] = lane;
+    }
     int at = 0, at_heavy = -1;
     if (lane == 0) {
-        Plan p;
-        p.N = N;
-        p.ob = ob;
-        p.parts = (max(leff, 1) + BLK2 - 1) / BLK2;
-        p.n_src = row.n_src >= 1 && row.n_src <= S_max ? row.n_src : 0;    // (reported by step 1)
-        p.n_noise = 0;
-        p.x[0] = a.speech + (int64_t)utt * a.stride;
-        p.nlen[0] = 1;
-        p.src[0] = 0;
-        for (int s = 1; s < p.n_src; ++s) {
-            const float *x;
-            int nlen;
-            if (source_of(row, s, nullptr, a.bank, a.bank_len, x, nlen)) {
-                ++p.n_noise;
-                p.x[p.n_noise] = x;
-                p.nlen[p.n_noise] = nlen;
-                p.src[p.n_noise] = s;
-            } else if (n > 0 && atomicCAS(&a.status[0], -1, utt) == -1) {
-                a.status[1] = aug::R_NOISE;
-            }
-        }
-        a.plans[utt] = p;
         if (n > 0) {
             int *list = a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED);
-            const bool heavy = p.n_noise > 1;
-            if (heavy) at_heavy = atomicAdd(list, n);
-            at = atomicAdd(list + 1, heavy ? n : 2 * n);
+            const bool heavy = n_noise > 1;
+            if (heavy) at_heavy = atomicAdd(list, n_v);
+            at = atomicAdd(list + 1, heavy ? n : n + n_v);
         }
+        p->n_src = in.n_src;
+        p->n_noise = n_noise;
+        p->N = N;
+        p->ob = ob;
+        p->parts = (max(leff, 1) + BLK2 - 1) / BLK2;
+        p->period = period;
+        p->copy_from = n_v * ob - period;
     }
     at = __shfl_sync(0xffffffffu, at, 0);
     at_heavy = __shfl_sync(0xffffffffu, at_heavy, 0);
     const int last = a.unit_cap - 1;
     for (int i = lane; i < n; i += 32) {
         a.units[last - at - i] = Unit{utt, 2 * i};
-        a.units[at_heavy >= 0 ? at_heavy + i : last - at - n - i] = Unit{utt, 2 * i + 1};
+        if (i < n_v) a.units[at_heavy >= 0 ? at_heavy + i : last - at - n - i] = Unit{utt, 2 * i + 1};
     }
 }
 
-// The same with the lengths in global memory.
-__device__ __forceinline__ void plan_measured(const PlanArgs &a, const AugUttParams *__restrict__ table, int utt,
-                                              int S_max, const int *leff, const int *leff_all, bool mixed,
-                                              bool stored_only, int lane) {
-    const AugUttParams &row = table[utt];
-    int len = lane < row.n_src && row.n_src <= S_max ? leff[utt * S_max + lane] : 0;
-    len = __reduce_max_sync(0xffffffffu, len);
-    plan_utterance(a, row, utt, S_max, len, mixed && (stored_only || !takes_fused_route(*leff_all)), lane);
+// Largest length of an utterance's responses.
+__device__ __forceinline__ int longest(const int *leff, const PlanInput &in, int utt, int S_max, int lane) {
+    return __reduce_max_sync(0xffffffffu, lane < in.n_src ? leff[utt * S_max + lane] : 0);
 }
 // One warp per utterance (long responses of the caller: the route follows from the whole batch; elsewhere
 // rir_spectra2_kernel plans on the way).
 __global__ void __launch_bounds__(256)
 plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restrict__ table, int B, int S_max,
             const int *leff, const int *leff_all, int stored_only) {
-    const int utt = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    PlanInput in;
+    if (utt < B) in = plan_input(args, table[utt], utt, S_max, lane);
     chain_next();
     chain_wait();
-    if (utt < B) plan_measured(args, table, utt, S_max, leff, leff_all, true, stored_only, threadIdx.x & 31);
+    if (utt < B)
+        plan_utterance(args, in, utt, longest(leff, in, utt, S_max, lane), stored_only || !takes_fused_route(*leff_all), lane);
 }
 
 // Spectra of the partitions of each impulse response: 8192 taps (those beyond L are zero) and as many
@@ -513,9 +538,13 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
     __shared__ int red_i[CF / 32];
     const int t = threadIdx.x;
     if (LENGTHS == KNOWN && blockIdx.x < n_plan) {
+        const int utt = blockIdx.x * (CF / 32) + (t >> 5), lane = t & 31;
+        PlanInput in;
+        if (utt < B) in = plan_input(plan, table[utt], utt, S_max, lane);
         chain_wait();
-        const int utt = blockIdx.x * (CF / 32) + (t >> 5);
-        if (utt < B) plan_measured(plan, table, utt, S_max, leff, leff_all, mixed, stored_only, t & 31);
+        if (utt < B)
+            plan_utterance(plan, in, utt, longest(leff, in, utt, S_max, lane),
+                           mixed && (stored_only || !takes_fused_route(*leff_all)), lane);
         return;
     }
     const int id = blockIdx.x - n_plan, part = id % P, us = id / P, utt = us / S_max, s = us - utt * S_max;
@@ -524,7 +553,8 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
     fftpair::fill_tables(sh, t, tw);
     if (row.n_src < 1 || row.n_src > S_max || s >= row.n_src) {
         chain_wait();
-        if (LENGTHS == FIND && s == 0 && t < 32) plan_utterance(plan, row, utt, S_max, 1, false, t);
+        if (LENGTHS == FIND && s == 0 && t < 32)
+            plan_utterance(plan, plan_input(plan, row, utt, S_max, t), utt, 1, false, t);
         return;
     }
     chain_wait();
@@ -601,9 +631,43 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
         sum = __shfl_sync(0xffffffffu, sum, 0);
         if ((int)(sum >> 56) == row.n_src) {
             const int len = t < 4 ? (int)(sum >> (14 * t)) & ((1 << 14) - 1) : 0;
-            plan_utterance(plan, row, utt, S_max, __reduce_max_sync(0xffffffffu, len), false, t);
+            plan_utterance(plan, plan_input(plan, row, utt, S_max, t), utt, __reduce_max_sync(0xffffffffu, len), false, t);
         }
     }
+}
+
+// Outputs [from, end) of a block of v that lie behind copy_from, wherever they come back; this thread's are the groups of
+// four i, i + 4 CF, ..., which it has just written.  Returns the sum of their squares.  (Read back one by one: kept in
+// registers, in the exchange buffer or read four at a time they cost the blocks that do not repeat up to 1 %.)
+__device__ __forceinline__ float repeat_block(float *row, int i, int from, int end, int copy_from, int period, int N) {
+    const bool groups = ((period | copy_from) & 3) == 0;
+    float sum = 0.f;
+#pragma unroll 1
+    for (; i < end; i += 4 * CF) {
+        if (i < from || i + 3 < copy_from) continue;
+        const float4 y = *reinterpret_cast<const float4 *>(row + i);
+        if (groups) {
+            for (int m = i; m < N - period;) {
+                m += period;
+                // (workspace rows are allocated up to a multiple of 4)
+                const float4 z = make_float4(y.x, m + 1 < N ? y.y : 0.f, m + 2 < N ? y.z : 0.f, m + 3 < N ? y.w : 0.f);
+                *reinterpret_cast<float4 *>(row + m) = z;
+                sum = fmaf(z.x, z.x, fmaf(z.y, z.y, fmaf(z.z, z.z, fmaf(z.w, z.w, sum))));
+            }
+        } else {
+            const float z[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (i + c < copy_from) continue;
+                for (int m = i + c; m < N - period;) {
+                    m += period;
+                    row[m] = z[c];
+                    sum = fmaf(z[c], z[c], sum);
+                }
+            }
+        }
+    }
+    return sum;
 }
 
 // KIND  FUSED    a block of one output from its samples (responses of one partition)
@@ -883,6 +947,8 @@ convolve_kernel(const Plan *plans, const Unit *units, const int *n_units, int un
                 if (j == j_last) {
                     const float2 e = fftpair::unpack(e2);
                     float sum = e.x + e.y;
+                    if (KIND == FUSED && noise && p.period > 0 && (b + 1) * ob > p.copy_from)
+                        sum += repeat_block(dst - (int64_t)b * ob, b * ob + o0, b * ob, (b + 1) * ob, p.copy_from, p.period, p.N);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
                     if ((t & 31) == 0) atomicAdd(&energy[2 * cur.utt + (noise ? 1 : 0)], (double)sum);
@@ -901,6 +967,15 @@ constexpr size_t FFT2_SMEM = sizeof(fftpair::Shared);
 }  // namespace
 
 static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_STORED; }
+
+// As many CTAs as fit (less the room to be left for kernels of other streams), but not more than there
+// can be units of work.
+static int convolve_fit(const AugCtx *ctx, const ConvInput &in) {
+    return std::min(FUSED_MINB * ctx->sm_count - in.room, aug::PARK_SLOTS);
+}
+static int64_t most_units(const ConvInput &in, int B, int ob) { return 2 * (int64_t)B * ((in.max_len + ob - 1) / ob); }
+// blocks of the fused kernel are shortest where a response fills min(rir_taps, 8192) taps
+static int shortest_block(const AugCtx *ctx) { return (F2 - std::min(ctx->cfg.rir_taps, BLK2) + 1) & ~3; }
 
 static PlanArgs plan_args(const AugCtx *ctx, const ConvInput &in) {
     return {in.speech, in.stride, in.lengths, in.bank, in.bank_len, in.max_len, ctx->status,
@@ -955,12 +1030,8 @@ static int launch_convolve(AugCtx *ctx, int grid) {
     ctx->launches++;
     return AUG_OK;
 }
-// As many CTAs as fit (less the room to be left for kernels of other streams), but not more than there
-// can be units of work.
 static int convolve_grid(const AugCtx *ctx, const ConvInput &in, int B, int ob) {
-    const int max_len = in.max_len;
-    const int fit = std::min(FUSED_MINB * ctx->sm_count - in.room, aug::PARK_SLOTS);
-    return (int)std::min<int64_t>(2 * (int64_t)B * ((max_len + ob - 1) / ob), fit);
+    return (int)std::min<int64_t>(most_units(in, B, ob), convolve_fit(ctx, in));
 }
 
 int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B, bool measured) {
@@ -976,12 +1047,10 @@ int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams
 }
 
 int launch_convolve_finish(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B) {
-    const AugConfig &c = ctx->cfg;
     if (in.max_len <= 0) return AUG_OK;
     int rc = AUG_OK;
     if (!ctx->stored_only) {
-        // blocks are shortest where a response fills min(rir_taps, 8192) taps
-        const int grid = convolve_grid(ctx, in, B, (F2 - std::min(c.rir_taps, BLK2) + 1) & ~3);
+        const int grid = convolve_grid(ctx, in, B, shortest_block(ctx));
         rc = ctx->park ? launch_convolve<FUSED, true>(ctx, grid) : launch_convolve<FUSED, false>(ctx, grid);
         if (rc != AUG_OK) return rc;
     }

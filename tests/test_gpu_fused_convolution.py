@@ -94,3 +94,20 @@ def test_parking_slots_used_by_many_units(hold):
     """Three noise sources, several units a CTA: a slot is written again by the unit after."""
     run([3 * OB + 5, 2 * OB, 700], [[(8, 40000), (3, 9000), (100, 777)], [(0, 50000), (16, 20000)],
                                     [(4, 400), (1, 333), (7, 50)]], copies=80, calls=2, hold=hold)
+
+
+@pytest.mark.parametrize("taps", [1, 300, 8192])
+def test_noise_that_comes_back(taps):
+    """One noise source whose stretch is shorter than the utterance: only the blocks up to the end of its first period
+    (and of the response behind it) are computed.  Periods of any alignment, around the length of a block, of
+    the utterance and far below, utterances that end right behind the computed blocks; a second noise, which needs all of them."""
+    ob = (16384 - taps + 1) & ~3
+    lengths, loops = [], []
+    for n in (6 * ob, 6 * ob + 1, 5 * ob - 3, 60001):
+        for m in (ob, ob + 1, ob - 2, 2 * ob - taps + 1, 2 * ob - taps + 2, 3 * ob + 3, 1, 3, 4, 1000, 1001, n - 1, n, n + 1):
+            m = min(max(m, 1), 59990)
+            lengths.append(n)
+            loops.append([(8 + len(loops) % 3, m)])
+    lengths.append(6 * ob + 1)
+    loops.append([(8, 2 * ob), (4, ob)])
+    run(lengths, loops, taps=taps, seed=taps)

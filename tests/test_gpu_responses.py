@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 from paper_1912_11040_b200 import binding, synth
-from helpers import RIR_REL_TOL
+from helpers import RIR_REL_TOL, WAVE_REL_TOL
 
 pytestmark = pytest.mark.gpu
 
@@ -74,3 +74,37 @@ def test_batches_on_both_sides_of_a_round(B, S, order):
                 ref = oracle.rir_image_method(r["room"], r["beta"], r["mic"], r["src_pos"][s], order, taps)
             for i in range(b, B, few):
                 assert np.max(np.abs(h[i, s] - ref)) <= RIR_REL_TOL * np.max(np.abs(ref)), (i, s)
+
+
+@pytest.mark.parametrize("taps", [1000, 9000, 17000])
+def test_ends_recorded_by_the_pipeline(taps):
+    """What a context keeps from an earlier batch does not show: responses that end elsewhere, a source less, and a
+    row that is rejected (silence) after a batch whose responses fill the buffer."""
+    import torch
+    w = synth.make_workload(2, seed=5, batch=6, dur_scale=0.15)
+    w.cfg.update(rir_taps=taps)
+    cfg = binding.make_config(w.cfg, w.B, w.stride)
+    T = binding.aug_frame_count(int(w.lengths.max()), cfg.win, cfg.hop)
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    speech, lengths, bank = cu(w.speech), cu(w.lengths), cu(w.bank)
+    first, second = w.table.copy(), w.table.copy()
+    first["beta"], first["room"] = 0.99, first["room"] * 1.5
+    second["n_src"][1] = 1
+    second["order"][2] = cfg.max_order + 1
+    second["order"][3] = 0
+
+    def run(ctx, table):
+        feats = torch.full((w.B, T, cfg.n_mel), float("nan"), device="cuda")
+        wave = torch.full((w.B, w.stride), float("nan"), device="cuda")
+        ctx.aug_pipeline(speech, w.stride, lengths, w.lengths, bank, w.bank.size, binding.table_to_device(table), w.B,
+                         feats, T, torch.empty(w.B, dtype=torch.int32, device="cuda"), wave)
+        return wave.cpu().numpy()
+
+    used, fresh = binding.AugContext(cfg), binding.AugContext(cfg)
+    run(used, first)
+    got, want = run(used, second), run(fresh, second)
+    for b in range(w.B):
+        n = int(w.lengths[b])
+        # (after a batch of long responses the convolution goes another way: each within WAVE_REL_TOL of the definition)
+        assert np.max(np.abs(got[b, :n] - want[b, :n])) <= 2 * WAVE_REL_TOL * np.sqrt(np.mean(want[b, :n] ** 2.0))
+        assert (np.max(np.abs(got[b, :n])) == 0.0) == (b == 2)
