@@ -25,6 +25,8 @@
 // barriers per transform, 16 frames for 13 hops) took 360 us for 64 utterances of 2-20 s, this
 // one takes 261.  Its error is 1.8e-7 of the waveform (root mean square; the form before 2.3e-7); with
 // the transforms' factors built from powers instead of a table it took 258 and had 3.1e-7.
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft_pair.cuh"
 
@@ -75,13 +77,19 @@ vtlp_positions_kernel(const AugUttParams *__restrict__ table, int *__restrict__ 
     }
 }
 
+// Which hops a CTA owns: those of runs of several rounds or, in the utterances that come last, of single ones: the device is
+// left half empty for a shorter time at the end (64 utterances of 2-20 s, warp and its tables 243 us, so 230).
+struct HopMap {
+    int long_utts;                 // utterances done in runs
+    int runs, singles;             // CTAs of an utterance in runs and in single rounds
+};
+
 template <int ROUNDS>
 __global__ void __launch_bounds__(RS_THREADS, 2)
 vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int *__restrict__ lengths,
                     const int *__restrict__ k0_tab, const float *__restrict__ fr_tab, int win,
                     const float2 *__restrict__ tw, float *__restrict__ out, int64_t out_stride, int n_cap,
-                    const __grid_constant__ ResynthLayout lay) {
-    constexpr int HB = ROUNDS * NF - 3;              // hops of output per CTA
+                    const __grid_constant__ ResynthLayout lay, const HopMap map) {
     extern __shared__ __align__(16) float sm[];
     const int hop = win >> 2, front = win - hop;
     float *xin = sm + lay.xin;                       // [(NF-1) hop + win] padded input stretch of a round
@@ -89,11 +97,22 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
     float2 *pos = reinterpret_cast<float2 *>(sm + lay.pos);      // [SPEC] lower source bin (int), fraction
     float *carry = sm + lay.carry;                   // [3 hop] what earlier frames add to the next hops
 
-    const int utt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int run = blockIdx.x, utt = run / map.runs, rounds = ROUNDS;
+    if (utt < map.long_utts) {
+        run -= utt * map.runs;
+    } else {
+        run -= map.long_utts * map.runs;
+        utt = run / map.singles;
+        run -= utt * map.singles;
+        utt += map.long_utts;
+        rounds = 1;
+    }
+    const int HB = rounds * NF - 3;                  // hops of output per CTA
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = min(max(lengths[utt], 0), n_cap);
     if (N == 0) return;
     const int T = (N + front + hop - 1) / hop;       // frames = hops that cover the padded utterance
-    const int t0 = blockIdx.x * HB;                  // first hop this CTA owns
+    const int t0 = run * HB;                         // first hop this CTA owns
     if (t0 >= T) return;
     const float *x = speech + (int64_t)utt * stride;
     float *y = out + (int64_t)utt * out_stride;
@@ -135,7 +154,7 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
     }
 
 #pragma unroll 1
-    for (int round = 0; round < ROUNDS; ++round) {
+    for (int round = 0; round < rounds; ++round) {
         const int ft = t0 - 3 + round * NF;          // first frame of the round
         if (ft >= T) break;
         // input stretch of frames ft .. ft + NF - 1
@@ -354,15 +373,16 @@ int launch_vtlp_resynth(AugCtx *ctx, const float *speech, int64_t stride, const 
     // Runs of three rounds (45 hops for 48 frames), single rounds (13 for 16) where the batch is so
     // small that it would not fill the device otherwise.
     constexpr int RUN = 3;
-    const bool runs = (int64_t)((T_cap + RUN * NF - 4) / (RUN * NF - 3)) * B >= 4 * (int64_t)ctx->sm_count;
-    const int HB = (runs ? RUN : 1) * NF - 3;
+    HopMap map = {0, (T_cap + RUN * NF - 4) / (RUN * NF - 3), (T_cap + NF - 4) / (NF - 3)};
+    const bool runs = (int64_t)map.runs * B >= 4 * (int64_t)ctx->sm_count;
+    if (runs) map.long_utts = std::max(0, B - (4 * ctx->sm_count + map.singles - 1) / map.singles);
     auto kern = runs ? vtlp_resynth_kernel<RUN> : vtlp_resynth_kernel<1>;
     if ((runs ? smem_opt_in<vtlp_resynth_kernel<RUN>>(ctx->device) : smem_opt_in<vtlp_resynth_kernel<1>>(ctx->device)) !=
         AUG_OK)
         return AUG_ECUDA;
-    dim3 grid((T_cap + HB - 1) / HB, B);
+    const dim3 grid(map.long_utts * map.runs + (B - map.long_utts) * map.singles);
     kern<<<grid, RS_THREADS, smem, ctx->stream>>>(speech, stride, lengths, k0_tab, fr_tab, win, ctx->tw, out, out_stride,
-                                                  max_len, lay);
+                                                  max_len, lay, map);
     AUG_CUDA_OK(cudaGetLastError());
     ctx->launches++;
     return AUG_OK;
