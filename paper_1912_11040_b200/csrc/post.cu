@@ -19,21 +19,25 @@ namespace {
 // multiply-adds a frame) as long as they are not read again for every coefficient: a CTA
 // stages a tile of 128 frames in shared memory (odd row stride, so the lanes of a warp read 32
 // frames without conflicts) and each thread carries eight coefficients of two frames, the
-// basis arriving as 128-bit broadcasts.  205 k frames, 13 coefficients: 35.2 us, the bytes 12; with
-// the angles of the basis unreduced, two divisions per output and four loads in flight instead of ten
-// 44.7.
+// basis arriving as 128-bit broadcasts.  The features are copied asynchronously while the basis is worked out, and read
+// back four bands at a time.  205 k frames, 80 bands, 13 coefficients (the bytes take 12 us), and what else it takes to make
+// them from the waveform: 318 us in all with loads through registers and one band at a time, 293.
 constexpr int MFCC_THREADS = 128, MFCC_FT = 128, MFCC_CB = 16;   // frames per tile, coefficients per round
+// Rows of a staged frame: an odd number of 16-byte words, so that both copies of whole words and the reads of 32 frames'
+// words are free of bank conflicts.
+__host__ __device__ constexpr int mfcc_ld(int M) { return 4 * (((M + 3) >> 2) | 1); }
 __host__ __device__ constexpr size_t mfcc_smem(int M) {
-    return sizeof(float) * ((size_t)MFCC_FT * (M | 1) + MFCC_CB * M + MFCC_FT * (MFCC_CB + 1) + 4);
+    return sizeof(float) * ((size_t)MFCC_FT * mfcc_ld(M) + MFCC_CB * ((M + 3) & ~3) + MFCC_FT * (MFCC_CB + 1) + 4);
 }
 __global__ void __launch_bounds__(MFCC_THREADS)
 mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int M, int n_cep,
             int T_max, float pad_v, float *__restrict__ out) {
     extern __shared__ __align__(16) float sm[];
     float *basis = sm;                               // [M][MFCC_CB]
-    float *os = basis + MFCC_CB * M;                 // [MFCC_FT][MFCC_CB + 1]
-    float *xs = os + MFCC_FT * (MFCC_CB + 1);        // [MFCC_FT][M | 1]
-    const int utt = blockIdx.y, tid = threadIdx.x, ld = M | 1;
+    const int M4 = (M + 3) & ~3;                     // bands, and zeros up to whole words
+    float *xs = basis + MFCC_CB * M4;                // [MFCC_FT][mfcc_ld(M)]
+    const int utt = blockIdx.y, tid = threadIdx.x, ld = mfcc_ld(M);
+    float *os = xs + MFCC_FT * ld;                   // [MFCC_FT][MFCC_CB + 1]
     const int t0 = blockIdx.x * MFCC_FT;
     const int rows = min(MFCC_FT, T_max - t0);
     const int T = min(max(counts[utt], 0), T_max);
@@ -45,14 +49,10 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
     if ((M & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
         const int m4 = M >> 2, step_f = MFCC_THREADS / m4, step_m = MFCC_THREADS - step_f * m4;
         int f = tid / m4, m = tid - f * m4;
-#pragma unroll 10
-        for (int i = tid; i < nf * m4; i += MFCC_THREADS) {
-            const float4 z = __ldg(reinterpret_cast<const float4 *>(x) + i);
-            float *d = xs + f * ld + 4 * m;
-            d[0] = z.x;
-            d[1] = z.y;
-            d[2] = z.z;
-            d[3] = z.w;
+        const float *src = x + 4 * tid;
+        for (int i = tid; i < nf * m4; i += MFCC_THREADS, src += 4 * MFCC_THREADS) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(xs + f * ld + 4 * m)), "l"(src) : "memory");
             f += step_f;
             m += step_m;
             if (m >= m4) {
@@ -61,6 +61,7 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
             }
         }
     } else {
+        for (int i = tid; i < MFCC_FT * (M4 - M); i += MFCC_THREADS) xs[i / (M4 - M) * ld + M + i % (M4 - M)] = 0.f;
         for (int i = tid; i < nf * M; i += MFCC_THREADS) {
             const int f = i / M;
             xs[i + f * (ld - M)] = __ldg(x + i);
@@ -75,27 +76,33 @@ mfcc_kernel(const float *__restrict__ feats, const int *__restrict__ counts, int
         const float s = c >= n_cep ? 0.f : c == 0 ? rsqrtf((float)M) : sqrtf(2.f / (float)M);
         const float unit = 1.f / (float)(2 * M), rest = fmaf(-unit, (float)(2 * M), 1.f) * unit;   // 1 / 2M in two parts
         int k = c * (2 * (tid / MFCC_CB) + 1) % (4 * M);
-        for (int i = tid; i < MFCC_CB * M; i += MFCC_THREADS) {
-            basis[i] = s * cospif(fmaf((float)k, unit, (float)k * rest));
+        for (int i = tid; i < MFCC_CB * M4; i += MFCC_THREADS) {
+            basis[i] = i < MFCC_CB * M ? s * cospif(fmaf((float)k, unit, (float)k * rest)) : 0.f;
             k += step;
             if (k >= 4 * M) k -= 4 * M;
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         // pairs of coefficients, as the basis is read
         fftpair::u64 a[4], b[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) a[c] = b[c] = 0;
         const float *x0 = xs + f0 * ld, *x1 = x0 + 64 * ld, *bz = basis + 8 * half;
-#pragma unroll 4
-        for (int m = 0; m < M; ++m) {
-            const fftpair::u64 u = fftpair::both(x0[m]), v = fftpair::both(x1[m]);
-            const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * m);
-            const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * m + 4);
-            const fftpair::u64 w[4] = {p.x, p.y, q.x, q.y};
+#pragma unroll 2
+        for (int m = 0; m < M4; m += 4) {
+            const float4 p0 = *reinterpret_cast<const float4 *>(x0 + m), p1 = *reinterpret_cast<const float4 *>(x1 + m);
+            const float e0[4] = {p0.x, p0.y, p0.z, p0.w}, e1[4] = {p1.x, p1.y, p1.z, p1.w};
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                a[c] = fftpair::fma2(u, w[c], a[c]);
-                b[c] = fftpair::fma2(v, w[c], b[c]);
+            for (int d = 0; d < 4; ++d) {
+                const fftpair::u64 u = fftpair::both(e0[d]), v = fftpair::both(e1[d]);
+                const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * (m + d));
+                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(bz + MFCC_CB * (m + d) + 4);
+                const fftpair::u64 w[4] = {p.x, p.y, q.x, q.y};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    a[c] = fftpair::fma2(u, w[c], a[c]);
+                    b[c] = fftpair::fma2(v, w[c], b[c]);
+                }
             }
         }
 #pragma unroll
