@@ -7,6 +7,10 @@
 // with their rising weights and those of interval m+1 with their falling
 // weights; the intervals are contiguous bin ranges because the warp of Eq. 1 is
 // monotone.  Every interval is walked once for both sums.
+#include <math.h>
+
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft_pair.cuh"
 
@@ -19,12 +23,19 @@ __host__ __device__ __forceinline__ int frame_count(int n, int win, int hop) {
 }
 
 // ---------------------------------------------------------------- filterbank tables
+// Edges of the bands in mel: the first one and their distance.
+struct MelEdges {
+    double first, step;
+    MelEdges(double f_lo, double f_hi, int M) {
+        first = 2595.0 * log10(1.0 + f_lo / 700.0);
+        step = (2595.0 * log10(1.0 + f_hi / 700.0) - first) / (M + 1);
+    }
+};
 // One CTA per utterance: per DFT bin the edge interval and weights at the warped
 // frequency (fp64: a bin that barely enters a band must not lose its weight to
 // rounding), then the first bin of every interval.
 __global__ void __launch_bounds__(256)
-mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double f_lo,
-                  double f_hi, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped,
+mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double e0, double delta, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped,
                   int *counters, double *energy) {
     __shared__ int seg_s[513];
     chain_next();
@@ -37,12 +48,10 @@ mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double f
     // (unwarped: the warp was already applied to the waveform)
     const double a = unwarped ? 0.0 : 1.0 - (double)table[utt].alpha;
     const double PI = 3.14159265358979323846;
-    const double e0 = 2595.0 * log10(1.0 + f_lo / 700.0);
-    const double e1 = 2595.0 * log10(1.0 + f_hi / 700.0);
-    const double delta = (e1 - e0) / (M + 1);
     for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-        const double om = 2.0 * PI * k / K;
-        const double omw = om + 2.0 * atan(a * sin(om) / (1.0 - a * cos(om)));   // Eq. 1
+        double sin_om, cos_om;
+        sincospi(2.0 * k / K, &sin_om, &cos_om);
+        const double omw = 2.0 * PI * k / K + 2.0 * atan(a * sin_om / (1.0 - a * cos_om));   // Eq. 1
         const double fw = omw * fs / (2.0 * PI);
         const double mu = 2595.0 * log10(1.0 + fw / 700.0);
         const double u = (mu - e0) / delta;
@@ -184,6 +193,7 @@ __device__ __forceinline__ void walk_bands(const ulonglong2 *w4, const int *mst,
 // bands); the bytes take 61 and 105.  Tiles of a run, on the former batch and on 4096 of 1-6 s: two
 // 264 and 1302 us, four 249 and 1179, six 249 and 1190.
 constexpr int WARPS = FEAT_THREADS / 32;
+constexpr int TAIL_ROUNDS = 2;         // tiles a CTA's place on the device that are not done in runs
 
 template <int K>
 struct Plan;
@@ -333,21 +343,41 @@ __device__ __forceinline__ void power_rows(fftpair::C2 *v, fftpair::u64 *p, cons
     }
 }
 
+// Which frames a CTA works on.  Runs of several tiles share their set-up, but the device is left half empty behind the
+// last round of them; the utterances that come last are done tile by tile.  The last utterances go first: what the
+// convolution has written last is still in L2.  256 utterances of 2-20 s 258 -> 252 us, 96 116 -> 112, 64 of 60 s (K = 1024)
+// 666 -> 649; with twice as many single tiles 686.2 against 689.3 and 1376 against 1373 (whole calls), with four times as
+// many both slower.
+struct RunMap {
+    int utts, long_utts;           // of which the first ones (in the order of work) are done in runs
+    int runs, tiles;               // per utterance: runs, tiles
+};
+
 template <int K, int MODE, int TILES>
 __global__ void __launch_bounds__(FEAT_THREADS, 2)
 frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const GainSource gain,
               const int *__restrict__ lengths, int win, int hop, int M, int T_max, const aug::MelBin *__restrict__ melw,
               const int *__restrict__ melstart, const float2 *__restrict__ tw, float floor_v, float pad_v, int comp,
               float *__restrict__ out, int *__restrict__ counts, int n_cap, float *__restrict__ wave, int64_t wave_stride,
-              const __grid_constant__ Layout lay) {
+              const __grid_constant__ Layout lay, const RunMap map) {
     constexpr int QF = Plan<K>::QF, FT = tile_frames<K>(), NBP = K / 2 + 1;
     extern __shared__ __align__(16) float sm[];
     float *chunk = sm + lay.chunk, *win_s = sm + lay.win;
     float4 *mw = reinterpret_cast<float4 *>(sm + lay.mw);                    // (up, up, down, down)
     int *mst = reinterpret_cast<int *>(sm + lay.mst), *cut = reinterpret_cast<int *>(sm + lay.cut);
 
-    const int utt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int run0 = blockIdx.x * (FT * TILES);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int run = blockIdx.x, nth = run / map.runs, run_tiles = TILES;
+    if (nth < map.long_utts) {
+        run -= nth * map.runs;
+    } else {
+        run -= map.long_utts * map.runs;
+        nth = run / map.tiles;
+        run -= nth * map.tiles;
+        nth += map.long_utts;
+        run_tiles = 1;
+    }
+    const int utt = map.utts - 1 - nth, run0 = run * (FT * run_tiles);
     for (int n = tid; n < K; n += FEAT_THREADS)
         win_s[n] = n < win ? 0.25f - 0.25f * cospif(2.f * (float)n / (float)win) : 0.f;
     if (tid < 32) {
@@ -356,9 +386,9 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
     }
     const int N = min(max(lengths[utt], 0), n_cap);
     const int T = min(frame_count(N, win, hop), T_max);
-    if (blockIdx.x == 0 && tid == 0) counts[utt] = T;
-    const int rows = min(FT * TILES, T_max - run0);
-    const int nfr = max(0, min(FT * TILES, T - run0));
+    if (run == 0 && tid == 0) counts[utt] = T;
+    const int rows = min(FT * run_tiles, T_max - run0);
+    const int nfr = max(0, min(FT * run_tiles, T - run0));
     const int out_w = MODE == 0 ? NBP : M;
     float *orun = out + ((int64_t)utt * T_max + run0) * out_w;
     if (rows > nfr)
@@ -378,7 +408,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
     // The mixed waveform, where it is wanted: a tile writes the hops that its frames start, the CTA with
     // the last frame (the first one if there is none) what lies behind them.
     float *wrow = MODE == 1 && wave != nullptr ? wave + (int64_t)utt * wave_stride : nullptr;
-    if (MODE == 1 && wrow != nullptr && run0 <= max(T - 1, 0) && run0 + FT * TILES > max(T - 1, 0)) {
+    if (MODE == 1 && wrow != nullptr && run0 <= max(T - 1, 0) && run0 + FT * run_tiles > max(T - 1, 0)) {
         const float gw = fabsf(snr_gain(es, ev, snr_ratio(gain.table[utt]), n_src));
         const float *wa = in_a + (int64_t)utt * in_stride, *wb = in_b + (int64_t)utt * in_stride;
         for (int i = T * hop + tid; i < N; i += FEAT_THREADS) wrow[i] = fmaf(gw, wb[i], wa[i]);
@@ -387,7 +417,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
 
     const float *ra = in_a + (int64_t)utt * in_stride;
     const float *rb = MODE == 1 ? in_b + (int64_t)utt * in_stride : nullptr;
-    const int n_tiles = min(TILES, (nfr + FT - 1) / FT);
+    const int n_tiles = min(run_tiles, (nfr + FT - 1) / FT);
 
     // Samples of a tile travel global -> shared asynchronously, one tile ahead, in the 16-byte groups of
     // the row: the tile's first sample may be any of its first group (with hops that are no
@@ -626,7 +656,8 @@ logmel_kernel(const float *__restrict__ power, const int *__restrict__ counts, i
     float *fs = sm + logmel_fs(NBP);                                // [LM_FT][M | 1] band energies
     float4 *mw = reinterpret_cast<float4 *>(sm + logmel_mw(NBP, M));   // [NBP] (up, up, down, down)
     int *mst = reinterpret_cast<int *>(mw + NBP), *cut = mst + M + 2;
-    const int utt = blockIdx.y, tid = threadIdx.x, ld = M | 1;
+    // (the last utterances first: of power spectra made just now they are the ones still in L2)
+    const int utt = gridDim.y - 1 - blockIdx.y, tid = threadIdx.x, ld = M | 1;
     const int t0 = blockIdx.x * LM_FT;
     const int rows = min(LM_FT, T_max - t0);
     const int T = min(max(counts[utt], 0), T_max);
@@ -713,8 +744,9 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
     // to give every multiprocessor something to do.
     const int n_tiles = (T_max + FT - 1) / FT;
     const bool runs = (int64_t)n_tiles * B >= 2 * (int64_t)ctx->sm_count * RUN_TILES;
-    const int RUN = FT * (runs ? RUN_TILES : 1);
-    dim3 grid((T_max + RUN - 1) / RUN, B);
+    RunMap map = {B, 0, (n_tiles + RUN_TILES - 1) / RUN_TILES, n_tiles};
+    if (runs) map.long_utts = std::max(0, B - (TAIL_ROUNDS * 2 * ctx->sm_count + n_tiles - 1) / n_tiles);
+    const dim3 grid(map.long_utts * map.runs + (B - map.long_utts) * n_tiles);
     auto kern = runs ? frames_kernel<K, MODE, RUN_TILES> : frames_kernel<K, MODE, 1>;
     if ((runs ? smem_opt_in<frames_kernel<K, MODE, RUN_TILES>>(ctx->device)
               : smem_opt_in<frames_kernel<K, MODE, 1>>(ctx->device)) != AUG_OK)
@@ -724,12 +756,12 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
     if (MODE == 1) {
         if (launch_chained(kern, grid, FEAT_THREADS, smem, ctx->stream, a, b, stride, gain, lengths, c.win, c.hop,
                            c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw, c.log_floor, c.pad_value, c.compression,
-                           out, counts, n_cap, wave, wave_stride, lay) != AUG_OK)
+                           out, counts, n_cap, wave, wave_stride, lay, map) != AUG_OK)
             return AUG_ECUDA;
     } else {
         kern<<<grid, FEAT_THREADS, smem, ctx->stream>>>(
             a, b, stride, gain, lengths, c.win, c.hop, c.n_mel, T_max, ctx->melw, ctx->melstart, ctx->tw,
-            c.log_floor, c.pad_value, c.compression, out, counts, n_cap, wave, wave_stride, lay);
+            c.log_floor, c.pad_value, c.compression, out, counts, n_cap, wave, wave_stride, lay, map);
         AUG_CUDA_OK(cudaGetLastError());
     }
     ctx->launches++;
@@ -740,8 +772,9 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
 
 int launch_mel_tables(AugCtx *ctx, const AugUttParams *table, int B, bool reset) {
     const AugConfig &c = ctx->cfg;
+    const MelEdges e(c.f_lo, c.f_hi, c.n_mel);
     mel_tables_kernel<<<B, 256, 0, ctx->stream>>>(
-        table, c.n_fft, c.n_mel, (double)c.fs, (double)c.f_lo, (double)c.f_hi, ctx->melw, ctx->melstart,
+        table, c.n_fft, c.n_mel, (double)c.fs, e.first, e.step, ctx->melw, ctx->melstart,
         c.vtlp_win > 0 ? 1 : 0, ctx->counters, reset ? ctx->energy : nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     ctx->launches++;
@@ -866,8 +899,8 @@ extern "C" int feat_vtlp_logmel_noalloc(const AugConfig *cfg, const float *power
     // needs clearing.
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int nbp = cfg->n_fft / 2 + 1;
-    mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs,
-                                         (double)cfg->f_lo, (double)cfg->f_hi, melw, melstart, 0, nullptr,
+    const MelEdges e(cfg->f_lo, cfg->f_hi, cfg->n_mel);
+    mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs, e.first, e.step, melw, melstart, 0, nullptr,
                                          nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     int dev = -1;
