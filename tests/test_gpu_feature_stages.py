@@ -242,3 +242,29 @@ def test_hops_beyond_the_window(n_fft, win, hop):
         assert e.value.code == binding.AUG_ECAP
         with pytest.raises(binding.AugError):
             Device(w).stft_power(dev.speech)
+
+
+@pytest.mark.parametrize("n_fft", [512, 1024])
+def test_power_spectra_do_not_depend_on_the_place_in_the_batch(n_fft):
+    """A batch of which the first utterances are done in runs of tiles and the last ones tile by tile: copies of an utterance
+    come out bit by bit the same wherever they stand, with lengths around a tile, a run, and none."""
+    import torch
+    lengths = np.array([20000, 400 + 31 * 160, 400 + 32 * 160, 399, 0, 400 + 127 * 160 + 3], np.int32)
+    few, B, stride = len(lengths), 420, 20732
+    rng = np.random.default_rng(n_fft)
+    wave = (rng.standard_normal((few, stride)) * 0.05).astype(np.float32)
+    w = synth.make_workload(1, batch=2, dur_scale=0.1)
+    w.cfg.update(n_fft=n_fft)
+    ctx = binding.AugContext(binding.make_config(w.cfg, B, stride))
+    T = binding.aug_frame_count(int(lengths.max()), 400, 160)
+    rep = lambda a: torch.from_numpy(np.tile(a, (B // few,) + (1,) * (a.ndim - 1))).cuda()
+    power = torch.full((B, T, n_fft // 2 + 1), float("nan"), device="cuda")
+    counts = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+    ctx.feat_stft_power(rep(wave), stride, rep(lengths), B, power, T, counts)
+    first = power[:few].repeat(B // few, 1, 1)
+    assert torch.equal(power, first)
+    assert counts.cpu().tolist() == [binding.aug_frame_count(int(n), 400, 160) for n in lengths] * (B // few)
+    ref = oracle.stft_power(wave[0, :20000].astype(np.float64), 400, 160, n_fft)
+    got = power[0, : len(ref)].cpu().numpy()
+    # amplitudes within a few roundings of the largest one, squared
+    assert np.max(np.abs(got - ref)) <= 32 * EPS * np.max(ref)
