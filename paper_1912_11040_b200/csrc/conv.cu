@@ -19,9 +19,9 @@
 //                     twice the products per sample and twice the bytes from L2, took 534.
 //
 // Responses are often shorter than their buffer: behind the last image source's window
-// every tap is exactly zero.  The kernels that transform the responses record, per
-// utterance, the number of taps up to the last non-zero one (the largest over its
-// sources); the fused route then takes 16384 - that + 1 outputs from every block
+// every tap is exactly zero.  The number of taps up to the last non-zero one (the largest over an utterance's
+// sources) is recorded where the responses are made; those of the caller are measured, by a kernel of their own or
+// by the one that transforms them.  The fused route then takes 16384 - that + 1 outputs from every block
 // instead of 16384 - rir_taps + 1, and the stored-spectra route skips the partitions
 // that are zero throughout.  A context sized for long responses sends a batch whose
 // responses all end within 8192 taps through the fused route as well: the kernels of

@@ -17,8 +17,7 @@ namespace {
 //
 // A small matrix product, bound by reading the features once (80 bands: 320 bytes and 1040
 // multiply-adds a frame) as long as they are not read again for every coefficient: a CTA
-// stages a tile of 128 frames in shared memory (odd row stride, so the lanes of a warp read 32
-// frames without conflicts) and each thread carries eight coefficients of two frames, the
+// stages a tile of 128 frames in shared memory and each thread carries eight coefficients of two frames, the
 // basis arriving as 128-bit broadcasts.  The features are copied asynchronously while the basis is worked out, and read
 // back four bands at a time.  205 k frames, 80 bands, 13 coefficients (the bytes take 12 us), and what else it takes to make
 // them from the waveform: 318 us in all with loads through registers and one band at a time, 293.
