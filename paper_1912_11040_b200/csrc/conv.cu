@@ -637,8 +637,10 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
 }
 
 // Outputs [from, end) of a block of v that lie behind copy_from, wherever they come back; this thread's are the groups of
-// four i, i + 4 CF, ..., which it has just written.  Returns the sum of their squares.  (Read back one by one: kept in
-// registers, in the exchange buffer or read four at a time they cost the blocks that do not repeat up to 1 %.)
+// four i, i + 4 CF, ..., which it has just written.  Returns the sum of the copies' squares.  Equal ones are counted,
+// not added one by one: in a running sum of all of them a constant stretch came out 2e-5 too loud or quiet over 60 s.
+// (Read back one by one: kept in registers, in the exchange buffer or read four at a time they cost the blocks that do
+// not repeat up to 1 %.)
 __device__ __forceinline__ float repeat_block(float *row, int i, int from, int end, int copy_from, int period, int N) {
     const bool groups = ((period | copy_from) & 3) == 0;
     float sum = 0.f;
@@ -647,23 +649,27 @@ __device__ __forceinline__ float repeat_block(float *row, int i, int from, int e
         if (i < from || i + 3 < copy_from) continue;
         const float4 y = *reinterpret_cast<const float4 *>(row + i);
         if (groups) {
+            float whole = 0.f;
             for (int m = i; m < N - period;) {
                 m += period;
                 // (workspace rows are allocated up to a multiple of 4)
                 const float4 z = make_float4(y.x, m + 1 < N ? y.y : 0.f, m + 2 < N ? y.z : 0.f, m + 3 < N ? y.w : 0.f);
                 *reinterpret_cast<float4 *>(row + m) = z;
-                sum = fmaf(z.x, z.x, fmaf(z.y, z.y, fmaf(z.z, z.z, fmaf(z.w, z.w, sum))));
+                if (m + 3 < N) whole += 1.f;
+                else sum = fmaf(z.x, z.x, fmaf(z.y, z.y, fmaf(z.z, z.z, sum)));
             }
+            sum = fmaf(whole, fmaf(y.x, y.x, fmaf(y.y, y.y, fmaf(y.z, y.z, y.w * y.w))), sum);
         } else {
             const float z[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 if (i + c < copy_from) continue;
-                for (int m = i + c; m < N - period;) {
+                float copies = 0.f;
+                for (int m = i + c; m < N - period; copies += 1.f) {
                     m += period;
                     row[m] = z[c];
-                    sum = fmaf(z[c], z[c], sum);
                 }
+                sum = fmaf(copies, z[c] * z[c], sum);
             }
         }
     }

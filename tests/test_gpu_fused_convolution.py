@@ -111,3 +111,36 @@ def test_noise_that_comes_back(taps):
     lengths.append(6 * ob + 1)
     loops.append([(8, 2 * ob), (4, ob)])
     run(lengths, loops, taps=taps, seed=taps)
+
+
+def test_energy_of_noise_that_comes_back():
+    """The gain of a stretch that is repeated up to a million times: the mix has the SNR that was asked for.  A constant
+    stretch, so that errors of equal terms add up instead of averaging out."""
+    import torch
+    n, taps, snr = 960003, TAPS, -6.0
+    stretches = [1, 3, 4, 1000, 1001, OB, 3 * OB + 1, n // 2 - 1, n // 2, n]
+    B, stride = len(stretches), (n + 3) // 4 * 4
+    rng = np.random.default_rng(7)
+    bank = torch.full((n,), 0.05, device="cuda")
+    speech = torch.from_numpy((rng.standard_normal((B, stride)) * 0.05).astype(np.float32)).cuda()
+    rir = torch.from_numpy(np.abs(rng.standard_normal((B, 2, taps))).astype(np.float32) * 0.01).cuda()
+    tab = np.zeros(B, dtype=synth.UTT_DTYPE)
+    tab["snr_db"], tab["noise_len"][:, 0], tab["noise_weight"][:, 0] = snr, stretches, 1.0
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
+                            max_order=1, max_sources=2, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=B, max_samples=stride,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx = binding.AugContext(cfg)
+    lengths = torch.full((B,), n, dtype=torch.int32, device="cuda")
+    out = []
+    for n_src in (1, 2):
+        tab["n_src"] = n_src
+        w = torch.full((B, stride), float("nan"), device="cuda")
+        ctx.aug_reverb_mix(speech, stride, lengths, bank, n, rir, binding.table_to_device(tab), B, w)
+        out.append(w[:, :n].double())
+    y, noise = out[0], out[1] - out[0]
+    got = y.square().sum(1) / noise.square().sum(1) / 10.0 ** (snr / 10.0)
+    # each of the two sums: 16 roundings a lane of the packed sum, as many of the copies', seven to add up a warp's; the
+    # gain's and the wave's
+    bound = (2 * 39 + 2 + 2) * 2.0 ** -24
+    assert (got - 1.0).abs().max() <= bound, (got - 1.0).tolist()
