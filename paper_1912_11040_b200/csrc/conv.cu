@@ -393,7 +393,12 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
 // A stretch of noise that is shorter than the utterance repeats, and so does its reverberation as soon as the
 // response has run in: v[n + P] = v[n], n >= taps - 1.  Where there is one noise source, only the blocks
 // up to P + taps - 1 are listed, and those that hold the last period also write it wherever it comes back (4096
-// utterances of 1-6 s, stretches of half to all of their length: convolution 1694 us, so 1585).
+// utterances of 1-6 s, stretches of half to all of their length: 3365 us a call without copies, 3267 with them).
+// P is a multiple of the stretch that leaves MOST_COPIES copies of a block at most, so that the writing is shared
+// out: 64 utterances of 60 s over stretches of 1 s 782 us without copies, 666 with one period and all the others
+// in a few CTAs' hands, 651 with three copies, 629 with seven; of 16001 samples 814, 972, 669 and 640.  Contexts for
+// batches of less than two rounds of CTAs compute all blocks, see plan_args.
+constexpr int MOST_COPIES = 7;
 struct Plan {
     const float *x[AUG_S_MAX];     // [0] speech row, [1..n_noise] usable stretches of the bank
     int nlen[AUG_S_MAX];           // their lengths ([0] unused)
@@ -424,6 +429,7 @@ struct PlanArgs {
     Unit *units;
     int unit_cap;
     int *counters;                 // [N_COUNTERS]
+    int repeats;                   // blocks of repeated noise are copied, not computed
 };
 // What planning reads of the caller's inputs: lane l the length of the utterance and source l (0: the speech) of its row.
 // (Read, where the responses are made by the kernel before, ahead of the wait for it.)
@@ -455,12 +461,15 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const PlanInpu
     if (lane > 0 && lane < in.n_src && in.x == nullptr && n > 0 && atomicCAS(&a.status[0], -1, utt) == -1)
         a.status[1] = aug::R_NOISE;
     int n_v = n, period = 0;                       // blocks of v
-    if (!stored && n_noise == 1 && nlen < N) {
-        // (several periods as one where they are shorter than a block: the copies are a whole CTA's work)
-        period = nlen >= ob ? nlen : (ob + nlen - 1) / nlen * nlen;
-        const int blocks = (int)(((unsigned)period + (unsigned)max(leff, 1) - 2u) / (unsigned)ob) + 1;
-        if (blocks < n) n_v = blocks;
-        else period = 0;
+    if (a.repeats && !stored && n_noise == 1 && nlen < N) {
+        // as many stretches as keep the copies of a block few, and none shorter than a block
+        const unsigned least = max(ob, (N - 1) / (MOST_COPIES + 1) + 1), one = max(nlen, 1);
+        const unsigned several = (least + one - 1) / one * one;
+        const unsigned blocks = several < (unsigned)N ? (several + (unsigned)max(leff, 1) - 2u) / (unsigned)ob + 1 : n;
+        if ((int)blocks < n) {
+            n_v = blocks;
+            period = several;
+        }
     }
     Plan *p = a.plans + utt;
     if (lane == 0 || (usable >> lane & 1)) {
@@ -636,40 +645,83 @@ rir_spectra2_kernel(const float *rir, const AugUttParams *__restrict__ table, in
     }
 }
 
-// Outputs [from, end) of a block of v that lie behind copy_from, wherever they come back; this thread's are the groups of
-// four i, i + 4 CF, ..., which it has just written.  Returns the sum of the copies' squares.  Equal ones are counted,
-// not added one by one: in a running sum of all of them a constant stretch came out 2e-5 too loud or quiet over 60 s.
-// (Read back one by one: kept in registers, in the exchange buffer or read four at a time they cost the blocks that do
-// not repeat up to 1 %.)
-__device__ __forceinline__ float repeat_block(float *row, int i, int from, int end, int copy_from, int period, int N) {
-    const bool groups = ((period | copy_from) & 3) == 0;
+// Outputs [from, end) of a block of v that lie behind copy_from, wherever they come back; o = its thread's first group of
+// four, the others are 4 CF apart, and all of the block has just been written.  own: the sum of this thread's squares.
+// Returns that of the copies'.  Equal ones are counted, not added one by one: in a running sum of all of them a
+// constant stretch came out 2e-5 too loud or quiet over 60 s.
+// Bound by instructions: 256 utterances of 20 s over stretches of 0.6 of their length 1081 us without copies, 987 with
+// squares added up for every block, 974 with those of blocks that come back whole taken from `own`; with stretches
+// that are no multiple of 4, 1078, and 1021 with single words at the places of groups, 1000 lane by lane.
+__device__ __forceinline__ float repeat_block(float *row, int o, int from, int end, int copy_from, int period, int N, float own) {
+    const int first = max(from, copy_from);
     float sum = 0.f;
+    if (((period | copy_from) & 3) == 0) {
+        const int copies = (N - end) / period;         // of the last output
+        if (first == from && (N - 1 - from) / period == copies) {
+            // all of the block comes back as often
 #pragma unroll 1
-    for (; i < end; i += 4 * CF) {
-        if (i < from || i + 3 < copy_from) continue;
-        const float4 y = *reinterpret_cast<const float4 *>(row + i);
-        if (groups) {
-            float whole = 0.f;
-            for (int m = i; m < N - period;) {
-                m += period;
-                // (workspace rows are allocated up to a multiple of 4)
-                const float4 z = make_float4(y.x, m + 1 < N ? y.y : 0.f, m + 2 < N ? y.z : 0.f, m + 3 < N ? y.w : 0.f);
-                *reinterpret_cast<float4 *>(row + m) = z;
-                if (m + 3 < N) whole += 1.f;
-                else sum = fmaf(z.x, z.x, fmaf(z.y, z.y, fmaf(z.z, z.z, sum)));
+            for (; o < end; o += 4 * CF) {
+                if (o < from) continue;
+                float *p = row + o;
+                const float4 y = *reinterpret_cast<const float4 *>(p);
+#pragma unroll 1
+                for (int k = 0; k < copies; ++k) {
+                    p += period;
+                    *reinterpret_cast<float4 *>(p) = y;
+                }
             }
+            return (float)copies * own;
+        }
+#pragma unroll 1
+        for (; o < end; o += 4 * CF) {
+            if (o < first) continue;
+            const float4 y = *reinterpret_cast<const float4 *>(row + o);
+            unsigned m = o + period;
+            float whole = 0.f;
+#pragma unroll 1
+            for (; m + 3 < (unsigned)N; m += period, whole += 1.f) *reinterpret_cast<float4 *>(row + m) = y;
             sum = fmaf(whole, fmaf(y.x, y.x, fmaf(y.y, y.y, fmaf(y.z, y.z, y.w * y.w))), sum);
-        } else {
-            const float z[4] = {y.x, y.y, y.z, y.w};
+            if (m < (unsigned)N) {
+                // (workspace rows are allocated up to a multiple of 4)
+                const float4 z = make_float4(y.x, m + 1 < (unsigned)N ? y.y : 0.f, m + 2 < (unsigned)N ? y.z : 0.f, 0.f);
+                *reinterpret_cast<float4 *>(row + m) = z;
+                sum = fmaf(z.x, z.x, fmaf(z.y, z.y, fmaf(z.z, z.z, sum)));
+            }
+        }
+    } else {
+        // 128 outputs of a warp at a time, lane by lane: stores of whole sectors wherever they go
+        const int lane = threadIdx.x & 31;
+        __syncwarp();
+#pragma unroll 1
+        for (o -= 4 * lane; o < end; o += 4 * CF) {
+            if (o + 127 < first) continue;
+            const bool all = o >= first && o + 128 <= end;
+            float *p = row + o + lane;
+            float z[4], whole = 0.f;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                if (i + c < copy_from) continue;
-                float copies = 0.f;
-                for (int m = i + c; m < N - period; copies += 1.f) {
-                    m += period;
-                    row[m] = z[c];
+                const int i = o + 32 * c + lane;
+                z[c] = i >= first && i < end ? p[32 * c] : 0.f;
+            }
+            unsigned q = period;
+            if (all) {
+#pragma unroll 1
+                for (; q + 127 < (unsigned)(N - o); q += period, whole += 1.f) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) p[q + 32 * c] = z[c];
                 }
-                sum = fmaf(copies, z[c] * z[c], sum);
+            }
+            sum = fmaf(whole, fmaf(z[0], z[0], fmaf(z[1], z[1], fmaf(z[2], z[2], z[3] * z[3]))), sum);
+#pragma unroll 1
+            for (; q < (unsigned)(N - o); q += period) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int i = o + 32 * c + lane;
+                    if (i >= first && i < end && q < (unsigned)(N - i)) {
+                        p[q + 32 * c] = z[c];
+                        sum = fmaf(z[c], z[c], sum);
+                    }
+                }
             }
         }
     }
@@ -954,7 +1006,7 @@ convolve_kernel(const Plan *plans, const Unit *units, const int *n_units, int un
                     const float2 e = fftpair::unpack(e2);
                     float sum = e.x + e.y;
                     if (KIND == FUSED && noise && p.period > 0 && (b + 1) * ob > p.copy_from)
-                        sum += repeat_block(dst - (int64_t)b * ob, b * ob + o0, b * ob, (b + 1) * ob, p.copy_from, p.period, p.N);
+                        sum += repeat_block(dst - (int64_t)b * ob, b * ob + o0, b * ob, (b + 1) * ob, p.copy_from, p.period, p.N, sum);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
                     if ((t & 31) == 0) atomicAdd(&energy[2 * cur.utt + (noise ? 1 : 0)], (double)sum);
@@ -979,13 +1031,20 @@ static bool stored_route(const AugCtx *ctx) { return ctx->route == aug::ROUTE_ST
 static int convolve_fit(const AugCtx *ctx, const ConvInput &in) {
     return std::min(FUSED_MINB * ctx->sm_count - in.room, aug::PARK_SLOTS);
 }
-static int64_t most_units(const ConvInput &in, int B, int ob) { return 2 * (int64_t)B * ((in.max_len + ob - 1) / ob); }
+static int64_t most_units(int max_len, int B, int ob) { return 2 * (int64_t)B * (((int64_t)max_len + ob - 1) / ob); }
 // blocks of the fused kernel are shortest where a response fills min(rir_taps, 8192) taps
 static int shortest_block(const AugCtx *ctx) { return (F2 - std::min(ctx->cfg.rir_taps, BLK2) + 1) & ~3; }
 
 static PlanArgs plan_args(const AugCtx *ctx, const ConvInput &in) {
+    // Copies lengthen the units that make them, which does not pay before other units wait for a place: one utterance
+    // of 60 s over a stretch of 1 s 46 us computed, 89 copied (of 16001 samples 48 and 234), eight of 2 s 31 and 33.
+    // What counts is the largest batch that the context is for, so that an utterance's numbers do not depend on those
+    // it comes with, nor on the chunks of the host entry point (one of 20 s over 0.25 to 1 s in a context for hundreds:
+    // 40 us computed, 46 copied).  Blocks are up to twice as long as the shortest, hence two rounds.
+    const int repeats = most_units(ctx->cfg.max_samples, ctx->cfg.max_batch, shortest_block(ctx)) >
+                        2 * (int64_t)FUSED_MINB * ctx->sm_count;
     return {in.speech, in.stride, in.lengths, in.bank, in.bank_len, in.max_len, ctx->status,
-            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units), ctx->unit_cap, ctx->counters};
+            reinterpret_cast<Plan *>(ctx->plans), reinterpret_cast<Unit *>(ctx->units), ctx->unit_cap, ctx->counters, repeats};
 }
 
 template <Lengths LENGTHS>
@@ -1037,7 +1096,7 @@ static int launch_convolve(AugCtx *ctx, int grid) {
     return AUG_OK;
 }
 static int convolve_grid(const AugCtx *ctx, const ConvInput &in, int B, int ob) {
-    return (int)std::min<int64_t>(most_units(in, B, ob), convolve_fit(ctx, in));
+    return (int)std::min<int64_t>(most_units(in.max_len, B, ob), convolve_fit(ctx, in));
 }
 
 int launch_convolve_prepare(AugCtx *ctx, const ConvInput &in, const AugUttParams *table, int B, bool measured) {

@@ -144,3 +144,37 @@ def test_energy_of_noise_that_comes_back():
     # gain's and the wave's
     bound = (2 * 39 + 2 + 2) * 2.0 ** -24
     assert (got - 1.0).abs().max() <= bound, (got - 1.0).tolist()
+
+
+@pytest.mark.parametrize("copies", [1, 8])
+def test_short_stretches_take_no_longer_than_long_ones(copies):
+    """One and eight utterances of 60 s: noise that comes back sixty times is no more work than noise that does not."""
+    import torch
+    n, taps = 960000, 4001
+    stride = n
+    rng = np.random.default_rng(3)
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.float32)).cuda()
+    bank, speech = cu(rng.standard_normal(n) * 0.05), cu(rng.standard_normal((copies, stride)) * 0.05)
+    rir = cu(rng.standard_normal((copies, 2, taps)) * 0.01)
+    lengths = torch.full((copies,), n, dtype=torch.int32, device="cuda")
+    cfg = binding.AugConfig(fs=16000, win=400, hop=160, n_fft=512, n_mel=40, f_lo=0.0, f_hi=8000.0, rir_taps=taps,
+                            max_order=1, max_sources=2, frac_half_width=40, sound_speed=343.0, log_floor=1e-7,
+                            pad_value=0.0, compression=binding.COMPRESS_LOG, max_batch=copies, max_samples=stride,
+                            host_staging=0, image_lattice=0, max_bank_samples=0, vtlp_win=0, host_rows=0)
+    ctx, out = binding.AugContext(cfg), torch.empty((copies, stride), device="cuda")
+    took = {}
+    for m in (n, 16000, 16001):
+        tab = np.zeros(copies, dtype=synth.UTT_DTYPE)
+        tab["n_src"], tab["noise_len"][:, 0], tab["noise_weight"][:, 0] = 2, m, 1.0
+        table, times = binding.table_to_device(tab), []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(8):
+                ctx.aug_reverb_mix(speech, stride, lengths, bank, n, rir, table, copies, out)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        took[m] = min(times)
+    # (a quarter for what a loaded machine adds; it was twice to ten times as long)
+    assert max(took[16000], took[16001]) <= 1.25 * took[n], took
