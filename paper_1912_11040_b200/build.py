@@ -6,7 +6,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libaugb200.so")
 SOURCES = ["api.cu", "rir.cu", "conv.cu", "feat.cu", "peak.cu", "sample.cu", "post.cu", "resynth.cu"]
-HEADERS = ["common.cuh", "fft_pair.cuh", os.path.join("..", "..", "include", "aug_b200.h")]
+HEADERS = ["common.cuh", "fft_pair.cuh", "image_delay.cuh", os.path.join("..", "..", "include", "aug_b200.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared", "-cudart", "static"]
 

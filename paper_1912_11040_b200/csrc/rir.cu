@@ -52,6 +52,7 @@
 
 #include "common.cuh"
 #include "fft_pair.cuh"
+#include "image_delay.cuh"
 
 namespace {
 
@@ -242,10 +243,9 @@ rir_image_kernel(const AugUttParams *__restrict__ table, int S_max, int L, int h
             const int iy = ky + order, iz = kz + order;
             const double d2 = dsq[ix] + dsq[AX + iy] + dsq[2 * AX + iz];
             const float g = gain[ix] * gain[AX + iy] * gain[2 * AX + iz];
-            // d from the fp32 reciprocal square root and one Newton step in fp64 (relative error below 1e-13)
             const float r0 = rsqrtf((float)d2);
-            const double t = d2 * (double)r0, e = fma(-t, (double)r0, 1.0);
-            const double tau = fma(0.5 * t, e, t) * fs_over_c;
+            double e;
+            const double tau = image_distance(d2, r0, e) * fs_over_c;
             // its whole part (rounded down): adding 1.5 2^52 leaves the nearest integer in the low word
             const double m = (tau - 0.5) + 6755399441055744.0;
             int n0 = __double2loint(m);

@@ -3,8 +3,10 @@
 Kernels that may start while the one before them is still writing (chained launches) must not
 read its results through the non-coherent path: that path is for data which nobody writes while
 the kernel lives.  Words made of a float's bits are multiplied without a sign, as they exceed 32 bits."""
+import ctypes
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -61,3 +63,24 @@ def test_bits_of_floats_are_multiplied_without_a_sign():
     with np.errstate(over="ignore"):
         got = (np.uint32(16) * bits(hi) + bits(lo) - np.uint32(17 * 0x4B400000 % 2 ** 32)).view(np.int32)
     assert np.array_equal(got, np.rint(v.astype(np.float64)).astype(np.int32))
+
+
+def test_distance_of_an_image_is_right_to_its_last_bits(tmp_path):
+    """The header's arithmetic, compiled for the host, from seeds two units off either way (what the fp32 reciprocal
+    square root may be): two roundings and that of the reference."""
+    src = tmp_path / "distance.cpp"
+    src.write_text('#include "image_delay.cuh"\n'
+                   'extern "C" void distances(const double *d2, const float *r0, double *d, double *e, int n) {\n'
+                   '    for (int i = 0; i < n; ++i) d[i] = image_distance(d2[i], r0[i], e[i]);\n}\n')
+    so = str(tmp_path / "distance.so")
+    subprocess.run(["g++", "-O2", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, "-o", so, str(src)], check=True)
+    rng = np.random.default_rng(0)
+    d2 = np.repeat(np.exp(rng.uniform(np.log(1e-4), np.log(1e6), 20000)), 5)
+    r0 = (1 / np.sqrt(d2)).astype(np.float32)
+    r0 = (r0.view(np.int32) + np.tile(np.arange(-2, 3, dtype=np.int32), 20000)).view(np.float32)
+    d, e = np.empty_like(d2), np.empty_like(d2)
+    p = lambda a, t: a.ctypes.data_as(ctypes.POINTER(t))
+    ctypes.CDLL(so).distances(p(d2, ctypes.c_double), p(r0, ctypes.c_float), p(d, ctypes.c_double),
+                              p(e, ctypes.c_double), len(d2))
+    assert np.max(np.abs(d / np.sqrt(d2) - 1)) <= 3 * np.finfo(np.float64).eps
+    assert np.max(np.abs(r0 * (1 + e / 2) * np.sqrt(d2) - 1)) <= np.max(np.abs(e)) ** 2
