@@ -158,6 +158,16 @@ inline int launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t sme
 }
 #endif
 
+// Whole part of n / by without a division: by a multiplication with 2^64 / by, rounded up.
+struct Divisor {
+    int by;
+    unsigned long long m;
+    explicit Divisor(int d) : by(d), m(~0ull / (unsigned)d + 1) {}      // (0 for 1)
+#ifdef __CUDACC__
+    __device__ __forceinline__ int of(int n) const { return by == 1 ? n : (int)__umul64hi((unsigned long long)n, m); }
+#endif
+};
+
 // Where a kernel gets the noise gain from: worked out before (value), or from the two sums of the convolution.
 struct GainSource {
     const float *value;             // [B], or NULL

@@ -194,6 +194,7 @@ __device__ __forceinline__ void walk_bands(const ulonglong2 *w4, const int *mst,
 // 264 and 1302 us, four 249 and 1179, six 249 and 1190.
 constexpr int WARPS = FEAT_THREADS / 32;
 constexpr int TAIL_ROUNDS = 2;         // tiles a CTA's place on the device that are not done in runs
+constexpr int TAIL_SAMPLES = 8192;     // samples of a large tile, see launch_frames
 
 template <int K>
 struct Plan;
@@ -350,7 +351,7 @@ __device__ __forceinline__ void power_rows(fftpair::C2 *v, fftpair::u64 *p, cons
 // many both slower.
 struct RunMap {
     int utts, long_utts;           // of which the first ones (in the order of work) are done in runs
-    int runs, tiles;               // per utterance: runs, tiles
+    Divisor runs, tiles;           // per utterance: runs, tiles
 };
 
 template <int K, int MODE, int TILES>
@@ -367,15 +368,20 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
     int *mst = reinterpret_cast<int *>(sm + lay.mst), *cut = reinterpret_cast<int *>(sm + lay.cut);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int run = blockIdx.x, nth = run / map.runs, run_tiles = TILES;
-    if (nth < map.long_utts) {
-        run -= nth * map.runs;
-    } else {
-        run -= map.long_utts * map.runs;
-        nth = run / map.tiles;
-        run -= nth * map.tiles;
-        nth += map.long_utts;
-        run_tiles = 1;
+    // (single tiles throughout: two grid dimensions.  With the same arithmetic for all, divisions in it, the power
+    // spectra of one utterance of 3 s took 8.2 us instead of 7.2)
+    int run = blockIdx.x, nth = blockIdx.y, run_tiles = TILES;
+    if (TILES > 1) {
+        nth = map.runs.of(run);
+        if (nth < map.long_utts) {
+            run -= nth * map.runs.by;
+        } else {
+            run -= map.long_utts * map.runs.by;
+            nth = map.tiles.of(run);
+            run -= nth * map.tiles.by;
+            nth += map.long_utts;
+            run_tiles = 1;
+        }
     }
     const int utt = map.utts - 1 - nth, run0 = run * (FT * run_tiles);
     for (int n = tid; n < K; n += FEAT_THREADS)
@@ -744,9 +750,18 @@ int launch_frames(AugCtx *ctx, const float *a, const float *b, int64_t stride, c
     // to give every multiprocessor something to do.
     const int n_tiles = (T_max + FT - 1) / FT;
     const bool runs = (int64_t)n_tiles * B >= 2 * (int64_t)ctx->sm_count * RUN_TILES;
-    RunMap map = {B, 0, (n_tiles + RUN_TILES - 1) / RUN_TILES, n_tiles};
+    const int n_runs = (n_tiles + RUN_TILES - 1) / RUN_TILES;
+    RunMap map = {B, B, Divisor(n_runs), Divisor(n_tiles)};
     if (runs) map.long_utts = std::max(0, B - (TAIL_ROUNDS * 2 * ctx->sm_count + n_tiles - 1) / n_tiles);
-    const dim3 grid(map.long_utts * map.runs + (B - map.long_utts) * n_tiles);
+    if (MODE == 0 && lay.ahead && lay.chunk_cap > TAIL_SAMPLES) {
+        // Nothing copies the samples of single tiles ahead, and large ones of a power spectrum take twice as long for it: only
+        // where that makes up for the last round of runs (100 utterances of 10 s: window and hop 320 51 us in runs
+        // alone, 57 with single tiles at the end; window 512, hop 441 52 and 43).
+        const int64_t places = 2 * (int64_t)ctx->sm_count, in_runs = (int64_t)map.long_utts * n_tiles;
+        const int64_t alone = ((int64_t)n_runs * B + places - 1) / places * std::min(RUN_TILES, n_tiles);
+        if ((in_runs + 2 * ((int64_t)B * n_tiles - in_runs)) / places + 2 > alone) map.long_utts = B;
+    }
+    const dim3 grid = runs ? dim3(map.long_utts * n_runs + (B - map.long_utts) * n_tiles) : dim3(n_tiles, B);
     auto kern = runs ? frames_kernel<K, MODE, RUN_TILES> : frames_kernel<K, MODE, 1>;
     if ((runs ? smem_opt_in<frames_kernel<K, MODE, RUN_TILES>>(ctx->device)
               : smem_opt_in<frames_kernel<K, MODE, 1>>(ctx->device)) != AUG_OK)
