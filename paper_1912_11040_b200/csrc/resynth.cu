@@ -78,10 +78,12 @@ vtlp_positions_kernel(const AugUttParams *__restrict__ table, int *__restrict__ 
 }
 
 // Which hops a CTA owns: those of runs of several rounds or, in the utterances that come last, of single ones: the device is
-// left half empty for a shorter time at the end (64 utterances of 2-20 s, warp and its tables 243 us, so 230).
+// left half empty for a shorter time at the end (64 utterances of 2-20 s, warp and its tables 243 us, so 230).  Single
+// rounds are a sixth more work, so no more utterances than two rounds for each place (4 of 100 s, window 400: 203 us in
+// runs, 208 with one of them in single rounds).
 struct HopMap {
     int long_utts;                 // utterances done in runs
-    int runs, singles;             // CTAs of an utterance in runs and in single rounds
+    Divisor runs, singles;         // CTAs of an utterance in runs and in single rounds
 };
 
 template <int ROUNDS>
@@ -97,13 +99,13 @@ vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int 
     float2 *pos = reinterpret_cast<float2 *>(sm + lay.pos);      // [SPEC] lower source bin (int), fraction
     float *carry = sm + lay.carry;                   // [3 hop] what earlier frames add to the next hops
 
-    int run = blockIdx.x, utt = run / map.runs, rounds = ROUNDS;
+    int run = blockIdx.x, utt = map.runs.of(run), rounds = ROUNDS;
     if (utt < map.long_utts) {
-        run -= utt * map.runs;
+        run -= utt * map.runs.by;
     } else {
-        run -= map.long_utts * map.runs;
-        utt = run / map.singles;
-        run -= utt * map.singles;
+        run -= map.long_utts * map.runs.by;
+        utt = map.singles.of(run);
+        run -= utt * map.singles.by;
         utt += map.long_utts;
         rounds = 1;
     }
@@ -373,14 +375,14 @@ int launch_vtlp_resynth(AugCtx *ctx, const float *speech, int64_t stride, const 
     // Runs of three rounds (45 hops for 48 frames), single rounds (13 for 16) where the batch is so
     // small that it would not fill the device otherwise.
     constexpr int RUN = 3;
-    HopMap map = {0, (T_cap + RUN * NF - 4) / (RUN * NF - 3), (T_cap + NF - 4) / (NF - 3)};
-    const bool runs = (int64_t)map.runs * B >= 4 * (int64_t)ctx->sm_count;
-    if (runs) map.long_utts = std::max(0, B - (4 * ctx->sm_count + map.singles - 1) / map.singles);
+    HopMap map = {0, Divisor((T_cap + RUN * NF - 4) / (RUN * NF - 3)), Divisor((T_cap + NF - 4) / (NF - 3))};
+    const bool runs = (int64_t)map.runs.by * B >= 4 * (int64_t)ctx->sm_count;
+    if (runs) map.long_utts = std::max(0, B - 4 * ctx->sm_count / map.singles.by);
     auto kern = runs ? vtlp_resynth_kernel<RUN> : vtlp_resynth_kernel<1>;
     if ((runs ? smem_opt_in<vtlp_resynth_kernel<RUN>>(ctx->device) : smem_opt_in<vtlp_resynth_kernel<1>>(ctx->device)) !=
         AUG_OK)
         return AUG_ECUDA;
-    const dim3 grid(map.long_utts * map.runs + (B - map.long_utts) * map.singles);
+    const dim3 grid(map.long_utts * map.runs.by + (B - map.long_utts) * map.singles.by);
     kern<<<grid, RS_THREADS, smem, ctx->stream>>>(speech, stride, lengths, k0_tab, fr_tab, win, ctx->tw, out, out_stride,
                                                   max_len, lay, map);
     AUG_CUDA_OK(cudaGetLastError());

@@ -64,3 +64,14 @@ def test_tiles_of_the_power_spectra(win, hop, B, seconds, grid, tmp_path):
     x, lengths = torch.zeros((B, n), device="cuda"), torch.full((B,), n, dtype=torch.int32, device="cuda")
     power, counts = torch.empty((B, T, 257), device="cuda"), torch.empty(B, dtype=torch.int32, device="cuda")
     assert grids_of("frames_kernel", lambda: ctx.feat_stft_power(x, n, lengths, B, power, T, counts), tmp_path) == [grid]
+
+
+def test_few_long_utterances_are_warped_in_runs(tmp_path):
+    import torch
+    B, n = 4, 1600000
+    ctx, table = context(B, n, vtlp_win=400)
+    x, lengths = torch.zeros((B, n), device="cuda"), torch.full((B,), n, dtype=torch.int32, device="cuda")
+    out, rows = torch.empty_like(x), binding.table_to_device(np.tile(table[:1], B))
+    got = grids_of("vtlp_resynth_kernel", lambda: ctx.aug_vtlp_resynth(x, n, lengths, rows, B, out, n), tmp_path)
+    hops = (n + 300 + 99) // 100
+    assert got == [(B * ((hops + 44) // 45), 1, 1)]
