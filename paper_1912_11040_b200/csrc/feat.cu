@@ -410,7 +410,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
         ev = gain.energy[2 * utt + 1];
     }
     float g = 0.f, *gain_s = sm + lay.cut + 63;
-    const bool noisy = MODE == 1 && snr_noisy(es, ev, n_src);
+    bool noisy = MODE == 1 && snr_noisy(es, ev, n_src);      // v is copied
     // The mixed waveform, where it is wanted: a tile writes the hops that its frames start, the CTA with
     // the last frame (the first one if there is none) what lies behind them.
     float *wrow = MODE == 1 && wave != nullptr ? wave + (int64_t)utt * wave_stride : nullptr;
@@ -521,6 +521,7 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
         __syncthreads();
         cut_bands<RUNS>(cut, mst, M, tid);
         g = *gain_s;
+        noisy = noisy && g != 0.f;            // (0 beside an infinite sum: v may hold an infinity, is not read)
     }
     fftpair::u64 *xb = reinterpret_cast<fftpair::u64 *>(sm + warp * SPAN);
 

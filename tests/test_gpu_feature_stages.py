@@ -183,6 +183,32 @@ def test_noise_that_is_not_finite_shows_in_the_waveform_alone(n_fft, hop):
         assert (F[0] - F_ref[0]).abs().max() <= 2 * LOGMEL_ABS_TOL
 
 
+@pytest.mark.parametrize("n_fft,hop", [(512, 160), (512, 125), (1024, 200)])
+def test_noise_whose_energy_overflows_shows_in_the_waveform_alone(n_fft, hop):
+    """Noise so loud that the sum of its squares is infinite makes the gain 0, and the features are those of y_s, also
+    where single samples of v overflow and the others do not: a click at levels up to the largest float."""
+    import torch
+    from helpers import LOGMEL_ABS_TOL, Device
+    w = synth.make_workload(2, seed=5, batch=2, dur_scale=0.2)
+    w.cfg.update(n_fft=n_fft, win=400, hop=hop)
+    w.table["n_src"][:] = [2, 1]
+    w.table["noise_weight"][0, 0] = 50.0
+    clean = synth.Workload(name=w.name, cfg=w.cfg, lengths=w.lengths, speech=w.speech, bank=w.bank, table=w.table.copy())
+    clean.table["n_src"][:] = 1
+    F_ref, _, _ = Device(clean).pipeline()
+    o, m = int(w.table["noise_offset"][0, 0]), int(w.table["noise_len"][0, 0])
+    lone = 0
+    for level in 1e36 * 1.2 ** np.arange(30):
+        w.bank = np.zeros_like(w.bank)
+        w.bank[o + m // 2] = level
+        F, _, wave = Device(w).pipeline()
+        wrong = int((~torch.isfinite(wave[0, : int(w.lengths[0])])).sum())
+        lone += 0 < wrong < 1000
+        # each side is within LOGMEL_ABS_TOL of the exact features
+        assert (F[0] - F_ref[0]).abs().max() <= 2 * LOGMEL_ABS_TOL, (level, wrong)
+    assert lone > 0
+
+
 # tiles that begin at any sample of a 16-byte group: rows of whole groups are copied in one tile ahead, other
 # rows sample by sample; single tiles and runs of them, last tiles of any number of frames
 @pytest.mark.parametrize("n_fft,win,hop", [(512, 400, 125), (512, 401, 110), (512, 3, 1), (512, 77, 131),
