@@ -109,9 +109,9 @@ struct Layout {
     int n_part, route, n_bins, t_cap, nblk_cap;
     int64_t ws_stride, unit_cap;
     int64_t off_xspec, off_park, off_park_flags, off_plans, off_units;
-    int64_t off_tw, off_tap_tab, off_rir, off_hspec, off_ys, off_vv, off_energy, off_arrived, off_counters, off_leff, off_gain, off_melw, off_melstart,
-        off_status, off_warped, off_vtlp_tab, off_st_speech, off_st_bank, off_st_table, off_st_lengths,
-        off_st_feats, off_st_counts, total;
+    int64_t off_tw, off_tap_tab, off_rir, off_hspec, off_ys, off_vv, off_energy, off_arrived, off_counters, off_leff,
+        off_gain, off_melw, off_melstart, off_status, off_warped, off_vtlp_tab, off_st_speech, off_st_bank, off_st_table,
+        off_st_lengths, off_st_feats, off_st_counts, total;
 };
 
 Layout make_layout(const AugConfig &c) {

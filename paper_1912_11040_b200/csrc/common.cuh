@@ -136,9 +136,9 @@ inline int smem_opt_in(int device) {
 // wait take room and slowed long kernels down, 1083 -> 1189 us on 128 x 8 s with 24000 taps); it calls
 // chain_wait() before it touches anything an earlier kernel writes or reads.  As that one may be writing
 // while this one lives, what it writes is not read through the non-coherent path (`const __restrict__`
-// parameters, __ldg), which is for data that nobody writes meanwhile.  Every CTA of a chained kernel calls chain_wait() on every path, so
-// that the end of a kernel implies the end of all before it.  (Both are no-ops in a kernel that
-// was launched the ordinary way.)
+// parameters, __ldg), which is for data that nobody writes meanwhile.  Every CTA of a chained kernel calls
+// chain_wait() on every path, so that the end of a kernel implies the end of all before it.  (Both are no-ops in a
+// kernel that was launched the ordinary way.)
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

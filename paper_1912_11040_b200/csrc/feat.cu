@@ -35,8 +35,8 @@ struct MelEdges {
 // frequency (fp64: a bin that barely enters a band must not lose its weight to
 // rounding), then the first bin of every interval.
 __global__ void __launch_bounds__(256)
-mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double e0, double delta, aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped,
-                  int *counters, double *energy) {
+mel_tables_kernel(const AugUttParams *__restrict__ table, int K, int M, double fs, double e0, double delta,
+                  aug::MelBin *__restrict__ melw, int *__restrict__ melstart, int unwarped, int *counters, double *energy) {
     __shared__ int seg_s[513];
     chain_next();
     // first kernel of aug_pipeline: the convolution's sums and counters start from zero
@@ -354,6 +354,7 @@ struct RunMap {
     Divisor runs, tiles;           // per utterance: runs, tiles
 };
 
+// TILES: tiles of a run; 1 where there are none, so that no loop and no arithmetic of runs is left.
 template <int K, int MODE, int TILES>
 __global__ void __launch_bounds__(FEAT_THREADS, 2)
 frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const GainSource gain,
@@ -605,7 +606,8 @@ frames_kernel(const float *in_a, const float *in_b, int64_t in_stride, const Gai
             const int f = QF * w + q;                // and f + QF / 2
             if (f < nf) {
                 walk_bands(reinterpret_cast<const ulonglong2 *>(mw), mst, cut[run], cut[run + 1],
-                           PairRow{reinterpret_cast<const u64 *>(sm + w * SPAN) + q * NBP}, chunk + f * lay.fs_ld, (QF / 2) * lay.fs_ld);
+                           PairRow{reinterpret_cast<const u64 *>(sm + w * SPAN) + q * NBP}, chunk + f * lay.fs_ld,
+                           (QF / 2) * lay.fs_ld);
             }
         }
         __syncthreads();                      // band energies in place
@@ -916,8 +918,8 @@ extern "C" int feat_vtlp_logmel_noalloc(const AugConfig *cfg, const float *power
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int nbp = cfg->n_fft / 2 + 1;
     const MelEdges e(cfg->f_lo, cfg->f_hi, cfg->n_mel);
-    mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs, e.first, e.step, melw, melstart, 0, nullptr,
-                                         nullptr);
+    mel_tables_kernel<<<B, 256, 0, st>>>(table_dev, cfg->n_fft, cfg->n_mel, (double)cfg->fs, e.first, e.step, melw,
+                                         melstart, 0, nullptr, nullptr);
     AUG_CUDA_OK(cudaGetLastError());
     int dev = -1;
     AUG_CUDA_OK(cudaGetDevice(&dev));

@@ -86,6 +86,7 @@ struct HopMap {
     Divisor runs, singles;         // CTAs of an utterance in runs and in single rounds
 };
 
+// ROUNDS: rounds of a run; 1 where there are none (and the loop of rounds goes).
 template <int ROUNDS>
 __global__ void __launch_bounds__(RS_THREADS, 2)
 vtlp_resynth_kernel(const float *__restrict__ speech, int64_t stride, const int *__restrict__ lengths,
