@@ -517,8 +517,10 @@ plan_kernel(const __grid_constant__ PlanArgs args, const AugUttParams *__restric
     const int utt = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     PlanInput in;
     if (utt < B) in = plan_input(args, table[utt], utt, S_max, lane);
-    chain_next();
     chain_wait();
+    // (not before: the next kernel's CTAs would wait in places that the responses' transforms still need.  aug_reverb_mix, 8
+    // utterances of 5 s, three noises, responses of 24000 taps 73 us, so 62; of 12000 67 and 60)
+    chain_next();
     if (utt < B)
         plan_utterance(args, in, utt, longest(leff, in, utt, S_max, lane), stored_only || !takes_fused_route(*leff_all), lane);
 }

@@ -49,6 +49,15 @@ def test_explicit_non_coherent_loads_are_of_constant_data():
         assert "tw[" in m.group(1), m.group(0)
 
 
+def test_work_is_planned_before_the_next_kernel_is_let_in():
+    """plan_kernel is short and follows the transforms of the responses: it lets the convolution's CTAs in when these
+    have ended, not while the waiting ones would take their places."""
+    s = source("conv.cu")
+    body = s[s.index("plan_kernel(const __grid_constant__"):]
+    body = body[: body.index("\n}")]
+    assert body.index("chain_wait();") < body.index("chain_next();")
+
+
 def test_bits_of_floats_are_multiplied_without_a_sign():
     """Rounding of loud taps: 16 times the bits of about 1.5 2^23 wraps, which only unsigned words may."""
     assert not re.search(r"\*\s*__float_as_int|__float_as_int\([^)]*\)\s*\*", source("rir.cu"))
