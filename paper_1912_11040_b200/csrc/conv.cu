@@ -388,11 +388,12 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
 // per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
 // (two thirds of them without work) and to each one's chain of loads before its first sample.
 //
-// Sums of several noise sources are the heavy units (three transforms and more against two): they are
-// listed from the front, the others from the back, so that the heavy ones are drawn first and none of them is the last
-// that the device waits for (in the order in which they are planned, and so: 64 utterances of 2-16 s, one or two noises,
-// 167 and 153 us; 96 of 2-20 s with up to two 302 and 287; 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and
-// 1376, whole calls each).
+// Sums of several noise sources are the heavy units (three transforms and more against two), and so are blocks of
+// noise that may have copies to write (below): they are listed from the front, the others from the back, so that the
+// heavy ones are drawn first and none of them is the last that the device waits for (in the order in which they are
+// planned, and so: 64 utterances of 2-16 s, one or two noises, 167 and 153 us; 96 of 2-20 s with up to two 302 and 287;
+// 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and 1376, whole calls each; blocks with copies among them: 256 of
+// 2-20 s with one or two noises 707 and 703, 64 of 10 s with one and responses of 1000 taps 154 and 149).
 //
 // A stretch of noise that is shorter than the utterance repeats, and so does its reverberation as soon as the
 // response has run in: v[n + P] = v[n], n >= taps - 1.  Where there is one noise source, only the blocks
@@ -486,7 +487,7 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const PlanInpu
     if (lane == 0) {
         if (n > 0) {
             int *list = a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED);
-            const bool heavy = n_noise > 1;
+            const bool heavy = n_noise > 1 || period > 0;
             if (heavy) at_heavy = atomicAdd(list, n_v);
             at = atomicAdd(list + 1, heavy ? n : n + n_v);
         }
