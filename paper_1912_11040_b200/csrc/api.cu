@@ -137,7 +137,7 @@ Layout make_layout(const AugConfig &c) {
     // its list of work: two outputs of every block, blocks as short as 8192 taps make them
     l.off_plans = take((int64_t)aug::PLAN_BYTES * B);
     l.unit_cap = 2 * B * ((c.max_samples + aug::CONV_TAPS - 1) / aug::CONV_TAPS);
-    l.off_units = take(2 * sizeof(int) * l.unit_cap);
+    l.off_units = take(2 * 2 * sizeof(int) * l.unit_cap);
     l.off_ys = take(sizeof(float) * B * l.ws_stride);
     l.off_vv = take(sizeof(float) * B * l.ws_stride);
     l.off_energy = take((sizeof(double) * 2 + sizeof(unsigned long long)) * B + sizeof(int) * aug::N_COUNTERS);

@@ -12,9 +12,9 @@ namespace aug {
 constexpr int CONV_TAPS = 8192;         // taps of a partition: half a transform of the convolution
 constexpr int CONV_BINS = 8192;         // complex numbers of a stored spectrum
 // Counters of the convolution: the batch's largest response length (long-response contexts), units of
-// work listed for the two routes (heavy and other ones), units drawn from the lists.
-enum Counter { LEFF_ALL, LIST_FUSED, LIST_STORED = LIST_FUSED + 2, DRAWN_FUSED = LIST_STORED + 2, DRAWN_SPECTRA, DRAWN_STORED,
-               N_COUNTERS };
+// work listed for the two routes (sums, blocks with copies, other ones), units drawn from the lists.
+enum Counter { LEFF_ALL, LIST_FUSED, LIST_STORED = LIST_FUSED + 3, DRAWN_FUSED = LIST_STORED + 3, DRAWN_SPECTRA,
+               DRAWN_STORED, N_COUNTERS };
 constexpr int PARK_SLOTS = 320;     // parking slots of the fused convolution = most CTAs it runs with
 constexpr int PLAN_BYTES = 96;      // per utterance, see conv.cu
 constexpr int MAX_TAPS = 24576;
@@ -69,7 +69,7 @@ struct AugCtx {
     float4 *park;          // [PARK_SLOTS][4096] products of noise sources waiting for the last one; NULL if unused
     int *park_flags;       // [PARK_SLOTS] 1 = slot held: that CTA sums in the time domain
     void *plans;           // [max_batch][PLAN_BYTES] what the fused convolution has to know of an utterance
-    void *units;           // [unit_cap] its list of work
+    void *units;           // [2 unit_cap] its list of work
     int unit_cap;
     float *warped;         // [max_batch][ws_stride] speech after the waveform warp; NULL unless cfg.vtlp_win
     void *vtlp_tab;        // [max_batch][513] lower source bin (int), then [max_batch][513] fraction (float)

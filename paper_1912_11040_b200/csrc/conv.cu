@@ -388,12 +388,13 @@ __device__ __forceinline__ void store_bins(float4 *p, const Bins &z) {
 // per possible block instead, 55 of 527 us (256 utterances of 2-20 s) went to launching CTAs
 // (two thirds of them without work) and to each one's chain of loads before its first sample.
 //
-// Sums of several noise sources are the heavy units (three transforms and more against two), and so are blocks of
-// noise that may have copies to write (below): they are listed from the front, the others from the back, so that the
-// heavy ones are drawn first and none of them is the last that the device waits for (in the order in which they are
-// planned, and so: 64 utterances of 2-16 s, one or two noises, 167 and 153 us; 96 of 2-20 s with up to two 302 and 287;
-// 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and 1376, whole calls each; blocks with copies among them: 256 of
-// 2-20 s with one or two noises 707 and 703, 64 of 10 s with one and responses of 1000 taps 154 and 149).
+// Sums of several noise sources are the heavy units (three transforms and more against two), and blocks of noise that may
+// have copies to write (below) come after them.  There are three lists, drawn from in this order: sums from the front,
+// blocks with copies behind the others' room, the others from the back, so that no long unit is the last that the
+// device waits for (in the order in which they are planned, and sums first: 64 utterances of 2-16 s, one or two noises,
+// 167 and 153 us; 96 of 2-20 s with up to two 302 and 287; 256 of 2-20 s 720 and 706; 64 of 60 s with two 1409 and 1376,
+// whole calls each.  Blocks with copies among the others, among the sums and between them: 64 of 2-16 s with recorded
+// responses 150.8, 152.8 and 149.2; 96 of 2-20 s 272.6, 269.8 and 268.6; 4096 of 1-6 s 3276, 3273 and 3256).
 //
 // A stretch of noise that is shorter than the utterance repeats, and so does its reverberation as soon as the
 // response has run in: v[n + P] = v[n], n >= taps - 1.  Where there is one noise source, only the blocks
@@ -483,13 +484,13 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const PlanInpu
         p->nlen[at] = in.nlen;
         p->src[at] = lane;
     }
-    int at = 0, at_heavy = -1;
+    int at = 0, at_v = 0;
+    const bool heavy = n_noise > 1, copies = period > 0;
     if (lane == 0) {
         if (n > 0) {
             int *list = a.counters + (stored ? aug::LIST_STORED : aug::LIST_FUSED);
-            const bool heavy = n_noise > 1 || period > 0;
-            if (heavy) at_heavy = atomicAdd(list, n_v);
-            at = atomicAdd(list + 1, heavy ? n : n + n_v);
+            if (heavy || copies) at_v = atomicAdd(list + (heavy ? 0 : 1), n_v);
+            at = atomicAdd(list + 2, heavy || copies ? n : n + n_v);
         }
         p->n_src = in.n_src;
         p->n_noise = n_noise;
@@ -500,11 +501,11 @@ __device__ __forceinline__ void plan_utterance(const PlanArgs &a, const PlanInpu
         p->copy_from = n_v * ob - period;
     }
     at = __shfl_sync(0xffffffffu, at, 0);
-    at_heavy = __shfl_sync(0xffffffffu, at_heavy, 0);
+    at_v = __shfl_sync(0xffffffffu, at_v, 0);
     const int last = a.unit_cap - 1;
     for (int i = lane; i < n; i += 32) {
         a.units[last - at - i] = Unit{utt, 2 * i};
-        if (i < n_v) a.units[at_heavy >= 0 ? at_heavy + i : last - at - n - i] = Unit{utt, 2 * i + 1};
+        if (i < n_v) a.units[heavy ? at_v + i : copies ? a.unit_cap + at_v + i : last - at - n - i] = Unit{utt, 2 * i + 1};
     }
 }
 
@@ -775,28 +776,31 @@ convolve_kernel(const Plan *plans, const Unit *units, const int *n_units, int un
     // has a barrier behind the one before.
     __shared__ Plan plan_s[3];
     __shared__ Unit unit_s[3];
-    __shared__ int2 list_s;                    // heavy units, all units
+    __shared__ int3 list_s;                    // sums, those and blocks with copies, all units
     const int t = threadIdx.x, G = gridDim.x;
     fftpair::fill_tables(sh, t, tw);
     chain_wait();
-    // (a CTA's first unit, which mostly is one of two, is read beside the counts)
+    // (a CTA's first unit, which mostly is one of three, is read beside the counts)
     // SPECTRA goes through the list backwards: the spectra that it writes last are still in L2 when STORED starts
     // (128 x 8 s, four sources: 250 -> 246 us).
-    const Unit front = units[blockIdx.x], back = units[unit_cap - 1 - blockIdx.x];
-    const int heavy = n_units[0], count = heavy + n_units[1];
+    const Unit front = units[blockIdx.x], middle = units[unit_cap + blockIdx.x], back = units[unit_cap - 1 - blockIdx.x];
+    const int heavy = n_units[0], early = heavy + n_units[1], count = early + n_units[2];
     if (blockIdx.x >= count) return;
-    auto unit_at = [&](int i, int2 list) {
-        if (KIND == SPECTRA) i = list.y - 1 - i;
-        return units[i < list.x ? i : unit_cap - 1 - (i - list.x)];
+    auto unit_at = [&](int i, int3 n) {
+        if (KIND == SPECTRA) i = n.z - 1 - i;
+        return units[i < n.x ? i : i < n.y ? unit_cap + (i - n.x) : unit_cap - 1 - (i - n.y)];
     };
-    const Unit first = KIND != SPECTRA && blockIdx.x < heavy ? front
-                       : KIND != SPECTRA && heavy == 0       ? back
-                                                             : unit_at(blockIdx.x, make_int2(heavy, count));
+    const int3 list = make_int3(heavy, early, count);
+    const Unit first = KIND == SPECTRA                          ? unit_at(blockIdx.x, list)
+                       : blockIdx.x < heavy                     ? front
+                       : heavy == 0 && blockIdx.x < early       ? middle
+                       : early == 0                             ? back
+                                                                : unit_at(blockIdx.x, list);
     if (t == 32) {
         const int second = blockIdx.x + G;
-        list_s = make_int2(heavy, count);
+        list_s = list;
         unit_s[0] = first;
-        unit_s[1] = second < count ? unit_at(second, make_int2(heavy, count)) : Unit{-1, 0};
+        unit_s[1] = second < count ? unit_at(second, list) : Unit{-1, 0};
     }
     if (t < (int)(sizeof(Plan) / 4))
         reinterpret_cast<int *>(&plan_s[0])[t] = reinterpret_cast<const int *>(plans + first.utt)[t];
@@ -816,7 +820,7 @@ convolve_kernel(const Plan *plans, const Unit *units, const int *n_units, int un
         int ticket = 0;
         if (t == 0) ticket = 2 * G + atomicAdd(drawn, 1);
         auto draw = [&]() {                    // (published by the barrier that follows)
-            if (t == 0) unit_s[k2] = ticket < list_s.y ? unit_at(ticket, list_s) : Unit{-1, 0};
+            if (t == 0) unit_s[k2] = ticket < list_s.z ? unit_at(ticket, list_s) : Unit{-1, 0};
             copies_done();
         };
         const bool noise = cur.block2 & 1;
@@ -1152,8 +1156,8 @@ int launch_mix(AugCtx *ctx, const int *lengths, const AugUttParams *table, int B
     if (max_len <= 0) return AUG_OK;
     dim3 grid((max_len + MIX_GROUPS * 1024 - 1) / (MIX_GROUPS * 1024), B);
     const GainSource gain = {ready ? ctx->gain : nullptr, ctx->energy, table};
-    if (launch_chained(ready ? mix_kernel<true> : mix_kernel<false>, grid, 256, 0, ctx->stream, ctx->ys, ctx->vv, ctx->ws_stride, gain, lengths,
-                       wave_out, out_stride, max_len) != AUG_OK)
+    if (launch_chained(ready ? mix_kernel<true> : mix_kernel<false>, grid, 256, 0, ctx->stream, ctx->ys, ctx->vv,
+                       ctx->ws_stride, gain, lengths, wave_out, out_stride, max_len) != AUG_OK)
         return AUG_ECUDA;
     ctx->launches++;
     return AUG_OK;
