@@ -38,11 +38,11 @@ FP32_LANES = 128          # fp32 lanes of one multiprocessor
 # from: the hashes guard that.
 NCU_TRAFFIC = {
     "bytes_per_audio_s": {
-        2: {"convolve": 255.9e6 / 1039.18, "features": 152.8e6 / 1039.18}},
+        2: {"convolve": 246.6e6 / 1039.18, "features": 150.2e6 / 1039.18}},
     "captured_on": {2: "96 utterances"},
     # kernel -> (its source files, sha256[:16] of them when the counters were taken)
-    "sources": {"convolve": (("conv.cu", "fft_pair.cuh"), "759948530f294a05"),
-                "features": (("feat.cu", "fft_pair.cuh"), "0d3193903d631b3c")}}
+    "sources": {"convolve": (("conv.cu", "fft_pair.cuh"), "aaac5060c92f9810"),
+                "features": (("feat.cu", "fft_pair.cuh"), "5c34b2d42d327638")}}
 
 
 def kernel_sources_sha(files):
@@ -71,8 +71,9 @@ def conv_work(w):
     (cut to a multiple of 4); longer ones in 4096-tap partitions of an 8192-point transform
     with 4096 outputs per block.  (The kernels do less than this when the responses end before
     their buffer does: blocks get longer, zero partitions are skipped and a long-response
-    context may take the one-partition route.  The nominal count stays that of the stated
-    configuration.)  Bytes: inputs read once, y_s and v written once, response spectra once."""
+    context may take the one-partition route; blocks of a single noise that repeats are copied.
+    The nominal count stays that of the stated configuration.)  Bytes: inputs read once, y_s and v
+    written once, response spectra once."""
     taps = int(w.cfg["rir_taps"])
     if taps <= 8192:
         F, P = 16384, 1
